@@ -18,10 +18,10 @@
 //     offsets of one image row (a multiple of the swizzle period), so the input is fetched three
 //     times instead of nine.
 //   * Small filter banks stay resident in shared memory for the whole launch.
-// Warp roles: warp 0 = first TMA producer (one lane), warp 1 = TMEM owner + first MMA issuer (one lane),
-// warps 2..9 = epilogue (two per TMEM lane quarter, splitting the columns), warp 10 = second MMA issuer (one lane;
-// the two issuers take alternate units), warp 11 = second TMA producer (one lane; the two producers take alternate
-// stages).  Every mbarrier wait is bounded.
+// Warp roles: warp 0 = first TMA producer, warp 1 = TMEM owner + first MMA issuer, warps 2..9 = epilogue (two per TMEM
+// lane quarter, splitting the columns), warp 10 = second MMA issuer (the two issuers take alternate units), warp 11 = second
+// TMA producer (the two producers take alternate stages).  Producer and issuer warps run their loops with all lanes and issue
+// from one elected lane.  Every mbarrier wait is bounded.
 #include "common.h"
 #include "ptx.cuh"
 
@@ -339,16 +339,16 @@ __device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tme
                 }
             } else {
 #pragma unroll
-            for (int ck = 0; ck < NCH; ++ck) {
-                if (n_it > 0 && ck < n_chunks) {
-                    tmem_ld16(t_row + (uint32_t)(ck * 16), r[ck]);
-                } else {
+                for (int ck = 0; ck < NCH; ++ck) {
+                    if (n_it > 0 && ck < n_chunks) {
+                        tmem_ld16(t_row + (uint32_t)(ck * 16), r[ck]);
+                    } else {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) r[ck][i] = 0u;
+                        for (int i = 0; i < 16; ++i) r[ck][i] = 0u;
+                    }
                 }
-            }
-            if (n_it > 0) tmem_ld_wait();
-            release();
+                if (n_it > 0) tmem_ld_wait();
+                release();
             }
             if (flush_pending) flush_stats();   // still the previous group's sums and channel tile
             cur_group = next_group;
@@ -502,7 +502,7 @@ __device__ __forceinline__ void mma_issuer(const ConvKParams& p, const UnitWalk&
     const int units_per_par = p.n_par > 1 ? p.total_units / p.n_par : 1;
     const int n_it_fixed = unit_iters(p, 0);
     bool ok = true;
-    if (p.resident && !mbar_wait_bounded(w_bar, 0u, p.spin_limit, abort_flag)) {
+    if (p.resident && !mbar_wait_warp(w_bar, 0u, p.spin_limit, abort_flag)) {
         atomicOr(p.status, B2C_DEV_TIMEOUT);
         ok = false;
     }
@@ -534,14 +534,14 @@ __device__ __forceinline__ void mma_issuer(const ConvKParams& p, const UnitWalk&
             // seeing the stamp pass i makes the parity wait unambiguous.
             if (p.issuers > 1) {
                 uint32_t polls = 0;
-                while (ld_volatile_shared(&slot_stage[s]) <= i_stage) {
-                    if (++polls > p.spin_limit || *(volatile uint32_t*)abort_flag != 0u) {
+                while (__any_sync(0xffffffffu, ld_volatile_shared(&slot_stage[s]) <= i_stage)) {
+                    if (++polls > p.spin_limit || __any_sync(0xffffffffu, *(volatile uint32_t*)abort_flag != 0u)) {
                         ok = false;
                         break;
                     }
                 }
             }
-            if (!ok || !mbar_wait_bounded(&full_bar[s], ph, p.spin_limit, abort_flag)) {
+            if (!ok || !mbar_wait_warp(&full_bar[s], ph, p.spin_limit, abort_flag)) {
                 *(volatile uint32_t*)abort_flag = 1u;
                 atomicOr(p.status, B2C_DEV_TIMEOUT);
                 ok = false;
@@ -553,7 +553,7 @@ __device__ __forceinline__ void mma_issuer(const ConvKParams& p, const UnitWalk&
             // the first MMA, the loop that bounds narrow tiles with two accumulators.
             if (it == 0) {
                 const long long w1 = timed ? clock64() : 0;
-                if (!mbar_wait_bounded(&acc_empty[buf], ((uint32_t)(j >> p.acc_shift) & 1u) ^ 1u, p.spin_limit, abort_flag)) {
+                if (!mbar_wait_warp(&acc_empty[buf], ((uint32_t)(j >> p.acc_shift) & 1u) ^ 1u, p.spin_limit, abort_flag)) {
                     atomicOr(p.status, B2C_DEV_TIMEOUT);
                     ok = false;
                     break;
@@ -562,33 +562,40 @@ __device__ __forceinline__ void mma_issuer(const ConvKParams& p, const UnitWalk&
             }
             tc_fence_after();
             // descriptors differ from stage to stage only in the 14-bit address field: add offsets to the low word
-            if constexpr (GROUP) {   // (never with full-halo or merged-tap stages)
-                uint32_t a_lo = ring_lo + (uint32_t)s * stage16;
-                for (int g = 0; g < n_k; ++g) {
+            if (elect_one()) {
+                if constexpr (GROUP) {   // (never with full-halo or merged-tap stages)
+                    uint32_t a_lo = ring_lo + (uint32_t)s * stage16;
+                    uint32_t b_bank = b_res;
+                    for (int g = 0; g < n_k; ++g) {
+                        const uint32_t b_lo = p.resident ? b_bank : a_lo + a_to_b16;
+                        issue_stage<KS, NB, PAIR>(d_tmem, a_lo, b_lo, desc_hi, idesc, a_step16, b_step16, (it | g) != 0 ? 1u : 0u);
+                        b_bank += b_cb16;
+                        a_lo += sub16;
+                    }
+                } else {
+                    const uint32_t a_lo = ring_lo + (uint32_t)s * stage16;
                     const uint32_t b_lo = p.resident ? b_res : a_lo + a_to_b16;
-                    issue_stage<KS, NB, PAIR>(d_tmem, a_lo, b_lo, desc_hi, idesc, a_step16, b_step16, (it | g) != 0 ? 1u : 0u);
-                    b_res += b_cb16;
-                    a_lo += sub16;
+                    if constexpr (FH) issue_stage_fh<KS, PAIR>(d_tmem, a_lo, b_lo, a_hi_fh, desc_hi, idesc, a_row16, a_rowpitch16, b_step16, b_s16, it != 0 ? 1u : 0u);
+                    else issue_stage<KS, NB, PAIR>(d_tmem, a_lo, b_lo, desc_hi, idesc, a_step16, b_step16, it != 0 ? 1u : 0u);
                 }
-            } else {
-                const uint32_t a_lo = ring_lo + (uint32_t)s * stage16;
-                const uint32_t b_lo = p.resident ? b_res : a_lo + a_to_b16;
-                if constexpr (FH) issue_stage_fh<KS, PAIR>(d_tmem, a_lo, b_lo, a_hi_fh, desc_hi, idesc, a_row16, a_rowpitch16, b_step16, b_s16, it != 0 ? 1u : 0u);
-                else issue_stage<KS, NB, PAIR>(d_tmem, a_lo, b_lo, desc_hi, idesc, a_step16, b_step16, it != 0 ? 1u : 0u);
-                b_res += b_cb16;
+                // frees the stage (in both CTAs of a pair) once these MMAs have read it
+                if constexpr (PAIR) umma_commit_pair(&empty_bar[s], (uint16_t)3);
+                else umma_commit(&empty_bar[s]);
             }
-            // frees the stage (in both CTAs of a pair) once these MMAs have read it
-            if constexpr (PAIR) umma_commit_pair(&empty_bar[s], (uint16_t)3);
-            else umma_commit(&empty_bar[s]);
+            b_res += (uint32_t)n_k * b_cb16;
+            __syncwarp();
             ++i_stage;
             if (++s == S) { s = 0; ph ^= 1u; }
         }
         if (!ok) break;
-        if constexpr (PAIR) umma_commit_pair(&acc_full[buf], (uint16_t)3);
-        else umma_commit(&acc_full[buf]);
+        if (elect_one()) {
+            if constexpr (PAIR) umma_commit_pair(&acc_full[buf], (uint16_t)3);
+            else umma_commit(&acc_full[buf]);
+        }
+        __syncwarp();
         ++j;
     }
-    if (timed) {
+    if (timed && elect_one()) {
         atomicAdd(p.stall + 1, (unsigned long long)wait_ring);
         atomicAdd(p.stall + 2, (unsigned long long)wait_acc);
     }
@@ -621,7 +628,7 @@ __device__ __forceinline__ void mma_issuer_split(const ConvKParams& p, const Uni
     const int units_per_par = p.n_par > 1 ? p.total_units / p.n_par : 1;
     long long wait_ring = 0, wait_acc = 0;
     bool ok = true;
-    if (resident && !mbar_wait_bounded(w_bar, 0u, p.spin_limit, abort_flag)) {
+    if (resident && !mbar_wait_warp(w_bar, 0u, p.spin_limit, abort_flag)) {
         atomicOr(p.status, B2C_DEV_TIMEOUT);
         ok = false;
     }
@@ -638,7 +645,7 @@ __device__ __forceinline__ void mma_issuer_split(const ConvKParams& p, const Uni
         if (k < i_end) {
             const long long w1 = timed ? clock64() : 0;
             const bool mine_first = k == i0;
-            if (!mbar_wait_bounded(mine_first ? &acc_empty[buf] : &init_bar[buf], mine_first ? acc_par ^ 1u : acc_par, p.spin_limit, abort_flag)) {
+            if (!mbar_wait_warp(mine_first ? &acc_empty[buf] : &init_bar[buf], mine_first ? acc_par ^ 1u : acc_par, p.spin_limit, abort_flag)) {
                 atomicOr(p.status, B2C_DEV_TIMEOUT);
                 ok = false;
                 break;
@@ -649,44 +656,50 @@ __device__ __forceinline__ void mma_issuer_split(const ConvKParams& p, const Uni
             do {
                 const int it = k - i0;
                 const long long w2 = timed ? clock64() : 0;
-                if (!mbar_wait_bounded(&full_bar[s], ph, p.spin_limit, abort_flag)) {
+                if (!mbar_wait_warp(&full_bar[s], ph, p.spin_limit, abort_flag)) {
                     atomicOr(p.status, B2C_DEV_TIMEOUT);
                     ok = false;
                     break;
                 }
                 if (timed) wait_ring += clock64() - w2;
                 tc_fence_after();
-                uint32_t a_lo = ring_lo + (uint32_t)s * stage16;
-                if constexpr (GROUP) {
-                    const int n_k = n_sub - it * G < G ? n_sub - it * G : G;
-                    uint32_t b_res = bank_lo + (uint32_t)(it * G) * b_cb16;
-                    for (int g = 0; g < n_k; ++g) {
-                        issue_stage<KS, NB, PAIR>(d_tmem, a_lo, resident ? b_res : a_lo + a_to_b16, desc_hi, idesc, a_step16, b_step16, (it | g) != 0 ? 1u : 0u);
-                        b_res += b_cb16;
-                        a_lo += sub16;
+                if (elect_one()) {
+                    uint32_t a_lo = ring_lo + (uint32_t)s * stage16;
+                    if constexpr (GROUP) {
+                        const int n_k = n_sub - it * G < G ? n_sub - it * G : G;
+                        uint32_t b_res = bank_lo + (uint32_t)(it * G) * b_cb16;
+                        for (int g = 0; g < n_k; ++g) {
+                            issue_stage<KS, NB, PAIR>(d_tmem, a_lo, resident ? b_res : a_lo + a_to_b16, desc_hi, idesc, a_step16, b_step16, (it | g) != 0 ? 1u : 0u);
+                            b_res += b_cb16;
+                            a_lo += sub16;
+                        }
+                    } else {
+                        issue_stage<KS, NB, PAIR>(d_tmem, a_lo, resident ? bank_lo + (uint32_t)it * b_cb16 : a_lo + a_to_b16, desc_hi, idesc, a_step16, b_step16,
+                                                  it != 0 ? 1u : 0u);
                     }
-                } else {
-                    issue_stage<KS, NB, PAIR>(d_tmem, a_lo, resident ? bank_lo + (uint32_t)it * b_cb16 : a_lo + a_to_b16, desc_hi, idesc, a_step16, b_step16,
-                                              it != 0 ? 1u : 0u);
+                    if constexpr (PAIR) umma_commit_pair(&empty_bar[s], (uint16_t)3);   // frees the stage in both CTAs of a pair
+                    else umma_commit(&empty_bar[s]);
+                    if (it == 0) {   // the overwriting stage (both issuing threads live in the leader CTA of a pair)
+                        if constexpr (PAIR) umma_commit_pair(&init_bar[buf], (uint16_t)1);
+                        else umma_commit(&init_bar[buf]);
+                    }
                 }
-                if constexpr (PAIR) umma_commit_pair(&empty_bar[s], (uint16_t)3);   // frees the stage in both CTAs of a pair
-                else umma_commit(&empty_bar[s]);
-                if (it == 0) {   // the overwriting stage (both issuing threads live in the leader CTA of a pair)
-                    if constexpr (PAIR) umma_commit_pair(&init_bar[buf], (uint16_t)1);
-                    else umma_commit(&init_bar[buf]);
-                }
+                __syncwarp();
                 k += 2;
                 s += 2;
                 if (s >= S) { s = my; ph ^= 1u; }
             } while (k < i_end);
             if (!ok) break;
         }
-        if constexpr (PAIR) umma_commit_pair(&acc_full[buf], (uint16_t)3);
-        else umma_commit(&acc_full[buf]);
+        if (elect_one()) {
+            if constexpr (PAIR) umma_commit_pair(&acc_full[buf], (uint16_t)3);
+            else umma_commit(&acc_full[buf]);
+        }
+        __syncwarp();
         i0 = i_end;
         ++j;
     }
-    if (timed) {
+    if (timed && elect_one()) {
         atomicAdd(p.stall + 1, (unsigned long long)wait_ring);
         atomicAdd(p.stall + 2, (unsigned long long)wait_acc);
     }
@@ -711,7 +724,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~uintptr_t(1023));
     uint8_t* ring = smem + p.resident_bytes;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // the compiler sees a warp-uniform role
     const int S = p.stages;
     const int sub_bytes = p.a_bytes + (p.resident ? 0 : p.nb * p.b_bytes);   // one k-block: the A tile and, unless the bank is resident, its filter tiles
     const int stage_bytes = p.gsub * sub_bytes;
@@ -754,26 +767,28 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
     int last_issued = -1;  // producer lanes: index of the last stage whose loads this lane issued
 
     if (warp == 0 || warp == kProducerWarp1) {
-        if (lane == 0) {
+        {
             // ------------------------------------------------------------ TMA producers
             // Producer w fills the ring slots w, w + kProducers, ...: the chain wait -> expect -> issue of one thread
             // (several hundred cycles) would otherwise bound short stages.  Splitting by slot (not by stage) keeps
             // every slot with one producer that uses it strictly in order, which a parity wait on its barrier needs.
             const int w = warp == 0 ? 0 : 1;
-            prefetch_tensormap(&p.tmB);
-            prefetch_tensormap(&p.tmA[0]);
+            if (elect_one()) {
+                prefetch_tensormap(&p.tmB);
+                prefetch_tensormap(&p.tmA[0]);
+            }
             // a pair counts the bytes of both CTAs on the leader's barriers; b_row = first filter row this CTA fetches
             const int b_rows = PAIR ? p.n_tile >> 1 : p.n_tile;
             const int R = p.r_filter;
             const uint32_t w_bar_cl = PAIR ? map_to_cta(smem_u32(&w_bar), 0) : 0u;
-            if (KIND == KIND_HMERGE && w == 0) {
+            if (KIND == KIND_HMERGE && w == 0 && elect_one()) {
                 // merged horizontal taps: per channel block one box of all nine taps, landing as [r][s][out][64 in]:
                 // three tiles (one per filter row) of 3 x n_tile rows
                 const int oc0 = (walk.first % p.n_ktiles) * p.n_tile;
                 mbar_expect_tx(&w_bar, (uint32_t)(p.c_blocks * 3 * p.tx_b));
                 for (int cb = 0; cb < p.c_blocks; ++cb)
                     tma_load_4d(smem + (size_t)cb * 3 * p.b_bytes, &p.tmB, &w_bar, cb * p.kb, oc0, 0, 0);
-            } else if (KIND != KIND_HMERGE && p.resident && w == 0) {
+            } else if (KIND != KIND_HMERGE && p.resident && w == 0 && elect_one()) {
                 // bank order: [tap or horizontal shift][channel block][vertical tap]
                 const int ktile = walk.first % p.n_ktiles;   // the walk stride is a multiple of n_ktiles: fixed per CTA
                 const TapList& tl = p.taps[0];
@@ -791,6 +806,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
                         }
                     }
             }
+            __syncwarp();
             bool ok = true;
             long long waited = 0;
             const bool timed = p.stall != nullptr;
@@ -817,41 +833,43 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
                     // stamp lets issuers that take alternate units tell the slot's phases apart (a relaxed store: the wait orders it)
                     auto wait_empty = [&]() -> bool {
                         const long long w0 = timed ? clock64() : 0;
-                        if (!mbar_wait_bounded(&empty_bar[s], ph ^ 1u, p.spin_limit, &abort_flag)) {
+                        if (!mbar_wait_warp(&empty_bar[s], ph ^ 1u, p.spin_limit, &abort_flag)) {
                             atomicOr(p.status, B2C_DEV_TIMEOUT);
                             ok = false;
                             return false;
                         }
                         if (timed) waited += clock64() - w0;
-                        if (p.issuers > 1 && !p.issue_split) st_volatile_shared(&slot_stage[s], i + 1);
+                        if (p.issuers > 1 && !p.issue_split && lane == 0) st_volatile_shared(&slot_stage[s], i + 1);
                         return true;
                     };
                     if (G > 1) {
                         if (!wait_empty()) break;
                         // the k-blocks that share this slot (one, except where short k-blocks are grouped)
                         const int k_first = it * G, n_k = n_sub - k_first < G ? n_sub - k_first : G;
-                        if constexpr (PAIR) {
-                            if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * (uint32_t)n_k * stage_tx);
-                        } else {
-                            mbar_expect_tx(&full_bar[s], (uint32_t)n_k * stage_tx);
-                        }
-                        for (int g = 0; g < n_k; ++g) {
-                            const int kblk = k_first + g;
-                            const int t0 = p.cb_shift >= 0 ? kblk >> p.cb_shift : kblk / p.c_blocks;   // tap
-                            const int cb = kblk - t0 * p.c_blocks;                                       // channel block
-                            uint8_t* a_dst = ring + (size_t)s * stage_bytes + (size_t)g * sub_bytes;
+                        if (elect_one()) {
                             if constexpr (PAIR) {
-                                const uint32_t full_cl = map_to_cta(smem_u32(&full_bar[s]), 0);
-                                tma_load_4d_pair(a_dst, &p.tmA[tl.map[t0]], full_cl, cb * p.kb, c.ow0 + tl.dw[t0], c.oh0 + tl.dh[t0], c.n0);
-                                for (int v = 0; v < n_b_loads; ++v) {
-                                    const int rs = tl.rs[t0 + 3 * v], fr = (rs * 11) >> 5;   // rs / 3 for rs < 9 (R is 1 or 3)
-                                    tma_load_4d_pair(a_dst + p.a_bytes + (size_t)v * p.b_bytes, &p.tmB, full_cl, cb * p.kb, rs - fr * R, oc0, fr);
-                                }
+                                if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * (uint32_t)n_k * stage_tx);
                             } else {
-                                tma_load_4d(a_dst, &p.tmA[tl.map[t0]], &full_bar[s], cb * p.kb, c.ow0 + tl.dw[t0], c.oh0 + tl.dh[t0], c.n0);
-                                for (int v = 0; v < n_b_loads; ++v) {
-                                    const int rs = tl.rs[t0 + 3 * v], fr = (rs * 11) >> 5;   // rs / 3 for rs < 9 (R is 1 or 3)
-                                    tma_load_4d(a_dst + p.a_bytes + (size_t)v * p.b_bytes, &p.tmB, &full_bar[s], cb * p.kb, rs - fr * R, oc0, fr);
+                                mbar_expect_tx(&full_bar[s], (uint32_t)n_k * stage_tx);
+                            }
+                            for (int g = 0; g < n_k; ++g) {
+                                const int kblk = k_first + g;
+                                const int t0 = p.cb_shift >= 0 ? kblk >> p.cb_shift : kblk / p.c_blocks;   // tap
+                                const int cb = kblk - t0 * p.c_blocks;                                       // channel block
+                                uint8_t* a_dst = ring + (size_t)s * stage_bytes + (size_t)g * sub_bytes;
+                                if constexpr (PAIR) {
+                                    const uint32_t full_cl = map_to_cta(smem_u32(&full_bar[s]), 0);
+                                    tma_load_4d_pair(a_dst, &p.tmA[tl.map[t0]], full_cl, cb * p.kb, c.ow0 + tl.dw[t0], c.oh0 + tl.dh[t0], c.n0);
+                                    for (int v = 0; v < n_b_loads; ++v) {
+                                        const int rs = tl.rs[t0 + 3 * v], fr = (rs * 11) >> 5;   // rs / 3 for rs < 9 (R is 1 or 3)
+                                        tma_load_4d_pair(a_dst + p.a_bytes + (size_t)v * p.b_bytes, &p.tmB, full_cl, cb * p.kb, rs - fr * R, oc0, fr);
+                                    }
+                                } else {
+                                    tma_load_4d(a_dst, &p.tmA[tl.map[t0]], &full_bar[s], cb * p.kb, c.ow0 + tl.dw[t0], c.oh0 + tl.dh[t0], c.n0);
+                                    for (int v = 0; v < n_b_loads; ++v) {
+                                        const int rs = tl.rs[t0 + 3 * v], fr = (rs * 11) >> 5;   // rs / 3 for rs < 9 (R is 1 or 3)
+                                        tma_load_4d(a_dst + p.a_bytes + (size_t)v * p.b_bytes, &p.tmB, &full_bar[s], cb * p.kb, rs - fr * R, oc0, fr);
+                                    }
                                 }
                             }
                         }
@@ -872,21 +890,24 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
                             b_r[v] = fr;
                         }
                         if (!wait_empty()) break;
-                        if constexpr (PAIR) {
-                            const uint32_t full_cl = map_to_cta(smem_u32(&full_bar[s]), 0);
-                            if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * stage_tx);
-                            tma_load_4d_pair(a_dst, map_a, full_cl, ca, wa, ha, c.n0);
+                        if (elect_one()) {
+                            if constexpr (PAIR) {
+                                const uint32_t full_cl = map_to_cta(smem_u32(&full_bar[s]), 0);
+                                if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * stage_tx);
+                                tma_load_4d_pair(a_dst, map_a, full_cl, ca, wa, ha, c.n0);
 #pragma unroll
-                            for (int v = 0; v < 3; ++v)
-                                if (v < n_b_loads) tma_load_4d_pair(a_dst + p.a_bytes + (size_t)v * p.b_bytes, &p.tmB, full_cl, ca, b_s[v], oc0, b_r[v]);
-                        } else {
-                            mbar_expect_tx(&full_bar[s], stage_tx);
-                            tma_load_4d(a_dst, map_a, &full_bar[s], ca, wa, ha, c.n0);
+                                for (int v = 0; v < 3; ++v)
+                                    if (v < n_b_loads) tma_load_4d_pair(a_dst + p.a_bytes + (size_t)v * p.b_bytes, &p.tmB, full_cl, ca, b_s[v], oc0, b_r[v]);
+                            } else {
+                                mbar_expect_tx(&full_bar[s], stage_tx);
+                                tma_load_4d(a_dst, map_a, &full_bar[s], ca, wa, ha, c.n0);
 #pragma unroll
-                            for (int v = 0; v < 3; ++v)
-                                if (v < n_b_loads) tma_load_4d(a_dst + p.a_bytes + (size_t)v * p.b_bytes, &p.tmB, &full_bar[s], ca, b_s[v], oc0, b_r[v]);
+                                for (int v = 0; v < 3; ++v)
+                                    if (v < n_b_loads) tma_load_4d(a_dst + p.a_bytes + (size_t)v * p.b_bytes, &p.tmB, &full_bar[s], ca, b_s[v], oc0, b_r[v]);
+                            }
                         }
                     }
+                    __syncwarp();
                     last_issued = i;
                     if (s + kProducers < S) {
                         i += kProducers;
@@ -899,55 +920,55 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
                 }
                 i_base += n_it;
             }
-            if (p.stall != nullptr && rank == 0 && w == 0) {
+            if (p.stall != nullptr && rank == 0 && w == 0 && lane == 0) {
                 atomicAdd(p.stall + 0, (unsigned long long)waited);
                 atomicAdd(p.stall + 4, (unsigned long long)(clock64() - t_start));
             }
         }
     } else if (warp == 1 || (warp >= 2 + kEpiWarps && warp < kProducerWarp1)) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             // ------------------------------------------------------------ MMA issuers (in the leader CTA of a pair)
             const int my = warp == 1 ? 0 : warp - (2 + kEpiWarps) + 1;
             if (my < p.issuers) {
-            const uint32_t smem_addr = smem_u32(smem), ring_addr = smem_u32(ring);
-            const int ksteps = p.kb >> 4;
-            if constexpr (KIND == KIND_SPLIT) {
+                const uint32_t smem_addr = smem_u32(smem), ring_addr = smem_u32(ring);
+                const int ksteps = p.kb >> 4;
+                if constexpr (KIND == KIND_SPLIT) {
 #define B2C_ISSUER_S(KS, NB, GR) mma_issuer_split<KS, NB, PAIR, GR>(p, walk, my, tmem_base, smem_addr, ring_addr, stage_bytes, full_bar, empty_bar, acc_full, acc_empty, &w_bar, init_bar, &abort_flag)
-                if (p.nb == 3) {
-                    if (ksteps == 4) B2C_ISSUER_S(4, 3, false);
-                    else if (ksteps == 2) B2C_ISSUER_S(2, 3, false);
-                    else B2C_ISSUER_S(1, 3, false);
-                } else if (p.gsub > 1) {
-                    if (ksteps == 4) B2C_ISSUER_S(4, 1, true);
-                    else if (ksteps == 2) B2C_ISSUER_S(2, 1, true);
-                    else B2C_ISSUER_S(1, 1, true);
-                } else {
-                    if (ksteps == 4) B2C_ISSUER_S(4, 1, false);
-                    else if (ksteps == 2) B2C_ISSUER_S(2, 1, false);
-                    else B2C_ISSUER_S(1, 1, false);
-                }
+                    if (p.nb == 3) {
+                        if (ksteps == 4) B2C_ISSUER_S(4, 3, false);
+                        else if (ksteps == 2) B2C_ISSUER_S(2, 3, false);
+                        else B2C_ISSUER_S(1, 3, false);
+                    } else if (p.gsub > 1) {
+                        if (ksteps == 4) B2C_ISSUER_S(4, 1, true);
+                        else if (ksteps == 2) B2C_ISSUER_S(2, 1, true);
+                        else B2C_ISSUER_S(1, 1, true);
+                    } else {
+                        if (ksteps == 4) B2C_ISSUER_S(4, 1, false);
+                        else if (ksteps == 2) B2C_ISSUER_S(2, 1, false);
+                        else B2C_ISSUER_S(1, 1, false);
+                    }
 #undef B2C_ISSUER_S
-            } else {
-#define B2C_ISSUER(KS, NB, GR, FH) mma_issuer<KS, NB, PAIR, GR, FH>(p, walk, my, tmem_base, smem_addr, ring_addr, stage_bytes, full_bar, empty_bar, acc_full, acc_empty, &w_bar, init_bar, &abort_flag, slot_stage)
-                if constexpr (KIND == KIND_HMERGE) {
-                    B2C_ISSUER(4, 3, false, false);   // 64-channel k-blocks, the three filter rows of a channel block per stage
-                } else if constexpr (KIND == KIND_FULL_HALO) {
-                    B2C_ISSUER(4, 3, false, true);
-                } else if (p.nb == 3) {
-                    if (ksteps == 4) B2C_ISSUER(4, 3, false, false);
-                    else if (ksteps == 2) B2C_ISSUER(2, 3, false, false);
-                    else B2C_ISSUER(1, 3, false, false);
-                } else if (p.gsub > 1) {
-                    if (ksteps == 4) B2C_ISSUER(4, 1, true, false);
-                    else if (ksteps == 2) B2C_ISSUER(2, 1, true, false);
-                    else B2C_ISSUER(1, 1, true, false);
                 } else {
-                    if (ksteps == 4) B2C_ISSUER(4, 1, false, false);
-                    else if (ksteps == 2) B2C_ISSUER(2, 1, false, false);
-                    else B2C_ISSUER(1, 1, false, false);
-                }
+#define B2C_ISSUER(KS, NB, GR, FH) mma_issuer<KS, NB, PAIR, GR, FH>(p, walk, my, tmem_base, smem_addr, ring_addr, stage_bytes, full_bar, empty_bar, acc_full, acc_empty, &w_bar, init_bar, &abort_flag, slot_stage)
+                    if constexpr (KIND == KIND_HMERGE) {
+                        B2C_ISSUER(4, 3, false, false);   // 64-channel k-blocks, the three filter rows of a channel block per stage
+                    } else if constexpr (KIND == KIND_FULL_HALO) {
+                        B2C_ISSUER(4, 3, false, true);
+                    } else if (p.nb == 3) {
+                        if (ksteps == 4) B2C_ISSUER(4, 3, false, false);
+                        else if (ksteps == 2) B2C_ISSUER(2, 3, false, false);
+                        else B2C_ISSUER(1, 3, false, false);
+                    } else if (p.gsub > 1) {
+                        if (ksteps == 4) B2C_ISSUER(4, 1, true, false);
+                        else if (ksteps == 2) B2C_ISSUER(2, 1, true, false);
+                        else B2C_ISSUER(1, 1, true, false);
+                    } else {
+                        if (ksteps == 4) B2C_ISSUER(4, 1, false, false);
+                        else if (ksteps == 2) B2C_ISSUER(2, 1, false, false);
+                        else B2C_ISSUER(1, 1, false, false);
+                    }
 #undef B2C_ISSUER
-            }
+                }
             }
         }
     } else {
@@ -984,7 +1005,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
                 for (uint32_t i = 0; i < kDrainPolls && !mbar_try_wait(&full_bar[sl], (uint32_t)(it / S) & 1u); ++i) {}
             }
         }
-        if ((warp == 1 || (warp >= 2 + kEpiWarps && warp < kProducerWarp1)) && lane == 0 && rank == 0) {   // a commit covers the MMAs of the thread that makes it
+        if ((warp == 1 || (warp >= 2 + kEpiWarps && warp < kProducerWarp1)) && rank == 0 && elect_one()) {   // a commit covers the MMAs of the thread that makes it
             if constexpr (PAIR) umma_commit_pair(&drain_bar, (uint16_t)1);
             else umma_commit(&drain_bar);
             if (warp == 1)

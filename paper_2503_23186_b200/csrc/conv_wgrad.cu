@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
     __shared__ uint32_t abort_flag;
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~uintptr_t(1023));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int S = p.stages;
 
     int t = blockIdx.x;
@@ -156,53 +156,58 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
 
     if (warp == 0 || warp >= kWgProducerWarp1) {
         const int w = warp == 0 ? 0 : warp - kWgProducerWarp1 + 1;
-        if (lane == 0 && w < S) {
+        if (w < S) {
             // Producer w fills the ring slots w, w + kWgProducers, ...: one thread's wait -> expect -> issue chain is
             // longer than the MMAs of a stage take.  Each slot keeps one producer, which uses it strictly in order.
-            prefetch_tensormap(&p.tmDy);
-            prefetch_tensormap(&p.tmX[0]);
+            if (elect_one()) {
+                prefetch_tensormap(&p.tmDy);
+                prefetch_tensormap(&p.tmX[0]);
+            }
             const uint32_t tx = p.fx ? (uint32_t)(p.a_bytes + p.b_boxes * p.fx_tx) : (uint32_t)(p.a_bytes + grp.nb * p.b_boxes * p.box_b);
             int it = w, s = w;   // it counts ring slots; a slot holds G consecutive chunks (the last one of the CTA possibly fewer)
             uint32_t ph = 0u;
-            const bool timed = p.stall != nullptr && w == 0;
+            const bool timed = p.stall != nullptr && w == 0 && lane == 0;
             long long waited = 0;
             const int G = p.gsub, n_slots = (n_chunks + G - 1) / G;
             while (it < n_slots) {
                 const long long w0 = timed ? clock64() : 0;
-                if (!mbar_wait_bounded(&empty_bar[s], ph ^ 1u, p.spin_limit, &abort_flag)) {
+                if (!mbar_wait_warp(&empty_bar[s], ph ^ 1u, p.spin_limit, &abort_flag)) {
                     atomicOr(p.status, B2C_DEV_TIMEOUT);
                     break;
                 }
                 if (timed) waited += clock64() - w0;
                 const int n_g = n_chunks - it * G < G ? n_chunks - it * G : G;
-                mbar_expect_tx(&full_bar[s], (uint32_t)n_g * tx);
-                for (int g = 0; g < n_g; ++g) {
-                int ch = chunk_begin + it * G + g;
-                const int ow0 = (ch & (p.tiles_w - 1)) * p.bw;
-                ch >>= p.tw_shift;
-                const int th = ch / p.tiles_h;
-                const int oh0 = (ch - th * p.tiles_h) * p.bh;
-                const int n0 = th * p.bn;
-                uint8_t* dst = smem + (size_t)s * p.stage_bytes + (size_t)g * p.sub_bytes;
-                if (p.stack) {
-                    // one box with a halo row on top: copy 1 of dy (gathered one row higher) is its first pb pixels,
-                    // copy 0 starts one image row further down
-                    tma_load_4d(dst, &p.tmDy, &full_bar[s], 0, ow0, oh0 - 1, n0);
-                } else {
-                    for (int j = 0; j < p.a_boxes; ++j)  // boxes past the last channel are zero-filled
-                        tma_load_4d(dst + (size_t)j * p.box_a, &p.tmDy, &full_bar[s], ktile * 128 + j * p.cw_a, ow0, oh0, n0);
+                if (elect_one()) {
+                    mbar_expect_tx(&full_bar[s], (uint32_t)n_g * tx);
+                    for (int g = 0; g < n_g; ++g) {
+                        int ch = chunk_begin + it * G + g;
+                        const int ow0 = (ch & (p.tiles_w - 1)) * p.bw;
+                        ch >>= p.tw_shift;
+                        const int th = ch / p.tiles_h;
+                        const int oh0 = (ch - th * p.tiles_h) * p.bh;
+                        const int n0 = th * p.bn;
+                        uint8_t* dst = smem + (size_t)s * p.stage_bytes + (size_t)g * p.sub_bytes;
+                        if (p.stack) {
+                            // one box with a halo row on top: copy 1 of dy (gathered one row higher) is its first pb pixels,
+                            // copy 0 starts one image row further down
+                            tma_load_4d(dst, &p.tmDy, &full_bar[s], 0, ow0, oh0 - 1, n0);
+                        } else {
+                            for (int j = 0; j < p.a_boxes; ++j)  // boxes past the last channel are zero-filled
+                                tma_load_4d(dst + (size_t)j * p.box_a, &p.tmDy, &full_bar[s], ktile * 128 + j * p.cw_a, ow0, oh0, n0);
+                        }
+                        dst += p.a_bytes;
+                        if (p.fx) {   // one framed box per channel block, gathered at the first shift (one pixel to the left)
+                            for (int j = 0; j < p.b_boxes; ++j)
+                                tma_load_4d(dst + (size_t)j * p.fx_box, &p.tmX[grp.map[0]], &full_bar[s], ctile * p.ct + j * p.cw_b, ow0 + grp.dw[0],
+                                            oh0 + grp.dh[0], n0);
+                        } else
+                        for (int b = 0; b < grp.nb; ++b)
+                            for (int j = 0; j < p.b_boxes; ++j)
+                                tma_load_4d(dst + (size_t)(b * p.b_boxes + j) * p.box_b, &p.tmX[grp.map[b]], &full_bar[s], ctile * p.ct + j * p.cw_b,
+                                            ow0 + grp.dw[b], oh0 + grp.dh[b], n0);
+                    }
                 }
-                dst += p.a_bytes;
-                if (p.fx) {   // one framed box per channel block, gathered at the first shift (one pixel to the left)
-                    for (int j = 0; j < p.b_boxes; ++j)
-                        tma_load_4d(dst + (size_t)j * p.fx_box, &p.tmX[grp.map[0]], &full_bar[s], ctile * p.ct + j * p.cw_b, ow0 + grp.dw[0],
-                                    oh0 + grp.dh[0], n0);
-                } else
-                for (int b = 0; b < grp.nb; ++b)
-                    for (int j = 0; j < p.b_boxes; ++j)
-                        tma_load_4d(dst + (size_t)(b * p.b_boxes + j) * p.box_b, &p.tmX[grp.map[b]], &full_bar[s], ctile * p.ct + j * p.cw_b,
-                                    ow0 + grp.dw[b], oh0 + grp.dh[b], n0);
-                }
+                __syncwarp();
                 last_issued = it;
                 if (s + kWgProducers < S) {
                     it += kWgProducers;
@@ -216,7 +221,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
             if (timed) atomicAdd(p.stall + 0, (unsigned long long)waited);
         }
     } else if (warp == 1 || warp == 2) {
-        if (lane == 0 && warp - 1 < p.issuers) {
+        if (warp - 1 < p.issuers) {
             const int my = warp - 1;
             // SBO = eight pixel rows, LBO = next block of cw channels (the next box)
             const uint64_t proto_a = make_smem_desc(0u, (uint32_t)p.a_lbo, 16u * (uint32_t)p.cw_a, (uint32_t)p.swz_a);
@@ -242,12 +247,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                 ++n_pieces;
             }
             bool ok = true;
-            const bool timed = p.stall != nullptr;
+            const bool timed = p.stall != nullptr && lane == 0;
             const long long t_begin = timed ? clock64() : 0;
             long long waited = 0, issuing = 0;
             const int G = p.gsub, n_slots = (n_chunks + G - 1) / G;
             const uint32_t sub16 = (uint32_t)p.sub_bytes >> 4;
-            if (my != 0 && n_slots > 1 && !mbar_wait_bounded(&init_bar, 0u, p.spin_limit, &abort_flag)) {   // slot 0 has initialised the accumulator
+            if (my != 0 && n_slots > 1 && !mbar_wait_warp(&init_bar, 0u, p.spin_limit, &abort_flag)) {   // slot 0 has initialised the accumulator
                 atomicOr(p.status, B2C_DEV_TIMEOUT);
                 ok = false;
             }
@@ -263,7 +268,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
             uint32_t ph = 0u;
             for (int it = my; ok && it < n_slots; it += n_issuers) {
                 const long long w0 = timed ? clock64() : 0;
-                if (!mbar_wait_bounded(&full_bar[s], ph, p.spin_limit, &abort_flag)) {
+                if (!mbar_wait_warp(&full_bar[s], ph, p.spin_limit, &abort_flag)) {
                     atomicOr(p.status, B2C_DEV_TIMEOUT);
                     ok = false;
                     break;
@@ -273,31 +278,35 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                 tc_fence_after();
                 const uint32_t st16 = smem16 + (uint32_t)s * stage16;
                 const int n_g = n_chunks - it * G < G ? n_chunks - it * G : G;
-                for (int g = 0; g < n_g; ++g) {
-                const uint32_t a_lo = a_lo_base + st16 + (uint32_t)g * sub16, b_lo = b_lo_base + st16 + (uint32_t)g * sub16;
-                const uint32_t acc0 = (it | g) != 0 ? 1u : 0u;
-                if (fx) {   // chunks of 64 pixels: four k-steps; one MMA per channel block, N = three shifts x cw_b channels
-                    const uint32_t b_first = b_lo + fx_b_first;
-                    for (int i = 0; i < b_boxes; ++i)
-                        wg_issue_framed<4>(tmem_base + (uint32_t)i * fx_d_next, a_lo, b_first + (uint32_t)i * fx_b_next, a_hi, b_hi, id_fx, kstep_a, fk0, fk1, fk2,
-                                           fk3, acc0);
-                } else if (ksteps == 4) {
-                    wg_issue<4>(tmem_base + dcol0, a_lo, b_lo + boff0, a_hi, b_hi, idesc0, kstep_a, kstep_b, acc0);
-                    if (n_pieces > 1) wg_issue<4>(tmem_base + dcol1, a_lo, b_lo + boff1, a_hi, b_hi, idesc1, kstep_a, kstep_b, acc0);
-                    if (n_pieces > 2) wg_issue<4>(tmem_base + dcol2, a_lo, b_lo + boff2, a_hi, b_hi, idesc2, kstep_a, kstep_b, acc0);
-                } else {
-                    wg_issue<2>(tmem_base + dcol0, a_lo, b_lo + boff0, a_hi, b_hi, idesc0, kstep_a, kstep_b, acc0);
-                    if (n_pieces > 1) wg_issue<2>(tmem_base + dcol1, a_lo, b_lo + boff1, a_hi, b_hi, idesc1, kstep_a, kstep_b, acc0);
-                    if (n_pieces > 2) wg_issue<2>(tmem_base + dcol2, a_lo, b_lo + boff2, a_hi, b_hi, idesc2, kstep_a, kstep_b, acc0);
+                if (elect_one()) {
+                    for (int g = 0; g < n_g; ++g) {
+                        const uint32_t a_lo = a_lo_base + st16 + (uint32_t)g * sub16, b_lo = b_lo_base + st16 + (uint32_t)g * sub16;
+                        const uint32_t acc0 = (it | g) != 0 ? 1u : 0u;
+                        if (fx) {   // chunks of 64 pixels: four k-steps; one MMA per channel block, N = three shifts x cw_b channels
+                            const uint32_t b_first = b_lo + fx_b_first;
+                            for (int i = 0; i < b_boxes; ++i)
+                                wg_issue_framed<4>(tmem_base + (uint32_t)i * fx_d_next, a_lo, b_first + (uint32_t)i * fx_b_next, a_hi, b_hi, id_fx, kstep_a, fk0, fk1, fk2,
+                                                   fk3, acc0);
+                        } else if (ksteps == 4) {
+                            wg_issue<4>(tmem_base + dcol0, a_lo, b_lo + boff0, a_hi, b_hi, idesc0, kstep_a, kstep_b, acc0);
+                            if (n_pieces > 1) wg_issue<4>(tmem_base + dcol1, a_lo, b_lo + boff1, a_hi, b_hi, idesc1, kstep_a, kstep_b, acc0);
+                            if (n_pieces > 2) wg_issue<4>(tmem_base + dcol2, a_lo, b_lo + boff2, a_hi, b_hi, idesc2, kstep_a, kstep_b, acc0);
+                        } else {
+                            wg_issue<2>(tmem_base + dcol0, a_lo, b_lo + boff0, a_hi, b_hi, idesc0, kstep_a, kstep_b, acc0);
+                            if (n_pieces > 1) wg_issue<2>(tmem_base + dcol1, a_lo, b_lo + boff1, a_hi, b_hi, idesc1, kstep_a, kstep_b, acc0);
+                            if (n_pieces > 2) wg_issue<2>(tmem_base + dcol2, a_lo, b_lo + boff2, a_hi, b_hi, idesc2, kstep_a, kstep_b, acc0);
+                        }
+                    }
+                    umma_commit(&empty_bar[s]);
+                    if (it == 0) umma_commit(&init_bar);
                 }
-                }
-                umma_commit(&empty_bar[s]);
-                if (it == 0) umma_commit(&init_bar);
+                __syncwarp();
                 if (timed) issuing += clock64() - w1;
                 s += n_issuers;
                 if (s >= S) { s -= S; ph ^= 1u; }
             }
-            if (ok && n_chunks > 0) umma_commit(&accum_bar);
+            if (ok && n_chunks > 0 && elect_one()) umma_commit(&accum_bar);
+            __syncwarp();
             if (timed && my == 0) {
                 atomicAdd(p.stall + 1, (unsigned long long)waited);
                 atomicAdd(p.stall + 4, (unsigned long long)(clock64() - t_begin));
@@ -373,7 +382,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                 for (uint32_t i = 0; i < kWgDrainPolls && !mbar_try_wait(&full_bar[sl], (uint32_t)(it / S) & 1u); ++i) {}
             }
         }
-        if ((warp == 1 || warp == 2) && lane == 0 && warp - 1 < p.issuers) {   // a commit covers the MMAs of the thread that makes it
+        if ((warp == 1 || warp == 2) && warp - 1 < p.issuers && elect_one()) {   // a commit covers the MMAs of the thread that makes it
             umma_commit(&drain_bar);
             if (warp == 1)
                 for (uint32_t i = 0; i < kWgDrainPolls && !mbar_try_wait(&drain_bar, 0u); ++i) {}
