@@ -8,8 +8,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 SO = os.path.join(HERE, "libb2c.so")
-SOURCES = ["api.cu", "conv_kmajor.cu", "conv_wgrad.cu", "elementwise.cu"]
-HEADERS = ["common.h", "ptx.cuh", os.path.join("..", "..", "include", "b2c.h")]
+SOURCES = ["api.cu", "conv_kmajor.cu", "conv_splitk.cu", "conv_wgrad.cu", "elementwise.cu"]
+HEADERS = ["common.h", "conv_kmajor.h", "ptx.cuh", os.path.join("..", "..", "include", "b2c.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", 
               "-Xcompiler", "-fPIC", "-shared"]
 

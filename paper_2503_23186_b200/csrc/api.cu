@@ -61,6 +61,12 @@ b2c_status b2c_create(b2c_ctx** out, int device)
         ctx->use_group_kblocks = env ? (env[0] != '0') : 1;
     }
     {
+        const char* env = std::getenv("B2C_SPLIT_K");
+        ctx->use_split_k = env ? (env[0] != '0') : 1;
+    }
+    for (int a = 0; a < 2; ++a)
+        for (int b = 0; b < 9; ++b) ctx->max_clusters[a][b] = -1;
+    {
         const char* env = std::getenv("B2C_WGRAD_ISSUERS");
         ctx->use_wgrad_two_issuers = env ? (env[0] != '1') : 1;   // B2C_WGRAD_ISSUERS=1: one issuing thread
     }

@@ -22,57 +22,11 @@
 // lane quarter, splitting the columns), warp 10 = second MMA issuer (the two issuers take alternate units), warp 11 = second
 // TMA producer (the two producers take alternate stages).  Producer and issuer warps run their loops with all lanes and issue
 // from one elected lane.  Every mbarrier wait is bounded.
-#include "common.h"
-#include "ptx.cuh"
+#include "conv_kmajor.h"
 
 namespace b2c {
 
-struct alignas(64) ConvKParams {
-    CUtensorMap tmA[4];
-    CUtensorMap tmB;
-    TapList taps[4];
-    int bw, bh, bn;                  // pixel box of an output tile; bw*bh*bn == 128
-    int tiles_w, tiles_h, tiles_n;   // tiles of the output grid
-    int tw_shift, th_shift, nk_shift, grp_shift, cb_shift;   // log2 of tiles_w, tiles_h, n_ktiles, stats_group_images, c_blocks (-1: not a power of two)
-    int n_ktiles, n_tile;            // output-channel tiles, UMMA N
-    int n_par;                       // output parities (stride-2 data gradient: 4)
-    int total_units;
-    int kb, c_blocks;                // channels per k-block, k-blocks per tap
-    int stages, swz;
-    int tmem_cols, acc_cols;         // allocation, columns per accumulator
-    int acc_bufs, acc_shift;         // accumulators in TMEM (2 or 4) and log2 of that: unit j uses accumulator j % acc_bufs
-    int vreuse;                      // a stage serves the three vertical taps of one horizontal shift
-    int fh;                          // full halo: a stage holds the tile with a one-pixel frame and serves all nine taps
-    int hm;                          // merged horizontal taps: one N = 3 x n_tile MMA per vertical tap and k-step, the three column blocks are
-                                     // shifted by one pixel and added in the epilogue (tiles of whole image rows, 64 output channels)
-    int mma_n;                       // UMMA N (n_tile, or 3 x n_tile with merged horizontal taps)
-    int nb;                          // B tiles per stage (1, or 3 with vreuse)
-    int b_merged;                    // the three B tiles of a stage come with one load (box of three filter rows)
-    int r_filter;                    // filter height = width
-    int a_bytes, b_bytes;            // shared-memory footprint of the A tile / one B tile (multiples of 1 KB)
-    int tx_a, tx_b;                  // bytes one A / B load delivers
-    int a_step;                      // byte offset of one image row inside the A tile (vreuse)
-    int issuers;                     // MMA-issuing threads at work (1 or 2)
-    int gsub;                        // k-blocks that share a ring slot, one barrier wait and one commit (short k-blocks: the waits would bound the issuing threads)
-    int issue_split;                 // the two issuing threads share every unit: alternate stages into one accumulator (tiles wider than 128 channels)
-    int pair;                        // CTA pairs (cta_group::2): M = 256 per MMA, each CTA holds half of every B tile
-    int resident;                    // filter bank of this CTA's channel tile stays in shared memory
-    int resident_bytes;
-    int n_valid, oc_valid;           // images / output channels that exist
-    long long os_n, os_h, os_w;      // output element strides along the tile grid
-    long long off[4];                // output element offset per parity
-    void* out;
-    int out_is_f32;
-    int out_v8;                      // the output base is 32-byte aligned: bf16 chunks go out as one 256-bit store per lane
-    const float* bias;
-    double* stats;
-    int stats_group_images;          // images per BatchNorm statistics group (0: one group)
-    unsigned* status;
-    unsigned spin_limit;
-    unsigned long long* stall;       // optional [5]: cycles waited by producer / MMA (ring) / MMA (accumulator) / epilogue, CTA lifetime
-};
-
-static constexpr int kMaxStages = 8;
+static constexpr int kMaxStages = 8;   // (conv_splitk.cu has room for as many)
 static constexpr int kMaxAccBufs = 4;
 static constexpr int kEpiWarps = 8;
 static constexpr int kIssuers = 2;       // MMA-issuing threads: warp 1 and the warps after the epilogue warps
@@ -81,33 +35,6 @@ static constexpr int kThreads = 64 + 32 * kEpiWarps + 32 * (kIssuers - 1) + 32 *
 static constexpr int kProducerWarp1 = 2 + kEpiWarps + (kIssuers - 1);   // warp index of the second producer
 static constexpr uint32_t kDrainPolls = 1u << 22;
 
-struct UnitCoord {
-    int par, ktile, ow0, oh0, n0;
-};
-// tiles_w and tiles_h are powers of two (the grid sides are); the channel-tile count and the stats group size usually are
-__device__ __forceinline__ UnitCoord decode_unit(const ConvKParams& p, int u)
-{
-    UnitCoord c;
-    if (p.nk_shift >= 0) {
-        c.ktile = u & (p.n_ktiles - 1);
-        u >>= p.nk_shift;
-    } else {
-        c.ktile = u % p.n_ktiles;
-        u /= p.n_ktiles;
-    }
-    c.ow0 = (u & (p.tiles_w - 1)) * p.bw;
-    u >>= p.tw_shift;
-    c.oh0 = (u & (p.tiles_h - 1)) * p.bh;
-    u >>= p.th_shift;
-    if (p.n_par > 1) {
-        c.n0 = (u % p.tiles_n) * p.bn;
-        c.par = u / p.tiles_n;
-    } else {
-        c.n0 = u * p.bn;
-        c.par = 0;
-    }
-    return c;
-}
 // Units of this CTA: plain kernels walk units blockIdx.x, +gridDim.x, ...; CTA pairs walk pair-units (two pixel tiles
 // next to each other, same channel tile) and CTA `rank` of the pair takes tile 2*m + rank.
 struct UnitWalk {
@@ -1079,6 +1006,65 @@ struct KMajorPlan {
     size_t smem_bytes;
 };
 
+// Tensor-pipe and staging cycles of one k-block of kb channels on a tile of 128 pixels (a pair: 2 x 128) x n channels: an MMA of 16
+// channels takes n / 2 cycles, or what its operands take through the 128 B/clk shared-memory port (A: 4 KB, B: 32 n bytes, half of
+// it per CTA of a pair); the loads come in at about 60 B/clk per SM (measured, L2 -> shared memory with every SM streaming).
+static int kblock_cycles(int n, int kb, bool pair, int a_rows)
+{
+    const int b_rows = pair ? n / 2 : n;
+    const int operand = 32 + b_rows / 4, mma = (operand > n / 2 ? operand : n / 2) * (kb / 16);
+    const int loads = (a_rows + b_rows) * kb * 2 / 60;
+    return mma > loads ? mma : loads;
+}
+
+// Split-K plan (conv_splitk.cu) for a problem whose tiles do not fill the chip, or false where the persistent plan (est_cycles for its
+// busiest CTA) is the better one by the same estimate.  A cluster of `splits` CTAs or pairs shares a tile's k-blocks, all
+// clusters run in one wave, and the exchange of the partial tiles costs a cluster barrier and (splits - 1) / splits of the tile
+// at about 32 B/clk.  Measured with 128 images (launch to launch):
+// 512 -> 512 at 4x4 27.8 -> 17.6 us, 256 -> 256 at 8x8 18.2 -> 14.3; with 50 images 26.2 -> 12.0 and 16.2 -> 12.4 us.
+static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p, int m_tiles, long long est_cycles)
+{
+    const int kb = (pb.ic % 64 == 0) ? 64 : (pb.ic % 32 == 0) ? 32 : 16;
+    const int taps = p.n_par > 1 ? ((pb.r + 1) / 2) * ((pb.r + 1) / 2) : pb.r * pb.r;   // of the parity with most
+    const int min_taps = p.n_par > 1 ? 1 : taps;
+    const int c_blocks = pb.ic / kb;
+    long long best = est_cycles;
+    bool found = false;
+    for (int pair = 0; pair <= 1; ++pair) {
+        if (pair && (p.n_par > 1 || ctx->use_pairs == 0)) continue;
+        for (int n = 256; n >= 32; n -= 16) {
+            if (pb.oc % n || (pair && n % 32)) continue;
+            const int clusters = p.n_par * (pair ? (m_tiles / p.n_par + 1) / 2 : m_tiles / p.n_par) * (pb.oc / n);
+            for (int splits = 1; splits * (pair + 1) <= 8; splits *= 2) {
+                if (n % (8 * splits) || splits > min_taps * c_blocks) continue;
+                if (clusters > splitk_max_clusters(ctx, splits * (pair + 1), pair != 0)) continue;
+                const int k_blocks = (taps * c_blocks + splits - 1) / splits;
+                const long long est = (long long)k_blocks * kblock_cycles(n, kb, pair != 0, 128) + (splits > 1 ? 1500 + 16ll * n * (splits - 1) / splits : 0);
+                if (est * 10 >= best * 9) continue;   // a tenth better at least
+                best = est;
+                found = true;
+                p.n_tile = n; p.n_ktiles = pb.oc / n; p.pair = pair; p.splits = splits;
+            }
+        }
+    }
+    if (!found) return false;
+    const int b_rows = p.pair ? p.n_tile / 2 : p.n_tile;
+    p.kb = kb; p.c_blocks = c_blocks;
+    p.swz = kb == 64 ? SWZ_128B : kb == 32 ? SWZ_64B : SWZ_32B;
+    p.nb = 1;
+    p.tx_a = p.a_bytes = 128 * kb * 2;
+    p.tx_b = b_rows * kb * 2;
+    p.b_bytes = (p.tx_b + 1023) & ~1023;
+    p.gsub = 1;   // k-blocks of a ring slot: narrow ones share a slot, its barrier wait and its commit
+    while (p.gsub < 4 && 2 * p.gsub * (p.a_bytes + p.b_bytes) <= 40 * 1024 && 2 * p.gsub * p.splits <= taps * c_blocks) p.gsub *= 2;
+    p.stages = 216 * 1024 / (p.gsub * (p.a_bytes + p.b_bytes));
+    if (p.stages > kMaxStages) p.stages = kMaxStages;
+    p.tmem_cols = 32;
+    while (p.tmem_cols < p.n_tile) p.tmem_cols *= 2;
+    p.total_units = p.n_par * (p.pair ? m_tiles + (m_tiles & 1) : m_tiles / p.n_par) * p.n_ktiles;
+    return true;
+}
+
 static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajorPlan& plan)
 {
     ConvKParams& p = plan.p;
@@ -1132,7 +1118,7 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     const bool pair_ok = n_par == 1 && !pb.out_f32 && pb.bias == nullptr && n_tile % 32 == 0 && m_tiles % 2 == 0 && ctx->sm_count >= 2;
     p.pair = (pair_ok && (ctx->use_pairs == 2 || (ctx->use_pairs == 1 && n_tile >= 128 && R == 3 && pb.stride == 1) ||
                           (ctx->use_pairs == 3 && n_tile == 128 && R == 3 && pb.stride == 1))) ? 1 : 0;
-    const int b_rows = p.pair ? n_tile / 2 : n_tile;   // filter rows one CTA fetches per tile
+    int b_rows = p.pair ? n_tile / 2 : n_tile;   // filter rows one CTA fetches per tile
 
     // launch shape: one persistent CTA per SM; the unit walk stride (CTAs, or pairs) is a multiple of n_ktiles so that a
     // CTA keeps its channel tile
@@ -1229,13 +1215,27 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
         if (stages >= 4 || !vr) break;
     }
     if (p.stages < 2) return B2C_ERR_UNSUPPORTED_SHAPE;
+    int cluster = 0;   // CTAs per cluster of a split-K plan
+    if (ctx->use_split_k && grid < ctx->sm_count) {
+        const int max_taps = n_par > 1 ? ((R + 1) / 2) * ((R + 1) / 2) : taps_total;
+        const int a_rows = p.vreuse ? (p.bh + 2) * p.bw / 3 : p.fh ? 180 / 9 : 128;
+        ConvKParams q = p;
+        q.bw = gw < 128 ? gw : 128; q.bh = (128 / q.bw) < gh ? (128 / q.bw) : gh; q.bn = 128 / (q.bw * q.bh);
+        q.tiles_w = gw / q.bw; q.tiles_h = gh / q.bh; q.tiles_n = (pb.n + q.bn - 1) / q.bn;
+        q.vreuse = q.fh = q.hm = q.resident = q.resident_bytes = q.b_merged = q.a_step = 0;
+        if (choose_splitk(ctx, pb, q, n_par * m_tiles, (long long)units_per_cta * max_taps * (pb.ic / p.kb) * kblock_cycles(n_tile, p.kb, p.pair != 0, a_rows))) {
+            p = q;
+            cluster = p.splits * (p.pair ? 2 : 1);
+            b_rows = p.pair ? p.n_tile / 2 : p.n_tile;
+        }
+    }
     p.mma_n = p.hm ? 3 * p.n_tile : p.n_tile;
     // Short k-blocks share a ring slot.  An issuing thread pays 700-900 cycles per slot on top of its MMAs (the slot's stamp,
     // the barrier wait, two commits; measured inside the running kernel), which bounds the stride-2 and 1x1 layers
     // (one k-block = 2-4 MMAs of 48-128 cycles): group k-blocks while a slot holds less than about 1000 tensor-pipe
     // cycles, three slots remain (four where two threads take alternate slots) and the unit has that many k-blocks.
-    p.gsub = 1;
-    if (ctx->use_group_kblocks && !p.fh && !p.hm && !p.vreuse) {
+    if (!cluster) p.gsub = 1;
+    if (ctx->use_group_kblocks && !cluster && !p.fh && !p.hm && !p.vreuse) {
         // k-blocks of the longest unit (stride-2 data gradient: the parity that takes every other tap in both directions)
         const int max_sub = (n_par > 1 ? ((R + 1) / 2) * ((R + 1) / 2) : taps_total) * p.c_blocks;
         const int per_sub = (p.kb / 16) * (p.mma_n / 2 > 48 ? p.mma_n / 2 : 48);
@@ -1253,7 +1253,7 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     // Two issuing threads where one cannot keep the tensor pipe busy: tiles of at most 128 channels.
     p.issuers = p.n_tile <= 128 ? kIssuers : 1;
     // Wider tiles: both threads work on every unit, alternate stages (needs an even ring).
-    if (p.n_tile > 128 && ctx->use_issue_split && p.stages >= 2) {
+    if (!cluster && p.n_tile > 128 && ctx->use_issue_split && p.stages >= 2) {
         p.stages &= ~1;
         p.issuers = kIssuers;
         p.issue_split = 1;
@@ -1332,7 +1332,7 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     p.grp_shift = log2_exact(p.stats_group_images);
     p.cb_shift = log2_exact(p.c_blocks);
     if (p.stats && p.stats_group_images > 0 && (p.stats_group_images % p.bn) != 0) return B2C_ERR_UNSUPPORTED_SHAPE;  // a tile must not straddle groups
-    plan.grid = grid;
+    plan.grid = cluster ? p.total_units * p.splits : grid;
     plan.smem_bytes = smem_bytes;
     return B2C_OK;
 }
@@ -1352,6 +1352,7 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
     key_add(key, pb.r); key_add(key, pb.stride); key_add(key, pb.pad); key_add(key, pb.dgrad); key_add(key, pb.in); key_add(key, pb.wt);
     key_add(key, pb.out); key_add(key, pb.out_f32); key_add(key, pb.bias); key_add(key, pb.stats); key_add(key, pb.stats_group_images);
     key_add(key, ctx->use_pairs); key_add(key, ctx->use_full_halo); key_add(key, ctx->use_issue_split); key_add(key, ctx->use_hmerge); key_add(key, ctx->use_group_kblocks);
+    key_add(key, ctx->use_split_k);
     auto it = ctx->plan_cache.find(key);
     if (it == ctx->plan_cache.end()) {
         KMajorPlan fresh;
@@ -1371,6 +1372,7 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
     p.spin_limit = ctx->spin_limit;
     p.stall = ctx->stall_counters;
 
+    if (p.splits > 0) return launch_conv_splitk(ctx, p, grid, smem_bytes, stream);
     // the kernel kind of the plan (merged taps run on single CTAs only)
     typedef void (*kernel_t)(const ConvKParams);
     static const kernel_t kernels[2][4] = {

@@ -1,0 +1,88 @@
+// Parameter block and unit numbering shared by the two implicit-GEMM kernels with K-major operands: the persistent one
+// (conv_kmajor.cu) and the split-K one for problems with fewer tiles than SMs (conv_splitk.cu).
+#pragma once
+#include "common.h"
+#include "ptx.cuh"
+
+namespace b2c {
+
+struct alignas(64) ConvKParams {
+    CUtensorMap tmA[4];
+    CUtensorMap tmB;
+    TapList taps[4];
+    int bw, bh, bn;                  // pixel box of an output tile; bw*bh*bn == 128
+    int tiles_w, tiles_h, tiles_n;   // tiles of the output grid
+    int tw_shift, th_shift, nk_shift, grp_shift, cb_shift;   // log2 of tiles_w, tiles_h, n_ktiles, stats_group_images, c_blocks (-1: not a power of two)
+    int n_ktiles, n_tile;            // output-channel tiles, UMMA N
+    int n_par;                       // output parities (stride-2 data gradient: 4)
+    int total_units;
+    int kb, c_blocks;                // channels per k-block, k-blocks per tap
+    int stages, swz;
+    int tmem_cols, acc_cols;         // allocation, columns per accumulator
+    int acc_bufs, acc_shift;         // accumulators in TMEM (2 or 4) and log2 of that: unit j uses accumulator j % acc_bufs
+    int vreuse;                      // a stage serves the three vertical taps of one horizontal shift
+    int fh;                          // full halo: a stage holds the tile with a one-pixel frame and serves all nine taps
+    int hm;                          // merged horizontal taps: one N = 3 x n_tile MMA per vertical tap and k-step, the three column blocks are
+                                     // shifted by one pixel and added in the epilogue (tiles of whole image rows, 64 output channels)
+    int mma_n;                       // UMMA N (n_tile, or 3 x n_tile with merged horizontal taps)
+    int nb;                          // B tiles per stage (1, or 3 with vreuse)
+    int b_merged;                    // the three B tiles of a stage come with one load (box of three filter rows)
+    int r_filter;                    // filter height = width
+    int a_bytes, b_bytes;            // shared-memory footprint of the A tile / one B tile (multiples of 1 KB)
+    int tx_a, tx_b;                  // bytes one A / B load delivers
+    int a_step;                      // byte offset of one image row inside the A tile (vreuse)
+    int issuers;                     // MMA-issuing threads at work (1 or 2)
+    int gsub;                        // k-blocks that share a ring slot, one barrier wait and one commit (short k-blocks: the waits would bound the issuing threads)
+    int issue_split;                 // the two issuing threads share every unit: alternate stages into one accumulator (tiles wider than 128 channels)
+    int splits;                      // split-K plans (conv_splitk.cu): CTAs (or CTA pairs) of a cluster that share a unit's k-blocks; 0: persistent kernel
+    int pair;                        // CTA pairs (cta_group::2): M = 256 per MMA, each CTA holds half of every B tile
+    int resident;                    // filter bank of this CTA's channel tile stays in shared memory
+    int resident_bytes;
+    int n_valid, oc_valid;           // images / output channels that exist
+    long long os_n, os_h, os_w;      // output element strides along the tile grid
+    long long off[4];                // output element offset per parity
+    void* out;
+    int out_is_f32;
+    int out_v8;                      // the output base is 32-byte aligned: bf16 chunks go out as one 256-bit store per lane
+    const float* bias;
+    double* stats;
+    int stats_group_images;          // images per BatchNorm statistics group (0: one group)
+    unsigned* status;
+    unsigned spin_limit;
+    unsigned long long* stall;       // optional [5]: cycles waited by producer / MMA (ring) / MMA (accumulator) / epilogue, CTA lifetime
+};
+
+struct UnitCoord {
+    int par, ktile, ow0, oh0, n0;
+};
+// tiles_w and tiles_h are powers of two (the grid sides are); the channel-tile count and the stats group size usually are
+__device__ __forceinline__ UnitCoord decode_unit(const ConvKParams& p, int u)
+{
+    UnitCoord c;
+    if (p.nk_shift >= 0) {
+        c.ktile = u & (p.n_ktiles - 1);
+        u >>= p.nk_shift;
+    } else {
+        c.ktile = u % p.n_ktiles;
+        u /= p.n_ktiles;
+    }
+    c.ow0 = (u & (p.tiles_w - 1)) * p.bw;
+    u >>= p.tw_shift;
+    c.oh0 = (u & (p.tiles_h - 1)) * p.bh;
+    u >>= p.th_shift;
+    if (p.n_par > 1) {
+        c.n0 = (u % p.tiles_n) * p.bn;
+        c.par = u / p.tiles_n;
+    } else {
+        c.n0 = u * p.bn;
+        c.par = 0;
+    }
+    return c;
+}
+
+// Clusters of `cluster` CTAs (pair: made of CTA pairs) that run at the same time on this context's device.
+int splitk_max_clusters(b2c_ctx* ctx, int cluster, bool pair);
+// Split-K plan: the parameter block, CTAs per cluster and in all, dynamic shared memory.
+b2c_status launch_conv_splitk(b2c_ctx* ctx, const ConvKParams& p, int grid, size_t smem_bytes, cudaStream_t stream);
+
+}  // namespace b2c

@@ -1,0 +1,392 @@
+// Implicit-GEMM convolution for problems with fewer output tiles than the chip has SMs: forward pass, data gradient and
+// classifier at small batches.
+//
+// The operands, tap tables and tile geometry are those of conv_kmajor.cu; what differs is the split of the work.  There, a
+// CTA owns a whole tile, so a layer with 16 tiles of 72 k-blocks runs 72 k-blocks in a row on 16 SMs (or pairs) and leaves
+// the rest idle: 512 -> 512 channels at 4x4 with 128 images took 28 us, of which 19.4 us were the 36.8 k cycles of one
+// pair's MMAs.  Here a cluster of `splits` CTAs (or CTA pairs) shares a tile: each accumulates its share of the k-blocks in
+// its own TMEM, then the partial tiles are added up through distributed shared memory, every CTA finishing one slice of the
+// columns.  Nothing is written to global memory but the result, so no workspace and no second launch are needed.
+//   * One tile per cluster, not persistent: barriers and TMEM are set up once, every warp joins the epilogue when the main
+//     loop has been issued, and the kernel is small (a launch inside a step starts on a cold instruction cache).
+//   * The exchange goes through the ring's memory, which is free once the MMAs of every CTA of the cluster have completed
+//     (first cluster barrier).  A lane holds one row, so a block of four columns is stored as 128 rows x 16 bytes:
+//     neighbouring lanes write neighbouring 16-byte words of the receiver.
+// What bounds it now: the operands' way from L2 (a pair with 256 channels stages 32 KB per 512 tensor-pipe cycles, the rate one
+// SM can load), then the set-up and the exchange, about 3 us together.  Inside a step (128 images, time to the next kernel's
+// start): 512 -> 512 at 4x4 33 -> 14 us, 256 -> 256 at 8x8 32 -> 13 us; the whole ResNet-18-shaped step 1.89 -> 1.73 ms, as four
+// micro-batches of 50 6.32 -> 5.41 ms.
+// Warp roles during the main loop: warp 0 = TMA producer, warp 1 = TMEM owner and MMA issuer.  Every mbarrier wait is
+// bounded; a CTA that gives up still takes part in both cluster barriers.
+#include "conv_kmajor.h"
+
+namespace b2c {
+
+static constexpr int kSkThreads = 256;
+static constexpr int kSkStages = 8;
+static constexpr uint32_t kSkDrainPolls = 1u << 22;
+
+template <bool PAIR>
+__device__ __forceinline__ void sk_issue(int ksteps, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate_first)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (k >= ksteps) break;
+        const uint64_t ad = ((uint64_t)desc_hi << 32) | (uint64_t)(a_lo + 2u * k), bd = ((uint64_t)desc_hi << 32) | (uint64_t)(b_lo + 2u * k);
+        if constexpr (PAIR) umma_bf16_pair(d_tmem, ad, bd, idesc, k == 0 ? accumulate_first : 1u);
+        else umma_bf16(d_tmem, ad, bd, idesc, k == 0 ? accumulate_first : 1u);
+    }
+}
+
+// Column sums over the 32 rows a warp holds: after it, lane l holds in a[0], b[0] the totals of column l >> 1.
+__device__ __forceinline__ void sk_column_sums(float (&a)[16], float (&b)[16], int lane)
+{
+#pragma unroll
+    for (int width = 8, bit = 16; width >= 1; width >>= 1, bit >>= 1) {
+        const bool upper = (lane & bit) != 0;
+#pragma unroll
+        for (int i = 0; i < width; ++i) {
+            const float sa = upper ? a[i] : a[i + width], ka = upper ? a[i + width] : a[i];
+            const float sb = upper ? b[i] : b[i + width], kb = upper ? b[i + width] : b[i];
+            a[i] = ka + __shfl_xor_sync(0xffffffffu, sa, bit);
+            b[i] = kb + __shfl_xor_sync(0xffffffffu, sb, bit);
+        }
+    }
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+    b[0] += __shfl_xor_sync(0xffffffffu, b[0], 1);
+}
+
+template <bool PAIR>
+__global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid_constant__ ConvKParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t full_bar[kSkStages], empty_bar[kSkStages], acc_bar, drain_bar;
+    __shared__ uint32_t tmem_slot, abort_flag;
+    __shared__ float s_sum[2][256];   // BatchNorm sums of this CTA's columns
+
+    // (the same offset in every CTA of the cluster: the exchange maps addresses from one CTA to another)
+    uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~uintptr_t(1023));
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int cta = p.splits * (PAIR ? 2 : 1) > 1 ? (int)cluster_ctarank() : 0;
+    const int rank = PAIR ? cta & 1 : 0;                // CTA of its pair: 0 issues the MMAs and owns the pair's barriers
+    const int split = PAIR ? cta >> 1 : cta;
+    const uint32_t leader = (uint32_t)(cta - rank);
+    const int S = p.stages, G = p.gsub;
+    const int sub_bytes = p.a_bytes + p.b_bytes, stage_bytes = G * sub_bytes;
+
+    // the unit of this cluster (a pair takes two neighbouring pixel tiles) and this CTA's share of its k-blocks
+    const int cluster_id = (int)blockIdx.x / (p.splits * (PAIR ? 2 : 1));
+    const UnitCoord c = decode_unit(p, PAIR ? (2 * (cluster_id / p.n_ktiles) + rank) * p.n_ktiles + cluster_id % p.n_ktiles : cluster_id);
+    const TapList& tl = p.taps[c.par];
+    const int k_total = tl.count * p.c_blocks;
+    const int k_begin = k_total * split / p.splits, k_count = k_total * (split + 1) / p.splits - k_begin;
+    const int n_slots = (k_count + G - 1) / G;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full_bar[s], 1);
+            mbar_init(&empty_bar[s], 1);
+        }
+        mbar_init(&acc_bar, 1);
+        mbar_init(&drain_bar, 1);
+        abort_flag = 0;
+        fence_mbar_init();
+    }
+    for (int i = threadIdx.x; i < 512; i += kSkThreads) (&s_sum[0][0])[i] = 0.f;
+    if (warp == 1) {
+        if constexpr (PAIR) {
+            tmem_alloc_pair(&tmem_slot, (uint32_t)p.tmem_cols);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(&tmem_slot, (uint32_t)p.tmem_cols);
+            tmem_relinquish();
+        }
+    } else if (warp == 0 && elect_one()) {
+        prefetch_tensormap(&p.tmB);
+        prefetch_tensormap(&p.tmA[tl.map[0]]);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();   // the peer's barriers exist before anything arrives on them
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_slot;
+    pdl_wait();
+    pdl_launch_dependents();
+
+    int issued = 0;   // producer warp: ring slots whose loads it has issued
+    if (warp == 0) {
+        const int R = p.r_filter, b_rows = PAIR ? p.n_tile >> 1 : p.n_tile;
+        const int oc0 = c.ktile * p.n_tile + rank * b_rows;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int it = 0; it < n_slots; ++it) {
+            if (!mbar_wait_warp(&empty_bar[s], ph ^ 1u, p.spin_limit, &abort_flag)) {
+                if (lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
+                break;
+            }
+            const int n_k = k_count - it * G < G ? k_count - it * G : G;
+            if (elect_one()) {
+                const uint32_t bar = PAIR ? map_to_cta(smem_u32(&full_bar[s]), leader) : 0u;
+                if (rank == 0) mbar_expect_tx(&full_bar[s], (PAIR ? 2u : 1u) * (uint32_t)(n_k * (p.tx_a + p.tx_b)));   // a pair counts both CTAs' bytes
+                for (int g = 0; g < n_k; ++g) {
+                    const int kblk = k_begin + it * G + g;
+                    const int tap = p.cb_shift >= 0 ? kblk >> p.cb_shift : kblk / p.c_blocks, cb = kblk - tap * p.c_blocks;
+                    const int rs = tl.rs[tap], fr = (rs * 11) >> 5;   // rs / 3 for rs < 9 (R is 1 or 3)
+                    uint8_t* dst = ring + (size_t)s * stage_bytes + (size_t)g * sub_bytes;
+                    if constexpr (PAIR) {
+                        tma_load_4d_pair(dst, &p.tmA[tl.map[tap]], bar, cb * p.kb, c.ow0 + tl.dw[tap], c.oh0 + tl.dh[tap], c.n0);
+                        tma_load_4d_pair(dst + p.a_bytes, &p.tmB, bar, cb * p.kb, rs - fr * R, oc0, fr);
+                    } else {
+                        tma_load_4d(dst, &p.tmA[tl.map[tap]], &full_bar[s], cb * p.kb, c.ow0 + tl.dw[tap], c.oh0 + tl.dh[tap], c.n0);
+                        tma_load_4d(dst + p.a_bytes, &p.tmB, &full_bar[s], cb * p.kb, rs - fr * R, oc0, fr);
+                    }
+                }
+            }
+            __syncwarp();
+            issued = it + 1;
+            if (++s == S) { s = 0; ph ^= 1u; }
+        }
+    } else if (warp == 1 && rank == 0) {
+        const uint32_t idesc = make_idesc_bf16(PAIR ? 256 : 128, p.n_tile, false, false);
+        const uint64_t proto = make_smem_desc(0u, 16u, 8u * (uint32_t)p.kb * 2u, (uint32_t)p.swz);   // eight rows of kb bf16
+        const uint32_t desc_hi = (uint32_t)(proto >> 32), ring_lo = (uint32_t)proto + (smem_u32(ring) >> 4);
+        const uint32_t a_to_b16 = (uint32_t)p.a_bytes >> 4, sub16 = (uint32_t)sub_bytes >> 4, stage16 = (uint32_t)stage_bytes >> 4;
+        const int ksteps = p.kb >> 4;
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int it = 0; it < n_slots; ++it) {
+            ok = mbar_wait_warp(&full_bar[s], ph, p.spin_limit, &abort_flag);
+            if (!ok) {
+                if (lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
+                break;
+            }
+            tc_fence_after();
+            const int n_k = k_count - it * G < G ? k_count - it * G : G;
+            if (elect_one()) {
+                uint32_t a_lo = ring_lo + (uint32_t)s * stage16;
+                for (int g = 0; g < n_k; ++g, a_lo += sub16)
+                    sk_issue<PAIR>(ksteps, tmem_base, a_lo, a_lo + a_to_b16, desc_hi, idesc, (it | g) != 0 ? 1u : 0u);
+                if constexpr (PAIR) umma_commit_pair(&empty_bar[s], (uint16_t)(3u << leader));
+                else umma_commit(&empty_bar[s]);
+            }
+            __syncwarp();
+            if (++s == S) { s = 0; ph ^= 1u; }
+        }
+        if (ok && n_slots > 0 && elect_one()) {
+            if constexpr (PAIR) umma_commit_pair(&acc_bar, (uint16_t)(3u << leader));
+            else umma_commit(&acc_bar);
+        }
+        __syncwarp();
+    }
+
+    // ---------------------------------------------------------------- epilogue: all eight warps
+    bool live = n_slots > 0;
+    if (live && !mbar_wait_warp(&acc_bar, 0u, p.spin_limit, &abort_flag)) {
+        if (lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
+        live = false;
+    }
+    tc_fence_before();
+    __syncthreads();
+    const bool clustered = PAIR || p.splits > 1;
+    if (clustered) cluster_sync_all();   // every CTA's MMAs have completed (or it has given up): the rings may be written by the others
+    if (abort_flag) {
+        // A wait gave up: let the bulk copies counted on this CTA's barriers land and its MMAs retire before it goes on.  (Results are
+        // unspecified now; every write still stays inside the cluster's rings and the output.)
+        if (warp == 0 && rank == 0)
+            for (int back = 0; back < S && back < issued; ++back) {
+                const int it = issued - 1 - back;
+                for (uint32_t i = 0; i < kSkDrainPolls && !__all_sync(0xffffffffu, mbar_try_wait(&full_bar[it % S], (uint32_t)(it / S) & 1u)); ++i) {}
+            }
+        if (warp == 1 && rank == 0) {
+            if (elect_one()) {
+                if constexpr (PAIR) umma_commit_pair(&drain_bar, (uint16_t)(1u << leader));
+                else umma_commit(&drain_bar);
+            }
+            __syncwarp();
+            for (uint32_t i = 0; i < kSkDrainPolls && !__all_sync(0xffffffffu, mbar_try_wait(&drain_bar, 0u)); ++i) {}
+        }
+        __syncthreads();
+    }
+    tc_fence_after();
+
+    const int q = warp & 3, half = warp >> 2;   // TMEM lane quarter of this warp, half of the columns
+    const int m = q * 32 + lane;                // accumulator row = pixel of the tile (w fastest, then h, then image)
+    const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
+    const int sw = p.n_tile / p.splits;         // columns this CTA finishes
+    const int col0 = split * sw;
+    const bool exchange = p.splits > 1 && k_total > 0;
+    if (exchange) {
+        // partial sums of the other CTAs' columns -> their rings: block (sender, four columns) = 128 rows x 16 bytes
+        const int n8 = sw >> 3, c_lo = half ? (n8 + 1) >> 1 : 0, c_hi = half ? n8 : (n8 + 1) >> 1;
+        const uint32_t mine = smem_u32(ring) + (uint32_t)(split * (sw >> 2) * 128 + m) * 16u;
+        for (int j = 1; j < p.splits; ++j) {
+            const int dst = split + j < p.splits ? split + j : split + j - p.splits;
+            const uint32_t base = map_to_cta(mine, (uint32_t)(PAIR ? 2 * dst + rank : dst));
+            for (int ch = c_lo; ch < c_hi; ch += 2) {
+                uint32_t r0[8], r1[8];
+                tmem_ld8(t_row + (uint32_t)(dst * sw + ch * 8), r0);
+                if (ch + 1 < c_hi) tmem_ld8(t_row + (uint32_t)(dst * sw + ch * 8 + 8), r1);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 8; i += 4)
+                    st_cluster_v4(base + (uint32_t)(2 * ch + i / 4) * 2048u, __uint_as_float(r0[i]), __uint_as_float(r0[i + 1]), __uint_as_float(r0[i + 2]), __uint_as_float(r0[i + 3]));
+                if (ch + 1 < c_hi) {
+#pragma unroll
+                    for (int i = 0; i < 8; i += 4)
+                        st_cluster_v4(base + (uint32_t)(2 * ch + 2 + i / 4) * 2048u, __uint_as_float(r1[i]), __uint_as_float(r1[i + 1]), __uint_as_float(r1[i + 2]),
+                                      __uint_as_float(r1[i + 3]));
+                }
+            }
+        }
+    }
+    if (clustered) cluster_sync_all();   // the partial sums have arrived; nobody reads or writes another CTA's memory after this
+
+    const int lw = m % p.bw, lh = (m / p.bw) % p.bh, ln = m / (p.bw * p.bh);
+    const bool row_valid = c.n0 + ln < p.n_valid;
+    const long long row_off = (long long)(c.n0 + ln) * p.os_n + (long long)(c.oh0 + lh) * p.os_h + (long long)(c.ow0 + lw) * p.os_w + p.off[c.par];
+    const bool do_stats = p.stats != nullptr;
+    // 16 columns at a time (the last step of an odd count of eights takes 8)
+    const int n16 = (sw + 15) >> 4, g_lo = half ? (n16 + 1) >> 1 : 0, g_hi = half ? n16 : (n16 + 1) >> 1;
+    for (int g = g_lo; g < g_hi; ++g) {
+        const bool wide = g * 16 + 16 <= sw;
+        uint32_t r[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) r[i] = 0u;
+        if (k_total > 0) {
+            uint32_t lo[8], hi[8];
+            tmem_ld8(t_row + (uint32_t)(col0 + g * 16), lo);
+            if (wide) tmem_ld8(t_row + (uint32_t)(col0 + g * 16 + 8), hi);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                r[i] = lo[i];
+                r[8 + i] = wide ? hi[i] : 0u;
+            }
+        }
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+        if (exchange) {
+            for (int src = 0; src < p.splits; ++src) {
+                if (src == split) continue;
+                const float4* in = reinterpret_cast<const float4*>(ring) + (size_t)(src * (sw >> 2) + 4 * g) * 128 + m;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i < 2 || wide) {
+                        const float4 f = in[i * 128];
+                        v[4 * i] += f.x;
+                        v[4 * i + 1] += f.y;
+                        v[4 * i + 2] += f.z;
+                        v[4 * i + 3] += f.w;
+                    }
+                }
+            }
+        }
+        const int ch0 = c.ktile * p.n_tile + col0 + g * 16;
+        if (p.bias != nullptr) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (i < 8 || wide) v[i] += __ldg(p.bias + ch0 + i);
+        }
+        if (p.out_is_f32) {
+            if (row_valid) {
+                float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + row_off + ch0);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < 2 || wide) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            }
+            continue;
+        }
+        uint32_t pk[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) pk[i] = pack_bf16x2(v[2 * i], v[2 * i + 1]);
+        if (row_valid) {
+            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + row_off + ch0;
+            if (p.out_v8 && wide && (ch0 & 15) == 0) {
+                st_global_v8(dst, pk);
+            } else {
+                *reinterpret_cast<uint4*>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                if (wide) *reinterpret_cast<uint4*>(dst + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+            }
+        }
+        if (do_stats) {   // sums of the values as stored
+            float a[16], b[16];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162*>(&pk[i]);
+                a[2 * i] = row_valid ? __low2float(h) : 0.f;
+                a[2 * i + 1] = row_valid ? __high2float(h) : 0.f;
+                b[2 * i] = a[2 * i] * a[2 * i];
+                b[2 * i + 1] = a[2 * i + 1] * a[2 * i + 1];
+            }
+            sk_column_sums(a, b, lane);
+            if ((lane & 1) == 0) {   // the four lane quarters meet in shared memory
+                atomicAdd(&s_sum[0][g * 16 + (lane >> 1)], a[0]);
+                atomicAdd(&s_sum[1][g * 16 + (lane >> 1)], b[0]);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (do_stats) {
+        const int grp = p.stats_group_images > 0 ? c.n0 / p.stats_group_images : 0;
+        double* st = p.stats + (size_t)grp * 2 * p.oc_valid + c.ktile * p.n_tile + col0;
+        if (c.n0 < p.n_valid)   // (the second tile of a pair may lie past the last image)
+            for (int i = threadIdx.x; i < sw; i += kSkThreads) {
+                atomicAdd(st + i, (double)s_sum[0][i]);
+                atomicAdd(st + p.oc_valid + i, (double)s_sum[1][i]);
+            }
+    }
+    if (warp == 1) {
+        tc_fence_after();
+        if constexpr (PAIR) tmem_dealloc_pair(tmem_base, (uint32_t)p.tmem_cols);
+        else tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
+    }
+    if constexpr (PAIR) cluster_sync_all();   // a pair gives its TMEM back together
+}
+
+static b2c_status splitk_optin(b2c_ctx* ctx)
+{
+    if (!(ctx->smem_optin_done & B2C_OPTIN_SPLITK)) {
+        B2C_CUDA(cudaFuncSetAttribute(conv_splitk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
+        B2C_CUDA(cudaFuncSetAttribute(conv_splitk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
+        ctx->smem_optin_done |= B2C_OPTIN_SPLITK;
+    }
+    return B2C_OK;
+}
+
+int splitk_max_clusters(b2c_ctx* ctx, int cluster, bool pair)
+{
+    if (cluster == 1) return ctx->sm_count;
+    int& known = ctx->max_clusters[pair ? 1 : 0][cluster];   // a property of the device: asked once per context
+    if (known < 0) {
+        known = 0;
+        if (splitk_optin(ctx) != B2C_OK) return 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)cluster);
+        cfg.blockDim = dim3(kSkThreads);
+        cfg.dynamicSmemBytes = 217 * 1024;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)cluster;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, pair ? conv_splitk_kernel<true> : conv_splitk_kernel<false>, &cfg) == cudaSuccess) known = n;
+    }
+    return known;
+}
+
+b2c_status launch_conv_splitk(b2c_ctx* ctx, const ConvKParams& p, int grid, size_t smem_bytes, cudaStream_t stream)
+{
+    b2c_status st = splitk_optin(ctx);
+    if (st != B2C_OK) return st;
+    const unsigned cluster = (unsigned)(p.splits * (p.pair ? 2 : 1));
+    B2C_CUDA(b2c_launch(ctx, p.pair ? conv_splitk_kernel<true> : conv_splitk_kernel<false>, dim3((unsigned)grid), dim3(kSkThreads), smem_bytes, stream, cluster, p));
+    B2C_CUDA(cudaGetLastError());
+    return B2C_OK;
+}
+
+}  // namespace b2c

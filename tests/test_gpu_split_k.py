@@ -1,0 +1,88 @@
+"""Small problems (fewer tiles than SMs) through both kernels that serve them: clusters sharing a tile's k-blocks
+(B2C_SPLIT_K=1, the default) and the persistent kernel (0), against the oracle at the per-tensor budget."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2503_23186_b200 import workloads as wl
+from parity import assert_close, dev_bf16, dev_f32, host
+
+pytestmark = pytest.mark.gpu
+
+# an odd number of tiles on pairs, one tile split eight ways, slices of 8 / 20 x 8 columns, 16- and 32-channel k-blocks, output parities
+# with and without taps, more splits than a ragged share of k-blocks, several images per tile with a ragged last one
+SHAPES = [(50, 4, 4, 512, 512, 3, 1), (8, 4, 4, 256, 64, 3, 1), (3, 8, 8, 32, 32, 3, 1), (8, 32, 32, 16, 16, 3, 1), (2, 16, 16, 160, 160, 3, 1),
+          (8, 8, 8, 128, 256, 3, 2), (8, 8, 8, 128, 256, 1, 2), (5, 16, 16, 32, 64, 3, 2), (6, 8, 8, 48, 96, 3, 1), (16, 8, 8, 2048, 512, 1, 1), (7, 4, 4, 640, 320, 3, 1)]
+
+
+@pytest.fixture(scope="module", params=["0", "1"], ids=["persistent", "split-k"])
+def ctx(request):
+    import os
+    from paper_2503_23186_b200 import binding
+    before = os.environ.get("B2C_SPLIT_K")
+    os.environ["B2C_SPLIT_K"] = request.param
+    try:
+        c = binding.Context(0)
+    finally:
+        if before is None:
+            del os.environ["B2C_SPLIT_K"]
+        else:
+            os.environ["B2C_SPLIT_K"] = before
+    yield c
+    assert c.device_status() == 0
+    c.close()
+
+
+def _desc(N, H, W, C, K, R, st):
+    from paper_2503_23186_b200 import binding
+    return binding.conv_desc(N, H, W, C, K, R, st)
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
+def test_forward_statistics_and_data_gradient(ctx, shape):
+    N, H, W, C, K, R, st = shape
+    x, w, g = wl.conv_problem(40, *shape)
+    pad, P = (R - 1) // 2, H // st
+    y = torch.full((N, P, P, K), float("nan"), dtype=torch.bfloat16, device="cuda")
+    stats = torch.zeros(2 * K, dtype=torch.float64, device="cuda")
+    ctx.conv2d_fwd(_desc(*shape), dev_bf16(x), dev_bf16(w), y, ch_stats=stats)
+    wd = torch.empty(w.size, dtype=torch.bfloat16, device="cuda")
+    ctx.weight_pack_dgrad([(0, K, R * R, C)], dev_bf16(w).reshape(-1), wd)
+    dx = torch.full(x.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+    ctx.conv2d_dgrad(_desc(*shape), dev_bf16(g), wd, dx)
+    assert ctx.device_status() == 0
+    assert_close(y, oracle.conv2d_fwd(x, w, st, pad), "y")
+    assert_close(dx, oracle.conv2d_dgrad(g, w, x.shape, st, pad), "dx")
+    ys = host(y).reshape(-1, K)   # sums of the stored values: fp32 over a tile's rows, fp64 across tiles
+    np.testing.assert_allclose(host(stats)[:K], ys.sum(0), rtol=1e-5, atol=1e-3 * np.sqrt(ys.shape[0]))
+    np.testing.assert_allclose(host(stats)[K:], (ys * ys).sum(0), rtol=1e-5)
+
+
+def test_classifier_with_bias(ctx):
+    shape = (70, 1, 1, 512, 128, 1, 1)
+    x, w, _ = wl.conv_problem(41, *shape)
+    bias = wl.rng_for(41, "bias").standard_normal(128).astype(np.float32)
+    y = torch.full((70, 1, 1, 128), float("nan"), dtype=torch.float32, device="cuda")
+    ctx.conv2d_fwd(_desc(*shape), dev_bf16(x), dev_bf16(w), y, bias=dev_f32(bias))
+    assert ctx.device_status() == 0
+    assert_close(y, oracle.conv2d_fwd(x, w, 1, 0) + bias, "logits", 1e-5, 1e-5)   # fp32 output: accumulation error only
+
+
+@pytest.mark.parametrize("shape", [(50, 4, 4, 512, 512, 3, 1), (8, 8, 8, 128, 256, 3, 2), (8, 32, 32, 64, 64, 3, 1)], ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
+def test_winds_down_on_timeout(ctx, shape):
+    """A poll budget of one: the status word reports it, every CTA of the cluster leaves, the next launch is correct."""
+    N, H, W, C, K, R, st = shape
+    x, w, _ = wl.conv_problem(42, *shape)
+    y = torch.zeros((N, H // st, W // st, K), dtype=torch.bfloat16, device="cuda")
+    X, Wt = dev_bf16(x), dev_bf16(w)
+    ctx.set_spin_limit(1)
+    try:
+        ctx.conv2d_fwd(_desc(*shape), X, Wt, y)
+        status = ctx.device_status()
+    finally:
+        ctx.set_spin_limit(1 << 22)
+    assert status == 7   # B2C_ERR_DEVICE_TIMEOUT
+    ctx.conv2d_fwd(_desc(*shape), X, Wt, y)
+    assert ctx.device_status() == 0
+    assert_close(y, oracle.conv2d_fwd(x, w, st, 1), "y after recovery")
