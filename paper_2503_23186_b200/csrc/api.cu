@@ -619,11 +619,9 @@ b2c_status b2c_net_apply_update(b2c_net* net, int n_avg, float lr, float momentu
 {
     if (!net || !net->ws || n_avg < 1) return B2C_ERR_INVALID_ARG;
     cudaStream_t stream = (cudaStream_t)stream_;
-    ProfScope ps_(net, stream, B2C_PROF_UPDATE, 2);
-    b2c_status st = b2c_grad_accum_sgd_momentum(net->ctx, net->param_count, net->w, net->v, net->g, 1.f / (float)n_avg, lr, momentum, wd,
-                                                net->w_bf16, 1, stream_);
-    if (st != B2C_OK) return st;
-    return net_pack_dgrad(net, stream_);
+    ProfScope ps_(net, stream, B2C_PROF_UPDATE, 1);
+    return launch_update_pack(net->ctx, net->segs.data(), (int)net->segs.size(), net->param_count, net->w, net->v, net->g, 1.f / (float)n_avg, lr, momentum, wd,
+                              net->w_bf16, net->w_dgrad, stream);
 }
 
 #define B2C_TRY(call)                   \

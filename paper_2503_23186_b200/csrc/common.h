@@ -147,6 +147,11 @@ b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da
                          const float* gamma, const float* save_mean, const float* save_invstd, int relu, void* dy, void* dres, float* dgamma,
                          float* dbeta, int acc, double* sums, bool sums_zeroed, const void* relu_mask, unsigned* arrivals, cudaStream_t stream);
 
+// Average + SGD-momentum update of `count` elements, gradient sums cleared, and both bf16 copies, in one launch.  The segments (filter banks)
+// lie back to back from element 0 and their sizes are multiples of 8; elements behind the last one have no data-gradient layout.
+b2c_status launch_update_pack(b2c_ctx* ctx, const b2c_weight_seg* segs, int n_segs, size_t count, float* w, float* v, float* g, float inv_n, float lr, float momentum,
+                              float wd, void* w_bf16, void* w_dgrad, cudaStream_t stream);
+
 // Running statistics of the BatchNorm layers of a step (momentum update with the unbiased variance), taken from the fp64
 // sums the forward pass left in the workspace.  One entry per layer; the G statistics groups of a pass are applied in
 // order, as if the micro-batches had run one after the other.

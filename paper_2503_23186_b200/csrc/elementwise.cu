@@ -1149,7 +1149,8 @@ struct PackSegs {
 };
 // dst[c][rs-1-t][k] = src[k][t][c] per segment: for a fixed tap this is a k x c -> c x k transpose, done in 32 x 32
 // tiles through shared memory so that both the reads (c contiguous) and the writes (k contiguous) are coalesced.
-// One block per (segment, tap, tile of the (k, c) plane), numbered consecutively over all segments.
+// One block per (segment, tap, tile of the (k, c) plane), numbered consecutively over all segments.  Serves segments whose sizes rule
+// out the vectors of update_pack_kernel.
 __global__ void weight_pack_dgrad_kernel(const __grid_constant__ PackSegs segs, const __nv_bfloat16* __restrict__ src,
                                          __nv_bfloat16* __restrict__ dst)
 {
@@ -1176,6 +1177,115 @@ __global__ void weight_pack_dgrad_kernel(const __grid_constant__ PackSegs segs, 
     for (int j = threadIdx.y; j < 32; j += 8) {
         const int c = c0 + j, k = k0 + threadIdx.x;
         if (c < sg.c && k < sg.k) dst[sg.offset + ((long long)c * sg.rs + (sg.rs - 1 - t)) * sg.k + k] = tile[threadIdx.x][j];
+    }
+}
+
+// The update of a whole network in one pass: average + momentum + weight decay (sgd_momentum_kernel's arithmetic), the bf16 copy and its
+// tap-flipped [c][r][s][k] copy, whose elements are transposed through shared memory while they are in registers.
+// Bound: HBM, 28 bytes per parameter.  A block takes a 64 x 64 tile of one tap's (k, c) plane: rows of 64 fp32 values are 256-byte
+// runs, columns of 64 bf16 values leave as 128-byte runs, and a thread has four 16-byte loads per array in flight.  The separate
+// transposing pass read the bf16 copy back in 64-byte runs with two-byte accesses: 23.7 M parameters took 107 us (update) +
+// 80 us (transposition) against 105 us now, of which the bytes account for 101 us at the copy rate.
+// UPDATE false: the transposition alone, from the bf16 copy (segments whose k, c and offset are multiples of 8).
+// Elements past the last filter bank (BatchNorm and bias parameters) have no transposed copy: the last blocks take 4096 each.
+static constexpr int kUpTile = 64;
+static constexpr int kUpPitch = kUpTile + 2;   // bf16 elements per row of the transposed tile: two-way conflicts on the way in, none on the way out
+struct UpdateArgs {
+    float *w, *v, *g;
+    __nv_bfloat16 *w_bf16, *w_dgrad;
+    long long tail_begin, tail_end;   // elements without a transposed copy
+    int tail_block;                   // first block of the tail
+    float inv_n, lr, mu, wd;
+};
+__device__ __forceinline__ void sgd_element(float& w, float& v, float g_sum, const UpdateArgs& a)
+{
+    const float g = fmaf(a.wd, w, g_sum * a.inv_n);   // g = g_sum*inv_n + wd*w
+    v = fmaf(a.mu, v, g);                            // v = mu*v + g
+    w = fmaf(-a.lr, v, w);                           // w = w - lr*v
+}
+__device__ __forceinline__ uint2 sgd_vector(const UpdateArgs& a, float4 w, float4 v, float4 g, long long e)
+{
+    sgd_element(w.x, v.x, g.x, a);
+    sgd_element(w.y, v.y, g.y, a);
+    sgd_element(w.z, v.z, g.z, a);
+    sgd_element(w.w, v.w, g.w, a);
+    *reinterpret_cast<float4*>(a.w + e) = w;
+    *reinterpret_cast<float4*>(a.v + e) = v;
+    *reinterpret_cast<float4*>(a.g + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint2 b = make_uint2(pack_bf16x2(w.x, w.y), pack_bf16x2(w.z, w.w));
+    *reinterpret_cast<uint2*>(a.w_bf16 + e) = b;
+    return b;
+}
+template <bool UPDATE>
+__global__ void __launch_bounds__(kEwThreads) update_pack_kernel(const __grid_constant__ PackSegs segs, const __grid_constant__ UpdateArgs a)
+{
+    pdl_wait();   // first global access comes after the previous kernel of the stream
+    pdl_launch_dependents();
+    __shared__ __nv_bfloat16 tile[kUpTile * kUpPitch];
+    constexpr int V = kUpTile * kUpTile / 4 / kEwThreads;   // 4-element vectors per thread
+    if (UPDATE && (int)blockIdx.x >= a.tail_block) {
+        const long long first = a.tail_begin + ((long long)blockIdx.x - a.tail_block) * (kUpTile * kUpTile) + 4 * (int)threadIdx.x;
+        for (int u = 0; u < V; ++u) {
+            const long long e = first + 4ll * u * kEwThreads;
+            if (e < a.tail_end)
+                sgd_vector(a, *reinterpret_cast<const float4*>(a.w + e), *reinterpret_cast<const float4*>(a.v + e), *reinterpret_cast<const float4*>(a.g + e), e);
+        }
+        return;
+    }
+    int lo = 0, hi = segs.n_segs;   // binary search for the segment of this block
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if ((int)blockIdx.x >= segs.first_block[mid]) lo = mid;
+        else hi = mid;
+    }
+    const b2c_weight_seg sg = segs.seg[lo];
+    // taps are the fastest index: the blocks in flight read neighbouring runs of the same filter rows
+    const int local = (int)blockIdx.x - segs.first_block[lo], tiles_c = (sg.c + kUpTile - 1) / kUpTile;
+    const int tile_id = local / sg.rs, t = local - tile_id * sg.rs;
+    const int k0 = tile_id / tiles_c * kUpTile, c0 = tile_id % tiles_c * kUpTile;
+    const int c = c0 + 4 * ((int)threadIdx.x & 15), row = (int)threadIdx.x >> 4;   // 16 threads per row of 64, 16 rows per step
+    long long e[V];
+    bool ok[V];
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+        const int k = k0 + row + 16 * u;
+        ok[u] = k < sg.k && c < sg.c;
+        e[u] = sg.offset + ((long long)k * sg.rs + t) * sg.c + c;
+    }
+    uint2 b[V];
+    if constexpr (UPDATE) {
+        float4 w[V], v[V], g[V];
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            if (ok[u]) {
+                w[u] = *reinterpret_cast<const float4*>(a.w + e[u]);
+                v[u] = *reinterpret_cast<const float4*>(a.v + e[u]);
+                g[u] = *reinterpret_cast<const float4*>(a.g + e[u]);
+            }
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            if (ok[u]) b[u] = sgd_vector(a, w[u], v[u], g[u], e[u]);
+    } else {
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            if (ok[u]) b[u] = *reinterpret_cast<const uint2*>(a.w_bf16 + e[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < V; ++u)
+        if (ok[u]) {
+            const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&b[u]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) tile[(c - c0 + i) * kUpPitch + row + 16 * u] = h[i];
+        }
+    __syncthreads();
+    const int kv = 8 * ((int)threadIdx.x & 7), rc = (int)threadIdx.x >> 3;   // 8 threads per transposed row, 32 rows per step
+#pragma unroll
+    for (int u = 0; u < kUpTile / 32; ++u) {
+        const int cc = rc + 32 * u;
+        if (c0 + cc < sg.c && k0 + kv < sg.k) {
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(&tile[cc * kUpPitch + kv]);
+            *reinterpret_cast<uint4*>(a.w_dgrad + sg.offset + ((long long)(c0 + cc) * sg.rs + (sg.rs - 1 - t)) * sg.k + k0 + kv) = make_uint4(src[0], src[1], src[2], src[3]);
+        }
     }
 }
 
@@ -1245,6 +1355,41 @@ b2c_status launch_bn_running_update(b2c_ctx* ctx, const BnRunEntry* entries, int
         for (int i = 0; i < n; ++i) tab.e[i] = entries[first + i];
         B2C_CUDA(b2c_launch(ctx, bn_running_update_kernel, dim3((unsigned)n), dim3(128), 0, stream, 1u, tab, ws, run, G, momentum));
     }
+    B2C_CUDA(cudaGetLastError());
+    return B2C_OK;
+}
+
+// Numbers the 64 x 64 tiles of the segments' taps; false if a segment's sizes do not allow 16-byte vectors in both layouts.
+static bool tile_segments(const b2c_weight_seg* segs, int n_segs, PackSegs& ps)
+{
+    long long blocks = 0;
+    for (int i = 0; i < n_segs; ++i) {
+        if (segs[i].k % 8 || segs[i].c % 8 || segs[i].offset % 8) return false;
+        ps.seg[i] = segs[i];
+        ps.first_block[i] = (int)blocks;
+        blocks += (long long)segs[i].rs * ((segs[i].k + kUpTile - 1) / kUpTile) * ((segs[i].c + kUpTile - 1) / kUpTile);
+        if (blocks > 0x7fffffffll) return false;
+    }
+    ps.first_block[n_segs] = (int)blocks;
+    ps.n_segs = n_segs;
+    return true;
+}
+
+b2c_status launch_update_pack(b2c_ctx* ctx, const b2c_weight_seg* segs, int n_segs, size_t count, float* w, float* v, float* g, float inv_n, float lr, float momentum,
+                              float wd, void* w_bf16, void* w_dgrad, cudaStream_t stream)
+{
+    PackSegs ps;
+    if (!tile_segments(segs, n_segs, ps)) return B2C_ERR_UNSUPPORTED_SHAPE;
+    UpdateArgs a{};
+    a.w = w; a.v = v; a.g = g;
+    a.w_bf16 = reinterpret_cast<__nv_bfloat16*>(w_bf16); a.w_dgrad = reinterpret_cast<__nv_bfloat16*>(w_dgrad);
+    const b2c_weight_seg& last = segs[n_segs - 1];   // the filter banks lie back to back from offset 0, everything else behind them
+    a.tail_begin = last.offset + (long long)last.k * last.rs * last.c;
+    a.tail_end = (long long)count;
+    a.tail_block = ps.first_block[n_segs];
+    a.inv_n = inv_n; a.lr = lr; a.mu = momentum; a.wd = wd;
+    const long long blocks = a.tail_block + (a.tail_end - a.tail_begin + kUpTile * kUpTile - 1) / (kUpTile * kUpTile);
+    B2C_CUDA(b2c_launch(ctx, update_pack_kernel<true>, dim3((unsigned)blocks), dim3(kEwThreads), 0, stream, 1u, ps, a));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;
 }
@@ -1514,9 +1659,19 @@ b2c_status b2c_weight_pack_dgrad(b2c_ctx* ctx, const b2c_weight_seg* segs, int n
     if (!ctx || !segs || !src_bf16 || !dst_bf16) return B2C_ERR_INVALID_ARG;
     if (n_segs < 1 || n_segs > 128) return B2C_ERR_UNSUPPORTED_SHAPE;
     PackSegs ps;
+    const bool vectors = b2c_aligned16(src_bf16) && b2c_aligned16(dst_bf16);
+    for (int i = 0; i < n_segs; ++i)
+        if (segs[i].k < 1 || segs[i].rs < 1 || segs[i].c < 1 || segs[i].offset < 0) return B2C_ERR_INVALID_ARG;
+    if (vectors && tile_segments(segs, n_segs, ps)) {
+        UpdateArgs a{};
+        a.w_bf16 = const_cast<__nv_bfloat16*>(reinterpret_cast<const __nv_bfloat16*>(src_bf16));   // only read
+        a.w_dgrad = reinterpret_cast<__nv_bfloat16*>(dst_bf16);
+        B2C_CUDA(b2c_launch(ctx, update_pack_kernel<false>, dim3((unsigned)ps.first_block[n_segs]), dim3(kEwThreads), 0, (cudaStream_t)stream_, 1u, ps, a));
+        B2C_CUDA(cudaGetLastError());
+        return B2C_OK;
+    }
     long long blocks = 0;
     for (int i = 0; i < n_segs; ++i) {
-        if (segs[i].k < 1 || segs[i].rs < 1 || segs[i].c < 1 || segs[i].offset < 0) return B2C_ERR_INVALID_ARG;
         ps.seg[i] = segs[i];
         ps.first_block[i] = (int)blocks;
         blocks += (long long)segs[i].rs * ((segs[i].k + 31) / 32) * ((segs[i].c + 31) / 32);
