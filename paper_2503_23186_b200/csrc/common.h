@@ -5,7 +5,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <string>
 #include <unordered_map>
 #include <vector>
 
@@ -18,6 +17,27 @@
 typedef CUresult (*b2c_encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                         const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                         CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// What a launch plan depends on, as words that compare and hash in a few instructions (the look-up is on the path of every launch).
+struct b2c_plan_key {
+    unsigned long long w[16];
+    bool operator==(const b2c_plan_key& o) const
+    {
+        unsigned long long d = 0;
+        for (int i = 0; i < 16; ++i) d |= w[i] ^ o.w[i];
+        return d == 0;
+    }
+};
+struct b2c_plan_key_hash {
+    size_t operator()(const b2c_plan_key& k) const
+    {
+        unsigned long long h = 0x9e3779b97f4a7c15ull;
+        for (int i = 0; i < 16; ++i) h = (h ^ k.w[i]) * 0x100000001b3ull + (h >> 29);
+        return (size_t)(h ^ (h >> 32));
+    }
+};
+static inline unsigned long long b2c_key_pair(int a, int b) { return ((unsigned long long)(unsigned)a << 32) | (unsigned)b; }
+static inline unsigned long long b2c_key_ptr(const void* p) { return (unsigned long long)reinterpret_cast<uintptr_t>(p); }
 
 struct b2c_ctx {
     int device;
@@ -38,9 +58,9 @@ struct b2c_ctx {
     int use_wgrad_two_issuers;           // weight gradient: two MMA-issuing threads on alternate chunks of one accumulator where the ring depth is even
     int use_bn_grouped;                  // BatchNorm backward of the training step: both passes in one cooperative launch, group by group
     // Launch plans (kernel parameter blocks with their tensor maps, grid and shared-memory size) of the convolution
-    // kernels, keyed by the bytes of the problem description: pointers and shapes of a bound network repeat every
+    // kernels, keyed by the problem description: pointers and shapes of a bound network repeat every
     // step, so a plan is built once and its launches cost one parameter copy.
-    std::unordered_map<std::string, std::vector<unsigned char>> plan_cache;
+    std::unordered_map<b2c_plan_key, std::vector<unsigned char>, b2c_plan_key_hash> plan_cache;
     unsigned smem_optin_done;            // kernels whose dynamic shared-memory opt-in was set on this context's device (B2C_OPTIN_* bits)
 };
 #define B2C_OPTIN_KMAJOR 1u

@@ -1337,22 +1337,13 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     return B2C_OK;
 }
 
-// Appends the bytes of a value to a cache key.
-template <typename T>
-static inline void key_add(std::string& key, const T& v)
-{
-    key.append(reinterpret_cast<const char*>(&v), sizeof(T));
-}
-
 b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_t stream)
 {
     // plans are keyed by everything the planner reads: the problem and the context's switches
-    std::string key("K");
-    key_add(key, pb.n); key_add(key, pb.ih); key_add(key, pb.iw); key_add(key, pb.ic); key_add(key, pb.oh); key_add(key, pb.ow); key_add(key, pb.oc);
-    key_add(key, pb.r); key_add(key, pb.stride); key_add(key, pb.pad); key_add(key, pb.dgrad); key_add(key, pb.in); key_add(key, pb.wt);
-    key_add(key, pb.out); key_add(key, pb.out_f32); key_add(key, pb.bias); key_add(key, pb.stats); key_add(key, pb.stats_group_images);
-    key_add(key, ctx->use_pairs); key_add(key, ctx->use_full_halo); key_add(key, ctx->use_issue_split); key_add(key, ctx->use_hmerge); key_add(key, ctx->use_group_kblocks);
-    key_add(key, ctx->use_split_k);
+    const int switches = ctx->use_pairs | ctx->use_full_halo << 4 | ctx->use_issue_split << 5 | ctx->use_hmerge << 6 | ctx->use_group_kblocks << 7 | ctx->use_split_k << 8;
+    const b2c_plan_key key = {{b2c_key_pair('K', switches), b2c_key_pair(pb.n, pb.stats_group_images), b2c_key_pair(pb.ih, pb.iw), b2c_key_pair(pb.oh, pb.ow),
+                               b2c_key_pair(pb.ic, pb.oc), b2c_key_pair(pb.r, pb.stride), b2c_key_pair(pb.pad, pb.dgrad | pb.out_f32 << 1), b2c_key_ptr(pb.in),
+                               b2c_key_ptr(pb.wt), b2c_key_ptr(pb.out), b2c_key_ptr(pb.bias), b2c_key_ptr(pb.stats)}};
     auto it = ctx->plan_cache.find(key);
     if (it == ctx->plan_cache.end()) {
         KMajorPlan fresh;
@@ -1361,7 +1352,7 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
         if (ctx->plan_cache.size() >= 8192) ctx->plan_cache.clear();   // callers that pass new buffers every call: keep the table bounded
         std::vector<unsigned char> bytes(sizeof(KMajorPlan));
         memcpy(bytes.data(), &fresh, sizeof(KMajorPlan));
-        it = ctx->plan_cache.emplace(std::move(key), std::move(bytes)).first;
+        it = ctx->plan_cache.emplace(key, std::move(bytes)).first;
     }
     KMajorPlan plan;   // a copy: the 64-byte alignment of the tensor maps is the parameter block's, not the table's
     memcpy(&plan, it->second.data(), sizeof(KMajorPlan));

@@ -562,18 +562,11 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     return B2C_OK;
 }
 
-template <typename T>
-static inline void key_add(std::string& key, const T& v)
-{
-    key.append(reinterpret_cast<const char*>(&v), sizeof(T));
-}
-
 b2c_status launch_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, cudaStream_t stream)
 {
-    std::string key("W");
-    key_add(key, pb.n); key_add(key, pb.h); key_add(key, pb.w); key_add(key, pb.c); key_add(key, pb.p); key_add(key, pb.q); key_add(key, pb.k);
-    key_add(key, pb.r); key_add(key, pb.stride); key_add(key, pb.pad); key_add(key, pb.dy); key_add(key, pb.x); key_add(key, pb.dw);
-    key_add(key, ctx->use_wgrad_frame); key_add(key, ctx->use_wgrad_two_issuers); key_add(key, ctx->use_group_kblocks);
+    const int switches = ctx->use_wgrad_frame | ctx->use_wgrad_two_issuers << 1 | ctx->use_group_kblocks << 2;
+    const b2c_plan_key key = {{b2c_key_pair('W', switches), b2c_key_pair(pb.n, pb.c), b2c_key_pair(pb.h, pb.w), b2c_key_pair(pb.p, pb.q), b2c_key_pair(pb.k, pb.r),
+                               b2c_key_pair(pb.stride, pb.pad), b2c_key_ptr(pb.dy), b2c_key_ptr(pb.x), b2c_key_ptr(pb.dw)}};
     auto it = ctx->plan_cache.find(key);
     if (it == ctx->plan_cache.end()) {
         WgradPlan fresh;
@@ -582,7 +575,7 @@ b2c_status launch_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, cudaStream_t 
         if (ctx->plan_cache.size() >= 8192) ctx->plan_cache.clear();
         std::vector<unsigned char> bytes(sizeof(WgradPlan));
         memcpy(bytes.data(), &fresh, sizeof(WgradPlan));
-        it = ctx->plan_cache.emplace(std::move(key), std::move(bytes)).first;
+        it = ctx->plan_cache.emplace(key, std::move(bytes)).first;
     }
     WgradPlan plan;
     memcpy(&plan, it->second.data(), sizeof(WgradPlan));
