@@ -36,7 +36,7 @@
  *       B2C_BN_GROUPED=1     b2c_train_step runs the BatchNorm backward as one cooperative launch per layer, group by group
  *                            (b2c_bn_relu_bwd_groups); off by default: measured slower inside the step
  *       B2C_FUSE_WIDE=0|1    BatchNorm statistics of tiles wider than 64 channels: never | always in the convolution epilogue
- *                            (default: where the unit's MMAs take longer than the epilogue's column sums)
+ *                            (default: where the epilogue's sums cost less than a pass of their own)
  *       B2C_FUSE_BN_STATS=0  BatchNorm statistics by a separate pass instead of the convolution epilogue (b2c_train_step)
  *       B2C_CHUNK_MB=<n>     b2c_train_step takes layers whose tensors exceed n MB a few micro-batches at a time (0 = off, default)
  */

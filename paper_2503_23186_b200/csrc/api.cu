@@ -442,22 +442,28 @@ b2c_status b2c_net_create_concurrent(b2c_ctx* ctx, const b2c_layer_desc* layers,
         if (L.d.kind == B2C_LAYER_CONV) {
             TensorPlan& o = net->tensors[i + 1];
             o.stats_off = alloc(16 * (size_t)L.d.k * n_concurrent);
-            // the epilogue can own the statistics only if no 128-pixel tile straddles two micro-batches
+            // The epilogue can own the statistics unless a 128-pixel tile straddles two micro-batches of a pass.
             const int pix = L.p * L.q;
             const int imgs_per_tile = pix >= 128 ? 1 : 128 / pix;
-            o.fused_stats = net->fuse_stats && (micro_batch % imgs_per_tile == 0);
-            // Tiles wider than 64 channels sum their columns with a shuffle butterfly (about 1400 cycles per 32 columns and
-            // unit, measured); where that exceeds the unit's MMA time the epilogue becomes the bottleneck and one more pass
-            // over the output (mostly still in L2) is cheaper.  Tiles of up to 64 channels keep their sums in registers.
-            {
-                int n_tile = 16;
-                for (int cand = 256; cand >= 16; cand -= 16)
-                    if (L.d.k % cand == 0) { n_tile = cand; break; }
-                const long long mma_cycles = (long long)(L.c_pad * L.gemm_r * L.gemm_r / 16) * (n_tile / 2 > 48 ? n_tile / 2 : 48);
-                const long long sum_cycles = 1400ll * n_tile / 32;
-                const char* e2 = std::getenv("B2C_FUSE_WIDE");   // 1: always fuse; 0: never on wide tiles; default: by the estimate
-                const bool wide_ok = e2 ? e2[0] != '0' : mma_cycles >= sum_cycles;
-                if (n_tile > 64 && !wide_ok) o.fused_stats = false;
+            o.fused_stats = net->fuse_stats && (n_concurrent == 1 || micro_batch % imgs_per_tile == 0);
+            // Tiles of up to 64 channels sum at next to no cost.  Wider ones are fused where that takes less than one more pass over the
+            // output.  Cycles of a unit, measured on 1024-image layers: 530 per 32 columns for the epilogue's stores and 600 for its sums
+            // (64 -> 256 1x1: 126 us without, 273 us with), both hidden as far as the MMAs or the unit's share of the HBM traffic (24 B/clk
+            // per SM) take longer; the pass of its own 410 per 32 columns (5.5 TB/s) and about 5500 for the launch, spread over the units of
+            // a CTA.  Both sides measured: 128 -> 128 3x3 72 fused, 55 + 15 us; 512 -> 128 1x1 60, 55 + 15; 64 -> 128 3x3 stride 2 62, 58 +
+            // 15; 64 -> 256 1x1 273, 126 + 95; 256 -> 1024 1x1 82, 50 + 27.
+            int n_tile = 16;
+            for (int cand = 256; cand >= 16; cand -= 16)
+                if (L.d.k % cand == 0) { n_tile = cand; break; }
+            if (n_tile > 64) {
+                const double x = n_tile / 32.0, units = (double)batch * pix / 128.0 * (L.d.k / n_tile) / ctx->sm_count;
+                const double mma = (double)L.c_pad * L.gemm_r * L.gemm_r / 16.0 * (n_tile / 2 > 48 ? n_tile / 2 : 48);
+                const double hbm = (256.0 * L.c_pad * L.d.stride * L.d.stride * n_tile / L.d.k + 256.0 * n_tile) / 24.0;
+                const double hidden = mma > hbm ? mma : hbm;
+                const double plain = hidden > 530.0 * x ? hidden : 530.0 * x, fused = hidden > 1130.0 * x ? hidden : 1130.0 * x;
+                const char* e2 = std::getenv("B2C_FUSE_WIDE");   // 1: always; 0: never; default: by the estimate
+                const bool wide_ok = e2 ? e2[0] != '0' : fused - plain <= 410.0 * x + 5500.0 / (units > 1.0 ? units : 1.0);
+                if (!wide_ok) o.fused_stats = false;
             }
         }
         if (L.d.kind == B2C_LAYER_BN) {
@@ -692,7 +698,7 @@ b2c_status b2c_train_step(b2c_net* net, const void* images, const int32_t* label
                     pb.r = L.gemm_r; pb.stride = d.stride; pb.pad = (L.gemm_r - 1) / 2; pb.dgrad = false;
                     pb.in = act_in(d.src, img0); pb.wt = w_bf16 + L.w_off; pb.out = act(i + 1, img0);
                     pb.stats = o.fused_stats ? reinterpret_cast<double*>(net->ws + o.stats_off) + (size_t)g0 * 2 * d.k : nullptr;
-                    pb.stats_group_images = mbs;
+                    pb.stats_group_images = G > 1 ? mbs : 0;   // one micro-batch per pass: one group, whatever the tiles hold
                     ProfScope ps_(net, stream, B2C_PROF_CONV_FWD, 1, i, 0);
                     B2C_TRY(launch_conv_kmajor(ctx, pb, stream));
                     break;

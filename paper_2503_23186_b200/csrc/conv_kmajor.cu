@@ -85,11 +85,19 @@ __device__ __forceinline__ void butterfly16(float (&a)[16], float (&b)[16], int 
 }
 
 // Epilogue of one warp over all units of the CTA.  Epilogue warp e reads the TMEM lane quarter its warp index selects and the column half e >> 2
-// of every accumulator.  NCH > 0: the warp owns exactly NCH 16-column chunks per unit and keeps the BatchNorm sums of
-// its rows in registers across units, reducing them over rows once per statistics group.  NCH == 0: any width; sums
-// are reduced over rows per unit into a per-warp shared-memory array.
-template <int NCH, bool HM = false>
-__device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tmem_base, uint64_t* acc_full, uint64_t* acc_empty,
+// of every accumulator.  The warp owns at most NCH 16-column chunks per unit.  EAGER: it reads all
+// its columns at once and hands the accumulator back before packing and storing (narrow tiles).
+// STATS: BatchNorm sums of the values as stored, kept in registers until the statistics group ends; those of the last group are left
+// in my_stats ([0, 128) sums, [128, 256) sums of squares) for the CTA to add up.  Returns that group and channel tile (-1: none).
+//   * EAGER: a lane sums its own row's columns (32 registers per chunk), a butterfly reduces over the rows once per group.
+//   * wide tiles: two exchanges between lanes first (add_chunk), a quarter of the registers and about 60 instructions per chunk.
+//     Bound: issue slots and latency of eight warps.  Measured with 1024 images, forward with sums, 128 -> 128 at 16x16 and 1x1
+//     64 -> 256 at 32x32: shuffle butterfly per chunk (150 instructions) 82 and 342 us; tensor cores (m16n8k16, which queue behind the
+//     convolution's own MMAs) 90 and 224; transposed through shared memory (two warp barriers and a chain of eight adds) 72 and 253;
+//     read from TMEM once more in the fragment layout 72 and 244; this 72 and 273 us (a rolled loop: 79 and 219).
+// Without STATS the code carries no accumulators: 1x1 64 -> 256 154 -> 126 us, 32 -> 64 57 -> 48 us, data gradient 256 -> 64 159 -> 132 us.
+template <int NCH, bool EAGER, bool HM, bool STATS>
+__device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tmem_base, uint64_t* acc_full, uint64_t* acc_empty,
                                               uint32_t* abort_flag, float* my_stats, int e, int lane, int rank)
 {
     const UnitWalk walk(p, rank);
@@ -98,55 +106,55 @@ __device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tme
     const int q = (e + 2) & 3;       // TMEM lane quarter this warp may read: (warp index in the CTA) % 4, epilogue warps start at 2
     const int m = q * 32 + lane;     // accumulator row = pixel of the tile (w fastest, then h, then image)
     const int lw = m % p.bw, lh = (m / p.bw) % p.bh, ln = m / (p.bw * p.bh);
-    const bool do_stats = p.stats != nullptr;
     const int n_chunks_all = p.n_tile >> 4;
     const int first_half = (n_chunks_all + 1) >> 1;
     const int ck_begin = (e >> 2) ? first_half : 0;
     const int n_chunks = (e >> 2) ? n_chunks_all - first_half : first_half;   // chunks this warp handles
     const int col_begin = ck_begin * 16;
-    constexpr int NA = NCH > 0 ? NCH * 16 : 1;
-    float acc_s[NA], acc_q[NA];
+    constexpr int NA = !STATS ? 1 : EAGER ? 8 * NCH : 2 * NCH;   // column pairs this lane sums
+    f32x2 acc_s[NA], acc_q[NA];
 #pragma unroll
-    for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = 0.f;
-    for (int i = lane; i < 256; i += 32) my_stats[i] = 0.f;
-    __syncwarp();
+    for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = 0ull;
     int jacc = 0, cur_group = -1, cur_ktile = 0;
     bool ok = true;
     long long epi_wait = 0;
 
-    auto flush_stats = [&]() {   // this warp's partial sums of the finished statistics group -> global fp64
-        double* st = p.stats + (size_t)cur_group * 2 * p.oc_valid;
-        if constexpr (NCH > 0) {
+    // Totals over the warp's 32 rows: emit(column of the warp, sum, sum of squares) in one lane per column.
+    auto each_total = [&](auto emit) {
+        if constexpr (STATS && EAGER) {
 #pragma unroll
             for (int ck = 0; ck < NCH; ++ck) {
                 float a[16], b[16];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    a[i] = acc_s[ck * 16 + i];
-                    b[i] = acc_q[ck * 16 + i];
-                    acc_s[ck * 16 + i] = 0.f;
-                    acc_q[ck * 16 + i] = 0.f;
+                for (int i = 0; i < 8; ++i) {
+                    const float2 s = split_f32x2(acc_s[ck * 8 + i]), sq = split_f32x2(acc_q[ck * 8 + i]);
+                    a[2 * i] = s.x; a[2 * i + 1] = s.y;
+                    b[2 * i] = sq.x; b[2 * i + 1] = sq.y;
                 }
                 butterfly16(a, b, lane);
-                const int ch = cur_ktile * p.n_tile + col_begin + ck * 16 + (lane >> 1);
-                if ((lane & 1) == 0 && ck < n_chunks && ch < p.oc_valid) {
-                    atomicAdd(st + ch, (double)a[0]);
-                    atomicAdd(st + p.oc_valid + ch, (double)b[0]);
+                if ((lane & 1) == 0 && ck < n_chunks) emit(ck * 16 + (lane >> 1), a[0], b[0]);
+            }
+        } else if constexpr (STATS) {
+#pragma unroll
+            for (int i = 0; i < NA; ++i) {
+                const float2 s = column_total(acc_s[i]), sq = column_total(acc_q[i]);
+                if ((lane & 7) == 0 && i < 2 * n_chunks) {
+                    const int col = (i >> 1) * 16 + column_of(lane) + 2 * (i & 1);
+                    emit(col, s.x, sq.x);
+                    emit(col + 1, s.y, sq.y);
                 }
             }
-        } else {
-            __syncwarp();
-            for (int c = lane; c < n_chunks * 16; c += 32) {
-                const int ch = cur_ktile * p.n_tile + col_begin + c;
-                if (ch < p.oc_valid) {
-                    atomicAdd(st + ch, (double)my_stats[c]);
-                    atomicAdd(st + p.oc_valid + ch, (double)my_stats[128 + c]);
-                }
-                my_stats[c] = 0.f;
-                my_stats[128 + c] = 0.f;
-            }
-            __syncwarp();
         }
+        __syncwarp();
+    };
+    auto flush_stats = [&]() {   // this warp's sums of the finished statistics group -> global fp64
+        double* st = p.stats + (size_t)cur_group * 2 * p.oc_valid + cur_ktile * p.n_tile + col_begin;
+        each_total([&](int col, float s, float sq) {
+            atomicAdd(st + col, (double)s);
+            atomicAdd(st + p.oc_valid + col, (double)sq);
+        });
+#pragma unroll
+        for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = 0ull;
     };
 
     // The coordinates of a unit are worked out one unit ahead, between the probe of the current unit's accumulator barrier
@@ -180,21 +188,13 @@ __device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tme
             tc_fence_after();
             ++jacc;
         }
-        // A new statistics group: the finished group's sums go out.  Narrow tiles (sums in registers) do that after this unit's
-        // accumulator has been read and handed back, so that the MMA threads do not wait for the reduction over rows.
+        // A new statistics group: the finished group's sums go out, after this unit's first columns have been read (narrow tiles: after its
+        // accumulator has been handed back), so that the MMA threads do not wait for it.
         bool flush_pending = false;
         int next_group = cur_group;
-        if (do_stats) {
-            const int grp = p.stats_group_images > 0 ? (p.grp_shift >= 0 ? c.n0 >> p.grp_shift : c.n0 / p.stats_group_images) : 0;
-            if (grp != cur_group) {
-                if (cur_group >= 0) {
-                    if constexpr (NCH > 0) flush_pending = true;
-                    else flush_stats();
-                }
-                next_group = grp;
-                if constexpr (NCH == 0) cur_group = grp;
-            }
-            if constexpr (NCH == 0) cur_ktile = c.ktile;
+        if constexpr (STATS) {
+            next_group = p.stats_group_images > 0 ? (p.grp_shift >= 0 ? c.n0 >> p.grp_shift : c.n0 / p.stats_group_images) : 0;
+            flush_pending = next_group != cur_group && cur_group >= 0;
         }
         const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * p.acc_cols + col_begin);
         // the accumulator is handed back to the MMA thread as soon as this warp has read its last column
@@ -218,7 +218,7 @@ __device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tme
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] += (ch0 + i < p.oc_valid) ? __ldg(p.bias + ch0 + i) : 0.f;
             }
-            if (!HM && p.out_is_f32) {
+            if (!HM && !STATS && p.out_is_f32) {   // (statistics are those of bf16 values)
                 if (row_valid) {
                     float* dst = reinterpret_cast<float*>(p.out) + row_off + ch0;
 #pragma unroll
@@ -240,7 +240,13 @@ __device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tme
             }
         };
 
-        if constexpr (NCH > 0) {
+        auto group_end = [&]() {
+            if constexpr (!STATS) return;
+            if (flush_pending) flush_stats();   // still the previous group's sums and channel tile
+            cur_group = next_group;
+            cur_ktile = c.ktile;
+        };
+        if constexpr (EAGER) {
             // narrow tiles: read all of this warp's columns at once, free the accumulator, then work from registers
             uint32_t r[NCH][16];
             if constexpr (HM) {
@@ -277,24 +283,45 @@ __device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tme
                 if (n_it > 0) tmem_ld_wait();
                 release();
             }
-            if (flush_pending) flush_stats();   // still the previous group's sums and channel tile
-            cur_group = next_group;
-            cur_ktile = c.ktile;
+            group_end();
 #pragma unroll
             for (int ck = 0; ck < NCH; ++ck) {
                 if (ck < n_chunks) {
                     uint32_t pk[8];
                     store_chunk(r[ck], ck * 16, pk);
-                    if (do_stats && row_valid) {   // sums of the values as stored, kept per row in registers
+                    if (STATS && row_valid) {
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162*>(&pk[i]);
-                            const float lo = __low2float(h), hi = __high2float(h);
-                            acc_s[ck * 16 + 2 * i] += lo;
-                            acc_s[ck * 16 + 2 * i + 1] += hi;
-                            acc_q[ck * 16 + 2 * i] = fmaf(lo, lo, acc_q[ck * 16 + 2 * i]);
-                            acc_q[ck * 16 + 2 * i + 1] = fmaf(hi, hi, acc_q[ck * 16 + 2 * i + 1]);
-                        }
+                        for (int i = 0; i < 8; ++i) add_pair(pk[i], acc_s[STATS ? ck * 8 + i : 0], acc_q[STATS ? ck * 8 + i : 0]);
+                    }
+                }
+            }
+        } else if constexpr (STATS) {
+            // (only convolutions with taps everywhere have statistics: n_it > 0)
+            uint32_t r[2][16];
+            if (n_chunks > 0) {
+                tmem_ld16(t_row, r[0]);
+                tmem_ld_wait();
+            }
+            if (n_chunks <= 1) release();
+            group_end();
+#pragma unroll
+            for (int ck = 0; ck < NCH; ++ck) {
+                if (ck < n_chunks) {   // the next chunk comes in while this one is stored and summed
+                    if (ck + 1 < n_chunks) tmem_ld16(t_row + (uint32_t)((ck + 1) * 16), r[(ck + 1) & 1]);
+                    uint32_t pk[8];
+                    store_chunk(r[ck & 1], ck * 16, pk);
+                    if (!row_valid) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) pk[i] = 0u;
+                    }
+                    __syncwarp();
+                    f32x2 s[2] = {acc_s[2 * ck], acc_s[2 * ck + 1]}, sq[2] = {acc_q[2 * ck], acc_q[2 * ck + 1]};
+                    add_chunk(pk, lane, s, sq);
+                    acc_s[2 * ck] = s[0]; acc_s[2 * ck + 1] = s[1];
+                    acc_q[2 * ck] = sq[0]; acc_q[2 * ck + 1] = sq[1];
+                    if (ck + 1 < n_chunks) {
+                        tmem_ld_wait();
+                        if (ck + 2 == n_chunks) release();
                     }
                 }
             }
@@ -302,24 +329,6 @@ __device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tme
             auto process = [&](const uint32_t (&r)[16], int c0) {
                 uint32_t pk[8];
                 store_chunk(r, c0, pk);
-                if (do_stats && !p.out_is_f32) {
-                    float a[16], b[16];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162*>(&pk[i]);
-                        const float lo = row_valid ? __low2float(h) : 0.f, hi = row_valid ? __high2float(h) : 0.f;
-                        a[2 * i] = lo;
-                        a[2 * i + 1] = hi;
-                        b[2 * i] = lo * lo;
-                        b[2 * i + 1] = hi * hi;
-                    }
-                    butterfly16(a, b, lane);
-                    if ((lane & 1) == 0) {   // the array is private to this warp
-                        const int col = c0 + (lane >> 1);
-                        my_stats[col] += a[0];
-                        my_stats[128 + col] += b[0];
-                    }
-                }
             };
             uint32_t ra[16], rb[16];
             if (n_it > 0 && n_chunks > 0) {
@@ -349,8 +358,14 @@ __device__ __forceinline__ void epilogue_loop(const ConvKParams& p, uint32_t tme
             }
         }
     }
-    if (do_stats && cur_group >= 0 && ok) flush_stats();
+    // the four lane quarters' sums meet in shared memory: a quarter of the global atomics at the kernel's end
+    if (STATS && cur_group >= 0 && ok)
+        each_total([&](int col, float s, float sq) {
+            my_stats[col] = s;
+            my_stats[128 + col] = sq;
+        });
     if (p.stall != nullptr && e == 0 && lane == 0) atomicAdd(p.stall + 3, (unsigned long long)epi_wait);
+    return STATS && ok ? make_int2(cur_group, cur_ktile) : make_int2(-1, 0);
 }
 
 // Issues the MMAs of one stage: NB sub-tiles (vertical taps) x KS k-steps of 16 channels, fully unrolled so that
@@ -617,6 +632,12 @@ __device__ __forceinline__ void mma_issuer_split(const ConvKParams& p, const Uni
                 if (s >= S) { s = my; ph ^= 1u; }
             } while (k < i_end);
             if (!ok) break;
+        } else if (!mbar_wait_warp(&acc_empty[buf], acc_par ^ 1u, p.spin_limit, abort_flag)) {
+            // No stage of this unit is this thread's (units of one slot).  Its commit still counts towards the accumulator's barrier, so it
+            // must not run ahead of the buffer's previous unit: two commits of this thread would complete that unit's phase early.
+            atomicOr(p.status, B2C_DEV_TIMEOUT);
+            ok = false;
+            break;
         }
         if (elect_one()) {
             if constexpr (PAIR) umma_commit_pair(&acc_full[buf], (uint16_t)3);
@@ -647,6 +668,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
     __shared__ uint32_t tmem_slot;
     __shared__ uint32_t abort_flag;
     __shared__ int slot_stage[kMaxStages];   // per ring slot: 1 + index of the stage whose loads were issued into it last
+    __shared__ int2 s_last;   // statistics group and channel tile whose sums the epilogue warps left in s_stats
     __shared__ float s_stats[kEpiWarps][256];   // per epilogue warp (128 columns at most): [0,128) sums, [128,256) sums of squares
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~uintptr_t(1023));
@@ -901,21 +923,40 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
     } else {
         // ---------------------------------------------------------------- epilogue (8 warps)
         const int e = warp - 2;
+        int2 last;
+#define B2C_EPILOGUE(NCH, EAGER, HM)                                                                                                           \
+    last = p.stats != nullptr ? epilogue_loop<NCH, EAGER, HM, true>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank) \
+                              : epilogue_loop<NCH, EAGER, HM, false>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank)
         if constexpr (KIND == KIND_SPLIT) {   // tiles wider than 128 channels
-            epilogue_loop<0>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank);
+            B2C_EPILOGUE(8, false, false);
         } else if constexpr (KIND == KIND_HMERGE) {
-            epilogue_loop<2, true>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank);
+            B2C_EPILOGUE(2, true, true);
         } else {
-            if (KIND == KIND_GENERAL && p.n_tile <= 32 && !p.out_is_f32)
-                epilogue_loop<1>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank);
-            else if (p.n_tile <= 64 && !p.out_is_f32)
-                epilogue_loop<2>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank);
-            else
-                epilogue_loop<0>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank);
+            if (KIND == KIND_GENERAL && p.n_tile <= 32 && !p.out_is_f32) B2C_EPILOGUE(1, true, false);
+            else if (p.n_tile <= 64 && !p.out_is_f32) B2C_EPILOGUE(2, true, false);
+            else if (KIND == KIND_FULL_HALO || p.n_tile <= 128) B2C_EPILOGUE(4, false, false);
+            else B2C_EPILOGUE(8, false, false);   // (only with issue splitting switched off)
         }
+#undef B2C_EPILOGUE
+        if (e == 0 && lane == 0) s_last = last;
     }
     tc_fence_before();
     __syncthreads();
+    if (p.stats != nullptr && !abort_flag && s_last.x >= 0) {   // the last statistics group of this CTA
+        const int first_half = (((p.n_tile >> 4) + 1) >> 1) * 16;
+        double* st = p.stats + (size_t)s_last.x * 2 * p.oc_valid + s_last.y * p.n_tile;
+        for (int i = threadIdx.x; i < p.n_tile; i += kThreads) {
+            const int half = i >= first_half ? 1 : 0, col = i - half * first_half;
+            double s = 0.0, sq = 0.0;
+            for (int q = 0; q < 4; ++q) {
+                s += (double)s_stats[half * 4 + q][col];
+                sq += (double)s_stats[half * 4 + q][128 + col];
+            }
+            atomicAdd(st + i, s);
+            atomicAdd(st + p.oc_valid + i, sq);
+        }
+        __syncwarp();
+    }
     if constexpr (PAIR) cluster_sync_all();   // both CTAs have left their loops: nothing new will be issued
     if (abort_flag) {
         // A wait gave up.  Before the CTA may exit, let every bulk copy it issued land and every
@@ -1059,6 +1100,7 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
     while (p.gsub < 4 && 2 * p.gsub * (p.a_bytes + p.b_bytes) <= 40 * 1024 && 2 * p.gsub * p.splits <= taps * c_blocks) p.gsub *= 2;
     p.stages = 216 * 1024 / (p.gsub * (p.a_bytes + p.b_bytes));
     if (p.stages > kMaxStages) p.stages = kMaxStages;
+    if (p.splits > 1 && p.stages * p.gsub * (p.a_bytes + p.b_bytes) < 512 * p.n_tile) return false;   // the partial tiles are exchanged in the ring's memory
     p.tmem_cols = 32;
     while (p.tmem_cols < p.n_tile) p.tmem_cols *= 2;
     p.total_units = p.n_par * (p.pair ? m_tiles + (m_tiles & 1) : m_tiles / p.n_par) * p.n_ktiles;
@@ -1133,7 +1175,8 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     // Full-halo plan (3x3, stride 1, 64-channel k-blocks, images of at least 8 x 16 pixels, filter bank resident): tiles
     // of 8 x 16 pixels, one framed box per channel block serves all nine taps, so the input crosses L2 -> SM once
     // (three times with vertical tap reuse, nine without) and a ring slot holds a whole channel block of a unit.
-    const bool fh_ok = R == 3 && pb.stride == 1 && n_par == 1 && pb.ic % 64 == 0 && gw >= 8 && gh >= 16 && ctx->use_full_halo &&
+    // (up to 128 channels per tile: wider tiles share a unit between the issuing threads, which full-halo stages do not do)
+    const bool fh_ok = n_tile <= 128 && R == 3 && pb.stride == 1 && n_par == 1 && pb.ic % 64 == 0 && gw >= 8 && gh >= 16 && ctx->use_full_halo &&
                        9 * (pb.ic / 64) * b_rows * 64 * 2 <= (p.pair ? 148 : 96) * 1024;
     // shared-memory plan.  Preference: haloed stages (vertical tap reuse) with 64-channel k-blocks, then with
     // 32-channel k-blocks (smaller stages, so that a ring of at least four still fits), else one tap per stage.

@@ -80,6 +80,74 @@ __device__ __forceinline__ UnitCoord decode_unit(const ConvKParams& p, int u)
     return c;
 }
 
+// Two fp32 values in a register pair and the packed arithmetic on them (one issue slot for two adds or fused multiply-adds).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 make_f32x2(float lo, float hi)
+{
+    f32x2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ float2 split_f32x2(f32x2 v)
+{
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+__device__ __forceinline__ f32x2 add_f32x2(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 fma_f32x2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// s += both values of a packed bf16 pair, q += their squares.
+__device__ __forceinline__ void add_pair(uint32_t pair, f32x2& s, f32x2& q)
+{
+    const f32x2 f = make_f32x2(__uint_as_float(pair << 16), __uint_as_float(pair & 0xffff0000u));
+    s = add_f32x2(s, f);
+    q = fma_f32x2(f, f, q);
+}
+
+// Adds a warp's 32 rows x 16 columns of stored bf16 values (packed pairs pk, one row per lane, rows that do not exist as zeros) to
+// the lane's sums s and sums of squares q.  Two exchanges of packed pairs leave a lane with four columns of four rows, so a chunk needs
+// four register pairs for its sums instead of sixteen: lane l holds columns 8 (l >> 4) + 4 (l >> 3 & 1) + {0, 1} in s[0], q[0] and
+// + {2, 3} in s[1], q[1], and the eight lanes that differ in the lower bits are added up by column_total.
+__device__ __forceinline__ void add_chunk(const uint32_t (&pk)[8], int lane, f32x2 (&s)[2], f32x2 (&q)[2])
+{
+    const bool up16 = (lane & 16) != 0, up8 = (lane & 8) != 0;
+    uint32_t half[2][4];   // [row: own, the partner's][pair]
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        half[0][i] = up16 ? pk[4 + i] : pk[i];
+        half[1][i] = __shfl_xor_sync(0xffffffffu, up16 ? pk[i] : pk[4 + i], 16);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t mine = up8 ? half[r][2 + i] : half[r][i], other = __shfl_xor_sync(0xffffffffu, up8 ? half[r][i] : half[r][2 + i], 8);
+            add_pair(mine, s[i], q[i]);
+            add_pair(other, s[i], q[i]);
+        }
+}
+__device__ __forceinline__ float2 column_total(f32x2 v)
+{
+    float2 f = split_f32x2(v);
+#pragma unroll
+    for (int bit = 1; bit <= 4; bit <<= 1) {
+        f.x += __shfl_xor_sync(0xffffffffu, f.x, bit);
+        f.y += __shfl_xor_sync(0xffffffffu, f.y, bit);
+    }
+    return f;
+}
+__device__ __forceinline__ int column_of(int lane) { return (lane & 24) >> 1; }   // first of a lane's four columns; lanes with (l & 7) == 0 speak for them
+
 // Clusters of `cluster` CTAs (pair: made of CTA pairs) that run at the same time on this context's device.
 int splitk_max_clusters(b2c_ctx* ctx, int cluster, bool pair);
 // Split-K plan: the parameter block, CTAs per cluster and in all, dynamic shared memory.

@@ -38,24 +38,6 @@ __device__ __forceinline__ void sk_issue(int ksteps, uint32_t d_tmem, uint32_t a
     }
 }
 
-// Column sums over the 32 rows a warp holds: after it, lane l holds in a[0], b[0] the totals of column l >> 1.
-__device__ __forceinline__ void sk_column_sums(float (&a)[16], float (&b)[16], int lane)
-{
-#pragma unroll
-    for (int width = 8, bit = 16; width >= 1; width >>= 1, bit >>= 1) {
-        const bool upper = (lane & bit) != 0;
-#pragma unroll
-        for (int i = 0; i < width; ++i) {
-            const float sa = upper ? a[i] : a[i + width], ka = upper ? a[i + width] : a[i];
-            const float sb = upper ? b[i] : b[i + width], kb = upper ? b[i + width] : b[i];
-            a[i] = ka + __shfl_xor_sync(0xffffffffu, sa, bit);
-            b[i] = kb + __shfl_xor_sync(0xffffffffu, sb, bit);
-        }
-    }
-    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
-    b[0] += __shfl_xor_sync(0xffffffffu, b[0], 1);
-}
-
 template <bool PAIR>
 __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid_constant__ ConvKParams p)
 {
@@ -311,20 +293,24 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
             }
         }
         if (do_stats) {   // sums of the values as stored
-            float a[16], b[16];
+            if (!row_valid) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162*>(&pk[i]);
-                a[2 * i] = row_valid ? __low2float(h) : 0.f;
-                a[2 * i + 1] = row_valid ? __high2float(h) : 0.f;
-                b[2 * i] = a[2 * i] * a[2 * i];
-                b[2 * i + 1] = a[2 * i + 1] * a[2 * i + 1];
+                for (int i = 0; i < 8; ++i) pk[i] = 0u;
             }
-            sk_column_sums(a, b, lane);
-            if ((lane & 1) == 0) {   // the four lane quarters meet in shared memory
-                atomicAdd(&s_sum[0][g * 16 + (lane >> 1)], a[0]);
-                atomicAdd(&s_sum[1][g * 16 + (lane >> 1)], b[0]);
+            f32x2 s[2] = {0ull, 0ull}, sq[2] = {0ull, 0ull};
+            add_chunk(pk, lane, s, sq);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float2 ts = column_total(s[i]), tq = column_total(sq[i]);
+                if ((lane & 7) == 0) {   // the four lane quarters meet in shared memory
+                    const int col = g * 16 + column_of(lane) + 2 * i;
+                    atomicAdd(&s_sum[0][col], ts.x);
+                    atomicAdd(&s_sum[0][col + 1], ts.y);
+                    atomicAdd(&s_sum[1][col], tq.x);
+                    atomicAdd(&s_sum[1][col + 1], tq.y);
+                }
             }
+            __syncwarp();
         }
     }
     tc_fence_before();
@@ -337,6 +323,7 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
                 atomicAdd(st + i, (double)s_sum[0][i]);
                 atomicAdd(st + p.oc_valid + i, (double)s_sum[1][i]);
             }
+        __syncwarp();
     }
     if (warp == 1) {
         tc_fence_after();
