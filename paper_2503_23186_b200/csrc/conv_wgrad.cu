@@ -80,6 +80,27 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
+// Four neighbouring lanes hold four 16-byte vectors each, r[4 i ..] = vector i: afterwards lane t of the four holds in r[4 i ..]
+// vector t of lane i.
+__device__ __forceinline__ void transpose_lanes4(uint32_t (&r)[16], int t)
+{
+#pragma unroll
+    for (int mask = 1; mask <= 2; mask <<= 1) {
+        const bool upper = (t & mask) != 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (i & mask) continue;   // vectors i and i | mask: the off-diagonal ones change places
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t lo = r[4 * i + j], hi = r[4 * (i | mask) + j];
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, upper ? lo : hi, mask);
+                r[4 * i + j] = upper ? got : lo;
+                r[4 * (i | mask) + j] = upper ? hi : got;
+            }
+        }
+    }
+}
+
 // One MMA per k-step of 16 pixels, unrolled: descriptors differ only in their low (address) word.
 // Framed x: the B operand of k-step kk starts at its own row offset inside the framed box.
 template <int KS>
@@ -337,19 +358,29 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
             for (int b = 0; b < grp.nb && ck_begin < ck_end; ++b) {
                 const int rs = grp.rs[copy][b];
                 const bool live = rs >= 0 && k < p.k_total;
-                float* dst_row = p.dw + ((long long)(live ? k : 0) * p.rs_total + (live ? rs : 0)) * p.c_total + ctile * p.ct;
+                float* dst = p.dw + ctile * p.ct;
+                const int row_off = live ? (k * p.rs_total + rs) * p.c_total : -1;   // (a filter bank has fewer than 2^31 elements)
                 // accumulator column of 16-channel chunk ck of shift b (framed x: [channel block][shift][64 channels])
                 auto col = [&](int ck) -> uint32_t {
                     const int per_block = p.cw_b >> 4;   // 16-channel chunks per x box
                     return p.fx ? (uint32_t)((ck / per_block) * 3 * p.cw_b + b * p.cw_b + (ck % per_block) * 16) : (uint32_t)(b * p.ct + ck * 16);
                 };
-                auto send = [&](const uint32_t (&r)[16], int ck) {
-                    if (live) {
+                // A lane holds 16 columns of one row, and rows are rs x c elements apart.  Four neighbouring lanes exchange their vectors
+                // first (a 4 x 4 transposition), so that they send 64 consecutive bytes of one row together: an instruction then touches
+                // 16 whole sectors in 8 lines instead of 32 half sectors in 32 lines.  This tail is the same whatever the batch (up to 148
+                // tiles of 196 KB): 128 -> 128 at 16x16 with 128 images 20.7 -> 15.6 us, with 50 images 17.4 -> 12.4; 512 -> 512 at 4x4 with
+                // 1024 images 70.5 -> 67.6 us.
+                const int t4 = lane & 3;
+                auto send = [&](uint32_t (&r)[16], int ck) {
+                    transpose_lanes4(r, t4);   // r[4 i ..] = vector t4 of the row of lane (lane - t4) + i
 #pragma unroll
-                        for (int i = 0; i < 16; i += 4)
-                            red_add_v4(dst_row + ck * 16 + i, __uint_as_float(r[i]), __uint_as_float(r[i + 1]), __uint_as_float(r[i + 2]),
-                                       __uint_as_float(r[i + 3]));
+                    for (int i = 0; i < 4; ++i) {
+                        const int off = __shfl_sync(0xffffffffu, row_off, (lane & ~3) + i);
+                        if (off >= 0)
+                            red_add_v4(dst + off + ck * 16 + 4 * t4, __uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]), __uint_as_float(r[4 * i + 2]),
+                                       __uint_as_float(r[4 * i + 3]));
                     }
+                    __syncwarp();
                 };
                 // two chunks in flight: the next one is fetched while the current one is sent out
                 uint32_t ra[16], rb[16];
