@@ -35,15 +35,25 @@ static constexpr int kThreads = 64 + 32 * kEpiWarps + 32 * (kIssuers - 1) + 32 *
 static constexpr int kProducerWarp1 = 2 + kEpiWarps + (kIssuers - 1);   // warp index of the second producer
 static constexpr uint32_t kDrainPolls = 1u << 22;
 
-// Units of this CTA: plain kernels walk units blockIdx.x, +gridDim.x, ...; CTA pairs walk pair-units (two pixel tiles
-// next to each other, same channel tile) and CTA `rank` of the pair takes tile 2*m + rank.
+// Units of this CTA (a CTA pair walks pair-units: two pixel tiles next to each other, same channel tile, of which CTA `rank` takes tile
+// 2*m + rank).  A walker keeps its channel tile and takes a run of consecutive pixel tiles, so that it meets at most two statistics
+// groups or so of a pass: taken in turns, every walker met every group, and all of them sent the group's sums to the same addresses
+// at the same time.  Eight groups of 128 images: ResNet-18-shaped step 5853 -> 5555 us (launch times summed), ResNet-50-shaped 24.49 -> 23.70 ms.
+// The output parities of a stride-2 data gradient differ in work: their units are taken in turns.
 struct UnitWalk {
     int first, stride, count, rank, pair;
     __device__ UnitWalk(const ConvKParams& p, int rank_) : rank(rank_), pair(p.pair)
     {
-        first = pair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-        stride = pair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+        const int w = pair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, walkers = pair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
         count = pair ? p.total_units >> 1 : p.total_units;
+        first = w;
+        stride = walkers;
+        if (p.n_par == 1) {
+            const int per_ktile = walkers / p.n_ktiles, j = w / p.n_ktiles, kt = w - j * p.n_ktiles, m = count / p.n_ktiles;   // (walkers is a multiple of n_ktiles)
+            first = (int)((long long)m * j / per_ktile) * p.n_ktiles + kt;
+            count = (int)((long long)m * (j + 1) / per_ktile) * p.n_ktiles;
+            stride = p.n_ktiles;
+        }
     }
     __device__ int unit(const ConvKParams& p, int pu) const
     {
