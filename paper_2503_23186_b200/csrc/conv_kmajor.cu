@@ -1108,7 +1108,7 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
     p.b_bytes = (p.tx_b + 1023) & ~1023;
     p.gsub = 1;   // k-blocks of a ring slot: narrow ones share a slot, its barrier wait and its commit
     while (p.gsub < 4 && 2 * p.gsub * (p.a_bytes + p.b_bytes) <= 40 * 1024 && 2 * p.gsub * p.splits <= taps * c_blocks) p.gsub *= 2;
-    p.stages = 216 * 1024 / (p.gsub * (p.a_bytes + p.b_bytes));
+    p.stages = 214 * 1024 / (p.gsub * (p.a_bytes + p.b_bytes));   // (beside 10.4 KB of static arrays)
     if (p.stages > kMaxStages) p.stages = kMaxStages;
     if (p.splits > 1 && p.stages * p.gsub * (p.a_bytes + p.b_bytes) < 512 * p.n_tile) return false;   // the partial tiles are exchanged in the ring's memory
     p.tmem_cols = 32;
