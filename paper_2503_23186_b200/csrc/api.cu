@@ -200,7 +200,10 @@ b2c_status b2c_conv2d_wgrad(b2c_ctx* ctx, const b2c_conv_desc* d, const void* dy
     if (d->c < 16 || d->c % 16 || d->k < 16 || d->k % 16) return B2C_ERR_UNSUPPORTED_SHAPE;
     if (!b2c_is_pow2(p) || !b2c_is_pow2(q) || p > 128 || q > 128) return B2C_ERR_UNSUPPORTED_SHAPE;
     if (!b2c_aligned16(dy) || !b2c_aligned16(x) || !b2c_aligned16(dw_krsc)) return B2C_ERR_MISALIGNED;
-    if (!accumulate) B2C_CUDA(cudaMemsetAsync(dw_krsc, 0, sizeof(float) * (size_t)d->k * d->r * d->s * d->c, (cudaStream_t)stream));
+    if (!accumulate) {
+        b2c_status zs = launch_zero(ctx, dw_krsc, sizeof(float) * (size_t)d->k * d->r * d->s * d->c, nullptr, (cudaStream_t)stream);
+        if (zs != B2C_OK) return zs;
+    }
     return launch_conv_wgrad(ctx, pb, (cudaStream_t)stream);
 }
 
@@ -664,7 +667,6 @@ b2c_status b2c_train_step(b2c_net* net, const void* images, const int32_t* label
 
     const size_t image_bytes = (size_t)N * net->image_h * net->image_w * net->image_c * 2;
     if (image_bytes % 16) return B2C_ERR_MISALIGNED;
-    B2C_CUDA(cudaMemsetAsync(loss_dev, 0, sizeof(float), stream));
     const int mbs = net->micro_batch;
 
     for (int mb = 0; mb < n_passes; ++mb) {
@@ -675,7 +677,10 @@ b2c_status b2c_train_step(b2c_net* net, const void* images, const int32_t* label
             if (t == 0 && !staged_input) return img + (size_t)img0 * net->image_h * net->image_w * net->image_c * 2;
             return act(t, img0);
         };
-        B2C_CUDA(cudaMemsetAsync(net->ws + net->stats_begin, 0, (size_t)(net->stats_end - net->stats_begin), stream));
+        {   // the pass's fp64 sums, and once per step the loss
+            b2c_status zs = launch_zero(ctx, net->ws + net->stats_begin, (size_t)(net->stats_end - net->stats_begin), mb == 0 ? loss_dev : nullptr, stream);
+            if (zs != B2C_OK) return zs;
+        }
 
         // forward pass of layer i over the micro-batches g0 .. g0 + Gc of the pass
         auto forward_layer = [&](int i, int g0, int Gc) -> b2c_status {

@@ -172,6 +172,9 @@ b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da
 b2c_status launch_update_pack(b2c_ctx* ctx, const b2c_weight_seg* segs, int n_segs, size_t count, float* w, float* v, float* g, float inv_n, float lr, float momentum,
                               float wd, void* w_bf16, void* w_dgrad, cudaStream_t stream);
 
+// Clears `bytes` (a multiple of 8, 8-byte aligned) at `a` and, if f is not null, one float, as a launch like any other of the stream.
+b2c_status launch_zero(b2c_ctx* ctx, void* a, size_t bytes, float* f, cudaStream_t stream);
+
 // Running statistics of the BatchNorm layers of a step (momentum update with the unbiased variance), taken from the fp64
 // sums the forward pass left in the workspace.  One entry per layer; the G statistics groups of a pass are applied in
 // order, as if the micro-batches had run one after the other.

@@ -453,8 +453,6 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
                                                                              double* __restrict__ sums_all, const uint8_t* __restrict__ relu_mask,
                                                                              unsigned spin_limit, unsigned* status)
 {
-    pdl_wait();   // first global access comes after the previous kernel of the stream
-    pdl_launch_dependents();
     extern __shared__ uint8_t st_raw[];
     __shared__ uint64_t full[kStStages], empty[kStStages];
     __shared__ uint32_t abort_flag;
@@ -464,6 +462,8 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
     for (int i = threadIdx.x; i < 2 * c; i += kStThreads) s_acc[i] = 0.f;
     staged_init(full, empty, &abort_flag);
     __syncthreads();
+    pdl_wait();   // (the set-up above touched no global data) first global access comes after the previous kernel of the stream
+    pdl_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long base = (long long)blockIdx.y * m * sw.groups;
     const uint8_t* mask = relu ? relu_mask : nullptr;
@@ -539,8 +539,6 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(cons
                                                                             const uint8_t* __restrict__ relu_mask, unsigned spin_limit,
                                                                             unsigned* status)
 {
-    pdl_wait();   // first global access comes after the previous kernel of the stream
-    pdl_launch_dependents();
     extern __shared__ uint8_t st_raw[];
     __shared__ uint64_t full[kStStages], empty[kStStages];
     __shared__ uint32_t abort_flag;
@@ -548,6 +546,8 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(cons
     const StagedWalk sw(c, m, da2 != nullptr ? 3 : 2, relu != 0);
     staged_init(full, empty, &abort_flag);
     __syncthreads();
+    pdl_wait();   // first global access comes after the previous kernel of the stream
+    pdl_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const double* sums = sums_all + (size_t)blockIdx.y * 2 * c;
     const float* mean = mean_all + (size_t)blockIdx.y * c;
@@ -1315,7 +1315,29 @@ __global__ void bn_running_update_kernel(const __grid_constant__ BnRunTable tab,
     }
 }
 
+// ------------------------------------------------------------------------------ clearing
+// Clears n8 eight-byte words of `a` and, with f, one float.  A memset node does not take part in programmatic launches: the kernels on
+// either side of it start cold, about 3 us per memset between two short kernels against 1.3 us for this.
+__global__ void __launch_bounds__(kEwThreads) zero_kernel(unsigned long long* __restrict__ a, long long n8, float* f)
+{
+    pdl_wait();   // first global access comes after the previous kernel of the stream
+    pdl_launch_dependents();
+    for (long long i = (long long)blockIdx.x * kEwThreads + threadIdx.x; i < n8; i += (long long)gridDim.x * kEwThreads) a[i] = 0ull;
+    if (f != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *f = 0.f;
+}
+
 // ------------------------------------------------------------------------------ launchers
+b2c_status launch_zero(b2c_ctx* ctx, void* a, size_t bytes, float* f, cudaStream_t stream)
+{
+    const long long n8 = (long long)(bytes / 8);
+    long long blocks = (n8 + 4 * kEwThreads - 1) / (4 * kEwThreads);
+    if (blocks < 1) blocks = 1;
+    if (blocks > 8ll * ctx->sm_count) blocks = 8ll * ctx->sm_count;
+    B2C_CUDA(b2c_launch(ctx, zero_kernel, dim3((unsigned)blocks), dim3(kEwThreads), 0, stream, 1u, reinterpret_cast<unsigned long long*>(a), n8, f));
+    B2C_CUDA(cudaGetLastError());
+    return B2C_OK;
+}
+
 // Blocks per statistics group: one wave of two resident blocks per SM across all groups.
 static int ew_grid(b2c_ctx* ctx, int n_groups, long long m, int rows_per_iter)
 {
@@ -1332,7 +1354,10 @@ b2c_status launch_bn_fwd(b2c_ctx* ctx, int G, long long m, int c, const void* y,
     const int rows_per_iter = kEwThreads / (c / 8);
     dim3 grid((unsigned)ew_grid(ctx, G, m, rows_per_iter), (unsigned)G);
     if (stats_ready != 1) {
-        if (stats_ready == 0) B2C_CUDA(cudaMemsetAsync(stats, 0, sizeof(double) * 2 * c * G, stream));
+        if (stats_ready == 0) {
+            b2c_status st = launch_zero(ctx, stats, sizeof(double) * 2 * c * G, nullptr, stream);
+            if (st != B2C_OK) return st;
+        }
         B2C_CUDA(b2c_launch(ctx, bn_stats_kernel, dim3(grid), dim3(kEwThreads), sizeof(float) * 2 * c, stream, 1u, y, m, c, stats));
     }
     uint8_t* mask_out = relu ? reinterpret_cast<uint8_t*>(relu_mask) : nullptr;
@@ -1402,7 +1427,8 @@ b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da
     dim3 grid((unsigned)ew_grid(ctx, G, m, rows_per_iter), (unsigned)G);
     const uint8_t* mask = relu ? reinterpret_cast<const uint8_t*>(relu_mask) : nullptr;
     if (!sums_zeroed) {
-        B2C_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * 2 * c * G, stream));
+        b2c_status st = launch_zero(ctx, sums, sizeof(double) * 2 * c * G, nullptr, stream);
+        if (st != B2C_OK) return st;
         if (arrivals != nullptr) B2C_CUDA(cudaMemsetAsync(arrivals, 0, sizeof(unsigned) * G, stream));
     }
     // Both passes in one cooperative launch, group by group (the apply pass of a group re-reads its tensors from L2).
