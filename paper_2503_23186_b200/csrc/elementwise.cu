@@ -958,28 +958,41 @@ __global__ void __launch_bounds__(kGrThreads, 2) bn_bwd_grouped_kernel(const voi
 }
 
 // ------------------------------------------------------------------------------ pooling, padding
-__global__ void avgpool_fwd_kernel(const void* __restrict__ a, int n, int hw, int c, void* __restrict__ pooled)
+// A block takes one image and up to 32 channel vectors; its rows of threads share the positions, so that the loads of an image are in
+// flight together (one thread per vector walked the positions one after the other: 64 positions of 16 images: 20 of the 226 us of a small net's step).
+__global__ void __launch_bounds__(kEwThreads) avgpool_fwd_kernel(const void* __restrict__ a, int hw, int c, int lanes, void* __restrict__ pooled)
 {
     pdl_wait();   // first global access comes after the previous kernel of the stream
     pdl_launch_dependents();
-    const int groups = c >> 3;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)n * groups) return;
-    const int g = (int)(idx % groups);
-    const long long img = idx / groups;
+    __shared__ float part[kEwThreads][9];
+    const int groups = c >> 3, rows = kEwThreads / lanes, gl = threadIdx.x % lanes, rl = threadIdx.x / lanes;
+    const int g = blockIdx.y * lanes + gl;
+    const long long img = blockIdx.x;
     float s[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) s[i] = 0.f;
-    for (int j = 0; j < hw; ++j) {
-        float f[8];
-        unpack8(ld16(a, (img * hw + j) * groups + g), f);
+    if (g < groups && rl < rows) {
+#pragma unroll 4
+        for (int j = rl; j < hw; j += rows) {
+            float f[8];
+            unpack8(ld16(a, (img * hw + j) * groups + g), f);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s[i] += f[i];
+            for (int i = 0; i < 8; ++i) s[i] += f[i];
+        }
     }
-    const float inv = 1.f / (float)hw;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) s[i] *= inv;
-    reinterpret_cast<uint4*>(pooled)[idx] = pack8(s);
+    for (int i = 0; i < 8; ++i) part[threadIdx.x][i] = s[i];
+    __syncthreads();
+    if (rl == 0 && g < groups) {
+        for (int r = 1; r < rows; ++r) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) s[i] += part[r * lanes + gl][i];
+        }
+        const float inv = 1.f / (float)hw;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] *= inv;
+        reinterpret_cast<uint4*>(pooled)[img * groups + g] = pack8(s);
+    }
 }
 
 __global__ void avgpool_bwd_kernel(const void* __restrict__ dpooled, int n, int hw, int c, void* __restrict__ da)
@@ -1590,8 +1603,9 @@ b2c_status b2c_avgpool_fwd(b2c_ctx* ctx, int n, int hw, int c, const void* a, vo
     if (!ctx || !a || !pooled) return B2C_ERR_INVALID_ARG;
     if (n < 1 || hw < 1 || c < 8 || c % 8) return B2C_ERR_UNSUPPORTED_SHAPE;
     if (!b2c_aligned16(a) || !b2c_aligned16(pooled)) return B2C_ERR_MISALIGNED;
-    const long long total = (long long)n * (c / 8);
-    B2C_CUDA(b2c_launch(ctx, avgpool_fwd_kernel, dim3((unsigned)((total + 127) / 128)), dim3(128), 0, (cudaStream_t)stream_, 1u, a, n, hw, c, pooled));
+    const int groups = c / 8, lanes = groups < 32 ? groups : 32;
+    B2C_CUDA(b2c_launch(ctx, avgpool_fwd_kernel, dim3((unsigned)n, (unsigned)((groups + lanes - 1) / lanes)), dim3(kEwThreads), 0, (cudaStream_t)stream_, 1u, a, hw, c, lanes,
+                        pooled));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;
 }

@@ -1,0 +1,62 @@
+"""Edges of the average pool (image rows and channel vectors shared by a block) and of convolution plans: units of one ring slot on
+256-channel tiles, filter rows that do not fill a tile of the weight gradient."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2503_23186_b200 import workloads as wl
+from parity import assert_close, dev_bf16, host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2503_23186_b200 import binding
+    c = binding.Context(0)
+    yield c
+    assert c.device_status() == 0
+    c.close()
+
+
+# one position, fewer and more positions than thread rows, channel vectors: 1, not a divisor of the block, over one block's 32
+@pytest.mark.parametrize("n,hw,c", [(1, 1, 8), (3, 7, 48), (5, 16, 512), (2, 64, 128), (3, 49, 2048), (2, 300, 264)])
+def test_avgpool(ctx, n, hw, c):
+    a = wl.normal_bf16(60, f"pool{hw}x{c}", (n, hw, c))
+    pooled = torch.full((n, c), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ctx.avgpool_fwd(n, hw, c, dev_bf16(a), pooled)
+    assert ctx.device_status() == 0
+    assert_close(pooled, oracle.round_bf16(a.astype(np.float64).mean(1)), "pooled")
+
+
+# one k-block per unit on 256-channel tiles (two issuing threads, one slot per unit), several units per walker; 64 -> 256 3x3
+@pytest.mark.parametrize("shape", [(96, 16, 16, 64, 256, 1, 1), (40, 16, 16, 64, 256, 3, 1)], ids=["one-slot-units", "wide-3x3"])
+def test_wide_tiles_with_statistics(ctx, shape):
+    from paper_2503_23186_b200 import binding
+    N, H, W, C, K, R, st = shape
+    x, w, _ = wl.conv_problem(61, *shape)
+    ref = oracle.conv2d_fwd(x, w, st, (R - 1) // 2)
+    for _ in range(3):
+        y = torch.full((N, H, W, K), float("nan"), dtype=torch.bfloat16, device="cuda")
+        stats = torch.zeros(2 * K, dtype=torch.float64, device="cuda")
+        ctx.conv2d_fwd(binding.conv_desc(*shape), dev_bf16(x), dev_bf16(w), y, ch_stats=stats)
+        assert ctx.device_status() == 0
+        assert_close(y, ref, "y")
+        ys = host(y).reshape(-1, K)   # sums of the stored values: fp32 within a walker, fp64 across
+        np.testing.assert_allclose(host(stats)[:K], ys.sum(0), rtol=1e-5, atol=1e-3 * np.sqrt(ys.shape[0]))
+        np.testing.assert_allclose(host(stats)[K:], (ys * ys).sum(0), rtol=1e-5)
+
+
+@pytest.mark.parametrize("shape", [(6, 8, 8, 48, 16, 3, 1), (4, 8, 8, 32, 144, 3, 1), (4, 8, 8, 16, 80, 1, 2)], ids=lambda s: "n{}h{}c{}k{}r{}s{}".format(*(s[i] for i in (0, 1, 3, 4, 5, 6))))
+def test_weight_gradient_partial_tiles(ctx, shape):
+    from paper_2503_23186_b200 import binding
+    N, H, W, C, K, R, st = shape
+    x, _, g = wl.conv_problem(62, *shape)
+    ref = oracle.conv2d_wgrad(g, x, R, R, st, (R - 1) // 2)
+    dw = torch.full((K, R, R, C), float("nan"), dtype=torch.float32, device="cuda")
+    ctx.conv2d_wgrad(binding.conv_desc(*shape), dev_bf16(g), dev_bf16(x), dw)
+    assert_close(dw, ref, "dw")
+    ctx.conv2d_wgrad(binding.conv_desc(*shape), dev_bf16(g), dev_bf16(x), dw, accumulate=True)
+    assert ctx.device_status() == 0
+    assert_close(dw, 2 * ref, "dw accumulated")
