@@ -391,12 +391,13 @@ struct StagedWalk {
 // Producer side: one thread.  Returns the number of chunks it issued (for the drain after an aborted wait).
 __device__ __forceinline__ int staged_produce(const StagedWalk& sw, uint8_t* ring, uint64_t* full, uint64_t* empty, const void* t0, const void* t1,
                                               const void* t2, const uint8_t* mask, long long base_vec, unsigned spin_limit, uint32_t* abort_flag,
-                                              unsigned* status)
+                                              unsigned* status, bool backwards = false)
 {
     int i = 0;
     const uint32_t tbytes = (uint32_t)sw.chunk_vecs * 16u;
     const uint32_t tx = (uint32_t)sw.nt * tbytes + (mask != nullptr ? (uint32_t)sw.chunk_vecs : 0u);
-    for (long long k = blockIdx.x; k < sw.n_full; k += gridDim.x, ++i) {
+    for (long long j = blockIdx.x; j < sw.n_full; j += gridDim.x, ++i) {
+        const long long k = backwards ? sw.n_full - 1 - j : j;
         const int s = i % kStStages;
         if (!mbar_wait_bounded(&empty[s], (((uint32_t)(i / kStStages)) & 1u) ^ 1u, spin_limit, abort_flag)) {
             atomicOr(status, B2C_DEV_TIMEOUT);
@@ -556,7 +557,7 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(cons
     const uint8_t* mask = relu ? relu_mask : nullptr;
     int issued = 0;
     if (warp == kEwThreads / 32) {
-        if (lane == 0) issued = staged_produce(sw, ring, full, empty, da1, y, da2, mask, base, spin_limit, &abort_flag, status);
+        if (lane == 0) issued = staged_produce(sw, ring, full, empty, da1, y, da2, mask, base, spin_limit, &abort_flag, status, true);
     } else {
         if (blockIdx.x == 0) {
             for (int ch = threadIdx.x; ch < c; ch += kEwThreads) {
@@ -604,7 +605,12 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(cons
         };
         int i = 0;
         bool ok = true;
-        for (long long k = blockIdx.x; k < sw.n_full; k += gridDim.x, ++i) {
+        // From the last chunk to the first: what the reduction pass read last is met while it is still in L2.  Both passes together, 67 MB
+        // tensors (256 channels at 32x32, 128 images) 66.4 -> 63.1 us, with the shortcut's gradient 77.9 -> 73.5; 134 MB 114.0 -> 110.5;
+        // 537 MB 430 -> 426.  (Keeping lines with eviction hints, or walking the forward pass backwards behind its statistics pass, gave
+        // nothing more: 537 MB forward 281 -> 290.)
+        for (long long j = blockIdx.x; j < sw.n_full; j += gridDim.x, ++i) {
+            const long long k = sw.n_full - 1 - j;
             ok = staged_wait(full, i, lane, spin_limit, &abort_flag, status);
             if (!ok) break;
             if (act) {
