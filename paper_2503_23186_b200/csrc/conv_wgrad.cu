@@ -45,6 +45,7 @@ struct alignas(64) WgradParams {
     int ct;                            // x channels per CTA
     int n_ktiles, n_ctiles, n_splits;
     int chunks_total;
+    int stream;                           // the (tile, pixel chunk) pairs are dealt out in equal runs: a CTA may finish one tile and begin the next
     int stages, tmem_cols;
     int box_a, box_b, a_boxes, b_boxes;   // bytes per dy / x box; dy boxes per stage; x boxes per shift
     int a_bytes, a_lbo;                   // dy bytes per stage; byte distance between the two 64-row halves of the A operand
@@ -127,6 +128,9 @@ __device__ __forceinline__ void wg_issue(uint32_t d_tmem, uint32_t a_lo, uint32_
     }
 }
 
+// STREAM: the launch deals out equal runs of (tile, chunk) pairs (p.stream); otherwise a CTA has one tile, and the code for more is left out
+// (it cost short launches 0.2-1.7 us).
+template <bool STREAM>
 __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_constant__ WgradParams p)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -138,17 +142,22 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int S = p.stages;
 
-    int t = blockIdx.x;
-    const int ktile = t % p.n_ktiles;
-    t /= p.n_ktiles;
-    const int ctile = t % p.n_ctiles;
-    t /= p.n_ctiles;
-    const int gi = t % p.n_groups;
-    const int split = t / p.n_groups;
-    const WgGroup& grp = p.groups[gi];
-    const int chunk_begin = (int)((long long)p.chunks_total * split / p.n_splits);
-    const int chunk_end = (int)((long long)p.chunks_total * (split + 1) / p.n_splits);
-    const int n_chunks = chunk_end - chunk_begin;
+    // this CTA's run of (tile, chunk) pairs: part of one tile, or an equal share of all of them
+    const int n_tiles = p.n_ktiles * p.n_ctiles * p.n_groups;
+    int tile, chunk_begin, left;   // first tile, its first chunk, pairs in all
+    if constexpr (STREAM) {
+        const long long total = (long long)n_tiles * p.chunks_total, first = total * blockIdx.x / gridDim.x;
+        tile = (int)(first / p.chunks_total);
+        chunk_begin = (int)(first - (long long)tile * p.chunks_total);
+        left = (int)(total * (blockIdx.x + 1) / gridDim.x - first);
+    } else {
+        const int split = (int)blockIdx.x / n_tiles;
+        tile = (int)blockIdx.x - split * n_tiles;
+        chunk_begin = (int)((long long)p.chunks_total * split / p.n_splits);
+        left = (int)((long long)p.chunks_total * (split + 1) / p.n_splits) - chunk_begin;
+    }
+    // (worked out ahead of the wait for the previous kernel)
+    int ktile = tile % p.n_ktiles, gi = tile / p.n_ktiles / p.n_ctiles, ctile = tile / p.n_ktiles - gi * p.n_ctiles;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -173,236 +182,266 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
     pdl_wait();
     pdl_launch_dependents();
     const long long t_kernel = clock64();
-    int last_issued = -1;  // producer lanes: last chunk whose loads this lane issued
+    int last_issued = -1;  // producer lanes: last ring slot (counted from the start) whose loads this lane issued
+    // State of the roles that lives on from tile to tile: ring slots are counted from the start of the kernel, `first_slot` is the tile's first.
+    const int role = warp == 0 ? 0 : warp >= kWgProducerWarp1 ? warp - kWgProducerWarp1 + 1 : warp - 1;   // producer or issuer number
+    int slot_ = role, s_ = role, first_slot_ = 0;
+    uint32_t ph_ = 0u, tile_parity_ = 0u;
 
-    if (warp == 0 || warp >= kWgProducerWarp1) {
-        const int w = warp == 0 ? 0 : warp - kWgProducerWarp1 + 1;
-        if (w < S) {
-            // Producer w fills the ring slots w, w + kWgProducers, ...: one thread's wait -> expect -> issue chain is
-            // longer than the MMAs of a stage take.  Each slot keeps one producer, which uses it strictly in order.
-            if (elect_one()) {
-                prefetch_tensormap(&p.tmDy);
-                prefetch_tensormap(&p.tmX[0]);
-            }
-            const uint32_t tx = p.fx ? (uint32_t)(p.a_bytes + p.b_boxes * p.fx_tx) : (uint32_t)(p.a_bytes + grp.nb * p.b_boxes * p.box_b);
-            int it = w, s = w;   // it counts ring slots; a slot holds G consecutive chunks (the last one of the CTA possibly fewer)
-            uint32_t ph = 0u;
-            const bool timed = p.stall != nullptr && w == 0 && lane == 0;
-            long long waited = 0;
-            const int G = p.gsub, n_slots = (n_chunks + G - 1) / G;
-            while (it < n_slots) {
-                const long long w0 = timed ? clock64() : 0;
-                if (!mbar_wait_warp(&empty_bar[s], ph ^ 1u, p.spin_limit, &abort_flag)) {
-                    atomicOr(p.status, B2C_DEV_TIMEOUT);
-                    break;
-                }
-                if (timed) waited += clock64() - w0;
-                const int n_g = n_chunks - it * G < G ? n_chunks - it * G : G;
+    do {
+        const int n_chunks = STREAM ? (left < p.chunks_total - chunk_begin ? left : p.chunks_total - chunk_begin) : left;
+        int slot = STREAM ? slot_ : role, s = STREAM ? s_ : role;
+        uint32_t ph = STREAM ? ph_ : 0u;
+        const int first_slot = STREAM ? first_slot_ : 0;
+        const uint32_t tile_parity = STREAM ? tile_parity_ : 0u;
+        const WgGroup& grp = p.groups[gi];
+        const int n_slots = (n_chunks + p.gsub - 1) / p.gsub;   // ring slots of this tile
+
+        if (warp == 0 || warp >= kWgProducerWarp1) {
+            const int w = role;
+            if (w < S) {
+                // Producer w fills the ring slots w, w + kWgProducers, ...: one thread's wait -> expect -> issue chain is
+                // longer than the MMAs of a stage take.  Each slot keeps one producer, which uses it strictly in order.
                 if (elect_one()) {
-                    mbar_expect_tx(&full_bar[s], (uint32_t)n_g * tx);
-                    for (int g = 0; g < n_g; ++g) {
-                        int ch = chunk_begin + it * G + g;
-                        const int ow0 = (ch & (p.tiles_w - 1)) * p.bw;
-                        ch >>= p.tw_shift;
-                        const int th = ch / p.tiles_h;
-                        const int oh0 = (ch - th * p.tiles_h) * p.bh;
-                        const int n0 = th * p.bn;
-                        uint8_t* dst = smem + (size_t)s * p.stage_bytes + (size_t)g * p.sub_bytes;
-                        if (p.stack) {
-                            // one box with a halo row on top: copy 1 of dy (gathered one row higher) is its first pb pixels,
-                            // copy 0 starts one image row further down
-                            tma_load_4d(dst, &p.tmDy, &full_bar[s], 0, ow0, oh0 - 1, n0);
-                        } else {
-                            for (int j = 0; j < p.a_boxes; ++j)  // boxes past the last channel are zero-filled
-                                tma_load_4d(dst + (size_t)j * p.box_a, &p.tmDy, &full_bar[s], ktile * 128 + j * p.cw_a, ow0, oh0, n0);
-                        }
-                        dst += p.a_bytes;
-                        if (p.fx) {   // one framed box per channel block, gathered at the first shift (one pixel to the left)
-                            for (int j = 0; j < p.b_boxes; ++j)
-                                tma_load_4d(dst + (size_t)j * p.fx_box, &p.tmX[grp.map[0]], &full_bar[s], ctile * p.ct + j * p.cw_b, ow0 + grp.dw[0],
-                                            oh0 + grp.dh[0], n0);
-                        } else
-                        for (int b = 0; b < grp.nb; ++b)
-                            for (int j = 0; j < p.b_boxes; ++j)
-                                tma_load_4d(dst + (size_t)(b * p.b_boxes + j) * p.box_b, &p.tmX[grp.map[b]], &full_bar[s], ctile * p.ct + j * p.cw_b,
-                                            ow0 + grp.dw[b], oh0 + grp.dh[b], n0);
+                    prefetch_tensormap(&p.tmDy);
+                    prefetch_tensormap(&p.tmX[0]);
+                }
+                const uint32_t tx = p.fx ? (uint32_t)(p.a_bytes + p.b_boxes * p.fx_tx) : (uint32_t)(p.a_bytes + grp.nb * p.b_boxes * p.box_b);
+                const bool timed = p.stall != nullptr && w == 0 && lane == 0;
+                long long waited = 0;
+                const int G = p.gsub;   // a slot holds G consecutive chunks (the tile's last one possibly fewer)
+                while (slot < first_slot + n_slots) {
+                    const int it = slot - first_slot;
+                    const long long w0 = timed ? clock64() : 0;
+                    if (!mbar_wait_warp(&empty_bar[s], ph ^ 1u, p.spin_limit, &abort_flag)) {
+                        atomicOr(p.status, B2C_DEV_TIMEOUT);
+                        break;
                     }
-                }
-                __syncwarp();
-                last_issued = it;
-                if (s + kWgProducers < S) {
-                    it += kWgProducers;
-                    s += kWgProducers;
-                } else {   // wrap to this producer's first slot
-                    it += S - s + w;
-                    s = w;
-                    ph ^= 1u;
-                }
-            }
-            if (timed) atomicAdd(p.stall + 0, (unsigned long long)waited);
-        }
-    } else if (warp == 1 || warp == 2) {
-        if (warp - 1 < p.issuers) {
-            const int my = warp - 1;
-            // SBO = eight pixel rows, LBO = next block of cw channels (the next box)
-            const uint64_t proto_a = make_smem_desc(0u, (uint32_t)p.a_lbo, 16u * (uint32_t)p.cw_a, (uint32_t)p.swz_a);
-            // framed x: the column blocks of an MMA are the three shifts, one pixel row (cw_b channels) apart
-            const uint64_t proto_b = p.fx ? make_smem_desc(0u, 2u * (uint32_t)p.cw_b, p.fx_sbo, (uint32_t)p.swz_b)
-                                          : make_smem_desc(0u, (uint32_t)p.box_b, 16u * (uint32_t)p.cw_b, (uint32_t)p.swz_b);
-            const uint32_t a_hi = (uint32_t)(proto_a >> 32), a_lo_base = (uint32_t)proto_a;
-            const uint32_t b_hi = (uint32_t)(proto_b >> 32), b_lo_base = (uint32_t)proto_b;
-            const uint32_t kstep_a = (uint32_t)(16 * p.cw_a * 2) >> 4, kstep_b = (uint32_t)(16 * p.cw_b * 2) >> 4;   // 16 pixel rows
-            const int ksteps = p.pb >> 4;
-            // up to three MMAs per k-step (kept in scalars: the issuing thread must not index local memory)
-            uint32_t idesc0 = 0, idesc1 = 0, idesc2 = 0, boff0 = 0, boff1 = 0, boff2 = 0, dcol0 = 0, dcol1 = 0, dcol2 = 0;
-            int n_pieces = 0;
-            for (int i = 0; i < p.n_pieces; ++i) {
-                if (p.piece_t0[i] >= grp.nb) break;
-                const int nt = min(p.piece_nt[i], grp.nb - p.piece_t0[i]);
-                const uint32_t id = make_idesc_bf16(128, nt * p.ct, true, true);
-                const uint32_t bo = (uint32_t)(p.a_bytes + p.piece_t0[i] * p.b_boxes * p.box_b) >> 4;
-                const uint32_t dc = (uint32_t)(p.piece_t0[i] * p.ct);
-                if (i == 0) { idesc0 = id; boff0 = bo; dcol0 = dc; }
-                else if (i == 1) { idesc1 = id; boff1 = bo; dcol1 = dc; }
-                else { idesc2 = id; boff2 = bo; dcol2 = dc; }
-                ++n_pieces;
-            }
-            bool ok = true;
-            const bool timed = p.stall != nullptr && lane == 0;
-            const long long t_begin = timed ? clock64() : 0;
-            long long waited = 0, issuing = 0;
-            const int G = p.gsub, n_slots = (n_chunks + G - 1) / G;
-            const uint32_t sub16 = (uint32_t)p.sub_bytes >> 4;
-            if (my != 0 && n_slots > 1 && !mbar_wait_warp(&init_bar, 0u, p.spin_limit, &abort_flag)) {   // slot 0 has initialised the accumulator
-                atomicOr(p.status, B2C_DEV_TIMEOUT);
-                ok = false;
-            }
-            if (my != 0) tc_fence_after();
-            // (this thread's chain of dependent instructions per slot bounds chunks with few MMAs: nothing is recomputed in the loop)
-            const bool fx = p.fx != 0;
-            const int n_issuers = p.issuers, b_boxes = p.b_boxes;
-            const uint32_t id_fx = make_idesc_bf16(128, 3 * p.cw_b, true, true);
-            const uint32_t fx_b_first = (uint32_t)p.a_bytes >> 4, fx_b_next = (uint32_t)p.fx_box >> 4, fx_d_next = 3u * (uint32_t)p.cw_b;
-            const uint32_t fk0 = p.fx_koff[0], fk1 = p.fx_koff[1], fk2 = p.fx_koff[2], fk3 = p.fx_koff[3];
-            const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, smem16 = smem_u32(smem) >> 4;
-            int s = my;            // S is even with two threads: a thread's slots are my, my + 2, ...
-            uint32_t ph = 0u;
-            for (int it = my; ok && it < n_slots; it += n_issuers) {
-                const long long w0 = timed ? clock64() : 0;
-                if (!mbar_wait_warp(&full_bar[s], ph, p.spin_limit, &abort_flag)) {
-                    atomicOr(p.status, B2C_DEV_TIMEOUT);
-                    ok = false;
-                    break;
-                }
-                const long long w1 = timed ? clock64() : 0;
-                waited += w1 - w0;
-                tc_fence_after();
-                const uint32_t st16 = smem16 + (uint32_t)s * stage16;
-                const int n_g = n_chunks - it * G < G ? n_chunks - it * G : G;
-                if (elect_one()) {
-                    for (int g = 0; g < n_g; ++g) {
-                        const uint32_t a_lo = a_lo_base + st16 + (uint32_t)g * sub16, b_lo = b_lo_base + st16 + (uint32_t)g * sub16;
-                        const uint32_t acc0 = (it | g) != 0 ? 1u : 0u;
-                        if (fx) {   // chunks of 64 pixels: four k-steps; one MMA per channel block, N = three shifts x cw_b channels
-                            const uint32_t b_first = b_lo + fx_b_first;
-                            for (int i = 0; i < b_boxes; ++i)
-                                wg_issue_framed<4>(tmem_base + (uint32_t)i * fx_d_next, a_lo, b_first + (uint32_t)i * fx_b_next, a_hi, b_hi, id_fx, kstep_a, fk0, fk1, fk2,
-                                                   fk3, acc0);
-                        } else if (ksteps == 4) {
-                            wg_issue<4>(tmem_base + dcol0, a_lo, b_lo + boff0, a_hi, b_hi, idesc0, kstep_a, kstep_b, acc0);
-                            if (n_pieces > 1) wg_issue<4>(tmem_base + dcol1, a_lo, b_lo + boff1, a_hi, b_hi, idesc1, kstep_a, kstep_b, acc0);
-                            if (n_pieces > 2) wg_issue<4>(tmem_base + dcol2, a_lo, b_lo + boff2, a_hi, b_hi, idesc2, kstep_a, kstep_b, acc0);
-                        } else {
-                            wg_issue<2>(tmem_base + dcol0, a_lo, b_lo + boff0, a_hi, b_hi, idesc0, kstep_a, kstep_b, acc0);
-                            if (n_pieces > 1) wg_issue<2>(tmem_base + dcol1, a_lo, b_lo + boff1, a_hi, b_hi, idesc1, kstep_a, kstep_b, acc0);
-                            if (n_pieces > 2) wg_issue<2>(tmem_base + dcol2, a_lo, b_lo + boff2, a_hi, b_hi, idesc2, kstep_a, kstep_b, acc0);
+                    if (timed) waited += clock64() - w0;
+                    const int n_g = n_chunks - it * G < G ? n_chunks - it * G : G;
+                    if (elect_one()) {
+                        mbar_expect_tx(&full_bar[s], (uint32_t)n_g * tx);
+                        for (int g = 0; g < n_g; ++g) {
+                            int ch = chunk_begin + it * G + g;
+                            const int ow0 = (ch & (p.tiles_w - 1)) * p.bw;
+                            ch >>= p.tw_shift;
+                            const int th = ch / p.tiles_h;
+                            const int oh0 = (ch - th * p.tiles_h) * p.bh;
+                            const int n0 = th * p.bn;
+                            uint8_t* dst = smem + (size_t)s * p.stage_bytes + (size_t)g * p.sub_bytes;
+                            if (p.stack) {
+                                // one box with a halo row on top: copy 1 of dy (gathered one row higher) is its first pb pixels,
+                                // copy 0 starts one image row further down
+                                tma_load_4d(dst, &p.tmDy, &full_bar[s], 0, ow0, oh0 - 1, n0);
+                            } else {
+                                for (int j = 0; j < p.a_boxes; ++j)  // boxes past the last channel are zero-filled
+                                    tma_load_4d(dst + (size_t)j * p.box_a, &p.tmDy, &full_bar[s], ktile * 128 + j * p.cw_a, ow0, oh0, n0);
+                            }
+                            dst += p.a_bytes;
+                            if (p.fx) {   // one framed box per channel block, gathered at the first shift (one pixel to the left)
+                                for (int j = 0; j < p.b_boxes; ++j)
+                                    tma_load_4d(dst + (size_t)j * p.fx_box, &p.tmX[grp.map[0]], &full_bar[s], ctile * p.ct + j * p.cw_b, ow0 + grp.dw[0],
+                                                oh0 + grp.dh[0], n0);
+                            } else
+                            for (int b = 0; b < grp.nb; ++b)
+                                for (int j = 0; j < p.b_boxes; ++j)
+                                    tma_load_4d(dst + (size_t)(b * p.b_boxes + j) * p.box_b, &p.tmX[grp.map[b]], &full_bar[s], ctile * p.ct + j * p.cw_b,
+                                                ow0 + grp.dw[b], oh0 + grp.dh[b], n0);
                         }
-                    }
-                    umma_commit(&empty_bar[s]);
-                    if (it == 0) umma_commit(&init_bar);
-                }
-                __syncwarp();
-                if (timed) issuing += clock64() - w1;
-                s += n_issuers;
-                if (s >= S) { s -= S; ph ^= 1u; }
-            }
-            if (ok && n_chunks > 0 && elect_one()) umma_commit(&accum_bar);
-            __syncwarp();
-            if (timed && my == 0) {
-                atomicAdd(p.stall + 1, (unsigned long long)waited);
-                atomicAdd(p.stall + 4, (unsigned long long)(clock64() - t_begin));
-                atomicAdd(p.stall + 6, (unsigned long long)issuing);
-            }
-        }
-    }
-    // ------------------------------------------------------------------ epilogue: all eight warps
-    // The producer and MMA warps have nothing left to do once their loops end, so they help the four epilogue warps:
-    // two warps per TMEM lane quarter, each sending half of the channel chunks of every shift to dw.
-    {
-        const int q = warp & 3, part = warp >> 2;
-        const int m = q * 32 + lane;
-        const int copy = p.stack ? 1 - (m >> 6) : 0;                   // which dy copy this accumulator row belongs to (copy 1 comes first)
-        const int k = p.stack ? (m & 63) : ktile * 128 + m;
-        __syncwarp();
-        bool ok = n_chunks > 0;
-        if (ok) {
-            if (lane == 0) ok = mbar_wait_bounded(&accum_bar, 0u, p.spin_limit, &abort_flag);   // one poller per warp
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok && lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
-            tc_fence_after();
-        }
-        if (ok) {
-            const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
-            const int n_ck = p.ct >> 4;
-            const int ck_begin = part == 0 ? 0 : (n_ck + 1) >> 1, ck_end = part == 0 ? (n_ck + 1) >> 1 : n_ck;   // this warp's chunks
-            for (int b = 0; b < grp.nb && ck_begin < ck_end; ++b) {
-                const int rs = grp.rs[copy][b];
-                const bool live = rs >= 0 && k < p.k_total;
-                float* dst = p.dw + ctile * p.ct;
-                const int row_off = live ? (k * p.rs_total + rs) * p.c_total : -1;   // (a filter bank has fewer than 2^31 elements)
-                // accumulator column of 16-channel chunk ck of shift b (framed x: [channel block][shift][64 channels])
-                auto col = [&](int ck) -> uint32_t {
-                    const int per_block = p.cw_b >> 4;   // 16-channel chunks per x box
-                    return p.fx ? (uint32_t)((ck / per_block) * 3 * p.cw_b + b * p.cw_b + (ck % per_block) * 16) : (uint32_t)(b * p.ct + ck * 16);
-                };
-                // A lane holds 16 columns of one row, and rows are rs x c elements apart.  Four neighbouring lanes exchange their vectors
-                // first (a 4 x 4 transposition), so that they send 64 consecutive bytes of one row together: an instruction then touches
-                // 16 whole sectors in 8 lines instead of 32 half sectors in 32 lines.  This tail is the same whatever the batch (up to 148
-                // tiles of 196 KB): 128 -> 128 at 16x16 with 128 images 20.7 -> 15.6 us, with 50 images 17.4 -> 12.4; 512 -> 512 at 4x4 with
-                // 1024 images 70.5 -> 67.6 us.
-                const int t4 = lane & 3;
-                auto send = [&](uint32_t (&r)[16], int ck) {
-                    transpose_lanes4(r, t4);   // r[4 i ..] = vector t4 of the row of lane (lane - t4) + i
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int off = __shfl_sync(0xffffffffu, row_off, (lane & ~3) + i);
-                        if (off >= 0)
-                            red_add_v4(dst + off + ck * 16 + 4 * t4, __uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]), __uint_as_float(r[4 * i + 2]),
-                                       __uint_as_float(r[4 * i + 3]));
                     }
                     __syncwarp();
-                };
-                // two chunks in flight: the next one is fetched while the current one is sent out
-                uint32_t ra[16], rb[16];
-                tmem_ld16(t_row + col(ck_begin), ra);
-                tmem_ld_wait();
-                for (int ck = ck_begin; ck < ck_end; ck += 2) {
-                    if (ck + 1 < ck_end) tmem_ld16(t_row + col(ck + 1), rb);
-                    send(ra, ck);
-                    if (ck + 1 < ck_end) {
-                        tmem_ld_wait();
-                        if (ck + 2 < ck_end) tmem_ld16(t_row + col(ck + 2), ra);
-                        send(rb, ck + 1);
-                        if (ck + 2 < ck_end) tmem_ld_wait();
+                    last_issued = slot;
+                    if (s + kWgProducers < S) {
+                        slot += kWgProducers;
+                        s += kWgProducers;
+                    } else {   // wrap to this producer's first slot
+                        slot += S - s + w;
+                        s = w;
+                        ph ^= 1u;
                     }
+                }
+                if (timed) atomicAdd(p.stall + 0, (unsigned long long)waited);
+            }
+        } else if (warp == 1 || warp == 2) {
+            if (warp - 1 < p.issuers) {
+                const int my = role;
+                // SBO = eight pixel rows, LBO = next block of cw channels (the next box)
+                const uint64_t proto_a = make_smem_desc(0u, (uint32_t)p.a_lbo, 16u * (uint32_t)p.cw_a, (uint32_t)p.swz_a);
+                // framed x: the column blocks of an MMA are the three shifts, one pixel row (cw_b channels) apart
+                const uint64_t proto_b = p.fx ? make_smem_desc(0u, 2u * (uint32_t)p.cw_b, p.fx_sbo, (uint32_t)p.swz_b)
+                                              : make_smem_desc(0u, (uint32_t)p.box_b, 16u * (uint32_t)p.cw_b, (uint32_t)p.swz_b);
+                const uint32_t a_hi = (uint32_t)(proto_a >> 32), a_lo_base = (uint32_t)proto_a;
+                const uint32_t b_hi = (uint32_t)(proto_b >> 32), b_lo_base = (uint32_t)proto_b;
+                const uint32_t kstep_a = (uint32_t)(16 * p.cw_a * 2) >> 4, kstep_b = (uint32_t)(16 * p.cw_b * 2) >> 4;   // 16 pixel rows
+                const int ksteps = p.pb >> 4;
+                // up to three MMAs per k-step (kept in scalars: the issuing thread must not index local memory)
+                uint32_t idesc0 = 0, idesc1 = 0, idesc2 = 0, boff0 = 0, boff1 = 0, boff2 = 0, dcol0 = 0, dcol1 = 0, dcol2 = 0;
+                int n_pieces = 0;
+                for (int i = 0; i < p.n_pieces; ++i) {
+                    if (p.piece_t0[i] >= grp.nb) break;
+                    const int nt = min(p.piece_nt[i], grp.nb - p.piece_t0[i]);
+                    const uint32_t id = make_idesc_bf16(128, nt * p.ct, true, true);
+                    const uint32_t bo = (uint32_t)(p.a_bytes + p.piece_t0[i] * p.b_boxes * p.box_b) >> 4;
+                    const uint32_t dc = (uint32_t)(p.piece_t0[i] * p.ct);
+                    if (i == 0) { idesc0 = id; boff0 = bo; dcol0 = dc; }
+                    else if (i == 1) { idesc1 = id; boff1 = bo; dcol1 = dc; }
+                    else { idesc2 = id; boff2 = bo; dcol2 = dc; }
+                    ++n_pieces;
+                }
+                bool ok = true;
+                const bool timed = p.stall != nullptr && lane == 0;
+                const long long t_begin = timed ? clock64() : 0;
+                long long waited = 0, issuing = 0;
+                const int G = p.gsub;
+                const uint32_t sub16 = (uint32_t)p.sub_bytes >> 4;
+                if (slot != first_slot && slot < first_slot + n_slots) {   // the tile's first slot, the other thread's, has initialised the accumulator
+                    if (!mbar_wait_warp(&init_bar, tile_parity, p.spin_limit, &abort_flag)) {
+                        atomicOr(p.status, B2C_DEV_TIMEOUT);
+                        ok = false;
+                    }
+                    tc_fence_after();
+                }
+                // (this thread's chain of dependent instructions per slot bounds chunks with few MMAs: nothing is recomputed in the loop)
+                const bool fx = p.fx != 0;
+                const int n_issuers = p.issuers, b_boxes = p.b_boxes;
+                const uint32_t id_fx = make_idesc_bf16(128, 3 * p.cw_b, true, true);
+                const uint32_t fx_b_first = (uint32_t)p.a_bytes >> 4, fx_b_next = (uint32_t)p.fx_box >> 4, fx_d_next = 3u * (uint32_t)p.cw_b;
+                const uint32_t fk0 = p.fx_koff[0], fk1 = p.fx_koff[1], fk2 = p.fx_koff[2], fk3 = p.fx_koff[3];
+                const uint32_t stage16 = (uint32_t)p.stage_bytes >> 4, smem16 = smem_u32(smem) >> 4;
+                // S is even with two threads: a thread's slots are my, my + 2, ...
+                for (; ok && slot < first_slot + n_slots; slot += n_issuers) {
+                    const int it = slot - first_slot;
+                    const long long w0 = timed ? clock64() : 0;
+                    if (!mbar_wait_warp(&full_bar[s], ph, p.spin_limit, &abort_flag)) {
+                        atomicOr(p.status, B2C_DEV_TIMEOUT);
+                        ok = false;
+                        break;
+                    }
+                    const long long w1 = timed ? clock64() : 0;
+                    waited += w1 - w0;
+                    tc_fence_after();
+                    const uint32_t st16 = smem16 + (uint32_t)s * stage16;
+                    const int n_g = n_chunks - it * G < G ? n_chunks - it * G : G;
+                    if (elect_one()) {
+                        for (int g = 0; g < n_g; ++g) {
+                            const uint32_t a_lo = a_lo_base + st16 + (uint32_t)g * sub16, b_lo = b_lo_base + st16 + (uint32_t)g * sub16;
+                            const uint32_t acc0 = (it | g) != 0 ? 1u : 0u;
+                            if (fx) {   // chunks of 64 pixels: four k-steps; one MMA per channel block, N = three shifts x cw_b channels
+                                const uint32_t b_first = b_lo + fx_b_first;
+                                for (int i = 0; i < b_boxes; ++i)
+                                    wg_issue_framed<4>(tmem_base + (uint32_t)i * fx_d_next, a_lo, b_first + (uint32_t)i * fx_b_next, a_hi, b_hi, id_fx, kstep_a, fk0, fk1, fk2,
+                                                       fk3, acc0);
+                            } else if (ksteps == 4) {
+                                wg_issue<4>(tmem_base + dcol0, a_lo, b_lo + boff0, a_hi, b_hi, idesc0, kstep_a, kstep_b, acc0);
+                                if (n_pieces > 1) wg_issue<4>(tmem_base + dcol1, a_lo, b_lo + boff1, a_hi, b_hi, idesc1, kstep_a, kstep_b, acc0);
+                                if (n_pieces > 2) wg_issue<4>(tmem_base + dcol2, a_lo, b_lo + boff2, a_hi, b_hi, idesc2, kstep_a, kstep_b, acc0);
+                            } else {
+                                wg_issue<2>(tmem_base + dcol0, a_lo, b_lo + boff0, a_hi, b_hi, idesc0, kstep_a, kstep_b, acc0);
+                                if (n_pieces > 1) wg_issue<2>(tmem_base + dcol1, a_lo, b_lo + boff1, a_hi, b_hi, idesc1, kstep_a, kstep_b, acc0);
+                                if (n_pieces > 2) wg_issue<2>(tmem_base + dcol2, a_lo, b_lo + boff2, a_hi, b_hi, idesc2, kstep_a, kstep_b, acc0);
+                            }
+                        }
+                        umma_commit(&empty_bar[s]);
+                        if (it == 0) umma_commit(&init_bar);
+                    }
+                    __syncwarp();
+                    if (timed) issuing += clock64() - w1;
+                    s += n_issuers;
+                    if (s >= S) { s -= S; ph ^= 1u; }
+                }
+                if (ok && n_chunks > 0 && elect_one()) umma_commit(&accum_bar);
+                __syncwarp();
+                if (timed && my == 0) {
+                    atomicAdd(p.stall + 1, (unsigned long long)waited);
+                    atomicAdd(p.stall + 4, (unsigned long long)(clock64() - t_begin));
+                    atomicAdd(p.stall + 6, (unsigned long long)issuing);
                 }
             }
         }
-        if (p.stall != nullptr && lane == 0) atomicMax(p.stall + 7, (unsigned long long)(clock64() - t_kernel));   // the slowest warp of the slowest CTA
-        if (p.stall != nullptr && warp == 2 && lane == 0) atomicAdd(p.stall + 5, (unsigned long long)(clock64() - t_kernel));
-    }
-    tc_fence_before();
-    __syncthreads();
+        // ------------------------------------------------------------------ epilogue: all eight warps
+        // The producer and MMA warps have nothing left to do once their loops end, so they help the four epilogue warps:
+        // two warps per TMEM lane quarter, each sending half of the channel chunks of every shift to dw.
+        {
+            const int q = warp & 3, part = warp >> 2;
+            const int m = q * 32 + lane;
+            const int copy = p.stack ? 1 - (m >> 6) : 0;                   // which dy copy this accumulator row belongs to (copy 1 comes first)
+            const int k = p.stack ? (m & 63) : ktile * 128 + m;
+            __syncwarp();
+            bool ok = n_chunks > 0;
+            if (ok) {
+                if (lane == 0) ok = mbar_wait_bounded(&accum_bar, tile_parity, p.spin_limit, &abort_flag);   // one poller per warp
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok && lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
+                tc_fence_after();
+            }
+            if (ok) {
+                const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
+                const int n_ck = p.ct >> 4;
+                const int ck_begin = part == 0 ? 0 : (n_ck + 1) >> 1, ck_end = part == 0 ? (n_ck + 1) >> 1 : n_ck;   // this warp's chunks
+                for (int b = 0; b < grp.nb && ck_begin < ck_end; ++b) {
+                    const int rs = grp.rs[copy][b];
+                    const bool live = rs >= 0 && k < p.k_total;
+                    float* dst = p.dw + ctile * p.ct;
+                    const int row_off = live ? (k * p.rs_total + rs) * p.c_total : -1;   // (a filter bank has fewer than 2^31 elements)
+                    // accumulator column of 16-channel chunk ck of shift b (framed x: [channel block][shift][64 channels])
+                    auto col = [&](int ck) -> uint32_t {
+                        const int per_block = p.cw_b >> 4;   // 16-channel chunks per x box
+                        return p.fx ? (uint32_t)((ck / per_block) * 3 * p.cw_b + b * p.cw_b + (ck % per_block) * 16) : (uint32_t)(b * p.ct + ck * 16);
+                    };
+                    // A lane holds 16 columns of one row, and rows are rs x c elements apart.  Four neighbouring lanes exchange their vectors
+                    // first (a 4 x 4 transposition), so that they send 64 consecutive bytes of one row together: an instruction then touches
+                    // 16 whole sectors in 8 lines instead of 32 half sectors in 32 lines.  This tail is the same whatever the batch (up to 148
+                    // tiles of 196 KB): 128 -> 128 at 16x16 with 128 images 20.7 -> 15.6 us, with 50 images 17.4 -> 12.4; 512 -> 512 at 4x4 with
+                    // 1024 images 70.5 -> 67.6 us.
+                    const int t4 = lane & 3;
+                    auto send = [&](uint32_t (&r)[16], int ck) {
+                        transpose_lanes4(r, t4);   // r[4 i ..] = vector t4 of the row of lane (lane - t4) + i
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int off = __shfl_sync(0xffffffffu, row_off, (lane & ~3) + i);
+                            if (off >= 0)
+                                red_add_v4(dst + off + ck * 16 + 4 * t4, __uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]), __uint_as_float(r[4 * i + 2]),
+                                           __uint_as_float(r[4 * i + 3]));
+                        }
+                        __syncwarp();
+                    };
+                    // two chunks in flight: the next one is fetched while the current one is sent out
+                    uint32_t ra[16], rb[16];
+                    tmem_ld16(t_row + col(ck_begin), ra);
+                    tmem_ld_wait();
+                    for (int ck = ck_begin; ck < ck_end; ck += 2) {
+                        if (ck + 1 < ck_end) tmem_ld16(t_row + col(ck + 1), rb);
+                        send(ra, ck);
+                        if (ck + 1 < ck_end) {
+                            tmem_ld_wait();
+                            if (ck + 2 < ck_end) tmem_ld16(t_row + col(ck + 2), ra);
+                            send(rb, ck + 1);
+                            if (ck + 2 < ck_end) tmem_ld_wait();
+                        }
+                    }
+                }
+            }
+            if (p.stall != nullptr && lane == 0) atomicMax(p.stall + 7, (unsigned long long)(clock64() - t_kernel));   // the slowest warp of the slowest CTA
+            if (p.stall != nullptr && warp == 2 && lane == 0) atomicAdd(p.stall + 5, (unsigned long long)(clock64() - t_kernel));
+        }
+        tc_fence_before();
+        __syncthreads();
+        if constexpr (STREAM) {   // the accumulator has been read: the next tile may overwrite it
+            tc_fence_after();
+            slot_ = slot;
+            s_ = s;
+            ph_ = ph;
+            first_slot_ += n_slots;
+            tile_parity_ ^= 1u;
+            left -= n_chunks;
+            chunk_begin = 0;
+            if (++ktile == p.n_ktiles) {
+                ktile = 0;
+                if (++ctile == p.n_ctiles) { ctile = 0; ++gi; }
+            }
+            if (abort_flag) break;
+        }
+    } while (STREAM && left > 0);
     if (abort_flag) {
         // A wait gave up: let the issued bulk copies land and the issued MMAs retire before exit.
         if ((warp == 0 || warp >= kWgProducerWarp1) && lane == 0) {
@@ -450,9 +489,11 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     p.swz_b = p.cw_b == 64 ? SWZ_128B : p.cw_b == 32 ? SWZ_64B : SWZ_32B;
     // stacking needs chunks that stay inside one image (at least 64 pixels per image)
     p.stack = (R == 3 && pb.stride == 1 && pb.k == 64 && pb.p * pb.q >= 64 && pb.q >= 8) ? 1 : 0;   // q >= 8: the second copy starts on a swizzle-atom boundary
-    // x-channel tile: largest divisor of c that is a multiple of cw_b, at most 160 (three shifts fit 512 TMEM columns)
+    // x-channel tile: largest divisor of c that is a multiple of cw_b, at most 160 (three shifts fit 512 TMEM columns) or, for 1x1 layers, 256:
+    // with 128 x 128 tiles a chunk's operands (32 KB for 256 tensor-pipe cycles) come in at twice the rate an SM can load.  256 -> 1024 at 8x8
+    // with 1024 images 40.8 -> 38.5 us, 512 -> 2048 at 4x4 44.8 -> 41.5.
     p.ct = p.cw_b;
-    for (int cand = 160; cand >= p.cw_b; cand -= 16)
+    for (int cand = R == 1 ? 256 : 160; cand >= p.cw_b; cand -= 16)
         if (pb.c % cand == 0 && cand % p.cw_b == 0) { p.ct = cand; break; }
     // framed x stages: 64 pixels of one image per chunk, 64-channel x boxes, at most two of them per CTA (2 x 192 TMEM columns)
     p.fx = (R == 3 && pb.stride == 1 && pb.q >= 8 && pb.p * pb.q >= 64 && p.cw_b >= 32 && ctx->use_wgrad_frame) ? 1 : 0;
@@ -574,6 +615,17 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     if (n_splits > p.chunks_total / 4) n_splits = p.chunks_total / 4;
     if (n_splits < 1) n_splits = 1;
     p.n_splits = n_splits;
+    // Tiles that do not divide the SMs evenly leave many of them idle (75 tiles: one CTA each on 148 SMs: 640 -> 640 at 8x8 with 256 images 135 us, now 91).  Equal runs of (tile, chunk)
+    // pairs keep all busy, at the price of one more accumulator to send for most CTAs (about 9000 cycles).
+    {
+        const int cols = p.fx ? p.b_boxes * 3 * p.cw_b : shifts * p.ct;
+        const double mma = (p.pb / 16) * (cols / 2.0), load = p.sub_bytes / 60.0, chunk = mma > load ? mma : load, tail = 9000.0;
+        const int waves = (base * n_splits + ctx->sm_count - 1) / ctx->sm_count;
+        const double plain = waves * (((p.chunks_total + n_splits - 1) / n_splits) * chunk + tail);
+        const double per_cta = (double)base * p.chunks_total / ctx->sm_count;   // chunks
+        const double equal = per_cta * chunk + ((double)base / ctx->sm_count + 1.0) * tail;
+        p.stream = per_cta >= 8.0 && equal < 0.85 * plain ? 1 : 0;   // (an estimated tenth was measured as a loss: 320 -> 320 at 16x16 107 -> 111 us)
+    }
 
     if (!encode_activation_map(ctx, &p.tmDy, pb.dy, pb.n, pb.p, pb.q, pb.k, 1, 0, 0, p.cw_a, p.bw, p.stack ? p.bh + 1 : p.bh, p.bn)) return B2C_ERR_CUDA;
     if (pb.stride == 2) {
@@ -589,7 +641,7 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     p.rs_total = R * R;
     p.dw = pb.dw;
     plan.smem_bytes = (size_t)p.stages * p.stage_bytes + 1024;
-    plan.grid = base * n_splits;
+    plan.grid = p.stream ? ctx->sm_count : base * n_splits;
     return B2C_OK;
 }
 
@@ -616,12 +668,13 @@ b2c_status launch_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, cudaStream_t 
     p.stall = ctx->stall_counters;
 
     if (!(ctx->smem_optin_done & B2C_OPTIN_WGRAD)) {
-        B2C_CUDA(cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
+        B2C_CUDA(cudaFuncSetAttribute(conv_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
+        B2C_CUDA(cudaFuncSetAttribute(conv_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
         ctx->smem_optin_done |= B2C_OPTIN_WGRAD;
     }
     const size_t smem_bytes = plan.smem_bytes;
     dim3 grid((unsigned)plan.grid);
-    B2C_CUDA(b2c_launch(ctx, conv_wgrad_kernel, grid, dim3(kWgThreads), smem_bytes, stream, 1u, p));
+    B2C_CUDA(b2c_launch(ctx, p.stream ? conv_wgrad_kernel<true> : conv_wgrad_kernel<false>, grid, dim3(kWgThreads), smem_bytes, stream, 1u, p));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;
 }
