@@ -704,6 +704,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
         for (int i = 0; i < kMaxStages; ++i) slot_stage[i] = 0;
         fence_mbar_init();
     }
+    const UnitWalk walk(p, rank);   // (its divisions are over before the wait for the previous kernel)
     if (warp == 1) {
         if constexpr (PAIR) {
             tmem_alloc_pair(&tmem_slot, (uint32_t)p.tmem_cols);
@@ -722,7 +723,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
     pdl_wait();
     pdl_launch_dependents();
     const long long t_start = clock64();
-    const UnitWalk walk(p, rank);
     int last_issued = -1;  // producer lanes: index of the last stage whose loads this lane issued
 
     if (warp == 0 || warp == kProducerWarp1) {
