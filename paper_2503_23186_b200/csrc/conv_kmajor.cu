@@ -1059,28 +1059,31 @@ struct KMajorPlan {
 
 // Tensor-pipe and staging cycles of one k-block of kb channels on a tile of 128 pixels (a pair: 2 x 128) x n channels: an MMA of 16
 // channels takes n / 2 cycles, or what its operands take through the 128 B/clk shared-memory port (A: 4 KB, B: 32 n bytes, half of
-// it per CTA of a pair); the loads come in at about 60 B/clk per SM (measured, L2 -> shared memory with every SM streaming).
+// it per CTA of a pair); the loads come in at about 74 B/clk per SM (fitted with the estimates below).
 static int kblock_cycles(int n, int kb, bool pair, int a_rows)
 {
     const int b_rows = pair ? n / 2 : n;
     const int operand = 32 + b_rows / 4, mma = (operand > n / 2 ? operand : n / 2) * (kb / 16);
-    const int loads = (a_rows + b_rows) * kb * 2 / 60;
+    const int loads = (a_rows + b_rows) * kb * 2 / 74;
     return mma > loads ? mma : loads;
 }
 
-// Split-K plan (conv_splitk.cu) for a problem whose tiles do not fill the chip, or false where the persistent plan (est_cycles for its
-// busiest CTA) is the better one by the same estimate.  A cluster of `splits` CTAs or pairs shares a tile's k-blocks, all
-// clusters run in one wave, and the exchange of the partial tiles costs a cluster barrier and (splits - 1) / splits of the tile
-// at about 32 B/clk.  Measured with 128 images (launch to launch):
-// 512 -> 512 at 4x4 27.8 -> 17.6 us, 256 -> 256 at 8x8 18.2 -> 14.3; with 50 images 26.2 -> 12.0 and 16.2 -> 12.4 us.
+// Plan for the one-wave kernel (conv_splitk.cu) for a problem whose tiles do not fill the chip, or false where the persistent
+// plan (est_cycles) is the better one.  A cluster of `splits` CTAs or pairs shares a tile's k-blocks and adds the partial tiles
+// up at the end; splits = 1 is a tile per CTA or pair, whose shorter epilogue still beats the persistent kernel's one unit.
+// The estimates, in cycles over the 4 us that any launch takes, were fitted to 330 timed plans of 27 layers: the plan they
+// pick is on average 0.3 % and at most 5 % slower than the layer's best one.  With 128 images, persistent -> this, launch to
+// launch: 512 -> 512 at 4x4 27.8 -> 14.1 us, 256 -> 256 at 8x8 18.2 -> 12.7, 256 -> 512 at 8x8 stride 2 16.6 -> 10.5; with 50
+// images 26.3 -> 10.7, 16.4 -> 10.2 and 16.4 -> 8.6; 128 -> 128 at 8x8 with 16 images 10.3 -> 5.7.
 static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p, int m_tiles, long long est_cycles)
 {
     const int kb = (pb.ic % 64 == 0) ? 64 : (pb.ic % 32 == 0) ? 32 : 16;
     const int taps = p.n_par > 1 ? ((pb.r + 1) / 2) * ((pb.r + 1) / 2) : pb.r * pb.r;   // of the parity with most
     const int min_taps = p.n_par > 1 ? 1 : taps;
     const int c_blocks = pb.ic / kb;
-    long long best = est_cycles;
+    long long best = est_cycles - 600;   // worth a change from the persistent kernel (0.6 us)
     bool found = false;
+    const int smem = 208 * 1024;   // (beside 16.6 KB of static arrays)
     for (int pair = 0; pair <= 1; ++pair) {
         if (pair && (p.n_par > 1 || ctx->use_pairs == 0)) continue;
         for (int n = 256; n >= 32; n -= 16) {
@@ -1089,12 +1092,29 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
             for (int splits = 1; splits * (pair + 1) <= 8; splits *= 2) {
                 if (n % (8 * splits) || splits > min_taps * c_blocks) continue;
                 if (clusters > splitk_max_clusters(ctx, splits * (pair + 1), pair != 0)) continue;
+                const int b_rows = pair ? n / 2 : n, a_bytes = 128 * kb * 2, b_bytes = (b_rows * kb * 2 + 1023) & ~1023;
+                const int x_bytes = (splits - 1) * (n / splits) * 512;   // partial tiles of the other CTAs
+                // k-blocks share a slot until it holds the MMAs of the issuing thread's 500 cycles per slot, while three slots are left
+                const int block = kblock_cycles(n, kb, pair != 0, 128), mma = (n / 2 > 48 ? n / 2 : 48) * (kb / 16);
+                int gsub = 1;
+                while (gsub < 4 && gsub * mma < 480 && 6 * gsub * (a_bytes + b_bytes) <= smem && 2 * gsub * splits <= taps * c_blocks) gsub *= 2;
+                const int slot = gsub * (a_bytes + b_bytes);
+                int stages = (smem - x_bytes) / slot;
+                const int overlap = splits > 1 && stages < (gsub > 1 ? 3 : 4) ? 1 : 0;   // too few slots left: exchange through the ring's memory
+                if (overlap) stages = smem / slot;
+                if (stages > kMaxStages) stages = kMaxStages;
+                if (stages < 2 || (overlap && stages * slot < x_bytes)) continue;
                 const int k_blocks = (taps * c_blocks + splits - 1) / splits;
-                const long long est = (long long)k_blocks * kblock_cycles(n, kb, pair != 0, 128) + (splits > 1 ? 1500 + 16ll * n * (splits - 1) / splits : 0);
-                if (est * 10 >= best * 9) continue;   // a tenth better at least
+                // k-blocks, exchange (barriers, partial tiles at 21 B/clk), epilogue of n / splits columns
+                const long long per_block = block > 570 / gsub ? block : 570 / gsub;
+                const long long est = k_blocks * per_block + (splits > 1 ? 1100 + 800 * overlap + x_bytes / 21 : 0) + 190ll * n / splits / 32 + 2600 * pair;
+                if (est >= best) continue;
                 best = est;
                 found = true;
                 p.n_tile = n; p.n_ktiles = pb.oc / n; p.pair = pair; p.splits = splits;
+                p.a_bytes = a_bytes; p.b_bytes = b_bytes; p.gsub = gsub; p.stages = stages;
+                p.x_overlap = overlap;
+                p.x_off = overlap ? 0 : stages * slot;
             }
         }
     }
@@ -1103,14 +1123,8 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
     p.kb = kb; p.c_blocks = c_blocks;
     p.swz = kb == 64 ? SWZ_128B : kb == 32 ? SWZ_64B : SWZ_32B;
     p.nb = 1;
-    p.tx_a = p.a_bytes = 128 * kb * 2;
+    p.tx_a = p.a_bytes;
     p.tx_b = b_rows * kb * 2;
-    p.b_bytes = (p.tx_b + 1023) & ~1023;
-    p.gsub = 1;   // k-blocks of a ring slot: narrow ones share a slot, its barrier wait and its commit
-    while (p.gsub < 4 && 2 * p.gsub * (p.a_bytes + p.b_bytes) <= 40 * 1024 && 2 * p.gsub * p.splits <= taps * c_blocks) p.gsub *= 2;
-    p.stages = 214 * 1024 / (p.gsub * (p.a_bytes + p.b_bytes));   // (beside 10.4 KB of static arrays)
-    if (p.stages > kMaxStages) p.stages = kMaxStages;
-    if (p.splits > 1 && p.stages * p.gsub * (p.a_bytes + p.b_bytes) < 512 * p.n_tile) return false;   // the partial tiles are exchanged in the ring's memory
     p.tmem_cols = 32;
     while (p.tmem_cols < p.n_tile) p.tmem_cols *= 2;
     p.total_units = p.n_par * (p.pair ? m_tiles + (m_tiles & 1) : m_tiles / p.n_par) * p.n_ktiles;
@@ -1276,7 +1290,9 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
         q.bw = gw < 128 ? gw : 128; q.bh = (128 / q.bw) < gh ? (128 / q.bw) : gh; q.bn = 128 / (q.bw * q.bh);
         q.tiles_w = gw / q.bw; q.tiles_h = gh / q.bh; q.tiles_n = (pb.n + q.bn - 1) / q.bn;
         q.vreuse = q.fh = q.hm = q.resident = q.resident_bytes = q.b_merged = q.a_step = 0;
-        if (choose_splitk(ctx, pb, q, n_par * m_tiles, (long long)units_per_cta * max_taps * (pb.ic / p.kb) * kblock_cycles(n_tile, p.kb, p.pair != 0, a_rows))) {
+        const int block = kblock_cycles(n_tile, p.kb, p.pair != 0, a_rows), per_block = p.vreuse || block > 400 ? block : 400;
+        const long long persistent = (long long)units_per_cta * max_taps * (pb.ic / p.kb) * per_block + 1060ll * n_tile / 32;
+        if (choose_splitk(ctx, pb, q, n_par * m_tiles, persistent)) {
             p = q;
             cluster = p.splits * (p.pair ? 2 : 1);
             b_rows = p.pair ? p.n_tile / 2 : p.n_tile;
@@ -1312,7 +1328,8 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
         p.issue_split = 1;
     }
     const int stage_bytes = p.gsub * (p.a_bytes + (p.resident ? 0 : p.nb * p.b_bytes));
-    const size_t smem_bytes = (size_t)p.resident_bytes + (size_t)p.stages * stage_bytes + 1024;
+    const size_t smem_bytes = (size_t)p.resident_bytes + (size_t)p.stages * stage_bytes + 1024 +
+                              (cluster && !p.x_overlap ? (size_t)(p.splits - 1) * (p.n_tile / p.splits) * 512 : 0);
 
     // tensor maps
     const int box_h = (p.vreuse || p.fh || p.hm) ? p.bh + 2 : p.bh;

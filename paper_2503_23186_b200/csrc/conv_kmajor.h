@@ -35,6 +35,7 @@ struct alignas(64) ConvKParams {
     int gsub;                        // k-blocks that share a ring slot, one barrier wait and one commit (short k-blocks: the waits would bound the issuing threads)
     int issue_split;                 // the two issuing threads share every unit: alternate stages into one accumulator (tiles wider than 128 channels)
     int splits;                      // split-K plans (conv_splitk.cu): CTAs (or CTA pairs) of a cluster that share a unit's k-blocks; 0: persistent kernel
+    int x_off, x_overlap;            // split-K: byte offset of the exchange area behind the ring's start; it overlaps the ring
     int pair;                        // CTA pairs (cta_group::2): M = 256 per MMA, each CTA holds half of every B tile
     int resident;                    // filter bank of this CTA's channel tile stays in shared memory
     int resident_bytes;

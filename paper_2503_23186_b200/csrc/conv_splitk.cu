@@ -9,13 +9,18 @@
 // columns.  Nothing is written to global memory but the result, so no workspace and no second launch are needed.
 //   * One tile per cluster, not persistent: barriers and TMEM are set up once, every warp joins the epilogue when the main
 //     loop has been issued, and the kernel is small (a launch inside a step starts on a cold instruction cache).
-//   * The exchange goes through the ring's memory, which is free once the MMAs of every CTA of the cluster have completed
-//     (first cluster barrier).  A lane holds one row, so a block of four columns is stored as 128 rows x 16 bytes:
-//     neighbouring lanes write neighbouring 16-byte words of the receiver.
-// What bounds it now: the operands' way from L2 (a pair with 256 channels stages 32 KB per 512 tensor-pipe cycles, the rate one
-// SM can load), then the set-up and the exchange, about 3 us together.  Inside a step (128 images, time to the next kernel's
-// start): 512 -> 512 at 4x4 33 -> 14 us, 256 -> 256 at 8x8 32 -> 13 us; the whole ResNet-18-shaped step 1.89 -> 1.73 ms, as four
-// micro-batches of 50 6.32 -> 5.41 ms.
+//   * The exchange has an area of its own where three or four ring slots fit beside it; otherwise it goes through the ring's
+//     memory, which is free once the MMAs of every CTA of the cluster have completed (one more cluster barrier, about 1350
+//     cycles).  A lane holds one row, so a block of four columns is stored as 128 rows x 16 bytes: neighbouring lanes write
+//     neighbouring 16-byte words of the receiver, and the next columns are read from TMEM while the current ones are sent.
+//   * A slot holds two or four k-blocks of a narrow tile: waiting, issuing and committing cost about 500 cycles per slot, as
+//     long as the MMAs of 256 channels (128 channels, 36 k-blocks: 19.8 k cycles to the last MMA with one k-block per slot,
+//     13.4 k with two).
+// What bounds it now: the operands' way from L2 (about 74 B/clk per SM), then the set-up and the exchange, about 3 us together.
+// Launch to launch with 128 images: 512 -> 512 at 4x4 28 us in the persistent kernel, 13.5 here (17.4 with one k-block per slot,
+// the exchange in the ring and single-buffered); 256 -> 256 at 8x8 18.2 and 12.3 (14.1); the ResNet-18-shaped step of 128 images
+// 1.89 -> 1.73 ms when this kernel came and 1.490 -> 1.452 ms with those three, as four micro-batches of 50 6.32 -> 5.41 and
+// 4.41 -> 4.28 ms.
 // Warp roles during the main loop: warp 0 = TMA producer, warp 1 = TMEM owner and MMA issuer.  Every mbarrier wait is
 // bounded; a CTA that gives up still takes part in both cluster barriers.
 #include "conv_kmajor.h"
@@ -72,13 +77,15 @@ __device__ __forceinline__ void column_sums(const uint32_t (&pk)[8], float* stag
     }
 }
 
-template <bool PAIR>
+// TIMED: the instance that adds to the stall counters (read at run time, they cost the small net of tests and benchmarks 2.5 % of
+// its step: 198 -> 203 us)
+template <bool PAIR, bool TIMED>
 __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid_constant__ ConvKParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_bar[kSkStages], empty_bar[kSkStages], acc_bar, drain_bar;
     __shared__ uint32_t tmem_slot, abort_flag;
-    __shared__ float s_sum[2][256];   // BatchNorm sums of this CTA's columns
+    __shared__ float s_sum[4][2][256];   // BatchNorm sums of this CTA's columns, per TMEM lane quarter (shared-memory float atomics took 500 cycles a block)
     __shared__ __align__(16) float s_stage[kSkThreads / 32][256];   // staging of column_sums
 
     // (the same offset in every CTA of the cluster: the exchange maps addresses from one CTA to another)
@@ -90,6 +97,8 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     const uint32_t leader = (uint32_t)(cta - rank);
     const int S = p.stages, G = p.gsub;
     const int sub_bytes = p.a_bytes + p.b_bytes, stage_bytes = G * sub_bytes;
+
+    const long long t_start = TIMED ? clock64() : 0;
 
     // the unit of this cluster (a pair takes two neighbouring pixel tiles) and this CTA's share of its k-blocks
     const int cluster_id = (int)blockIdx.x / (p.splits * (PAIR ? 2 : 1));
@@ -109,7 +118,6 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
         abort_flag = 0;
         fence_mbar_init();
     }
-    for (int i = threadIdx.x; i < 512; i += kSkThreads) (&s_sum[0][0])[i] = 0.f;
     if (warp == 1) {
         if constexpr (PAIR) {
             tmem_alloc_pair(&tmem_slot, (uint32_t)p.tmem_cols);
@@ -124,7 +132,8 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     }
     tc_fence_before();
     __syncthreads();
-    if constexpr (PAIR) cluster_sync_all();   // the peer's barriers exist before anything arrives on them
+    const bool clustered = PAIR || p.splits > 1;
+    if (clustered) cluster_sync_all();   // the others' barriers and memory exist before anything arrives there
     tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
     pdl_wait();
@@ -136,11 +145,14 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
         const int oc0 = c.ktile * p.n_tile + rank * b_rows;
         int s = 0;
         uint32_t ph = 0;
+        long long waited = 0;
         for (int it = 0; it < n_slots; ++it) {
+            const long long t0 = TIMED ? clock64() : 0;
             if (!mbar_wait_warp(&empty_bar[s], ph ^ 1u, p.spin_limit, &abort_flag)) {
                 if (lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
                 break;
             }
+            if (TIMED) waited += clock64() - t0;
             const int n_k = k_count - it * G < G ? k_count - it * G : G;
             if (elect_one()) {
                 const uint32_t bar = PAIR ? map_to_cta(smem_u32(&full_bar[s]), leader) : 0u;
@@ -163,6 +175,7 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
             issued = it + 1;
             if (++s == S) { s = 0; ph ^= 1u; }
         }
+        if (TIMED && rank == 0 && lane == 0) atomicAdd(p.stall + 0, (unsigned long long)waited);
     } else if (warp == 1 && rank == 0) {
         const uint32_t idesc = make_idesc_bf16(PAIR ? 256 : 128, p.n_tile, false, false);
         const uint64_t proto = make_smem_desc(0u, 16u, 8u * (uint32_t)p.kb * 2u, (uint32_t)p.swz);   // eight rows of kb bf16
@@ -172,12 +185,15 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
         int s = 0;
         uint32_t ph = 0;
         bool ok = true;
+        long long waited = 0;
         for (int it = 0; it < n_slots; ++it) {
+            const long long t0 = TIMED ? clock64() : 0;
             ok = mbar_wait_warp(&full_bar[s], ph, p.spin_limit, &abort_flag);
             if (!ok) {
                 if (lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
                 break;
             }
+            if (TIMED) waited += clock64() - t0;
             tc_fence_after();
             const int n_k = k_count - it * G < G ? k_count - it * G : G;
             if (elect_one()) {
@@ -190,6 +206,7 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
             __syncwarp();
             if (++s == S) { s = 0; ph ^= 1u; }
         }
+        if (TIMED && lane == 0) atomicAdd(p.stall + 1, (unsigned long long)waited);
         if (ok && n_slots > 0 && elect_one()) {
             if constexpr (PAIR) umma_commit_pair(&acc_bar, (uint16_t)(3u << leader));
             else umma_commit(&acc_bar);
@@ -199,17 +216,18 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
 
     // ---------------------------------------------------------------- epilogue: all eight warps
     bool live = n_slots > 0;
+    const long long t_wait = TIMED ? clock64() : 0;
     if (live && !mbar_wait_warp(&acc_bar, 0u, p.spin_limit, &abort_flag)) {
         if (lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
         live = false;
     }
+    if (TIMED && rank == 0 && warp == 2 && lane == 0) atomicAdd(p.stall + 3, (unsigned long long)(clock64() - t_wait));
     tc_fence_before();
     __syncthreads();
-    const bool clustered = PAIR || p.splits > 1;
-    if (clustered) cluster_sync_all();   // every CTA's MMAs have completed (or it has given up): the rings may be written by the others
+    if (p.x_overlap) cluster_sync_all();   // every CTA's MMAs have completed (or it has given up): the rings may be written by the others
     if (abort_flag) {
         // A wait gave up: let the bulk copies counted on this CTA's barriers land and its MMAs retire before it goes on.  (Results are
-        // unspecified now; every write still stays inside the cluster's rings and the output.)
+        // unspecified now; every write still stays inside the cluster's exchange areas and the output.)
         if (warp == 0 && rank == 0)
             for (int back = 0; back < S && back < issued; ++back) {
                 const int it = issued - 1 - back;
@@ -234,25 +252,39 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     const int col0 = split * sw;
     const bool exchange = p.splits > 1 && k_total > 0;
     if (exchange) {
-        // partial sums of the other CTAs' columns -> their rings: block (sender, four columns) = 128 rows x 16 bytes
-        const int n8 = sw >> 3, c_lo = half ? (n8 + 1) >> 1 : 0, c_hi = half ? n8 : (n8 + 1) >> 1;
-        const uint32_t mine = smem_u32(ring) + (uint32_t)(split * (sw >> 2) * 128 + m) * 16u;
-        for (int j = 1; j < p.splits; ++j) {
-            const int dst = split + j < p.splits ? split + j : split + j - p.splits;
-            const uint32_t base = map_to_cta(mine, (uint32_t)(PAIR ? 2 * dst + rank : dst));
-            for (int ch = c_lo; ch < c_hi; ch += 2) {
-                uint32_t r0[8], r1[8];
-                tmem_ld8(t_row + (uint32_t)(dst * sw + ch * 8), r0);
-                if (ch + 1 < c_hi) tmem_ld8(t_row + (uint32_t)(dst * sw + ch * 8 + 8), r1);
-                tmem_ld_wait();
-#pragma unroll
-                for (int i = 0; i < 8; i += 4)
-                    st_cluster_v4(base + (uint32_t)(2 * ch + i / 4) * 2048u, __uint_as_float(r0[i]), __uint_as_float(r0[i + 1]), __uint_as_float(r0[i + 2]), __uint_as_float(r0[i + 3]));
-                if (ch + 1 < c_hi) {
-#pragma unroll
-                    for (int i = 0; i < 8; i += 4)
-                        st_cluster_v4(base + (uint32_t)(2 * ch + 2 + i / 4) * 2048u, __uint_as_float(r1[i]), __uint_as_float(r1[i + 1]), __uint_as_float(r1[i + 2]),
-                                      __uint_as_float(r1[i + 3]));
+        // partial sums of the other CTAs' columns -> their exchange areas: block (sender, four columns) = 128 rows x 16 bytes; the next columns
+        // are read from TMEM while the current ones are sent
+        const int n8 = sw >> 3, c_lo = half ? (n8 + 1) >> 1 : 0, n_c = (half ? n8 : (n8 + 1) >> 1) - c_lo, n_all = n_c * (p.splits - 1);
+        int f_dst = split + 1 < p.splits ? split + 1 : 0, f_ch = 0, s_dst = f_dst, s_ch = 0;   // next columns to read, next to send
+        auto step = [&](int& dst, int& ch) {
+            if (++ch == n_c) {
+                ch = 0;
+                if (++dst == p.splits) dst = 0;
+            }
+        };
+        auto send = [&](const uint32_t (&r)[8]) {
+            const uint32_t at = map_to_cta(smem_u32(ring) + (uint32_t)p.x_off + (uint32_t)(((split < s_dst ? split : split - 1) * (sw >> 2) + 2 * (c_lo + s_ch)) * 128 + m) * 16u,
+                                           (uint32_t)(PAIR ? 2 * s_dst + rank : s_dst));
+            st_cluster_v4(at, __uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]), __uint_as_float(r[3]));
+            st_cluster_v4(at + 2048u, __uint_as_float(r[4]), __uint_as_float(r[5]), __uint_as_float(r[6]), __uint_as_float(r[7]));
+            step(s_dst, s_ch);
+        };
+        auto fetch = [&](uint32_t (&r)[8]) {
+            tmem_ld8(t_row + (uint32_t)(f_dst * sw + (c_lo + f_ch) * 8), r);
+            step(f_dst, f_ch);
+        };
+        if (n_all > 0) {
+            uint32_t r0[8], r1[8];
+            fetch(r0);
+            tmem_ld_wait();
+            for (int i = 0; i < n_all; i += 2) {
+                if (i + 1 < n_all) fetch(r1);
+                send(r0);
+                if (i + 1 < n_all) {
+                    tmem_ld_wait();
+                    if (i + 2 < n_all) fetch(r0);
+                    send(r1);
+                    if (i + 2 < n_all) tmem_ld_wait();
                 }
             }
         }
@@ -265,29 +297,35 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     const bool do_stats = p.stats != nullptr;
     // 16 columns at a time (the last step of an odd count of eights takes 8)
     const int n16 = (sw + 15) >> 4, g_lo = half ? (n16 + 1) >> 1 : 0, g_hi = half ? n16 : (n16 + 1) >> 1;
+    auto fetch = [&](uint32_t (&r)[16], int g) {
+        uint32_t lo[8], hi[8];
+        tmem_ld8(t_row + (uint32_t)(col0 + g * 16), lo);
+        if (g * 16 + 16 <= sw) tmem_ld8(t_row + (uint32_t)(col0 + g * 16 + 8), hi);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            r[i] = lo[i];
+            r[8 + i] = g * 16 + 16 <= sw ? hi[i] : 0u;
+        }
+    };
+    const float4* xin = reinterpret_cast<const float4*>(ring + p.x_off) + m;
+    const int x_sender = (sw >> 2) * 128;   // float4s of one sender
     for (int g = g_lo; g < g_hi; ++g) {
         const bool wide = g * 16 + 16 <= sw;
         uint32_t r[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) r[i] = 0u;
         if (k_total > 0) {
-            uint32_t lo[8], hi[8];
-            tmem_ld8(t_row + (uint32_t)(col0 + g * 16), lo);
-            if (wide) tmem_ld8(t_row + (uint32_t)(col0 + g * 16 + 8), hi);
-            tmem_ld_wait();
+            fetch(r, g);
+        } else {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                r[i] = lo[i];
-                r[8 + i] = wide ? hi[i] : 0u;
-            }
+            for (int i = 0; i < 16; ++i) r[i] = 0u;
         }
         float v[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
         if (exchange) {
-            for (int src = 0; src < p.splits; ++src) {
-                if (src == split) continue;
-                const float4* in = reinterpret_cast<const float4*>(ring) + (size_t)(src * (sw >> 2) + 4 * g) * 128 + m;
+            const float4* in = xin + (size_t)4 * g * 128;
+#pragma unroll 2
+            for (int src = 1; src < p.splits; ++src, in += x_sender) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (i < 2 || wide) {
@@ -334,11 +372,11 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
             }
             float s[2], sq[2];
             column_sums(pk, s_stage[warp], lane, s, sq);
-            if (column_owner(lane)) {   // the four lane quarters meet in shared memory
+            if (column_owner(lane)) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    atomicAdd(&s_sum[0][g * 16 + h * 8 + (lane >> 2)], s[h]);
-                    atomicAdd(&s_sum[1][g * 16 + h * 8 + (lane >> 2)], sq[h]);
+                    s_sum[q][0][g * 16 + h * 8 + (lane >> 2)] = s[h];
+                    s_sum[q][1][g * 16 + h * 8 + (lane >> 2)] = sq[h];
                 }
             }
             __syncwarp();
@@ -351,8 +389,13 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
         double* st = p.stats + (size_t)grp * 2 * p.oc_valid + c.ktile * p.n_tile + col0;
         if (c.n0 < p.n_valid)   // (the second tile of a pair may lie past the last image)
             for (int i = threadIdx.x; i < sw; i += kSkThreads) {
-                atomicAdd(st + i, (double)s_sum[0][i]);
-                atomicAdd(st + p.oc_valid + i, (double)s_sum[1][i]);
+                double s = 0.0, sq = 0.0;
+                for (int w = 0; w < 4; ++w) {   // the four lane quarters
+                    s += (double)s_sum[w][0][i];
+                    sq += (double)s_sum[w][1][i];
+                }
+                atomicAdd(st + i, s);
+                atomicAdd(st + p.oc_valid + i, sq);
             }
         __syncwarp();
     }
@@ -361,14 +404,15 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
         if constexpr (PAIR) tmem_dealloc_pair(tmem_base, (uint32_t)p.tmem_cols);
         else tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
     }
+    if (TIMED && rank == 0 && threadIdx.x == 0) atomicAdd(p.stall + 4, (unsigned long long)(clock64() - t_start));
     if constexpr (PAIR) cluster_sync_all();   // a pair gives its TMEM back together
 }
 
 static b2c_status splitk_optin(b2c_ctx* ctx)
 {
     if (!(ctx->smem_optin_done & B2C_OPTIN_SPLITK)) {
-        B2C_CUDA(cudaFuncSetAttribute(conv_splitk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024));
-        B2C_CUDA(cudaFuncSetAttribute(conv_splitk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024));
+        for (auto* k : {conv_splitk_kernel<false, false>, conv_splitk_kernel<false, true>, conv_splitk_kernel<true, false>, conv_splitk_kernel<true, true>})
+            B2C_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024));
         ctx->smem_optin_done |= B2C_OPTIN_SPLITK;
     }
     return B2C_OK;
@@ -384,7 +428,7 @@ int splitk_max_clusters(b2c_ctx* ctx, int cluster, bool pair)
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)cluster);
         cfg.blockDim = dim3(kSkThreads);
-        cfg.dynamicSmemBytes = 215 * 1024;
+        cfg.dynamicSmemBytes = 209 * 1024;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)cluster;
@@ -392,7 +436,7 @@ int splitk_max_clusters(b2c_ctx* ctx, int cluster, bool pair)
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, pair ? conv_splitk_kernel<true> : conv_splitk_kernel<false>, &cfg) == cudaSuccess) known = n;
+        if (cudaOccupancyMaxActiveClusters(&n, pair ? conv_splitk_kernel<true, false> : conv_splitk_kernel<false, false>, &cfg) == cudaSuccess) known = n;
     }
     return known;
 }
@@ -402,7 +446,10 @@ b2c_status launch_conv_splitk(b2c_ctx* ctx, const ConvKParams& p, int grid, size
     b2c_status st = splitk_optin(ctx);
     if (st != B2C_OK) return st;
     const unsigned cluster = (unsigned)(p.splits * (p.pair ? 2 : 1));
-    B2C_CUDA(b2c_launch(ctx, p.pair ? conv_splitk_kernel<true> : conv_splitk_kernel<false>, dim3((unsigned)grid), dim3(kSkThreads), smem_bytes, stream, cluster, p));
+    const bool timed = p.stall != nullptr;
+    auto* kernel = p.pair ? (timed ? conv_splitk_kernel<true, true> : conv_splitk_kernel<true, false>)
+                          : (timed ? conv_splitk_kernel<false, true> : conv_splitk_kernel<false, false>);
+    B2C_CUDA(b2c_launch(ctx, kernel, dim3((unsigned)grid), dim3(kSkThreads), smem_bytes, stream, cluster, p));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;
 }
