@@ -1059,12 +1059,12 @@ struct KMajorPlan {
 
 // Tensor-pipe and staging cycles of one k-block of kb channels on a tile of 128 pixels (a pair: 2 x 128) x n channels: an MMA of 16
 // channels takes n / 2 cycles, or what its operands take through the 128 B/clk shared-memory port (A: 4 KB, B: 32 n bytes, half of
-// it per CTA of a pair); the loads come in at about 74 B/clk per SM (fitted with the estimates below).
+// it per CTA of a pair); the loads come in at about 74 B/clk per SM, 52 with 160-channel tiles (fitted with the estimates below).
 static int kblock_cycles(int n, int kb, bool pair, int a_rows)
 {
     const int b_rows = pair ? n / 2 : n;
     const int operand = 32 + b_rows / 4, mma = (operand > n / 2 ? operand : n / 2) * (kb / 16);
-    const int loads = (a_rows + b_rows) * kb * 2 / 74;
+    const int loads = (a_rows + b_rows) * kb * 2 / ((n & (n - 1)) && kb == 64 ? 52 : 74);
     return mma > loads ? mma : loads;
 }
 
@@ -1075,7 +1075,7 @@ static int kblock_cycles(int n, int kb, bool pair, int a_rows)
 // pick is on average 0.3 % and at most 5 % slower than the layer's best one.  With 128 images, persistent -> this, launch to
 // launch: 512 -> 512 at 4x4 27.8 -> 14.1 us, 256 -> 256 at 8x8 18.2 -> 12.7, 256 -> 512 at 8x8 stride 2 16.6 -> 10.5; with 50
 // images 26.3 -> 10.7, 16.4 -> 10.2 and 16.4 -> 8.6; 128 -> 128 at 8x8 with 16 images 10.3 -> 5.7.
-static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p, int m_tiles, long long est_cycles)
+static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p, int m_tiles, bool reuse, long long est_cycles)
 {
     const int kb = (pb.ic % 64 == 0) ? 64 : (pb.ic % 32 == 0) ? 32 : 16;
     const int taps = p.n_par > 1 ? ((pb.r + 1) / 2) * ((pb.r + 1) / 2) : pb.r * pb.r;   // of the parity with most
@@ -1083,7 +1083,6 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
     const int c_blocks = pb.ic / kb;
     long long best = est_cycles - 600;   // worth a change from the persistent kernel (0.6 us)
     bool found = false;
-    const int smem = 208 * 1024;   // (beside 16.6 KB of static arrays)
     for (int pair = 0; pair <= 1; ++pair) {
         if (pair && (p.n_par > 1 || ctx->use_pairs == 0)) continue;
         for (int n = 256; n >= 32; n -= 16) {
@@ -1091,7 +1090,14 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
             const int clusters = p.n_par * (pair ? (m_tiles / p.n_par + 1) / 2 : m_tiles / p.n_par) * (pb.oc / n);
             for (int splits = 1; splits * (pair + 1) <= 8; splits *= 2) {
                 if (n % (8 * splits) || splits > min_taps * c_blocks) continue;
-                if (clusters > splitk_max_clusters(ctx, splits * (pair + 1), pair != 0)) continue;
+                // (short reductions stay whole: a split saves them a microsecond at most, and a layer then adds up in the same
+                // order whatever the number of images in the launch)
+                if (splits > 1 && est_cycles < 15000) continue;
+                // two tiles per SM: their CTAs (72 registers, half of the shared memory each) take turns at the tensor pipe, one in
+                // its epilogue while the other loads
+                const bool two = splits == 1 && !pair && !reuse && clusters > ctx->sm_count && clusters <= 2 * ctx->sm_count;
+                if (!two && clusters > splitk_max_clusters(ctx, splits * (pair + 1), pair != 0)) continue;
+                const int smem = (two ? 94 : 208) * 1024;   // (beside 16.6 KB of static arrays)
                 const int b_rows = pair ? n / 2 : n, a_bytes = 128 * kb * 2, b_bytes = (b_rows * kb * 2 + 1023) & ~1023;
                 const int x_bytes = (splits - 1) * (n / splits) * 512;   // partial tiles of the other CTAs
                 // k-blocks share a slot until it holds the MMAs of the issuing thread's 500 cycles per slot, while three slots are left
@@ -1107,7 +1113,7 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
                 const int k_blocks = (taps * c_blocks + splits - 1) / splits;
                 // k-blocks, exchange (barriers, partial tiles at 21 B/clk), epilogue of n / splits columns
                 const long long per_block = block > 570 / gsub ? block : 570 / gsub;
-                const long long est = k_blocks * per_block + (splits > 1 ? 1100 + 800 * overlap + x_bytes / 21 : 0) + 190ll * n / splits / 32 + 2600 * pair;
+                const long long est = k_blocks * per_block * (two ? 2 : 1) + (two ? 2000 : 0) + (splits > 1 ? 1100 + 800 * overlap + x_bytes / 21 : 0) + 190ll * n / splits / 32 + 2600 * pair;
                 if (est >= best) continue;
                 best = est;
                 found = true;
@@ -1180,9 +1186,12 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     // Measured on B200 (1024-image layers): pairs gain ~30 % at 128-channel tiles, where the filter traffic from L2
     // bounds single CTAs, and lose 5-30 % at 64 and 256 and on the short reductions of 1x1 and stride-2 layers; so by
     // default only 3x3 stride-1 layers with 128-channel tiles use them (use_pairs: 0 = never, 1 = those, 2 = every
-    // eligible problem).
     const bool pair_ok = n_par == 1 && !pb.out_f32 && pb.bias == nullptr && n_tile % 32 == 0 && m_tiles % 2 == 0 && ctx->sm_count >= 2;
-    p.pair = (pair_ok && (ctx->use_pairs == 2 || (ctx->use_pairs == 1 && n_tile >= 128 && R == 3 && pb.stride == 1) ||
+    // eligible problem).  Where single CTAs get by with one tile each, short reductions are faster without the pair's set-up and
+    // longer operand path: 160 -> 160 at 32x32 with 16 images 15.1 us as pairs, 11.6 as singles, 128 -> 128 at 16x16 with 50
+    // 10.4 and 8.3, but 320 -> 320 at 16x16 with 32 16.6 and 17.2.
+    const bool short_wave = p.total_units <= ctx->sm_count && R * R * pb.ic < 2048;
+    p.pair = (pair_ok && (ctx->use_pairs == 2 || (ctx->use_pairs == 1 && n_tile >= 128 && R == 3 && pb.stride == 1 && !short_wave) ||
                           (ctx->use_pairs == 3 && n_tile == 128 && R == 3 && pb.stride == 1))) ? 1 : 0;
     int b_rows = p.pair ? n_tile / 2 : n_tile;   // filter rows one CTA fetches per tile
 
@@ -1238,7 +1247,9 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
             planned = true;
         }
     }
-    if (!planned && fh_ok && units_per_cta >= 2) {
+    // (a pair's bank of 147 KB takes six units to pay: 128 -> 128 at 16x16 with 128 images, two units, 15.7 us, 13.7 without; with
+    // 384, six units, 25.8 and 25.4 forward, 25.8 and 26.7 backward; with 1024 55.1 and 60.9)
+    if (!planned && fh_ok && units_per_cta >= (9 * (pb.ic / 64) * b_rows * 128 > 96 * 1024 ? 6 : 2)) {
         const int tx_b = b_rows * 64 * 2, bank = taps_total * (pb.ic / 64) * tx_b, a_bytes = ((10 * 18 * 128) + 1023) & ~1023;
         int stages = (ring_budget - bank) / a_bytes;
         if (stages > kMaxStages) stages = kMaxStages;
@@ -1283,7 +1294,7 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     }
     if (p.stages < 2) return B2C_ERR_UNSUPPORTED_SHAPE;
     int cluster = 0;   // CTAs per cluster of a split-K plan
-    if (ctx->use_split_k && grid < ctx->sm_count) {
+    if (ctx->use_split_k && units_per_cta <= 2) {
         const int max_taps = n_par > 1 ? ((R + 1) / 2) * ((R + 1) / 2) : taps_total;
         const int a_rows = p.vreuse ? (p.bh + 2) * p.bw / 3 : p.fh ? 180 / 9 : 128;
         ConvKParams q = p;
@@ -1291,8 +1302,10 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
         q.tiles_w = gw / q.bw; q.tiles_h = gh / q.bh; q.tiles_n = (pb.n + q.bn - 1) / q.bn;
         q.vreuse = q.fh = q.hm = q.resident = q.resident_bytes = q.b_merged = q.a_step = 0;
         const int block = kblock_cycles(n_tile, p.kb, p.pair != 0, a_rows), per_block = p.vreuse || block > 400 ? block : 400;
-        const long long persistent = (long long)units_per_cta * max_taps * (pb.ic / p.kb) * per_block + 1060ll * n_tile / 32;
-        if (choose_splitk(ctx, pb, q, n_par * m_tiles, persistent)) {
+        const bool reuse = p.vreuse || p.fh || p.hm;   // taps share their loads
+        const long long persistent = (long long)units_per_cta * max_taps * (pb.ic / p.kb) * per_block + 1060ll * n_tile / 32 +
+                                     (p.pair ? 2600 : !reuse && units_per_cta > 1 ? 3000 : 0);
+        if (choose_splitk(ctx, pb, q, n_par * m_tiles, reuse, persistent)) {
             p = q;
             cluster = p.splits * (p.pair ? 2 : 1);
             b_rows = p.pair ? p.n_tile / 2 : p.n_tile;

@@ -12,9 +12,10 @@ pytestmark = pytest.mark.gpu
 
 # an odd number of tiles on pairs, one tile split eight ways, slices of 8 / 20 x 8 columns, 16- and 32-channel k-blocks, output parities
 # with and without taps, more splits than a ragged share of k-blocks, several images per tile with a ragged last one,
-# partial tiles too large to have an area beside the ring
+# partial tiles too large to have an area beside the ring, two tiles per SM
 SHAPES = [(50, 4, 4, 512, 512, 3, 1), (8, 4, 4, 256, 64, 3, 1), (3, 8, 8, 32, 32, 3, 1), (8, 32, 32, 16, 16, 3, 1), (2, 16, 16, 160, 160, 3, 1),
-          (8, 8, 8, 128, 256, 3, 2), (8, 8, 8, 128, 256, 1, 2), (5, 16, 16, 32, 64, 3, 2), (6, 8, 8, 48, 96, 3, 1), (16, 8, 8, 2048, 512, 1, 1), (7, 4, 4, 640, 320, 3, 1), (33, 8, 8, 512, 256, 3, 1)]
+          (8, 8, 8, 128, 256, 3, 2), (8, 8, 8, 128, 256, 1, 2), (5, 16, 16, 32, 64, 3, 2), (6, 8, 8, 48, 96, 3, 1), (16, 8, 8, 2048, 512, 1, 1), (7, 4, 4, 640, 320, 3, 1), (33, 8, 8, 512, 256, 3, 1),
+          (81, 32, 32, 16, 32, 3, 2), (75, 16, 16, 64, 64, 1, 1)]
 
 
 @pytest.fixture(scope="module", params=["0", "1"], ids=["persistent", "split-k"])
