@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                     const int rs = grp.rs[copy][b];
                     const bool live = rs >= 0 && k < p.k_total;
                     float* dst = p.dw + ctile * p.ct;
-                    const int row_off = live ? (k * p.rs_total + rs) * p.c_total : -1;   // (a filter bank has fewer than 2^31 elements)
+                    // offset of the row in dw in units of 16 elements: a filter bank may exceed 2^31 elements, but not 2^36 (256 GB)
+                    const unsigned row16 = live ? (unsigned)(k * p.rs_total + rs) * (unsigned)(p.c_total >> 4) : 0xffffffffu;
                     // accumulator column of 16-channel chunk ck of shift b (framed x: [channel block][shift][64 channels])
                     auto col = [&](int ck) -> uint32_t {
                         const int per_block = p.cw_b >> 4;   // 16-channel chunks per x box
@@ -398,9 +399,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                         transpose_lanes4(r, t4);   // r[4 i ..] = vector t4 of the row of lane (lane - t4) + i
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const int off = __shfl_sync(0xffffffffu, row_off, (lane & ~3) + i);
-                            if (off >= 0)
-                                red_add_v4(dst + off + ck * 16 + 4 * t4, __uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]), __uint_as_float(r[4 * i + 2]),
+                            const unsigned to = __shfl_sync(0xffffffffu, row16, (lane & ~3) + i);
+                            if (to != 0xffffffffu)
+                                red_add_v4(dst + (size_t)to * 16 + ck * 16 + 4 * t4, __uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]), __uint_as_float(r[4 * i + 2]),
                                            __uint_as_float(r[4 * i + 3]));
                         }
                         __syncwarp();

@@ -61,3 +61,19 @@ def test_weight_gradient_tiles(ctx, shape):
     ctx.conv2d_wgrad(binding.conv_desc(*shape), dev_bf16(g), dev_bf16(x), dw, accumulate=True)
     assert ctx.device_status() == 0
     assert_close(dw, 2 * ref, "dw accumulated")
+
+
+def test_weight_gradient_of_a_bank_beyond_2_to_the_31_elements(ctx):
+    """Row offsets into dw need 64 bits: rows before, around and behind element 2^31 of a 65536 x 32832 filter bank."""
+    from paper_2503_23186_b200 import binding
+    shape = N, H, W, C, K, R, st = 2, 8, 8, 32832, 65536, 1, 1
+    r = wl.rng_for(63, "big-bank")
+    x, g = (torch.from_numpy(r.standard_normal((N, H, W, ch), dtype=np.float32)).to(torch.bfloat16) for ch in (C, K))
+    dw = torch.full((K, C), float("nan"), dtype=torch.float32, device="cuda")
+    ctx.conv2d_wgrad(binding.conv_desc(*shape), g.cuda(), x.cuda(), dw)
+    assert ctx.device_status() == 0
+    assert bool(torch.isfinite(dw.sum(1)).all())   # every row was written
+    mid = (1 << 31) // C
+    rows = np.r_[0:4, mid - 4:mid + 4, K - 4:K]
+    want = g.double().numpy().reshape(-1, K)[:, rows].T @ x.double().numpy().reshape(-1, C)
+    assert_close(dw[torch.from_numpy(rows).cuda()], want, "dw rows")
