@@ -187,6 +187,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
     const int role = warp == 0 ? 0 : warp >= kWgProducerWarp1 ? warp - kWgProducerWarp1 + 1 : warp - 1;   // producer or issuer number
     int slot_ = role, s_ = role, first_slot_ = 0;
     uint32_t ph_ = 0u, tile_parity_ = 0u;
+    bool stop = false;   // a wait has given up
 
     do {
         const int n_chunks = STREAM ? (left < p.chunks_total - chunk_begin ? left : p.chunks_total - chunk_begin) : left;
@@ -426,7 +427,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
             if (p.stall != nullptr && warp == 2 && lane == 0) atomicAdd(p.stall + 5, (unsigned long long)(clock64() - t_kernel));
         }
         tc_fence_before();
-        __syncthreads();
+        // One answer for the block: a warp that is already at the next tile may run out of polls and raise the flag before a slower one
+        // has looked at it here.
+        stop = __syncthreads_or(*(volatile uint32_t*)&abort_flag != 0u) != 0;
         if constexpr (STREAM) {   // the accumulator has been read: the next tile may overwrite it
             tc_fence_after();
             slot_ = slot;
@@ -440,10 +443,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                 ktile = 0;
                 if (++ctile == p.n_ctiles) { ctile = 0; ++gi; }
             }
-            if (abort_flag) break;
         }
-    } while (STREAM && left > 0);
-    if (abort_flag) {
+    } while (STREAM && left > 0 && !stop);
+    if (stop) {
         // A wait gave up: let the issued bulk copies land and the issued MMAs retire before exit.
         if ((warp == 0 || warp >= kWgProducerWarp1) && lane == 0) {
             const int w = warp == 0 ? 0 : warp - kWgProducerWarp1 + 1;

@@ -224,7 +224,9 @@ def test_forward_variants_wind_down_on_timeout(ctx, shape):
                                  lambda: assert_close(y, oracle.conv2d_fwd(x, w, st, 1), "y after recovery"))
 
 
-@pytest.mark.parametrize("shape", [(8, 32, 32, 64, 64, 3, 1), (4, 8, 8, 512, 512, 3, 1), (8, 32, 32, 64, 128, 1, 2)], ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
+# the last one deals out equal runs of (tile, pixel chunk) pairs: the wind-down may begin at any of a CTA's tiles
+@pytest.mark.parametrize("shape", [(8, 32, 32, 64, 64, 3, 1), (4, 8, 8, 512, 512, 3, 1), (8, 32, 32, 64, 128, 1, 2), (32, 8, 8, 640, 640, 3, 1)],
+                         ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
 def test_weight_gradient_winds_down_on_timeout(ctx, shape):
     N, H, W, C, K, R, st = shape
     x, _, g = wl.conv_problem(36, *shape)
