@@ -80,7 +80,8 @@ def test_winds_down_on_timeout(ctx, shape):
     X, Wt = dev_bf16(x), dev_bf16(w)
     ctx.set_spin_limit(1)
     try:
-        ctx.conv2d_fwd(_desc(*shape), X, Wt, y)
+        for _ in range(8):   # (a poll may suspend for longer than a short launch takes: one launch can get through without a time-out)
+            ctx.conv2d_fwd(_desc(*shape), X, Wt, y)
         status = ctx.device_status()
     finally:
         ctx.set_spin_limit(1 << 22)
