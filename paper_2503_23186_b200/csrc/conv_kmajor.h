@@ -101,16 +101,23 @@ __device__ __forceinline__ f32x2 add_f32x2(f32x2 a, f32x2 b)
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ f32x2 mul_f32x2(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 __device__ __forceinline__ f32x2 fma_f32x2(f32x2 a, f32x2 b, f32x2 c)
 {
     f32x2 d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ f32x2 widen_bf16x2(uint32_t pair) { return make_f32x2(__uint_as_float(pair << 16), __uint_as_float(pair & 0xffff0000u)); }
 // s += both values of a packed bf16 pair, q += their squares.
 __device__ __forceinline__ void add_pair(uint32_t pair, f32x2& s, f32x2& q)
 {
-    const f32x2 f = make_f32x2(__uint_as_float(pair << 16), __uint_as_float(pair & 0xffff0000u));
+    const f32x2 f = widen_bf16x2(pair);
     s = add_f32x2(s, f);
     q = fma_f32x2(f, f, q);
 }

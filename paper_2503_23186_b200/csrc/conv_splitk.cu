@@ -44,21 +44,22 @@ __device__ __forceinline__ void sk_issue(int ksteps, uint32_t d_tmem, uint32_t a
 }
 
 // BatchNorm sums of a warp's 32 rows x 16 columns of stored bf16 values (packed pairs, one row per lane, rows that do not exist as
-// zeros), on the tensor cores, which are idle by now.  The block goes through 1 KB of shared memory as [half][row][8 columns]; ldmatrix
-// with transposition gives registers that are at the same time the A operand V^T and the B operand V of an m16n8k16 MMA, so with ones
-// as A's lower eight rows one MMA per 16 rows and 8 columns yields V^T V, whose diagonal holds the sums of squares, and the column sums
-// (bf16 products are exact in fp32).  Lane l holds column 8 h + (l >> 2) in s[h], q[h] if column_owner(l).  128 -> 256 stride 2 with 250
-// images, forward with sums: lane exchanges and fp32 adds 18.8 us, this 16.5 us (12.5 us without sums).
-__device__ __forceinline__ bool column_owner(int lane) { return (lane >> 3) == (lane & 3); }
-__device__ __forceinline__ void column_sums(const uint32_t (&pk)[8], float* stage, int lane, float (&s)[2], float (&q)[2])
+// zeros).  The block goes through 1 KB of shared memory as [half][row][8 columns]; ldmatrix with transposition then hands lane l eight
+// rows of column l >> 2 of each half, which it adds up in fp32, and the four lanes of a column share the rest: on return the lane holds
+// one total, of column column_of_total(l): the sum, or the sum of squares if total_is_square(l).
+// The squares of bf16 values end in the same few bits, so a running sum loses a quarter of a unit in its last place with every other
+// addition, always downwards; here four squares meet exactly or nearly so before anything larger is added.  On the tensor cores, whose
+// accumulators truncate, the sums of squares came out 5.0e-8 low; now 1.1e-8 off, as in the persistent kernel.
+__device__ __forceinline__ int column_of_total(int lane) { return 8 * (lane & 1) + (lane >> 2); }
+__device__ __forceinline__ int total_is_square(int lane) { return (lane >> 1) & 1; }
+__device__ __forceinline__ float column_sums(const uint32_t (&pk)[8], float* stage, int lane)
 {
     const uint32_t base = smem_u32(stage) + 16u * (uint32_t)lane;
     __syncwarp();   // the previous block has been read
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(base), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]) : "memory");
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(base + 512u), "r"(pk[4]), "r"(pk[5]), "r"(pk[6]), "r"(pk[7]) : "memory");
     __syncwarp();
-    const bool odd = ((lane >> 2) & 1) != 0;
-    const uint32_t ones = 0x3F803F80u;
+    float s[2], q[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         uint32_t t[4];   // t[i]: rows 8 i + 2 (lane & 3) + {0, 1} of column lane >> 2
@@ -66,15 +67,17 @@ __device__ __forceinline__ void column_sums(const uint32_t (&pk)[8], float* stag
                      : "=r"(t[0]), "=r"(t[1]), "=r"(t[2]), "=r"(t[3])
                      : "r"(base + 512u * h)
                      : "memory");
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < 4; i += 2)
-            asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %5}, {%4, %6}, {%0, %1, %2, %3};"
-                         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                         : "r"(t[i]), "r"(ones), "r"(t[i + 1]));
-        q[h] = odd ? c[1] : c[0];
-        s[h] = odd ? c[3] : c[2];
+        const f32x2 f0 = widen_bf16x2(t[0]), f1 = widen_bf16x2(t[1]), f2 = widen_bf16x2(t[2]), f3 = widen_bf16x2(t[3]);
+        const float2 ss = split_f32x2(add_f32x2(add_f32x2(f0, f1), add_f32x2(f2, f3)));
+        const float2 qq = split_f32x2(add_f32x2(fma_f32x2(f1, f1, mul_f32x2(f0, f0)), fma_f32x2(f3, f3, mul_f32x2(f2, f2))));
+        s[h] = ss.x + ss.y;
+        q[h] = qq.x + qq.y;
     }
+    // four totals over four lanes: each exchange halves what a lane carries
+    const bool odd = (lane & 1) != 0, upper = (lane & 2) != 0;
+    const float ms = (odd ? s[1] : s[0]) + __shfl_xor_sync(0xffffffffu, odd ? s[0] : s[1], 1);
+    const float mq = (odd ? q[1] : q[0]) + __shfl_xor_sync(0xffffffffu, odd ? q[0] : q[1], 1);
+    return (upper ? mq : ms) + __shfl_xor_sync(0xffffffffu, upper ? ms : mq, 2);
 }
 
 // TIMED: the instance that adds to the stall counters (read at run time, they cost the small net of tests and benchmarks 2.5 % of
@@ -370,15 +373,7 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
 #pragma unroll
                 for (int i = 0; i < 8; ++i) pk[i] = 0u;
             }
-            float s[2], sq[2];
-            column_sums(pk, s_stage[warp], lane, s, sq);
-            if (column_owner(lane)) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    s_sum[q][0][g * 16 + h * 8 + (lane >> 2)] = s[h];
-                    s_sum[q][1][g * 16 + h * 8 + (lane >> 2)] = sq[h];
-                }
-            }
+            s_sum[q][total_is_square(lane)][g * 16 + column_of_total(lane)] = column_sums(pk, s_stage[warp], lane);
             __syncwarp();
         }
     }

@@ -61,6 +61,23 @@ def test_forward_statistics_and_data_gradient(ctx, shape):
     np.testing.assert_allclose(host(stats)[K:], (ys * ys).sum(0), rtol=1e-5)
 
 
+@pytest.mark.parametrize("shape", [(250, 16, 16, 128, 256, 3, 2), (50, 4, 4, 512, 512, 3, 1), (64, 8, 8, 64, 160, 1, 1)], ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
+def test_statistics_are_summed_in_fp32(ctx, shape):
+    """Sums of squares of 32 rows in fp32, fp64 beyond: five levels of rounding to nearest leave a column about 1e-8 off in either
+    direction.  Truncating additions, or chains of them (a square of a bf16 value ends in the same bits), lose 5e-8 and more."""
+    N, H, W, C, K, R, st = shape
+    x, w, _ = wl.conv_problem(43, *shape)
+    P = H // st
+    y = torch.empty((N, P, P, K), dtype=torch.bfloat16, device="cuda")
+    stats = torch.zeros(2 * K, dtype=torch.float64, device="cuda")
+    ctx.conv2d_fwd(_desc(*shape), dev_bf16(x), dev_bf16(w), y, ch_stats=stats)
+    ys = y.double().reshape(-1, K)
+    err = (stats[K:] / (ys * ys).sum(0) - 1).cpu().numpy()
+    assert np.mean(np.abs(err)) <= 2.5e-8 and abs(np.mean(err)) <= 2e-8, (np.mean(np.abs(err)), np.mean(err))
+    err = ((stats[:K] - ys.sum(0)) / ys.abs().sum(0)).cpu().numpy()
+    assert np.mean(np.abs(err)) <= 1e-8, np.mean(np.abs(err))
+
+
 def test_classifier_with_bias(ctx):
     shape = (70, 1, 1, 512, 128, 1, 1)
     x, w, _ = wl.conv_problem(41, *shape)
