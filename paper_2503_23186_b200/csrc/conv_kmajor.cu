@@ -34,6 +34,7 @@ static constexpr int kProducers = 2;     // TMA-issuing threads: warp 0 and the 
 static constexpr int kThreads = 64 + 32 * kEpiWarps + 32 * (kIssuers - 1) + 32 * (kProducers - 1);
 static constexpr int kProducerWarp1 = 2 + kEpiWarps + (kIssuers - 1);   // warp index of the second producer
 static constexpr uint32_t kDrainPolls = 1u << 22;
+static constexpr int kFoldUnits = 8;     // units of a narrow tile (wide: half as many) whose squares a lane of the epilogue adds up before they move on
 
 // Units of this CTA (a CTA pair walks pair-units: two pixel tiles next to each other, same channel tile, of which CTA `rank` takes tile
 // 2*m + rank).  A walker keeps its channel tile and takes a run of consecutive pixel tiles, so that it meets at most two statistics
@@ -100,11 +101,16 @@ __device__ __forceinline__ void butterfly16(float (&a)[16], float (&b)[16], int 
 // STATS: BatchNorm sums of the values as stored, kept in registers until the statistics group ends; those of the last group are left
 // in my_stats ([0, 128) sums, [128, 256) sums of squares) for the CTA to add up.  Returns that group and channel tile (-1: none).
 //   * EAGER: a lane sums its own row's columns (32 registers per chunk), a butterfly reduces over the rows once per group.
-//   * wide tiles: two exchanges between lanes first (add_chunk), a quarter of the registers and about 60 instructions per chunk.
+//   * wide tiles: two exchanges between lanes first (add_chunk), a quarter of the registers and about 65 instructions per chunk.
 //     Bound: issue slots and latency of eight warps.  Measured with 1024 images, forward with sums, 128 -> 128 at 16x16 and 1x1
 //     64 -> 256 at 32x32: shuffle butterfly per chunk (150 instructions) 82 and 342 us; tensor cores (m16n8k16, which queue behind the
 //     convolution's own MMAs) 90 and 224; transposed through shared memory (two warp barriers and a chain of eight adds) 72 and 253;
 //     read from TMEM once more in the fragment layout 72 and 244; this 72 and 273 us (a rolled loop: 79 and 219).
+// The squares of bf16 values end in the same few bits: added one by one to a running fp32 sum they are rounded down more often than up,
+// and a chain of 200 comes out 5e-7 low.  So four squares of a wide tile meet before they reach the running sum, which moves on to a second
+// one in local memory after every few units; narrow tiles, which have no registers to spare, add their rows up in my_stats instead.
+// Sums of squares of 1024 images are 1.2e-8 off (without: 3.3e-7 on 64 -> 256 1x1, 4.6e-8 on 32 -> 64 1x1), for 275 -> 280 us on
+// 64 -> 256 1x1, 64.9 -> 66.1 on 128 -> 128 at 16x16, 76.6 -> 80.8 on 64 -> 64 at 32x32.
 // Without STATS the code carries no accumulators: 1x1 64 -> 256 154 -> 126 us, 32 -> 64 57 -> 48 us, data gradient 256 -> 64 159 -> 132 us.
 template <int NCH, bool EAGER, bool HM, bool STATS>
 __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tmem_base, uint64_t* acc_full, uint64_t* acc_empty,
@@ -125,6 +131,17 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
     f32x2 acc_s[NA], acc_q[NA];
 #pragma unroll
     for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = 0ull;
+    f32x2 long_q[NA];   // wide tiles only
+    int opaque_zero = 0, held = 0;   // (an index that the compiler cannot see through keeps long_q out of the registers)
+    if constexpr (STATS && !EAGER) {
+        asm volatile("mov.u32 %0, 0;" : "=r"(opaque_zero));
+#pragma unroll
+        for (int i = 0; i < NA; ++i) long_q[i + opaque_zero] = 0ull;
+    }
+    if constexpr (STATS && EAGER) {
+        for (int i = lane; i < 256; i += 32) my_stats[i] = 0.f;
+        __syncwarp();
+    }
     int jacc = 0, cur_group = -1, cur_ktile = 0;
     bool ok = true;
     long long epi_wait = 0;
@@ -147,7 +164,7 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
         } else if constexpr (STATS) {
 #pragma unroll
             for (int i = 0; i < NA; ++i) {
-                const float2 s = column_total(acc_s[i]), sq = column_total(acc_q[i]);
+                const float2 s = column_total(acc_s[i]), sq = column_total(add_f32x2(acc_q[i], long_q[i + opaque_zero]));
                 if ((lane & 7) == 0 && i < 2 * n_chunks) {
                     const int col = (i >> 1) * 16 + column_of(lane) + 2 * (i & 1);
                     emit(col, s.x, sq.x);
@@ -157,14 +174,40 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
         }
         __syncwarp();
     };
-    auto flush_stats = [&]() {   // this warp's sums of the finished statistics group -> global fp64
+    // The running sums move on; at the end of a statistics group this warp's share of it goes to global fp64.
+    auto flush_stats = [&](bool group_done) {
+        held = 0;
         double* st = p.stats + (size_t)cur_group * 2 * p.oc_valid + cur_ktile * p.n_tile + col_begin;
-        each_total([&](int col, float s, float sq) {
-            atomicAdd(st + col, (double)s);
-            atomicAdd(st + p.oc_valid + col, (double)sq);
-        });
+        if constexpr (EAGER) {
+            each_total([&](int col, float s, float sq) {   // (a column's total always comes from the same lane)
+                my_stats[col] += s;
+                my_stats[128 + col] += sq;
+            });
+            if (group_done) {
+                for (int col = lane; col < n_chunks * 16; col += 32) {
+                    atomicAdd(st + col, (double)my_stats[col]);
+                    atomicAdd(st + p.oc_valid + col, (double)my_stats[128 + col]);
+                    my_stats[col] = my_stats[128 + col] = 0.f;
+                }
+                __syncwarp();
+            }
 #pragma unroll
-        for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = 0ull;
+            for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = 0ull;
+        } else {
+#pragma unroll
+            for (int i = 0; i < NA; ++i) {
+                long_q[i + opaque_zero] = add_f32x2(long_q[i + opaque_zero], acc_q[i]);
+                acc_q[i] = 0ull;
+            }
+            if (group_done) {
+                each_total([&](int col, float s, float sq) {
+                    atomicAdd(st + col, (double)s);
+                    atomicAdd(st + p.oc_valid + col, (double)sq);
+                });
+#pragma unroll
+                for (int i = 0; i < NA; ++i) acc_s[i] = long_q[i + opaque_zero] = 0ull;
+            }
+        }
     };
 
     // The coordinates of a unit are worked out one unit ahead, between the probe of the current unit's accumulator barrier
@@ -204,7 +247,7 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
         int next_group = cur_group;
         if constexpr (STATS) {
             next_group = p.stats_group_images > 0 ? (p.grp_shift >= 0 ? c.n0 >> p.grp_shift : c.n0 / p.stats_group_images) : 0;
-            flush_pending = next_group != cur_group && cur_group >= 0;
+            flush_pending = cur_group >= 0 && (next_group != cur_group || held == (EAGER ? kFoldUnits : kFoldUnits / 2));
         }
         const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * p.acc_cols + col_begin);
         // the accumulator is handed back to the MMA thread as soon as this warp has read its last column
@@ -252,7 +295,8 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
 
         auto group_end = [&]() {
             if constexpr (!STATS) return;
-            if (flush_pending) flush_stats();   // still the previous group's sums and channel tile
+            if (flush_pending) flush_stats(next_group != cur_group);   // still the previous units' sums, group and channel tile
+            ++held;
             cur_group = next_group;
             cur_ktile = c.ktile;
         };
@@ -371,8 +415,8 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
     // the four lane quarters' sums meet in shared memory: a quarter of the global atomics at the kernel's end
     if (STATS && cur_group >= 0 && ok)
         each_total([&](int col, float s, float sq) {
-            my_stats[col] = s;
-            my_stats[128 + col] = sq;
+            my_stats[col] = EAGER ? my_stats[col] + s : s;
+            my_stats[128 + col] = EAGER ? my_stats[128 + col] + sq : sq;
         });
     if (p.stall != nullptr && e == 0 && lane == 0) atomicAdd(p.stall + 3, (unsigned long long)epi_wait);
     return STATS && ok ? make_int2(cur_group, cur_ktile) : make_int2(-1, 0);

@@ -136,13 +136,16 @@ __device__ __forceinline__ void add_chunk(const uint32_t (&pk)[8], int lane, f32
         half[1][i] = __shfl_xor_sync(0xffffffffu, up16 ? pk[i] : pk[4 + i], 16);
     }
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
+    for (int i = 0; i < 2; ++i) {
+        f32x2 f[4];   // four rows of the lane's column pair
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const uint32_t mine = up8 ? half[r][2 + i] : half[r][i], other = __shfl_xor_sync(0xffffffffu, up8 ? half[r][i] : half[r][2 + i], 8);
-            add_pair(mine, s[i], q[i]);
-            add_pair(other, s[i], q[i]);
+        for (int r = 0; r < 2; ++r) {
+            f[2 * r] = widen_bf16x2(up8 ? half[r][2 + i] : half[r][i]);
+            f[2 * r + 1] = widen_bf16x2(__shfl_xor_sync(0xffffffffu, up8 ? half[r][i] : half[r][2 + i], 8));
         }
+        s[i] = add_f32x2(s[i], add_f32x2(add_f32x2(f[0], f[1]), add_f32x2(f[2], f[3])));
+        q[i] = add_f32x2(q[i], add_f32x2(fma_f32x2(f[1], f[1], mul_f32x2(f[0], f[0])), fma_f32x2(f[3], f[3], mul_f32x2(f[2], f[2]))));
+    }
 }
 __device__ __forceinline__ float2 column_total(f32x2 v)
 {

@@ -48,6 +48,26 @@ def test_wide_tiles_with_statistics(ctx, shape):
         np.testing.assert_allclose(host(stats)[K:], (ys * ys).sum(0), rtol=1e-5)
 
 
+# walkers of 28 wide and 55 narrow tiles: chains of single squares in fp32 would come out 9e-8 and 5e-8 low (a square of a bf16 value
+# ends in the same bits); sums over 32 rows in fp32 are about 1.1e-8 off, whatever the length of the walk
+@pytest.mark.parametrize("shape", [(256, 32, 32, 32, 512, 1, 1), (1024, 32, 32, 16, 64, 1, 1)], ids=["wide", "narrow"])
+def test_statistics_of_long_walks(ctx, shape):
+    from paper_2503_23186_b200 import binding
+    N, H, W, C, K, R, st = shape
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(64)
+    x = torch.randn((N, H, W, C), generator=gen, device="cuda").to(torch.bfloat16)
+    w = (torch.randn((K, R, R, C), generator=gen, device="cuda") * (2.0 / C) ** 0.5).to(torch.bfloat16)
+    y = torch.empty((N, H, W, K), dtype=torch.bfloat16, device="cuda")
+    stats = torch.zeros(2 * K, dtype=torch.float64, device="cuda")
+    ctx.conv2d_fwd(binding.conv_desc(*shape), x, w, y, ch_stats=stats)
+    assert ctx.device_status() == 0
+    ys = y.reshape(-1, K)
+    squares = sum((part.double() ** 2).sum(0) for part in ys.split(1 << 16))
+    err = (stats[K:] / squares - 1).cpu().numpy()
+    assert np.mean(np.abs(err)) <= 2e-8, np.mean(np.abs(err))
+
+
 # 75 / 80 tiles on 148 SMs: equal runs of (tile, pixel chunk) pairs, a CTA finishing one tile and beginning the next; partial tiles
 @pytest.mark.parametrize("shape", [(32, 8, 8, 640, 640, 3, 1), (28, 8, 8, 1280, 2048, 1, 1), (31, 8, 8, 640, 624, 3, 1), (6, 8, 8, 48, 16, 3, 1), (4, 8, 8, 32, 144, 3, 1), (4, 8, 8, 16, 80, 1, 2)], ids=lambda s: "n{}h{}c{}k{}r{}s{}".format(*(s[i] for i in (0, 1, 3, 4, 5, 6))))
 def test_weight_gradient_tiles(ctx, shape):
