@@ -49,14 +49,16 @@ __device__ __forceinline__ uint4 ld16_or_zero(const void* base, long long vec_in
     return ok ? __ldg(reinterpret_cast<const uint4*>(base) + vec_index) : make_uint4(0u, 0u, 0u, 0u);
 }
 
-// A thread's 8 + 8 per-channel sums into the block's shared accumulators.  Threads of a warp whose lanes differ by a
-// multiple of the group count hold the same channels: where the group count is a power of two below 32 those lanes add
-// up with shuffles first and one lane per channel group issues the shared-memory atomics, which leaves one contender
-// per warp and address instead of one per row (32 rows on the same address took several microseconds per block).
-// `whole_warps`: every lane of every calling warp is active (the group count divides the block).
-__device__ __forceinline__ void block_accumulate(float* s_acc, int c, int groups, int g, float (&a)[8], float (&b)[8], bool active)
+// A thread's 8 + 8 per-channel sums, added up over the block and then to the 2c global fp64 sums.  Threads of a warp whose lanes differ by
+// a multiple of the group count hold the same channels: where the group count is a power of two below 32 those lanes add up with
+// shuffles first.  What is left, a slot per warp or per row of threads, goes to shared memory ([slots][2c], at most 16 KB) and is added
+// up there in fp64, always in the same order.  (Shared-memory fp32 atomics, a compare-and-swap each, queued up to 85 threads at one
+// address: 24 channels at 8x8 with 312 images 28.0 us for the two passes of the backward pass, 7.7 now.)
+// Every thread of the block calls this; `active` ones hold sums.
+static constexpr size_t kReduceSlotBytes = 16 * sizeof(float) * kEwThreads;
+__device__ __forceinline__ void block_reduce(float* slots, int c, int groups, float (&a)[8], float (&b)[8], bool active, double* out)
 {
-    const bool warp_reduce = groups < 32 && (groups & (groups - 1)) == 0;   // uniform over the block; all threads are active then
+    const bool warp_reduce = groups < 32 && (groups & (groups - 1)) == 0;   // uniform over the block; all of its first kEwThreads threads are active then
     if (warp_reduce) {
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) {
@@ -68,13 +70,24 @@ __device__ __forceinline__ void block_accumulate(float* s_acc, int c, int groups
                 }
             }
         }
-        if ((int)(threadIdx.x & 31) >= groups) return;
     }
-    if (!active) return;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        atomicAdd(&s_acc[g * 8 + i], a[i]);
-        atomicAdd(&s_acc[c + g * 8 + i], b[i]);
+    const int n_slots = warp_reduce ? kEwThreads / 32 : kEwThreads / groups;
+    if (active && (!warp_reduce || (int)(threadIdx.x & 31) < groups)) {
+        float4* mine = reinterpret_cast<float4*>(slots + (size_t)(warp_reduce ? threadIdx.x >> 5 : threadIdx.x / groups) * 2 * c) + 2 * (threadIdx.x % groups);
+        mine[0] = make_float4(a[0], a[1], a[2], a[3]);
+        mine[1] = make_float4(a[4], a[5], a[6], a[7]);
+        mine[2 * groups] = make_float4(b[0], b[1], b[2], b[3]);
+        mine[2 * groups + 1] = make_float4(b[4], b[5], b[6], b[7]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * c; i += blockDim.x) {
+        double even = 0.0, odd = 0.0;
+#pragma unroll 4
+        for (int sl = 0; sl < n_slots; sl += 2) {
+            even += (double)slots[(size_t)sl * 2 * c + i];
+            if (sl + 1 < n_slots) odd += (double)slots[(size_t)(sl + 1) * 2 * c + i];
+        }
+        atomicAdd(out + i, even + odd);
     }
 }
 
@@ -85,37 +98,44 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_stats_kernel(const void* __r
 {
     pdl_wait();   // first global access comes after the previous kernel of the stream
     pdl_launch_dependents();
-    extern __shared__ float s_acc[];  // [2*c]
-    for (int i = threadIdx.x; i < 2 * c; i += kEwThreads) s_acc[i] = 0.f;
-    __syncthreads();
+    __shared__ __align__(16) float slots[kReduceSlotBytes / sizeof(float)];
     const RowWalk rw(c);
     const int g = threadIdx.x % rw.groups, rl = threadIdx.x / rw.groups;
     const long long base = (long long)blockIdx.y * m * rw.groups;
-    if (rl < rw.rows_per_iter) {
-        float s[8], ss[8];
+    float s[8], ss[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s[i] = ss[i] = 0.f;
+    for (int i = 0; i < 8; ++i) s[i] = ss[i] = 0.f;
+    if (rl < rw.rows_per_iter) {
         const long long step = (long long)gridDim.x * rw.rows_per_iter;
         for (long long r = (long long)blockIdx.x * rw.rows_per_iter + rl; r < m; r += kStatsUnroll * step) {
             uint4 v[kStatsUnroll];
 #pragma unroll
             for (int u = 0; u < kStatsUnroll; ++u) v[u] = ld16_or_zero(y, base + (r + u * step) * rw.groups + g, r + u * step < m);
+            // The rows of a step meet before they reach the running sums: squares of bf16 values end in the same few bits, and added one by
+            // one to a running fp32 sum they are rounded down more often than up.  Sums of squares of 128 images at 8x8 with 256 channels
+            // 1.6e-8 off, now 6e-9; of 64 images with 160 channels 2.4e-8, now 4e-9.
+            float hs[8], hq[8];
 #pragma unroll
-            for (int u = 0; u < kStatsUnroll; ++u) {
-                float f[8];
-                unpack8(v[u], f);
+            for (int u = 0; u < kStatsUnroll; u += 4) {
+                float f[4][8];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) unpack8(v[u + k], f[k]);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    s[i] += f[i];
-                    ss[i] = fmaf(f[i], f[i], ss[i]);
+                    const float s4 = (f[0][i] + f[1][i]) + (f[2][i] + f[3][i]);
+                    const float q4 = fmaf(f[1][i], f[1][i], f[0][i] * f[0][i]) + fmaf(f[3][i], f[3][i], f[2][i] * f[2][i]);
+                    hs[i] = u == 0 ? s4 : hs[i] + s4;
+                    hq[i] = u == 0 ? q4 : hq[i] + q4;
                 }
             }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                s[i] += hs[i];
+                ss[i] += hq[i];
+            }
         }
-        block_accumulate(s_acc, c, rw.groups, g, s, ss, true);
     }
-    __syncthreads();
-    double* out = stats + (size_t)blockIdx.y * 2 * c;
-    for (int i = threadIdx.x; i < 2 * c; i += kEwThreads) atomicAdd(out + i, (double)s_acc[i]);
+    block_reduce(slots, c, rw.groups, s, ss, rl < rw.rows_per_iter, stats + (size_t)blockIdx.y * 2 * c);
 }
 
 // mean and 1/sqrt(var+eps) from the fp64 sums, identically in every thread that needs them.
@@ -214,16 +234,14 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_bwd_reduce_kernel(const void
 {
     pdl_wait();   // first global access comes after the previous kernel of the stream
     pdl_launch_dependents();
-    extern __shared__ float s_acc[];
-    for (int i = threadIdx.x; i < 2 * c; i += kEwThreads) s_acc[i] = 0.f;
-    __syncthreads();
+    __shared__ __align__(16) float slots[kReduceSlotBytes / sizeof(float)];
     const RowWalk rw(c);
     const int g = threadIdx.x % rw.groups, rl = threadIdx.x / rw.groups;
     const long long base = (long long)blockIdx.y * m * rw.groups;
-    if (rl < rw.rows_per_iter) {
-        float sb[8], sg[8];
+    float sb[8], sg[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) sb[i] = sg[i] = 0.f;
+    for (int i = 0; i < 8; ++i) sb[i] = sg[i] = 0.f;
+    if (rl < rw.rows_per_iter) {
         const long long step = (long long)gridDim.x * rw.rows_per_iter;
         constexpr int U = 2;
         for (long long r = (long long)blockIdx.x * rw.rows_per_iter + rl; r < m; r += U * step) {
@@ -242,6 +260,7 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_bwd_reduce_kernel(const void
                     else va[u] = ld16_or_zero(a, vi, ok);
                 }
             }
+            float pb[8], pg[8];   // both rows meet before they reach the running sums
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 float d[8], d2[8], fy[8], fa[8];
@@ -260,16 +279,18 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_bwd_reduce_kernel(const void
                     float dz = d[i];
                     if (da2 != nullptr) dz += d2[i];
                     if (!((mk[u] >> i) & 1u)) dz = 0.f;
-                    sb[i] += dz;
-                    sg[i] = fmaf(dz, fy[i], sg[i]);
+                    pb[i] = u == 0 ? dz : pb[i] + dz;
+                    pg[i] = u == 0 ? dz * fy[i] : fmaf(dz, fy[i], pg[i]);
                 }
             }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                sb[i] += pb[i];
+                sg[i] += pg[i];
+            }
         }
-        block_accumulate(s_acc, c, rw.groups, g, sb, sg, true);
     }
-    __syncthreads();
-    double* out = sums_all + (size_t)blockIdx.y * 2 * c;
-    for (int i = threadIdx.x; i < 2 * c; i += kEwThreads) atomicAdd(out + i, (double)s_acc[i]);
+    block_reduce(slots, c, rw.groups, sb, sg, rl < rw.rows_per_iter, sums_all + (size_t)blockIdx.y * 2 * c);
 }
 
 // Pass 2: dy = gamma*invstd*(dz - dbeta/m - xhat*dgamma/m), dres = dz; block 0 of each group emits dgamma, dbeta.
@@ -460,8 +481,6 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
     __shared__ uint32_t abort_flag;
     uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(st_raw) + 127u) & ~uintptr_t(127));
     const StagedWalk sw(c, m, da2 != nullptr ? 3 : 2, relu != 0);
-    float* s_acc = reinterpret_cast<float*>(ring + (size_t)kStStages * sw.stage_bytes);
-    for (int i = threadIdx.x; i < 2 * c; i += kStThreads) s_acc[i] = 0.f;
     staged_init(full, empty, &abort_flag);
     __syncthreads();
     pdl_wait();   // (the set-up above touched no global data) first global access comes after the previous kernel of the stream
@@ -470,16 +489,17 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
     const long long base = (long long)blockIdx.y * m * sw.groups;
     const uint8_t* mask = relu ? relu_mask : nullptr;
     int issued = 0;
+    const bool act = threadIdx.x < sw.active;   // (consumer warps only)
+    float sb[8], sg[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sb[i] = sg[i] = 0.f;
     if (warp == kEwThreads / 32) {
         if (lane == 0) issued = staged_produce(sw, ring, full, empty, da1, y, da2, mask, base, spin_limit, &abort_flag, status);
     } else {
         const int g = threadIdx.x % sw.groups;
-        const bool act = threadIdx.x < sw.active;
         const uint32_t tbytes = (uint32_t)sw.chunk_vecs * 16u;
-        float sb[8], sg[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) sb[i] = sg[i] = 0.f;
-        auto accumulate = [&](const uint4& v1, const uint4& vy, const uint4& v2, bool two, unsigned mk) {
+        // dz and dz * y of one vector are put into or added to pb and pg
+        auto accumulate = [&](float (&pb)[8], float (&pg)[8], bool first, const uint4& v1, const uint4& vy, const uint4& v2, bool two, unsigned mk) {
             float d[8], d2[8], fy[8];
             unpack8(v1, d);
             if (two) unpack8(v2, d2);
@@ -489,8 +509,8 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
                 float dz = d[i];
                 if (two) dz += d2[i];
                 if (!((mk >> i) & 1u)) dz = 0.f;
-                sb[i] += dz;
-                sg[i] = fmaf(dz, fy[i], sg[i]);
+                pb[i] = first ? dz : pb[i] + dz;
+                pg[i] = first ? dz * fy[i] : fmaf(dz, fy[i], pg[i]);
             }
         };
         int i = 0;
@@ -500,6 +520,7 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
             if (!ok) break;
             if (act) {
                 const uint8_t* st = ring + (size_t)(i % kStStages) * sw.stage_bytes;
+                float pb[8], pg[8];   // both rows meet before they reach the running sums
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int v = u * sw.active + threadIdx.x;
@@ -508,7 +529,12 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
                     uint4 v2 = make_uint4(0u, 0u, 0u, 0u);
                     if (sw.nt > 2) v2 = reinterpret_cast<const uint4*>(st + 2 * tbytes)[v];
                     const unsigned mk = mask != nullptr ? (unsigned)st[sw.nt * tbytes + v] : 0xffu;
-                    accumulate(v1, vy, v2, sw.nt > 2, mk);
+                    accumulate(pb, pg, u == 0, v1, vy, v2, sw.nt > 2, mk);
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    sb[j] += pb[j];
+                    sg[j] += pg[j];
                 }
             }
             staged_release(empty, i, lane);
@@ -520,16 +546,14 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
                 const uint4 v1 = ld16(da1, vi), vy = ld16(y, vi);
                 const uint4 v2 = da2 != nullptr ? ld16(da2, vi) : make_uint4(0u, 0u, 0u, 0u);
                 const unsigned mk = mask != nullptr ? (unsigned)__ldg(mask + vi) : 0xffu;
-                accumulate(v1, vy, v2, da2 != nullptr, mk);
+                accumulate(sb, sg, false, v1, vy, v2, da2 != nullptr, mk);
             }
         }
-        block_accumulate(s_acc, c, sw.groups, g, sb, sg, act);
     }
     __syncthreads();
     if (abort_flag && warp == kEwThreads / 32 && lane == 0) staged_drain(issued, full);
-    double* out = sums_all + (size_t)blockIdx.y * 2 * c;
-    for (int i = threadIdx.x; i < 2 * c; i += kStThreads) atomicAdd(out + i, (double)s_acc[i]);
-    __syncthreads();
+    __syncthreads();   // the ring has been read (and nothing is on its way into it): it holds the block's partial sums now
+    block_reduce(reinterpret_cast<float*>(ring), c, sw.groups, sb, sg, act, sums_all + (size_t)blockIdx.y * 2 * c);
 }
 
 __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(const void* __restrict__ da1, const void* __restrict__ da2,
@@ -1370,8 +1394,8 @@ static int ew_grid(b2c_ctx* ctx, int n_groups, long long m, int rows_per_iter)
 // Blocks per statistics group of a reduction over `bytes` of input: every block ends with one fp64 addition per channel sum, and those
 // of one group meet at the same addresses at about 30 ns per block, against 22 bytes a block streams per ns; the sum of the two is
 // least at sqrt(bytes / 660) blocks.  Measured with 18 / 74 / 148 / 296 blocks, backward (both passes): 512 channels at 4x4 with 128
-// images 18.5 / 12.9 / 13.5 / 17.2 us, 256 at 8x8 27.5 / 16.7 / 16.4 / 19.7, 64 at 32x32 73 / 29.3 / 23.0 / 22.9; forward with its statistics
-// 12.3 / 11.5 / 12.2 / 16.0, 15.4 / 12.3 / 13.0 / 17.2 and 27.8 / 15.7 / 15.2 / 17.1.
+// images 16.8 / 11.5 / 12.0 / 14.4 us, 256 at 8x8 25.2 / 14.4 / 13.9 / 16.2, 64 at 32x32 71 / 27.2 / 21.1 / 21.1; forward with its statistics
+// 11.1 / 9.8 / 11.0 / 13.9, 13.9 / 10.7 / 11.4 / 14.0 and 29.3 / 14.9 / 13.7 / 14.0.
 static dim3 reduce_grid(dim3 grid, double bytes)
 {
     const unsigned best = (unsigned)std::ceil(std::sqrt(bytes / 660.0));
@@ -1389,7 +1413,7 @@ b2c_status launch_bn_fwd(b2c_ctx* ctx, int G, long long m, int c, const void* y,
             b2c_status st = launch_zero(ctx, stats, sizeof(double) * 2 * c * G, nullptr, stream);
             if (st != B2C_OK) return st;
         }
-        B2C_CUDA(b2c_launch(ctx, bn_stats_kernel, reduce_grid(grid, 2.0 * m * c), dim3(kEwThreads), sizeof(float) * 2 * c, stream, 1u, y, m, c, stats));
+        B2C_CUDA(b2c_launch(ctx, bn_stats_kernel, reduce_grid(grid, 2.0 * m * c), dim3(kEwThreads), 0, stream, 1u, y, m, c, stats));
     }
     uint8_t* mask_out = relu ? reinterpret_cast<uint8_t*>(relu_mask) : nullptr;
     if (residual != nullptr)
@@ -1527,7 +1551,7 @@ b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da
     if (staged) {
         const int nt = da2 != nullptr ? 3 : 2;
         const size_t stage = (size_t)nt * chunk_vecs * 16 + (relu ? ((chunk_vecs + 127) & ~127) : 0);
-        const size_t smem = kStStages * stage + sizeof(float) * 2 * c + 128;
+        const size_t smem = kStStages * stage + 128;   // (the ring also has room for the reduction's slots: more than 128 threads' vectors, twice, per tensor)
         if (smem <= 110 * 1024) {
             if (!(ctx->smem_optin_done & B2C_OPTIN_BN_BWD)) {
                 B2C_CUDA(cudaFuncSetAttribute(bn_bwd_reduce_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024));
@@ -1541,7 +1565,7 @@ b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da
             return B2C_OK;
         }
     }
-    B2C_CUDA(b2c_launch(ctx, bn_bwd_reduce_kernel, reduce_grid(grid, (da2 != nullptr ? 6.0 : 4.0) * m * c), dim3(kEwThreads), sizeof(float) * 2 * c, stream, 1u, da1, da2, y, a, m, c, relu, sums, mask));
+    B2C_CUDA(b2c_launch(ctx, bn_bwd_reduce_kernel, reduce_grid(grid, (da2 != nullptr ? 6.0 : 4.0) * m * c), dim3(kEwThreads), 0, stream, 1u, da1, da2, y, a, m, c, relu, sums, mask));
     B2C_CUDA(b2c_launch(ctx, bn_bwd_apply_kernel, dim3(grid), dim3(kEwThreads), 0, stream, 1u, da1, da2, y, a, m, c, gamma, save_mean, save_invstd, relu, sums, dy, dres, dgamma, dbeta,
                                                          acc, mask));
     B2C_CUDA(cudaGetLastError());

@@ -97,3 +97,25 @@ def test_weight_gradient_of_a_bank_beyond_2_to_the_31_elements(ctx):
     rows = np.r_[0:4, mid - 4:mid + 4, K - 4:K]
     want = g.double().numpy().reshape(-1, K)[:, rows].T @ x.double().numpy().reshape(-1, C)
     assert_close(dw[torch.from_numpy(rows).cuda()], want, "dw rows")
+
+
+# rows of threads that fill a block, that do not (20, 3 and 256 channel vectors), that a warp adds up with shuffles first
+@pytest.mark.parametrize("n,hw,c,bound", [(128, 8, 256, 1e-8), (64, 8, 160, 1e-8), (312, 8, 24, 1e-8), (2, 4, 2048, 1e-8), (40, 16, 64, 2e-8), (800, 32, 16, 2e-8)])
+def test_batchnorm_sums_are_accurate(ctx, n, hw, c, bound):
+    """Sums of squares in fp32 over eight rows, over a thread's steps and over the rows of a warp, in fp64 beyond.  A rounding leaves
+    2^-26 of the partial sum on average; they add up along three levels per step, and five more where a warp's rows meet."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(65)
+    shape = (n, hw, hw, c)
+    y = (1.5 * torch.randn(shape, generator=gen, device="cuda") + 0.5).to(torch.bfloat16)
+    a = torch.empty_like(y)
+    stats = torch.full((2 * c,), float("nan"), dtype=torch.float64, device="cuda")
+    mean, invstd = torch.empty(c, device="cuda"), torch.empty(c, device="cuda")
+    ones, zeros = torch.ones(c, device="cuda"), torch.zeros(c, device="cuda")
+    ctx.bn_relu_fwd(n, hw, hw, c, y, stats, False, ones, zeros, None, True, 1e-5, a, mean, invstd)
+    assert ctx.device_status() == 0
+    yd = y.double().reshape(-1, c)
+    err = (stats[c:] / (yd * yd).sum(0) - 1).cpu().numpy()
+    assert np.mean(np.abs(err)) <= bound, np.mean(np.abs(err))
+    err = ((stats[:c] - yd.sum(0)) / yd.abs().sum(0)).cpu().numpy()
+    assert np.mean(np.abs(err)) <= bound, np.mean(np.abs(err))
