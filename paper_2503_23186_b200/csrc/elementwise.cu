@@ -989,40 +989,46 @@ __global__ void __launch_bounds__(kGrThreads, 2) bn_bwd_grouped_kernel(const voi
 }
 
 // ------------------------------------------------------------------------------ pooling, padding
-// A block takes one image and up to 32 channel vectors; its rows of threads share the positions, so that the loads of an image are in
-// flight together (one thread per vector walked the positions one after the other: 64 positions of 16 images: 20 of the 226 us of a small net's step).
-__global__ void __launch_bounds__(kEwThreads) avgpool_fwd_kernel(const void* __restrict__ a, int hw, int c, int lanes, void* __restrict__ pooled)
+// 2^rows_shift rows of threads share the positions of a channel vector, so that the loads of an image are in flight together; a block
+// takes kEwThreads / rows consecutive vectors (of one or several images).  Bound: latency on small inputs, HBM on large ones, where the
+// vectors alone fill the chip and a thread walks its positions by itself.
+__global__ void __launch_bounds__(kEwThreads) avgpool_fwd_kernel(const void* __restrict__ a, long long vectors, int hw, int groups, int rows_shift, void* __restrict__ pooled)
 {
     pdl_wait();   // first global access comes after the previous kernel of the stream
     pdl_launch_dependents();
-    __shared__ float part[kEwThreads][9];
-    const int groups = c >> 3, rows = kEwThreads / lanes, gl = threadIdx.x % lanes, rl = threadIdx.x / lanes;
-    const int g = blockIdx.y * lanes + gl;
-    const long long img = blockIdx.x;
+    __shared__ __align__(16) float part[8 * kEwThreads];   // [row][vector][8]
+    const int rows = 1 << rows_shift, per_block = kEwThreads >> rows_shift;
+    const int vl = (int)threadIdx.x & (per_block - 1), rl = (int)threadIdx.x / per_block;
+    const long long first = (long long)blockIdx.x * per_block, v = first + vl;
     float s[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) s[i] = 0.f;
-    if (g < groups && rl < rows) {
+    if (v < vectors) {
+        const long long img = v / groups, base = img * hw * groups + (v - img * groups);
 #pragma unroll 4
         for (int j = rl; j < hw; j += rows) {
             float f[8];
-            unpack8(ld16(a, (img * hw + j) * groups + g), f);
+            unpack8(ld16(a, base + (long long)j * groups), f);
 #pragma unroll
             for (int i = 0; i < 8; ++i) s[i] += f[i];
         }
     }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) part[threadIdx.x][i] = s[i];
-    __syncthreads();
-    if (rl == 0 && g < groups) {
-        for (int r = 1; r < rows; ++r) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) s[i] += part[r * lanes + gl][i];
-        }
-        const float inv = 1.f / (float)hw;
+    const float inv = 1.f / (float)hw;
+    if (rows == 1) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) s[i] *= inv;
-        reinterpret_cast<uint4*>(pooled)[img * groups + g] = pack8(s);
+        if (v < vectors) reinterpret_cast<uint4*>(pooled)[v] = pack8(s);
+        return;
+    }
+    float4* mine = reinterpret_cast<float4*>(part) + 2 * threadIdx.x;
+    mine[0] = make_float4(s[0], s[1], s[2], s[3]);
+    mine[1] = make_float4(s[4], s[5], s[6], s[7]);
+    __syncthreads();
+    for (int o = (int)threadIdx.x; o < 8 * per_block; o += kEwThreads) {   // one output each
+        float t = 0.f;
+#pragma unroll 4
+        for (int r = 0; r < rows; ++r) t += part[8 * per_block * r + o];
+        if (first + (o >> 3) < vectors) reinterpret_cast<__nv_bfloat16*>(pooled)[8 * first + o] = __float2bfloat16_rn(t * inv);
     }
 }
 
@@ -1645,9 +1651,15 @@ b2c_status b2c_avgpool_fwd(b2c_ctx* ctx, int n, int hw, int c, const void* a, vo
     if (!ctx || !a || !pooled) return B2C_ERR_INVALID_ARG;
     if (n < 1 || hw < 1 || c < 8 || c % 8) return B2C_ERR_UNSUPPORTED_SHAPE;
     if (!b2c_aligned16(a) || !b2c_aligned16(pooled)) return B2C_ERR_MISALIGNED;
-    const int groups = c / 8, lanes = groups < 32 ? groups : 32;
-    B2C_CUDA(b2c_launch(ctx, avgpool_fwd_kernel, dim3((unsigned)n, (unsigned)((groups + lanes - 1) / lanes)), dim3(kEwThreads), 0, (cudaStream_t)stream_, 1u, a, hw, c, lanes,
-                        pooled));
+    // Rows until there are 512 threads per SM, as long as they have positions of their own, past 32 rows four of them.  Measured with one thread
+    // per vector / a block per image, its vectors at most 32 wide / this rule: 16 images x 64 positions x 128 channels 12.3 / 2.4 / 2.2 us,
+    // 1024 x 16 x 512 4.6 / 6.3 / 4.2, 1024 x 16 x 2048 11.8 / 19.6 / 10.4, 65536 x 4 x 16 3.4 / 261 / 3.0, 1 x 4096 x 64 663 / 20.6 / 6.3.
+    const long long vectors = (long long)n * (c / 8);
+    int rows_shift = 0;
+    while (rows_shift < 8 && ((rows_shift < 5 ? 2ll : 8ll) << rows_shift) <= hw && (vectors << rows_shift) < 512ll * ctx->sm_count) ++rows_shift;
+    const long long per_block = kEwThreads >> rows_shift;
+    B2C_CUDA(b2c_launch(ctx, avgpool_fwd_kernel, dim3((unsigned)((vectors + per_block - 1) / per_block)), dim3(kEwThreads), 0, (cudaStream_t)stream_, 1u, a, vectors, hw, c / 8,
+                        rows_shift, pooled));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;
 }

@@ -20,8 +20,9 @@ def ctx():
     c.close()
 
 
-# one position, fewer and more positions than thread rows, channel vectors: 1, not a divisor of the block, over one block's 32
-@pytest.mark.parametrize("n,hw,c", [(1, 1, 8), (3, 7, 48), (5, 16, 512), (2, 64, 128), (3, 49, 2048), (2, 300, 264)])
+# rows of threads per vector: one (many images, few channels; one position), up to 32, up to 256; positions that the rows do not divide,
+# vectors that do not fill a block or straddle images
+@pytest.mark.parametrize("n,hw,c", [(1, 1, 8), (3, 7, 48), (5, 16, 512), (2, 64, 128), (3, 49, 2048), (2, 300, 264), (9000, 4, 16), (70000, 1, 8), (1, 4096, 24), (257, 9, 136)])
 def test_avgpool(ctx, n, hw, c):
     a = wl.normal_bf16(60, f"pool{hw}x{c}", (n, hw, c))
     pooled = torch.full((n, c), float("nan"), dtype=torch.bfloat16, device="cuda")
