@@ -219,6 +219,26 @@ b2c_status b2c_conv2d_dgrad(b2c_ctx* ctx, const b2c_conv_desc* d, const void* dy
 b2c_status b2c_conv2d_wgrad(b2c_ctx* ctx, const b2c_conv_desc* d, const void* dy, const void* x, float* dw_krsc,
                             int accumulate, void* stream);
 
+/* The launch plan that a call of this context would take for the layer (pass 0: b2c_conv2d_fwd, 1: b2c_conv2d_dgrad,
+ * 2: b2c_conv2d_wgrad), without launching anything: for tests and for reading timings. */
+typedef enum {
+    B2C_PLAN_GENERAL = 0, B2C_PLAN_SHARED_UNITS = 1, B2C_PLAN_MERGED_TAPS = 2, B2C_PLAN_FULL_HALO = 3,   /* persistent forward / data gradient */
+    B2C_PLAN_ONE_WAVE = 4,                                      /* one tile, or share of a tile, per CTA or pair */
+    B2C_PLAN_WGRAD = 5, B2C_PLAN_WGRAD_RUNS = 6                 /* weight gradient: part of one tile per CTA | equal runs over all tiles */
+} b2c_plan_kind;
+typedef struct {
+    int kind;              /* b2c_plan_kind */
+    int tile_channels;     /* channels of a tile (weight gradient: input channels) */
+    int pair;              /* CTA pairs */
+    int splits;            /* CTAs or pairs (weight gradient: CTAs) that share a tile's reduction */
+    int overlap;           /* the partial sums change hands through the ring's memory */
+    int ctas;              /* CTAs launched */
+    int smem_bytes;        /* dynamic shared memory of a CTA */
+    int k_block;           /* channels (weight gradient: pixels) per k-block */
+    int slot_k_blocks;     /* k-blocks per ring slot */
+} b2c_conv_plan;
+b2c_status b2c_conv2d_plan(b2c_ctx* ctx, const b2c_conv_desc* d, int pass, b2c_conv_plan* out);
+
 /* db[k] (+)= sum_m dz[m, k] for bf16 dz [m, pitch]; fp32 db [k]. */
 b2c_status b2c_bias_grad(b2c_ctx* ctx, int m, int k, int pitch, const void* dz, float* db, int accumulate, void* stream);
 

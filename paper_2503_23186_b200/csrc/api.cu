@@ -151,6 +151,24 @@ size_t b2c_conv2d_workspace_bytes(const b2c_conv_desc* d, int which)
     return 0;   // forward, data gradient and weight gradient keep everything they need in shared memory and TMEM
 }
 
+static KMajorProblem kmajor_problem(const b2c_conv_desc* d, int p, int q, bool dgrad)
+{
+    KMajorProblem pb{};
+    pb.n = d->n; pb.r = d->r; pb.stride = d->stride; pb.pad = d->pad;
+    pb.dgrad = dgrad;
+    pb.ih = dgrad ? p : d->h; pb.iw = dgrad ? q : d->w; pb.ic = dgrad ? d->k : d->c;
+    pb.oh = dgrad ? d->h : p; pb.ow = dgrad ? d->w : q; pb.oc = dgrad ? d->c : d->k;
+    return pb;
+}
+static WgradProblem wgrad_problem(const b2c_conv_desc* d, int p, int q)
+{
+    WgradProblem pb{};
+    pb.n = d->n; pb.h = d->h; pb.w = d->w; pb.c = d->c;
+    pb.p = p; pb.q = q; pb.k = d->k;
+    pb.r = d->r; pb.stride = d->stride; pb.pad = d->pad;
+    return pb;
+}
+
 b2c_status b2c_conv2d_fwd(b2c_ctx* ctx, const b2c_conv_desc* d, const void* x, const void* w_krsc, void* y, int y_is_f32, const float* bias,
                           double* ch_stats, void* stream)
 {
@@ -159,11 +177,7 @@ b2c_status b2c_conv2d_fwd(b2c_ctx* ctx, const b2c_conv_desc* d, const void* x, c
     b2c_status st = check_desc(d, &p, &q);
     if (st != B2C_OK) return st;
     if (ch_stats && y_is_f32) return B2C_ERR_INVALID_ARG;
-    KMajorProblem pb{};
-    pb.n = d->n; pb.ih = d->h; pb.iw = d->w; pb.ic = d->c;
-    pb.oh = p; pb.ow = q; pb.oc = d->k;
-    pb.r = d->r; pb.stride = d->stride; pb.pad = d->pad;
-    pb.dgrad = false;
+    KMajorProblem pb = kmajor_problem(d, p, q, false);
     pb.in = x; pb.wt = w_krsc; pb.out = y;
     pb.out_f32 = y_is_f32 != 0; pb.bias = bias; pb.stats = ch_stats;
     return launch_conv_kmajor(ctx, pb, (cudaStream_t)stream);
@@ -175,13 +189,8 @@ b2c_status b2c_conv2d_dgrad(b2c_ctx* ctx, const b2c_conv_desc* d, const void* dy
     int p, q;
     b2c_status st = check_desc(d, &p, &q);
     if (st != B2C_OK) return st;
-    KMajorProblem pb{};
-    pb.n = d->n; pb.ih = p; pb.iw = q; pb.ic = d->k;
-    pb.oh = d->h; pb.ow = d->w; pb.oc = d->c;
-    pb.r = d->r; pb.stride = d->stride; pb.pad = d->pad;
-    pb.dgrad = true;
+    KMajorProblem pb = kmajor_problem(d, p, q, true);
     pb.in = dy; pb.wt = w_crsk_flipped; pb.out = dx;
-    pb.out_f32 = false; pb.bias = nullptr; pb.stats = nullptr;
     return launch_conv_kmajor(ctx, pb, (cudaStream_t)stream);
 }
 
@@ -191,10 +200,7 @@ b2c_status b2c_conv2d_wgrad(b2c_ctx* ctx, const b2c_conv_desc* d, const void* dy
     int p, q;
     b2c_status st = check_desc(d, &p, &q);
     if (st != B2C_OK) return st;
-    WgradProblem pb{};
-    pb.n = d->n; pb.h = d->h; pb.w = d->w; pb.c = d->c;
-    pb.p = p; pb.q = q; pb.k = d->k;
-    pb.r = d->r; pb.stride = d->stride; pb.pad = d->pad;
+    WgradProblem pb = wgrad_problem(d, p, q);
     pb.dy = dy; pb.x = x; pb.dw = dw_krsc;
     // everything the launcher would reject is rejected here, before anything is enqueued
     if (d->c < 16 || d->c % 16 || d->k < 16 || d->k % 16) return B2C_ERR_UNSUPPORTED_SHAPE;
@@ -205,6 +211,16 @@ b2c_status b2c_conv2d_wgrad(b2c_ctx* ctx, const b2c_conv_desc* d, const void* dy
         if (zs != B2C_OK) return zs;
     }
     return launch_conv_wgrad(ctx, pb, (cudaStream_t)stream);
+}
+
+b2c_status b2c_conv2d_plan(b2c_ctx* ctx, const b2c_conv_desc* d, int pass, b2c_conv_plan* out)
+{
+    if (!ctx || !out || pass < 0 || pass > 2) return B2C_ERR_INVALID_ARG;
+    int p, q;
+    b2c_status st = check_desc(d, &p, &q);
+    if (st != B2C_OK) return st;
+    *out = b2c_conv_plan{};
+    return pass == 2 ? plan_conv_wgrad(ctx, wgrad_problem(d, p, q), *out) : plan_conv_kmajor(ctx, kmajor_problem(d, p, q, pass == 1), *out);
 }
 
 }  // extern "C"

@@ -143,6 +143,7 @@ struct KMajorProblem {
     int stats_group_images;  // images per statistics group (0: one group)
 };
 b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_t stream);
+b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan& out);   // pointers of the problem: null
 
 struct WgradProblem {
     int n, h, w, c;        // x
@@ -153,6 +154,7 @@ struct WgradProblem {
     float* dw;             // [k][r*r][c] fp32, accumulated into
 };
 b2c_status launch_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, cudaStream_t stream);
+b2c_status plan_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, b2c_conv_plan& out);
 
 // BatchNorm over G statistics groups (micro-batches) of m rows each; stats / sums are fp64 [G][2c],
 // save_mean / save_invstd fp32 [G][c].  G > 1 requires acc != 0 in the backward pass.  stats_ready: 1 = `stats` holds the

@@ -1388,6 +1388,10 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     const size_t smem_bytes = (size_t)p.resident_bytes + (size_t)p.stages * stage_bytes + 1024 +
                               (cluster && !p.x_overlap ? (size_t)(p.splits - 1) * (p.n_tile / p.splits) * 512 : 0);
 
+    plan.grid = cluster ? p.total_units * p.splits : grid;
+    plan.smem_bytes = smem_bytes;
+    if (pb.in == nullptr) return B2C_OK;   // a question about the plan
+
     // tensor maps
     const int box_h = (p.vreuse || p.fh || p.hm) ? p.bh + 2 : p.bh;
     const int box_w = p.fh ? p.bw + 2 : p.bw;
@@ -1459,8 +1463,23 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     p.grp_shift = log2_exact(p.stats_group_images);
     p.cb_shift = log2_exact(p.c_blocks);
     if (p.stats && p.stats_group_images > 0 && (p.stats_group_images % p.bn) != 0) return B2C_ERR_UNSUPPORTED_SHAPE;  // a tile must not straddle groups
-    plan.grid = cluster ? p.total_units * p.splits : grid;
-    plan.smem_bytes = smem_bytes;
+    return B2C_OK;
+}
+
+static int kernel_kind(const ConvKParams& p) { return p.hm ? KIND_HMERGE : p.fh ? KIND_FULL_HALO : p.issue_split ? KIND_SPLIT : KIND_GENERAL; }
+
+b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan& out)
+{
+    static_assert((int)KIND_GENERAL == B2C_PLAN_GENERAL && (int)KIND_SPLIT == B2C_PLAN_SHARED_UNITS && (int)KIND_HMERGE == B2C_PLAN_MERGED_TAPS &&
+                      (int)KIND_FULL_HALO == B2C_PLAN_FULL_HALO, "the header's names of the kernel kinds");
+    KMajorPlan plan;
+    b2c_status st = build_kmajor_plan(ctx, pb, plan);
+    if (st != B2C_OK) return st;
+    const ConvKParams& p = plan.p;
+    out.kind = p.splits > 0 ? B2C_PLAN_ONE_WAVE : kernel_kind(p);
+    out.tile_channels = p.n_tile; out.pair = p.pair; out.splits = p.splits > 0 ? p.splits : 1; out.overlap = p.x_overlap;
+    out.ctas = plan.grid; out.smem_bytes = (int)plan.smem_bytes;
+    out.k_block = p.kb; out.slot_k_blocks = p.gsub;
     return B2C_OK;
 }
 
@@ -1496,8 +1515,7 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
     static const kernel_t kernels[2][4] = {
         {conv_kmajor_kernel<false, KIND_GENERAL>, conv_kmajor_kernel<false, KIND_SPLIT>, conv_kmajor_kernel<false, KIND_HMERGE>, conv_kmajor_kernel<false, KIND_FULL_HALO>},
         {conv_kmajor_kernel<true, KIND_GENERAL>, conv_kmajor_kernel<true, KIND_SPLIT>, nullptr, conv_kmajor_kernel<true, KIND_FULL_HALO>}};
-    const int kind = p.hm ? KIND_HMERGE : p.fh ? KIND_FULL_HALO : p.issue_split ? KIND_SPLIT : KIND_GENERAL;
-    const kernel_t kernel = kernels[p.pair ? 1 : 0][kind];
+    const kernel_t kernel = kernels[p.pair ? 1 : 0][kernel_kind(p)];
     if (kernel == nullptr) return B2C_ERR_UNSUPPORTED_SHAPE;
     if (!(ctx->smem_optin_done & B2C_OPTIN_KMAJOR)) {   // the attribute belongs to the device: kept per context, not per process
         for (int a = 0; a < 2; ++a)

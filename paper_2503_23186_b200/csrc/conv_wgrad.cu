@@ -630,6 +630,10 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
         p.stream = per_cta >= 8.0 && equal < 0.85 * plain ? 1 : 0;   // (an estimated tenth was measured as a loss: 320 -> 320 at 16x16 107 -> 111 us)
     }
 
+    plan.smem_bytes = (size_t)p.stages * p.stage_bytes + 1024;
+    plan.grid = p.stream ? ctx->sm_count : base * n_splits;
+    if (pb.dy == nullptr) return B2C_OK;   // a question about the plan
+
     if (!encode_activation_map(ctx, &p.tmDy, pb.dy, pb.n, pb.p, pb.q, pb.k, 1, 0, 0, p.cw_a, p.bw, p.stack ? p.bh + 1 : p.bh, p.bn)) return B2C_ERR_CUDA;
     if (pb.stride == 2) {
         for (int ph = 0; ph < 2; ++ph)
@@ -643,8 +647,19 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     p.c_total = pb.c;
     p.rs_total = R * R;
     p.dw = pb.dw;
-    plan.smem_bytes = (size_t)p.stages * p.stage_bytes + 1024;
-    plan.grid = p.stream ? ctx->sm_count : base * n_splits;
+    return B2C_OK;
+}
+
+b2c_status plan_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, b2c_conv_plan& out)
+{
+    WgradPlan plan;
+    b2c_status st = build_wgrad_plan(ctx, pb, plan);
+    if (st != B2C_OK) return st;
+    const WgradParams& p = plan.p;
+    out.kind = p.stream ? B2C_PLAN_WGRAD_RUNS : B2C_PLAN_WGRAD;
+    out.tile_channels = p.ct; out.splits = p.n_splits;
+    out.ctas = plan.grid; out.smem_bytes = (int)plan.smem_bytes;
+    out.k_block = p.pb; out.slot_k_blocks = p.gsub;
     return B2C_OK;
 }
 
