@@ -1115,8 +1115,11 @@ static int kblock_cycles(int n, int kb, bool pair, int a_rows)
 // Plan for the one-wave kernel (conv_splitk.cu) for a problem whose tiles do not fill the chip, or false where the persistent
 // plan (est_cycles) is the better one.  A cluster of `splits` CTAs or pairs shares a tile's k-blocks and adds the partial tiles
 // up at the end; splits = 1 is a tile per CTA or pair, whose shorter epilogue still beats the persistent kernel's one unit.
-// The estimates, in cycles over the 4 us that any launch takes, were fitted to 330 timed plans of 27 layers: the plan they
-// pick is on average 0.3 % and at most 5 % slower than the layer's best one.  With 128 images, persistent -> this, launch to
+// The estimates, in cycles over the 4 us that any launch takes, were fitted to timed plans.  K-blocks of 64 channels: 187 layers, the plan
+// they pick is on average 5 % slower than the layer's best one (most of that on short reductions, which stay whole).  Narrower ones, whose
+// rows of 32 and 64 bytes come in more slowly, have constants of their own: 503 layers, on average 1.1 % and at most 28 % slower than
+// the best plan, where those of the wide ones picked plans up to 2.7 times as slow (25 images, 784 -> 512 at 16x16 55 us in the persistent
+// kernel, 97 in the plan that they preferred; 17 images, 160 -> 160 at 32x32 12.0 and 15.6).  With 128 images, persistent -> this, launch to
 // launch: 512 -> 512 at 4x4 27.8 -> 14.1 us, 256 -> 256 at 8x8 18.2 -> 12.7, 256 -> 512 at 8x8 stride 2 16.6 -> 10.5; with 50
 // images 26.3 -> 10.7, 16.4 -> 10.2 and 16.4 -> 8.6; 128 -> 128 at 8x8 with 16 images 10.3 -> 5.7.
 static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p, int m_tiles, bool reuse, long long est_cycles)
@@ -1125,7 +1128,9 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
     const int taps = p.n_par > 1 ? ((pb.r + 1) / 2) * ((pb.r + 1) / 2) : pb.r * pb.r;   // of the parity with most
     const int min_taps = p.n_par > 1 ? 1 : taps;
     const int c_blocks = pb.ic / kb;
-    long long best = est_cycles - 600;   // worth a change from the persistent kernel (0.6 us)
+    const bool narrow = kb < 64;
+    // worth a change from the persistent kernel: 0.6 us, and a quarter where that one shares loads and the estimates are less sure
+    long long best = (narrow && reuse ? est_cycles * 18 / 25 : est_cycles) - 600;
     bool found = false;
     for (int pair = 0; pair <= 1; ++pair) {
         if (pair && (p.n_par > 1 || ctx->use_pairs == 0)) continue;
@@ -1155,9 +1160,12 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
                 if (stages > kMaxStages) stages = kMaxStages;
                 if (stages < 2 || (overlap && stages * slot < x_bytes)) continue;
                 const int k_blocks = (taps * c_blocks + splits - 1) / splits;
-                // k-blocks, exchange (barriers, partial tiles at 21 B/clk), epilogue of n / splits columns
-                const long long per_block = block > 570 / gsub ? block : 570 / gsub;
-                const long long est = k_blocks * per_block * (two ? 2 : 1) + (two ? 2000 : 0) + (splits > 1 ? 1100 + 800 * overlap + x_bytes / 21 : 0) + 190ll * n / splits / 32 + 2600 * pair;
+                // k-blocks, exchange (barriers, partial tiles at 21 B/clk), epilogue of n / splits columns.  A slot of narrow k-blocks takes
+                // 1900 cycles however little it holds, most of them latency, which two tiles per SM hide for each other.
+                const int slot_cycles = narrow ? 1900 : 570, own = narrow && two ? 2 * block : block;
+                const long long per_block = own > slot_cycles / gsub ? own : slot_cycles / gsub;
+                const long long est = k_blocks * per_block * (two && !narrow ? 2 : 1) + (two ? 2000 : 0) + (splits > 1 ? (narrow ? 1700 : 1100) + 800 * overlap + x_bytes / 21 : 0) +
+                                      190ll * n / splits / 32 + (narrow ? 5000 : 2600) * pair;
                 if (est >= best) continue;
                 best = est;
                 found = true;
@@ -1345,7 +1353,8 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
         q.bw = gw < 128 ? gw : 128; q.bh = (128 / q.bw) < gh ? (128 / q.bw) : gh; q.bn = 128 / (q.bw * q.bh);
         q.tiles_w = gw / q.bw; q.tiles_h = gh / q.bh; q.tiles_n = (pb.n + q.bn - 1) / q.bn;
         q.vreuse = q.fh = q.hm = q.resident = q.resident_bytes = q.b_merged = q.a_step = 0;
-        const int block = kblock_cycles(n_tile, p.kb, p.pair != 0, a_rows), per_block = p.vreuse || block > 400 ? block : 400;
+        const int block = kblock_cycles(n_tile, p.kb, p.pair != 0, a_rows);
+        const int least = kb_natural < 64 ? (p.vreuse ? 490 : 900) : p.vreuse ? 0 : 400, per_block = block > least ? block : least;
         const bool reuse = p.vreuse || p.fh || p.hm;   // taps share their loads
         const long long persistent = (long long)units_per_cta * max_taps * (pb.ic / p.kb) * per_block + 1060ll * n_tile / 32 +
                                      (p.pair ? 2600 : !reuse && units_per_cta > 1 ? 3000 : 0);
