@@ -375,7 +375,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                 if (!ok && lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
                 tc_fence_after();
             }
-            if (ok) {
+            // Up to 32 filter rows are the work of two warps: what bounds them is the latency of each step, not the L2's sectors, so they send
+            // their vectors as they are, unless many CTAs add to the same rows; warps whose rows all lie past the last filter row have nothing to
+            // send.  640 -> 16 channels at 2x2 with 7 images 9.2 us with the exchange, 6.6 without; 49 CTAs per row (160 -> 16 at 32x32 with 13
+            // images) 15.7 and 12.6, but 148 (64 -> 32 1x1 at 32x32 with 256 images) 12.3 and 13.5.
+            const bool few_rows = !p.stack && p.k_total - ktile * 128 <= 32 && p.n_splits <= 64;
+            if (ok && (p.stack || ktile * 128 + q * 32 < p.k_total)) {
                 const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
                 const int n_ck = p.ct >> 4;
                 const int ck_begin = part == 0 ? 0 : (n_ck + 1) >> 1, ck_end = part == 0 ? (n_ck + 1) >> 1 : n_ck;   // this warp's chunks
@@ -397,6 +402,15 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                     // 1024 images 70.5 -> 67.6 us.
                     const int t4 = lane & 3;
                     auto send = [&](uint32_t (&r)[16], int ck) {
+                        if (few_rows) {
+                            if (live) {
+#pragma unroll
+                                for (int i = 0; i < 4; ++i)
+                                    red_add_v4(dst + (size_t)row16 * 16 + ck * 16 + 4 * i, __uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
+                                               __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3]));
+                            }
+                            return;
+                        }
                         transpose_lanes4(r, t4);   // r[4 i ..] = vector t4 of the row of lane (lane - t4) + i
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {

@@ -69,8 +69,10 @@ def test_statistics_of_long_walks(ctx, shape):
     assert np.mean(np.abs(err)) <= 2e-8, np.mean(np.abs(err))
 
 
-# 75 / 80 tiles on 148 SMs: equal runs of (tile, pixel chunk) pairs, a CTA finishing one tile and beginning the next; partial tiles
-@pytest.mark.parametrize("shape", [(32, 8, 8, 640, 640, 3, 1), (28, 8, 8, 1280, 2048, 1, 1), (31, 8, 8, 640, 624, 3, 1), (6, 8, 8, 48, 16, 3, 1), (4, 8, 8, 32, 144, 3, 1), (4, 8, 8, 16, 80, 1, 2)], ids=lambda s: "n{}h{}c{}k{}r{}s{}".format(*(s[i] for i in (0, 1, 3, 4, 5, 6))))
+# 75 / 80 tiles on 148 SMs: equal runs of (tile, pixel chunk) pairs, a CTA finishing one tile and beginning the next; partial tiles;
+# up to 32 filter rows, as a whole bank, as the rest of one, and with many CTAs on the same rows; 1x1 tiles of up to 160 channels
+@pytest.mark.parametrize("shape", [(32, 8, 8, 640, 640, 3, 1), (28, 8, 8, 1280, 2048, 1, 1), (31, 8, 8, 640, 624, 3, 1), (6, 8, 8, 48, 16, 3, 1), (4, 8, 8, 32, 144, 3, 1), (4, 8, 8, 16, 80, 1, 2), (7, 2, 2, 640, 16, 3, 1), (12, 4, 4, 128, 32, 3, 1),
+                                   (40, 32, 32, 32, 32, 1, 1), (35, 4, 4, 256, 256, 1, 1), (9, 8, 8, 128, 144, 1, 1), (9, 8, 8, 176, 64, 1, 1)], ids=lambda s: "n{}h{}c{}k{}r{}s{}".format(*(s[i] for i in (0, 1, 3, 4, 5, 6))))
 def test_weight_gradient_tiles(ctx, shape):
     from paper_2503_23186_b200 import binding
     N, H, W, C, K, R, st = shape
