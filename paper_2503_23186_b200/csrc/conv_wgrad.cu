@@ -506,12 +506,29 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     p.swz_b = p.cw_b == 64 ? SWZ_128B : p.cw_b == 32 ? SWZ_64B : SWZ_32B;
     // stacking needs chunks that stay inside one image (at least 64 pixels per image)
     p.stack = (R == 3 && pb.stride == 1 && pb.k == 64 && pb.p * pb.q >= 64 && pb.q >= 8) ? 1 : 0;   // q >= 8: the second copy starts on a swizzle-atom boundary
-    // x-channel tile: largest divisor of c that is a multiple of cw_b, at most 160 (three shifts fit 512 TMEM columns) or, for 1x1 layers, 256:
-    // with 128 x 128 tiles a chunk's operands (32 KB for 256 tensor-pipe cycles) come in at twice the rate an SM can load.  256 -> 1024 at 8x8
-    // with 1024 images 40.8 -> 38.5 us, 512 -> 2048 at 4x4 44.8 -> 41.5.
-    p.ct = p.cw_b;
-    for (int cand = R == 1 ? 256 : 160; cand >= p.cw_b; cand -= 16)
-        if (pb.c % cand == 0 && cand % p.cw_b == 0) { p.ct = cand; break; }
+    // x-channel tile: largest divisor of c that is a multiple of cw_b, at most 160 (three shifts fit 512 TMEM columns)
+    auto widest = [&](int limit) {
+        for (int cand = limit; cand > p.cw_b; cand -= 16)
+            if (pb.c % cand == 0 && cand % p.cw_b == 0) return cand;
+        return p.cw_b;
+    };
+    p.ct = widest(160);
+    // 1x1 layers: up to 256, where that is estimated faster.  With 128 x 128 tiles a chunk's operands (32 KB for 256 tensor-pipe cycles) come in at
+    // twice the rate an SM can load, but a wider tile leaves fewer CTAs, each with a longer tail.  Measured with at most 160 / 256 channels: 256 -> 1024
+    // at 8x8 with 1024 images 40.8 / 38.5 us, 512 -> 2048 at 4x4 44.8 / 41.5, 176 -> 512 at 8x8 with 198 images 15.9 / 10.8, but 256 -> 256 at 4x4
+    // with 35 images 7.5 / 9.7, 240 -> 48 at 8x8 with 163 images 8.4 / 11.0, 208 -> 512 at 8x8 stride 2 with 36 images 7.5 / 10.1.
+    if (R == 1) {
+        const int chunks = (int)(((long long)pb.n * pb.p * pb.q + 63) / 64);
+        auto cycles = [&](int ct) {
+            const int tiles = (pb.k + 127) / 128 * (pb.c / ct), fit = ctx->sm_count / tiles;
+            int splits = fit < chunks / 4 ? fit : chunks / 4;
+            if (splits < 1) splits = 1;
+            const long long load = (128 + ct) * 128 / 60, mma = 2 * (ct > 96 ? ct : 96);
+            return (long long)((tiles * splits + ctx->sm_count - 1) / ctx->sm_count) * ((chunks + splits - 1) / splits * (load > mma ? load : mma) + 1500 + 23 * ct);
+        };
+        const int other = widest(256);
+        if (cycles(other) < cycles(p.ct)) p.ct = other;
+    }
     // framed x stages: 64 pixels of one image per chunk, 64-channel x boxes, at most two of them per CTA (2 x 192 TMEM columns)
     p.fx = (R == 3 && pb.stride == 1 && pb.q >= 8 && pb.p * pb.q >= 64 && p.cw_b >= 32 && ctx->use_wgrad_frame) ? 1 : 0;
     if (p.fx) {   // as many boxes per CTA as TMEM holds (three shifts of cw_b columns each): 2 of 64 channels, up to 5 of 32
