@@ -37,10 +37,11 @@ static constexpr uint32_t kDrainPolls = 1u << 22;
 static constexpr int kFoldUnits = 8;     // units of a narrow tile (wide: half as many) whose squares a lane of the epilogue adds up before they move on
 
 // Units of this CTA (a CTA pair walks pair-units: two pixel tiles next to each other, same channel tile, of which CTA `rank` takes tile
-// 2*m + rank).  A walker keeps its channel tile and takes a run of consecutive pixel tiles, so that it meets at most two statistics
-// groups or so of a pass: taken in turns, every walker met every group, and all of them sent the group's sums to the same addresses
-// at the same time.  Eight groups of 128 images: ResNet-18-shaped step 5853 -> 5555 us (launch times summed), ResNet-50-shaped 24.49 -> 23.70 ms.
-// The output parities of a stride-2 data gradient differ in work: their units are taken in turns.
+// 2*m + rank).  A walker keeps its channel tile.  The walkers take their units in turns, so that tiles in work at one time are neighbours in
+// memory; where a pass sums several statistics groups, each takes a run of consecutive pixel tiles instead, so that it meets at most two
+// groups or so: in turns, every walker met every group, and all of them sent the group's sums to the same addresses at the same time.  Eight
+// groups of 128 images: ResNet-18-shaped step 5853 -> 5555 us (launch times summed), ResNet-50-shaped 24.49 -> 23.70 ms.  Without groups runs
+// are slower: data gradient 112 <- 256 1x1 at 32x32 with 442 images 79.3 us in runs, 72.5 in turns, 64 <- 256 with 1024 images 104.0 and 102.7.
 struct UnitWalk {
     int first, stride, count, rank, pair;
     __device__ UnitWalk(const ConvKParams& p, int rank_) : rank(rank_), pair(p.pair)
@@ -49,7 +50,7 @@ struct UnitWalk {
         count = pair ? p.total_units >> 1 : p.total_units;
         first = w;
         stride = walkers;
-        if (p.n_par == 1) {
+        if (p.stats != nullptr && p.stats_group_images > 0) {
             const int per_ktile = walkers / p.n_ktiles, j = w / p.n_ktiles, kt = w - j * p.n_ktiles, m = count / p.n_ktiles;   // (walkers is a multiple of n_ktiles)
             first = (int)((long long)m * j / per_ktile) * p.n_ktiles + kt;
             count = (int)((long long)m * (j + 1) / per_ktile) * p.n_ktiles;
