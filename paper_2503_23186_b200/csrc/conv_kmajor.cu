@@ -34,6 +34,7 @@ static constexpr int kProducers = 2;     // TMA-issuing threads: warp 0 and the 
 static constexpr int kThreads = 64 + 32 * kEpiWarps + 32 * (kIssuers - 1) + 32 * (kProducers - 1);
 static constexpr int kProducerWarp1 = 2 + kEpiWarps + (kIssuers - 1);   // warp index of the second producer
 static constexpr uint32_t kDrainPolls = 1u << 22;
+static constexpr size_t kClusterSmem = 115 * 1024;   // more than half of the 228 KB of an SM
 static constexpr int kFoldUnits = 8;     // units of a narrow tile (wide: half as many) whose squares a lane of the epilogue adds up before they move on
 
 // Units of this CTA (a CTA pair walks pair-units: two pixel tiles next to each other, same channel tile, of which CTA `rank` takes tile
@@ -1395,8 +1396,12 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
         p.issue_split = 1;
     }
     const int stage_bytes = p.gsub * (p.a_bytes + (p.resident ? 0 : p.nb * p.b_bytes));
-    const size_t smem_bytes = (size_t)p.resident_bytes + (size_t)p.stages * stage_bytes + 1024 +
-                              (cluster && !p.x_overlap ? (size_t)(p.splits - 1) * (p.n_tile / p.splits) * 512 : 0);
+    size_t smem_bytes = (size_t)p.resident_bytes + (size_t)p.stages * stage_bytes + 1024 +
+                        (cluster && !p.x_overlap ? (size_t)(p.splits - 1) * (p.n_tile / p.splits) * 512 : 0);
+    // CTAs that wait for one another (pairs, and clusters that share a tile) take more than half of an SM's shared memory, so that no two of
+    // them share an SM.  Their TMEM allocations wait for columns without a limit: two clusters of different streams (or three) that met on
+    // several SMs could each hold the columns that the other one's partner waits for.
+    if ((p.pair || p.splits > 1) && smem_bytes < kClusterSmem) smem_bytes = kClusterSmem;
 
     plan.grid = cluster ? p.total_units * p.splits : grid;
     plan.smem_bytes = smem_bytes;

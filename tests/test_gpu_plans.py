@@ -1,4 +1,6 @@
 """Which kernel a convolution layer gets: the rules of the planner at layers where a wrong estimate costs much."""
+import random
+
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -28,3 +30,20 @@ def test_narrow_k_blocks_stay_in_the_persistent_kernel(ctx, which, shape):
 def test_few_tiles_go_to_the_one_wave_kernel(ctx, which, shape, splits):
     plan = _plan(ctx, which, shape)
     assert plan["kind"] == "one-wave" and plan["splits"] >= splits, plan
+
+
+def test_clusters_have_their_sms_to_themselves(ctx):
+    """CTAs that wait for one another must not share an SM with CTAs of another cluster (their TMEM allocations could wait in a circle):
+    each takes more than half of an SM's 228 KB of shared memory, also where the plan needs less."""
+    rng = random.Random(1)
+    clusters = raised = 0
+    for _ in range(1500):
+        hw = rng.choice([4, 8, 16, 32])
+        shape = (rng.randint(1, 600), hw, hw, 16 * rng.randint(1, 40), 16 * rng.randint(1, 40), rng.choice([1, 3]), rng.choice([1, 1, 2]))
+        for which in ("fwd", "dgrad"):
+            plan = _plan(ctx, which, shape)
+            if plan["pair"] or plan["splits"] > 1:
+                clusters += 1
+                raised += plan["smem_bytes"] == 115 * 1024
+                assert plan["smem_bytes"] > 114 * 1024, (shape, plan)
+    assert clusters >= 200 and raised >= 5, (clusters, raised)
