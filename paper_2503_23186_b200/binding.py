@@ -134,7 +134,11 @@ def _ptr(t):
 
 
 def _stream():
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    """Handle of the current stream.  The functions that read it without an object are torch's own, but not public."""
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _check(status: int, where: str):
