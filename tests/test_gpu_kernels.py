@@ -384,7 +384,8 @@ def test_bounded_wait_reports_timeout(ctx):
     y = torch.zeros((8, 32, 32, 64), dtype=torch.bfloat16, device="cuda")
     ctx.set_spin_limit(1)
     try:
-        ctx.conv2d_fwd(_desc(*shape), dev_bf16(x), dev_bf16(w), y)
+        for _ in range(8):   # (a poll may suspend for longer than a short launch takes)
+            ctx.conv2d_fwd(_desc(*shape), dev_bf16(x), dev_bf16(w), y)
         status = ctx.device_status()
     finally:
         ctx.set_spin_limit(1 << 22)
@@ -402,8 +403,11 @@ def test_conv_full_halo_on_and_off(mode, monkeypatch):
     monkeypatch.setenv("B2C_FULL_HALO", mode)
     c = binding.Context(0)
     try:
-        for shape in [(64, 32, 32, 64, 64, 3, 1), (160, 16, 16, 128, 128, 3, 1), (40, 16, 32, 64, 64, 3, 1)]:
+        for shape in [(64, 32, 32, 64, 64, 3, 1), (160, 16, 16, 128, 128, 3, 1), (40, 16, 32, 64, 64, 3, 1), (390, 16, 16, 64, 128, 3, 1)]:
             N, H, W, C, K, R, st = shape
+            if shape[0] == 390:   # six units per pair: below, the default plans leave 128 channels to streamed filter tiles
+                plan = c.conv2d_plan(_desc(*shape), "fwd")
+                assert plan["pair"] == 1 and (plan["kind"] == "full-halo") == (mode == "1"), plan
             x, w, g = wl.conv_problem(13, *shape)
             ref = oracle.conv2d_fwd(x, w, st, 1)
             y = torch.full(ref.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
@@ -422,11 +426,13 @@ def test_conv_full_halo_on_and_off(mode, monkeypatch):
         c.close()
 
 
+@pytest.mark.parametrize("split_k", ["1", "0"], ids=["default", "persistent"])
 @pytest.mark.parametrize("mode", ["0", "2"])
-def test_conv_cta_pairs_forced_on_and_off(mode, monkeypatch):
-    """The forward / data-gradient kernel on single CTAs only (0) and on CTA pairs wherever possible (2): same results."""
+def test_conv_cta_pairs_forced_on_and_off(mode, split_k, monkeypatch):
+    """The forward / data-gradient kernels on single CTAs only (0) and on CTA pairs wherever possible (2): same results."""
     from paper_2503_23186_b200 import binding
     monkeypatch.setenv("B2C_CTA_PAIRS", mode)
+    monkeypatch.setenv("B2C_SPLIT_K", split_k)
     c = binding.Context(0)
     try:
         for shape in [(8, 32, 32, 64, 64, 3, 1), (4, 16, 16, 128, 256, 3, 1), (4, 16, 16, 256, 128, 3, 1), (8, 32, 32, 64, 128, 3, 2),

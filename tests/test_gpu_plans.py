@@ -2,6 +2,7 @@
 import random
 
 import pytest
+import torch
 
 pytestmark = pytest.mark.gpu
 
@@ -30,6 +31,54 @@ def test_narrow_k_blocks_stay_in_the_persistent_kernel(ctx, which, shape):
 def test_few_tiles_go_to_the_one_wave_kernel(ctx, which, shape, splits):
     plan = _plan(ctx, which, shape)
     assert plan["kind"] == "one-wave" and plan["splits"] >= splits, plan
+
+
+# Every kernel of the forward pass whose waits run out: the persistent ones (B2C_SPLIT_K=0) on pairs and single CTAs, with shared and alternate
+# units, merged taps and full-halo stages, and the one-wave kernel with clusters and with two tiles per SM
+@pytest.mark.parametrize("split_k,shape,want", [
+    ("0", (16, 16, 16, 256, 256, 3, 1), dict(kind="shared-units", pair=1)), ("0", (100, 16, 16, 128, 128, 3, 1), dict(kind="general", pair=1)),
+    ("0", (400, 16, 16, 128, 128, 3, 1), dict(kind="full-halo", pair=1)), ("0", (80, 32, 32, 64, 64, 3, 1), dict(kind="merged-taps")),
+    ("0", (4, 16, 16, 128, 256, 3, 1), dict(kind="shared-units", pair=0)), ("0", (8, 32, 32, 64, 128, 3, 2), dict(kind="general", pair=0)),
+    ("1", (8, 8, 8, 256, 512, 3, 2), dict(kind="one-wave", splits=8)), ("1", (75, 16, 16, 64, 64, 1, 1), dict(kind="one-wave", ctas=150)),
+], ids=lambda v: v if isinstance(v, str) else "n{}h{}w{}c{}k{}r{}s{}".format(*v) if isinstance(v, tuple) else "-".join(map(str, v.values())))
+def test_winds_down_on_timeout(split_k, shape, want, monkeypatch):
+    """A poll budget of one: the status word reports it, every CTA leaves, and the next launch gives what one before gave."""
+    from paper_2503_23186_b200 import binding
+    monkeypatch.setenv("B2C_SPLIT_K", split_k)
+    c = binding.Context(0)
+    N, H, W, C, K, R, st = shape
+    plan = _plan(c, "fwd", shape)
+    assert all(plan[k] == v for k, v in want.items()), plan
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(70)
+    x = torch.randn((N, H, W, C), generator=gen, device="cuda").to(torch.bfloat16)
+    w = (torch.randn((K, R, R, C), generator=gen, device="cuda") * (2.0 / (R * R * C)) ** 0.5).to(torch.bfloat16)
+    d = binding.conv_desc(*shape)
+    good, y = (torch.full((N, H // st, W // st, K), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    c.conv2d_fwd(d, x, w, good)
+    assert c.device_status() == 0
+    c.set_spin_limit(1)
+    try:
+        for _ in range(8):
+            c.conv2d_fwd(d, x, w, y)
+        assert c.device_status() == 7   # B2C_ERR_DEVICE_TIMEOUT
+    finally:
+        c.set_spin_limit(1 << 22)
+    y.fill_(float("nan"))
+    c.conv2d_fwd(d, x, w, y)
+    assert c.device_status() == 0
+    diff = (y.float() - good.float()).norm() / good.float().norm()
+    if want["kind"] == "shared-units":   # two threads issue into one accumulator: sums in either order, a few bf16 values one step (2^-8) apart
+        assert diff.item() <= 1e-3, diff.item()
+    else:
+        assert diff.item() == 0.0, diff.item()
+    c.close()
+
+
+@pytest.mark.parametrize("shape", [(32, 8, 8, 640, 640, 3, 1), (28, 8, 8, 1280, 2048, 1, 1), (31, 8, 8, 640, 624, 3, 1)], ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
+def test_weight_gradients_in_equal_runs(ctx, shape):
+    """The layers with which the parity and wind-down tests mean the kernel that walks several tiles per CTA."""
+    assert _plan(ctx, "wgrad", shape)["kind"] == "wgrad-runs"
 
 
 def test_clusters_have_their_sms_to_themselves(ctx):

@@ -152,6 +152,8 @@ def test_kernel_switches_off_and_on(name, value, monkeypatch):
     against the oracle."""
     from paper_2503_23186_b200 import binding
     monkeypatch.setenv(name, value)
+    if name in ("B2C_ISSUE_SPLIT", "B2C_GROUP_KBLOCKS", "B2C_CTA_PAIRS", "B2C_HMERGE"):
+        monkeypatch.setenv("B2C_SPLIT_K", "0")   # switches of the persistent kernel, which leaves most of these layers to the one-wave kernel
     c = binding.Context(0)
     try:
         # (the 64-output-channel layers are large enough for merged horizontal taps: at least two tiles per SM, rows of 32 / 16 / 8 pixels)
@@ -215,7 +217,7 @@ def _expect_timeout_then_recover(ctx, run, check):
 
 @pytest.mark.parametrize("shape", [(16, 16, 16, 128, 128, 3, 1), (8, 8, 8, 256, 256, 3, 1), (8, 32, 32, 64, 128, 3, 2)], ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
 def test_forward_variants_wind_down_on_timeout(ctx, shape):
-    """CTA pairs (128- and 256-channel tiles, the latter with two issuing threads per unit) and a stride-2 layer."""
+    """Small layers as the default plans take them (the one-wave kernel); the persistent kernels' wind-down is tested by plan."""
     N, H, W, C, K, R, st = shape
     x, w, _ = wl.conv_problem(35, *shape)
     P = H // st

@@ -16,6 +16,16 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(50, 4, 4, 512, 512, 3, 1), (8, 4, 4, 256, 64, 3, 1), (3, 8, 8, 32, 32, 3, 1), (8, 32, 32, 16, 16, 3, 1), (2, 16, 16, 160, 160, 3, 1),
           (8, 8, 8, 128, 256, 3, 2), (8, 8, 8, 128, 256, 1, 2), (5, 16, 16, 32, 64, 3, 2), (6, 8, 8, 48, 96, 3, 1), (16, 8, 8, 2048, 512, 1, 1), (7, 4, 4, 640, 320, 3, 1), (33, 8, 8, 512, 256, 3, 1),
           (81, 32, 32, 16, 32, 3, 2), (75, 16, 16, 64, 64, 1, 1)]
+# Layers whose plans split a tile, with what the plan has to be (forward, data gradient; None: whatever it is): parities through the
+# exchange, in an area of its own and through the ring's memory, parities without taps, slices of 40, 24 and 8 columns, k-blocks of 32 and
+# 16 channels, split pairs
+SPLIT = [((50, 8, 8, 256, 512, 3, 2), dict(splits=2), dict(splits=2, overlap=1)), ((8, 8, 8, 256, 512, 3, 2), dict(splits=8), dict(splits=4, overlap=0)),
+         ((8, 8, 8, 1024, 2048, 1, 2), dict(splits=4), dict(splits=2)), ((32, 8, 8, 160, 160, 3, 1), dict(splits=2, tile_channels=80, k_block=32), None),
+         ((8, 8, 8, 512, 80, 3, 1), dict(splits=2, tile_channels=80), dict(splits=4, k_block=16)), ((24, 4, 4, 240, 512, 1, 2), None, dict(splits=2, tile_channels=48)),
+         ((1, 4, 4, 128, 544, 1, 2), None, dict(splits=4, tile_channels=32, k_block=32)), ((39, 4, 4, 640, 480, 3, 1), dict(splits=4, tile_channels=96, pair=1), None),
+         ((35, 4, 4, 224, 304, 3, 2), None, dict(splits=4, overlap=1, k_block=16))]
+# B2C_SPLIT_K=0 on pairs: two threads that share units, and alternate units
+PERSISTENT_PAIRS = [((8, 16, 16, 256, 256, 3, 1), dict(kind="shared-units", pair=1)), ((80, 16, 16, 128, 128, 3, 1), dict(kind="general", pair=1))]
 
 
 @pytest.fixture(scope="module", params=["0", "1"], ids=["persistent", "split-k"])
@@ -31,6 +41,7 @@ def ctx(request):
             del os.environ["B2C_SPLIT_K"]
         else:
             os.environ["B2C_SPLIT_K"] = before
+    c.split_k = request.param == "1"
     yield c
     assert c.device_status() == 0
     c.close()
@@ -41,9 +52,24 @@ def _desc(N, H, W, C, K, R, st):
     return binding.conv_desc(N, H, W, C, K, R, st)
 
 
-@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
+def _check_plan(ctx, shape, which, want):
+    plan = ctx.conv2d_plan(_desc(*shape), which)
+    assert want is None or all(plan[k] == v for k, v in want.items()), (shape, which, plan)
+
+
+@pytest.mark.parametrize("shape", SHAPES + [s for s, _, _ in SPLIT] + [s for s, _ in PERSISTENT_PAIRS], ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
 def test_forward_statistics_and_data_gradient(ctx, shape):
     N, H, W, C, K, R, st = shape
+    if ctx.split_k:
+        for s, fwd, dgrad in SPLIT:
+            if s == shape:
+                _check_plan(ctx, shape, "fwd", fwd)
+                _check_plan(ctx, shape, "dgrad", dgrad)
+    else:
+        for s, want in PERSISTENT_PAIRS:
+            if s == shape:
+                _check_plan(ctx, shape, "fwd", want)
+        assert ctx.conv2d_plan(_desc(*shape), "fwd")["kind"] != "one-wave"
     x, w, g = wl.conv_problem(40, *shape)
     pad, P = (R - 1) // 2, H // st
     y = torch.full((N, P, P, K), float("nan"), dtype=torch.bfloat16, device="cuda")
