@@ -30,7 +30,8 @@
  *                            a barrier wait and a commit; weight gradient of layers with few MMAs per 64-pixel chunk: one chunk per slot
  *                            instead of two
  *       B2C_ISSUE_SPLIT=0    forward / data gradient, tiles wider than 128 channels: one MMA-issuing thread instead of two sharing every unit
- *       B2C_SPLIT_K=0        forward / data gradient with fewer tiles than SMs: one CTA or pair per tile instead of a cluster sharing its k-blocks
+ *       B2C_SPLIT_K=0        forward / data gradient with up to two tiles per SM: the persistent kernel instead of the one-wave kernel, in which
+ *                            a cluster of CTAs may share a tile's k-blocks
  *       B2C_WGRAD_FRAME=0    weight gradient: one x box per horizontal shift instead of one framed box per channel block
  *       B2C_WGRAD_ISSUERS=1  weight gradient: one MMA-issuing thread instead of two on alternate chunks of one accumulator
  *       B2C_BN_GROUPED=1     b2c_train_step runs the BatchNorm backward as one cooperative launch per layer, group by group

@@ -450,7 +450,7 @@ b2c_status b2c_net_create_concurrent(b2c_ctx* ctx, const b2c_layer_desc* layers,
             if (kind == B2C_LAYER_BN && L.d.res >= 0 && (L.res_slot = add_contrib(L.d.res)) < 0) return fail(B2C_ERR_UNSUPPORTED_SHAPE);
         }
     }
-    // small per-layer buffers; the fp64 statistics are contiguous so one memset clears them
+    // small per-layer buffers; the fp64 statistics are contiguous so that one launch clears them
     for (int i = 0; i < n_layers; ++i) {
         LayerPlan& L = net->layers[i];
         if (L.d.kind == B2C_LAYER_BN) { L.mean_off = alloc(4 * (size_t)L.d.c * n_concurrent); L.invstd_off = alloc(4 * (size_t)L.d.c * n_concurrent); }

@@ -53,7 +53,7 @@ struct b2c_ctx {
     int use_pdl;                         // kernels are launched with programmatic stream serialization (their set-up overlaps the previous kernel's tail)
     int use_hmerge;                      // forward / data gradient of 3x3 stride-1 layers with 64 output channels: horizontal taps merged into N = 192 MMAs
     int use_group_kblocks;               // short k-blocks of stride-2 and 1x1 layers share ring slots (fewer barrier waits per MMA)
-    int use_split_k;                     // forward / data gradient with fewer tiles than SMs: clusters of CTAs share a tile's k-blocks (conv_splitk.cu)
+    int use_split_k;                     // forward / data gradient with up to two tiles per SM: one wave, clusters of CTAs may share a tile's k-blocks (conv_splitk.cu)
     int max_clusters[2][9];              // clusters of 1..8 CTAs that run at once, for single CTAs and pairs; -1: not asked yet
     int use_wgrad_two_issuers;           // weight gradient: two MMA-issuing threads on alternate chunks of one accumulator where the ring depth is even
     int use_bn_grouped;                  // BatchNorm backward of the training step: both passes in one cooperative launch, group by group

@@ -1105,7 +1105,8 @@ struct KMajorPlan {
 
 // Tensor-pipe and staging cycles of one k-block of kb channels on a tile of 128 pixels (a pair: 2 x 128) x n channels: an MMA of 16
 // channels takes n / 2 cycles, or what its operands take through the 128 B/clk shared-memory port (A: 4 KB, B: 32 n bytes, half of
-// it per CTA of a pair); the loads come in at about 74 B/clk per SM, 52 with 160-channel tiles (fitted with the estimates below).
+// it per CTA of a pair); the loads come in at about 74 B/clk per SM, 52 where the tile's width is no power of
+// two (fitted with the estimates below, where 160- and 80-channel tiles weigh most).
 static int kblock_cycles(int n, int kb, bool pair, int a_rows)
 {
     const int b_rows = pair ? n / 2 : n;
@@ -1141,11 +1142,11 @@ static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p,
             const int clusters = p.n_par * (pair ? (m_tiles / p.n_par + 1) / 2 : m_tiles / p.n_par) * (pb.oc / n);
             for (int splits = 1; splits * (pair + 1) <= 8; splits *= 2) {
                 if (n % (8 * splits) || splits > min_taps * c_blocks) continue;
-                // (short reductions stay whole: a split saves them a microsecond at most, and a layer then adds up in the same
-                // order whatever the number of images in the launch)
+                // (short reductions stay whole: a split saves them a microsecond at most)
                 if (splits > 1 && est_cycles < 15000) continue;
                 // two tiles per SM: their CTAs (72 registers, half of the shared memory each) take turns at the tensor pipe, one in
-                // its epilogue while the other loads
+                // its epilogue while the other loads.  (The occupancy calculator answers one for kernels that allocate TMEM, so it is
+                // not asked; 191 CTAs that live 19.0 k cycles each start every 17 k cycles.)
                 const bool two = splits == 1 && !pair && !reuse && clusters > ctx->sm_count && clusters <= 2 * ctx->sm_count;
                 if (!two && clusters > splitk_max_clusters(ctx, splits * (pair + 1), pair != 0)) continue;
                 const int smem = (two ? 94 : 208) * 1024;   // (beside 16.6 KB of static arrays)
@@ -1238,12 +1239,12 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     // tile that splits into two multiples of 16; the fp32 / bias / multi-parity cases stay on single CTAs.
     const int m_tiles = p.tiles_n * p.tiles_h * p.tiles_w;
     // Measured on B200 (1024-image layers): pairs gain ~30 % at 128-channel tiles, where the filter traffic from L2
-    // bounds single CTAs, and lose 5-30 % at 64 and 256 and on the short reductions of 1x1 and stride-2 layers; so by
-    // default only 3x3 stride-1 layers with 128-channel tiles use them (use_pairs: 0 = never, 1 = those, 2 = every
+    // bounds single CTAs, and lose 5-30 % at 64 channels and on the short reductions of 1x1 and stride-2 layers; so by
+    // default only 3x3 stride-1 layers with tiles of 128 channels and more use them (use_pairs: 0 = never, 1 = those, 2 = every
+    // eligible problem, 3 = 128-channel tiles only).  Where single CTAs get by with one tile each, short reductions are faster without
+    // the pair's set-up and longer operand path: 160 -> 160 at 32x32 with 16 images 15.1 us as pairs, 11.6 as singles, 128 -> 128 at
+    // 16x16 with 50 10.4 and 8.3, but 320 -> 320 at 16x16 with 32 16.6 and 17.2.
     const bool pair_ok = n_par == 1 && !pb.out_f32 && pb.bias == nullptr && n_tile % 32 == 0 && m_tiles % 2 == 0 && ctx->sm_count >= 2;
-    // eligible problem).  Where single CTAs get by with one tile each, short reductions are faster without the pair's set-up and
-    // longer operand path: 160 -> 160 at 32x32 with 16 images 15.1 us as pairs, 11.6 as singles, 128 -> 128 at 16x16 with 50
-    // 10.4 and 8.3, but 320 -> 320 at 16x16 with 32 16.6 and 17.2.
     const bool short_wave = p.total_units <= ctx->sm_count && R * R * pb.ic < 2048;
     p.pair = (pair_ok && (ctx->use_pairs == 2 || (ctx->use_pairs == 1 && n_tile >= 128 && R == 3 && pb.stride == 1 && !short_wave) ||
                           (ctx->use_pairs == 3 && n_tile == 128 && R == 3 && pb.stride == 1))) ? 1 : 0;

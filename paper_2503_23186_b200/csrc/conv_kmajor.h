@@ -1,5 +1,6 @@
 // Parameter block and unit numbering shared by the two implicit-GEMM kernels with K-major operands: the persistent one
-// (conv_kmajor.cu) and the split-K one for problems with fewer tiles than SMs (conv_splitk.cu).
+// (conv_kmajor.cu) and the split-K one for problems with up to one or two tiles per SM (conv_splitk.cu).  The packed arithmetic
+// serves both, the column exchanges behind it the persistent one.
 #pragma once
 #include "common.h"
 #include "ptx.cuh"

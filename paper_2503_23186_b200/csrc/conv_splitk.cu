@@ -1,5 +1,5 @@
-// Implicit-GEMM convolution for problems with fewer output tiles than the chip has SMs: forward pass, data gradient and
-// classifier at small batches.
+// Implicit-GEMM convolution for problems with up to one output tile per SM (two, where they are small): forward pass, data
+// gradient and classifier at small batches.
 //
 // The operands, tap tables and tile geometry are those of conv_kmajor.cu; what differs is the split of the work.  There, a
 // CTA owns a whole tile, so a layer with 16 tiles of 72 k-blocks runs 72 k-blocks in a row on 16 SMs (or pairs) and leaves
@@ -218,12 +218,8 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     }
 
     // ---------------------------------------------------------------- epilogue: all eight warps
-    bool live = n_slots > 0;
     const long long t_wait = TIMED ? clock64() : 0;
-    if (live && !mbar_wait_warp(&acc_bar, 0u, p.spin_limit, &abort_flag)) {
-        if (lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
-        live = false;
-    }
+    if (n_slots > 0 && !mbar_wait_warp(&acc_bar, 0u, p.spin_limit, &abort_flag) && lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
     if (TIMED && rank == 0 && warp == 2 && lane == 0) atomicAdd(p.stall + 3, (unsigned long long)(clock64() - t_wait));
     tc_fence_before();
     __syncthreads();
