@@ -1123,8 +1123,8 @@ static int kblock_cycles(int n, int kb, bool pair, int a_rows)
 // rows of 32 and 64 bytes come in more slowly, have constants of their own: 503 layers, on average 1.1 % and at most 28 % slower than
 // the best plan, where those of the wide ones picked plans up to 2.7 times as slow (25 images, 784 -> 512 at 16x16 55 us in the persistent
 // kernel, 97 in the plan that they preferred; 17 images, 160 -> 160 at 32x32 12.0 and 15.6).  With 128 images, persistent -> this, launch to
-// launch: 512 -> 512 at 4x4 27.8 -> 14.1 us, 256 -> 256 at 8x8 18.2 -> 12.7, 256 -> 512 at 8x8 stride 2 16.6 -> 10.5; with 50
-// images 26.3 -> 10.7, 16.4 -> 10.2 and 16.4 -> 8.6; 128 -> 128 at 8x8 with 16 images 10.3 -> 5.7.
+// launch: 512 -> 512 at 4x4 27.8 -> 13.6 us, 256 -> 256 at 8x8 18.2 -> 12.3, 256 -> 512 at 8x8 stride 2 16.6 -> 10.3; with 50
+// images 26.3 -> 10.4, 16.4 -> 9.8 and 16.4 -> 8.2; 128 -> 128 at 8x8 with 16 images 10.3 -> 6.3.
 static bool choose_splitk(b2c_ctx* ctx, const KMajorProblem& pb, ConvKParams& p, int m_tiles, bool reuse, long long est_cycles)
 {
     const int kb = (pb.ic % 64 == 0) ? 64 : (pb.ic % 32 == 0) ? 32 : 16;

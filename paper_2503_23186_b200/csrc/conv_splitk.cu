@@ -17,7 +17,7 @@
 //     long as the MMAs of 256 channels (128 channels, 36 k-blocks: 19.8 k cycles to the last MMA with one k-block per slot,
 //     13.4 k with two).
 // What bounds it now: the operands' way from L2 (about 74 B/clk per SM), then the set-up and the exchange, about 3 us together.
-// Launch to launch with 128 images: 512 -> 512 at 4x4 28 us in the persistent kernel, 13.5 here (17.4 with one k-block per slot,
+// Launch to launch with 128 images: 512 -> 512 at 4x4 28 us in the persistent kernel, 13.6 here (17.4 with one k-block per slot,
 // the exchange in the ring and single-buffered); 256 -> 256 at 8x8 18.2 and 12.3 (14.1); the ResNet-18-shaped step of 128 images
 // 1.89 -> 1.73 ms when this kernel came and 1.490 -> 1.452 ms with those three, as four micro-batches of 50 6.32 -> 5.41 and
 // 4.41 -> 4.28 ms.

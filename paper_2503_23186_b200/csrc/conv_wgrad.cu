@@ -649,7 +649,7 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     if (n_splits > p.chunks_total / 4) n_splits = p.chunks_total / 4;
     if (n_splits < 1) n_splits = 1;
     p.n_splits = n_splits;
-    // Tiles that do not divide the SMs evenly leave many of them idle (75 tiles: one CTA each on 148 SMs: 640 -> 640 at 8x8 with 256 images 135 us, now 91).  Equal runs of (tile, chunk)
+    // Tiles that do not divide the SMs evenly leave many of them idle (75 tiles: one CTA each on 148 SMs: 640 -> 640 at 8x8 with 256 images 135 us, now 82).  Equal runs of (tile, chunk)
     // pairs keep all busy, at the price of one more accumulator to send for most CTAs (about 9000 cycles).
     {
         const int cols = p.fx ? p.b_boxes * 3 * p.cw_b : shifts * p.ct;
