@@ -122,3 +122,25 @@ def test_batchnorm_sums_are_accurate(ctx, n, hw, c, bound):
     assert np.mean(np.abs(err)) <= bound, np.mean(np.abs(err))
     err = ((stats[:c] - yd.sum(0)) / yd.abs().sum(0)).cpu().numpy()
     assert np.mean(np.abs(err)) <= bound, np.mean(np.abs(err))
+
+
+def test_staged_backward_of_the_widest_layers_with_two_gradients(ctx):
+    """2048 channels, two upstream gradients: three tensors per ring stage, which the reduction's partial sums use once it is empty."""
+    n, hw, c = 10, 8, 2048
+    r = wl.rng_for(66, "bn-wide")
+    y, da1, da2 = (wl.to_bf16_grid(r.standard_normal((n * hw * hw, c))) for _ in range(3))
+    gamma = (1.0 + 0.1 * r.standard_normal(c)).astype(np.float32)
+    mean, _, invstd = oracle.bn_stats(y, 1e-5)
+    mean, invstd = oracle.round_f32(mean), oracle.round_f32(invstd)
+    dy_ref, dres_ref, dg_ref, db_ref = oracle.bn_relu_bwd(da1, da2, y, y, gamma, mean, invstd, True, True)
+    mask = torch.from_numpy(np.packbits((y > 0).reshape(-1, 8), axis=1, bitorder="little").reshape(-1)).cuda()
+    dy, dres = (torch.full((n * hw * hw, c), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    dg, db = torch.zeros(c, device="cuda"), torch.zeros(c, device="cuda")
+    ws = torch.empty(ctx.bn_relu_bwd_workspace_bytes(c), dtype=torch.uint8, device="cuda")
+    dev = lambda v: torch.from_numpy(np.ascontiguousarray(v, dtype=np.float32)).cuda()
+    ctx.bn_relu_bwd(n, hw, hw, c, dev_bf16(da1), dev_bf16(da2), dev_bf16(y), None, dev(gamma), dev(mean), dev(invstd), True, dy, dres, dg, db, False, ws, relu_mask=mask)
+    assert ctx.device_status() == 0
+    assert_close(dy, dy_ref, "dy")
+    assert_close(dres, dres_ref, "dres")
+    assert_close(dg, dg_ref, "dgamma", 1e-5, 1e-5)   # fp32 over a few rows, fp64 beyond
+    assert_close(db, db_ref, "dbeta", 1e-5, 1e-5)
