@@ -141,6 +141,8 @@ struct KMajorProblem {
     const float* bias;
     double* stats;         // fp64 [groups][2*oc] or nullptr
     int stats_group_images;  // images per statistics group (0: one group)
+    bool no_wait;          // the launch right before this one shares nothing that is written with this one, and itself waits for the one before it:
+                           // the kernel starts as SMs fall free and waits for that launch only at its end
 };
 b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_t stream);
 b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan& out);   // pointers of the problem: null

@@ -766,8 +766,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
     tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
     // set-up done (it touched no global data): order behind the previous kernel of the stream, then let the next one in
-    pdl_wait();
-    pdl_launch_dependents();
+    pdl_begin(p.no_wait);
     const long long t_start = clock64();
     int last_issued = -1;  // producer lanes: index of the last stage whose loads this lane issued
 
@@ -1043,6 +1042,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
         if constexpr (PAIR) tmem_dealloc_pair(tmem_base, (uint32_t)p.tmem_cols);
         else tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
     }
+    pdl_end(p.no_wait);
 }
 
 // ------------------------------------------------------------------------------------------ host side
@@ -1521,6 +1521,7 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
     ConvKParams& p = plan.p;
     const int grid = plan.grid;
     const size_t smem_bytes = plan.smem_bytes;
+    p.no_wait = pb.no_wait ? 1 : 0;
     p.status = ctx->d_status;
     p.spin_limit = ctx->spin_limit;
     p.stall = ctx->stall_counters;

@@ -49,6 +49,7 @@ struct alignas(64) ConvKParams {
     const float* bias;
     double* stats;
     int stats_group_images;          // images per BatchNorm statistics group (0: one group)
+    int no_wait;                     // starts beside the previous launch of the stream, see pdl_begin
     unsigned* status;
     unsigned spin_limit;
     unsigned long long* stall;       // optional [5]: cycles waited by producer / MMA (ring) / MMA (accumulator) / epilogue, CTA lifetime

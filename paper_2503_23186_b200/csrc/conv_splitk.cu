@@ -139,8 +139,7 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     if (clustered) cluster_sync_all();   // the others' barriers and memory exist before anything arrives there
     tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
-    pdl_wait();
-    pdl_launch_dependents();
+    pdl_begin(p.no_wait);
 
     int issued = 0;   // producer warp: ring slots whose loads it has issued
     if (warp == 0) {
@@ -396,6 +395,7 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
         else tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
     }
     if (TIMED && rank == 0 && threadIdx.x == 0) atomicAdd(p.stall + 4, (unsigned long long)(clock64() - t_start));
+    pdl_end(p.no_wait);
     if constexpr (PAIR) cluster_sync_all();   // a pair gives its TMEM back together
 }
 

@@ -18,6 +18,19 @@ namespace b2c {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// The same for a kernel that needs nothing of the launch right before it (no_wait).  That launch let this one in only after its own wait,
+// so everything older has completed; reads must go through the async proxy (no stale L1 lines).  pdl_end keeps the order for the launches
+// behind this one: the grid does not complete before the one that it overtook.
+__device__ __forceinline__ void pdl_begin(int no_wait)
+{
+    if (!no_wait) pdl_wait();
+    pdl_launch_dependents();
+}
+__device__ __forceinline__ void pdl_end(int no_wait)
+{
+    if (no_wait) pdl_wait();
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // ---------------------------------------------------------------- mbarrier
