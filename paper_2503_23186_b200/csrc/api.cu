@@ -465,12 +465,11 @@ b2c_status b2c_net_create_concurrent(b2c_ctx* ctx, const b2c_layer_desc* layers,
             const int pix = L.p * L.q;
             const int imgs_per_tile = pix >= 128 ? 1 : 128 / pix;
             o.fused_stats = net->fuse_stats && (n_concurrent == 1 || micro_batch % imgs_per_tile == 0);
-            // Tiles of up to 64 channels sum at next to no cost.  Wider ones are fused where that takes less than one more pass over the
-            // output.  Cycles of a unit, measured on 1024-image layers: 530 per 32 columns for the epilogue's stores and 600 for its sums
-            // (64 -> 256 1x1: 126 us without, 273 us with), both hidden as far as the MMAs or the unit's share of the HBM traffic (24 B/clk
-            // per SM) take longer; the pass of its own 410 per 32 columns (5.5 TB/s) and about 5500 for the launch, spread over the units of
-            // a CTA.  Both sides measured: 128 -> 128 3x3 72 fused, 55 + 15 us; 512 -> 128 1x1 60, 55 + 15; 64 -> 128 3x3 stride 2 62, 58 +
-            // 15; 64 -> 256 1x1 273, 126 + 95; 256 -> 1024 1x1 82, 50 + 27.
+            // Tiles of up to 64 channels sum at next to no cost, and so do those of 128 and 256 channels, whose epilogue works in blocks (64 -> 256
+            // 1x1 130 us without, 145 with sums, a pass of its own 95; 256 -> 1024 51 and 57, 27).  Other wide ones are fused where that takes less
+            // than one more pass over the output.  Cycles of a unit, measured on 1024-image layers: 530 per 32 columns for the epilogue's
+            // stores and 600 for its sums, both hidden as far as the MMAs or the unit's share of the HBM traffic (24 B/clk per SM) take longer;
+            // the pass of its own 410 per 32 columns (5.5 TB/s) and about 5500 for the launch, spread over the units of a CTA.
             int n_tile = 16;
             for (int cand = 256; cand >= 16; cand -= 16)
                 if (L.d.k % cand == 0) { n_tile = cand; break; }
@@ -480,8 +479,8 @@ b2c_status b2c_net_create_concurrent(b2c_ctx* ctx, const b2c_layer_desc* layers,
                 const double hbm = (256.0 * L.c_pad * L.d.stride * L.d.stride * n_tile / L.d.k + 256.0 * n_tile) / 24.0;
                 const double hidden = mma > hbm ? mma : hbm;
                 const double plain = hidden > 530.0 * x ? hidden : 530.0 * x, fused = hidden > 1130.0 * x ? hidden : 1130.0 * x;
-                const char* e2 = std::getenv("B2C_FUSE_WIDE");   // 1: always; 0: never; default: by the estimate
-                const bool wide_ok = e2 ? e2[0] != '0' : fused - plain <= 410.0 * x + 5500.0 / (units > 1.0 ? units : 1.0);
+                const char* e2 = std::getenv("B2C_FUSE_WIDE");   // 1: always; 0: never; default: by the rule above
+                const bool wide_ok = e2 ? e2[0] != '0' : n_tile == 128 || n_tile == 256 || fused - plain <= 410.0 * x + 5500.0 / (units > 1.0 ? units : 1.0);
                 if (!wide_ok) o.fused_stats = false;
             }
         }

@@ -97,7 +97,7 @@ __device__ __forceinline__ void butterfly16(float (&a)[16], float (&b)[16], int 
     b[0] += __shfl_xor_sync(0xffffffffu, b[0], 1);
 }
 
-// Epilogue of one warp over all units of the CTA.  Epilogue warp e reads the TMEM lane quarter its warp index selects and the column half e >> 2
+// Epilogue of one warp over all units of the CTA, for the tile widths and plans that epilogue_blocks does not take.  Epilogue warp e reads the TMEM lane quarter its warp index selects and the column half e >> 2
 // of every accumulator.  The warp owns at most NCH 16-column chunks per unit.  EAGER: it reads all
 // its columns at once and hands the accumulator back before packing and storing (narrow tiles).
 // STATS: BatchNorm sums of the values as stored, kept in registers until the statistics group ends; those of the last group are left
@@ -424,6 +424,236 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
     return STATS && ok ? make_int2(cur_group, cur_ktile) : make_int2(-1, 0);
 }
 
+// Epilogue of one warp for tiles of 64, 128 or 256 channels without a bias: the same share of every unit as in epilogue_loop, but the rounded
+// values go through shared memory, BC columns of the warp's 32 rows at a time, so that a lane then holds 8 neighbouring columns of every
+// (32 / (BC / 8))-th row: an instruction stores whole runs of BC columns (BC = 64: 4 lines, where a row per lane touches 32), and the
+// BatchNorm sums of a column are additions in one lane with no exchange.  Rows that do not exist (images past the last one) are skipped.
+// NB blocks of BC columns are the warp's half of the tile; wider blocks need fewer running sums per lane (with NB = 4 and BC = 32 they spill).
+// Bound: HBM writes on 1x1 layers (537 MB alone take 125-145 us), else the two warps' latency per scheduler, no longer the store path.
+// Layers of 1024 images inside a step, epilogue_loop -> this: with sums 64 -> 256 1x1 at 32x32 312 -> 145 us (sums in a pass of their own: 139 +
+// 95), 128 -> 512 at 16x16 166 -> 84, 64 -> 64 3x3 80 -> 71, 128 -> 128 3x3 at 16x16 77 -> 63, 64 -> 128 1x1 stride 2 60 -> 41, 512 -> 512 at 4x4
+// 65 -> 63; without sums data gradient 256 <- 64 1x1 137 -> 126, 512 <- 128 81 -> 71, 64 <- 64 3x3 66 -> 63.
+template <int BC, int NB, bool HM, bool STATS>
+__device__ __forceinline__ int2 epilogue_blocks(const ConvKParams& p, uint32_t tmem_base, uint64_t* acc_full, uint64_t* acc_empty, uint32_t* abort_flag,
+                                                float* my_stats, uint8_t* stage, int e, int lane, int rank)
+{
+    constexpr int LPR = BC / 8;       // lanes per row on the way out
+    constexpr int RPI = 32 / LPR;     // rows per instruction; LPR instructions cover the warp's rows
+    const UnitWalk walk(p, rank);
+    const bool remote_empty = p.pair && rank != 0;
+    const int q = (e + 2) & 3;
+    const int col_begin = (e >> 2) * (BC * NB);
+    const int my_row = q * 32 + lane / LPR;   // and every RPI-th after it
+    int my_off = 8 * (lane % LPR) + col_begin;
+#pragma unroll
+    for (int bit = 0; bit < 7; ++bit)
+        if ((my_row >> bit) & 1) my_off += p.row_bit[bit];
+    constexpr int LOG_RPI = RPI == 4 ? 2 : RPI == 8 ? 3 : 4;
+    int step_off[5 - LOG_RPI];   // (moved by hand: read from the parameters again for every store, they cost 64 -> 64 3x3 with 256 images 18.2 -> 19.2 us)
+#pragma unroll
+    for (int i = 0; i < 5 - LOG_RPI; ++i) asm volatile("mov.u32 %0, %1;" : "=r"(step_off[i]) : "r"(p.row_bit[LOG_RPI + i]));
+    // 16-byte words of the staging block: word j of row r lies at j ^ swizzle(r), without bank conflicts either way
+    auto swizzle = [](int row) { return BC == 64 ? row & 7 : BC == 32 ? (row >> 1) & 3 : (row >> 2) & 1; };
+    const uint32_t st_w = smem_u32(stage) + (uint32_t)lane * (BC * 2);
+    const int sw_w = swizzle(lane);
+
+    constexpr int NA = STATS ? 4 * NB : 1;   // column pairs this lane sums
+    f32x2 acc_s[NA], acc_q[NA], long_q[NA];
+    int opaque_zero = 0, held = 0;   // (an index that the compiler cannot see through keeps long_q out of the registers)
+    if constexpr (STATS) {
+        asm volatile("mov.u32 %0, 0;" : "=r"(opaque_zero));
+#pragma unroll
+        for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = long_q[i + opaque_zero] = 0ull;
+    }
+    int jacc = 0, cur_group = -1, cur_ktile = 0;
+    bool ok = true;
+    long long epi_wait = 0;
+
+    auto each_total = [&](auto emit) {   // emit(column of the warp, sum, sum of squares) in one lane per column
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            float2 s = split_f32x2(acc_s[i]), sq = split_f32x2(add_f32x2(acc_q[i], long_q[i + opaque_zero]));
+#pragma unroll
+            for (int bit = LPR; bit < 32; bit <<= 1) {
+                s.x += __shfl_xor_sync(0xffffffffu, s.x, bit);
+                s.y += __shfl_xor_sync(0xffffffffu, s.y, bit);
+                sq.x += __shfl_xor_sync(0xffffffffu, sq.x, bit);
+                sq.y += __shfl_xor_sync(0xffffffffu, sq.y, bit);
+            }
+            if (lane < LPR) {
+                const int col = (i >> 2) * BC + 8 * lane + 2 * (i & 3);
+                emit(col, s.x, sq.x);
+                emit(col + 1, s.y, sq.y);
+            }
+        }
+        __syncwarp();
+    };
+    auto flush_stats = [&](bool group_done) {
+        held = 0;
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            long_q[i + opaque_zero] = add_f32x2(long_q[i + opaque_zero], acc_q[i]);
+            acc_q[i] = 0ull;
+        }
+        if (group_done) {
+            double* st = p.stats + (size_t)cur_group * 2 * p.oc_valid + cur_ktile * p.n_tile + col_begin;
+            each_total([&](int col, float s, float sq) {
+                atomicAdd(st + col, (double)s);
+                atomicAdd(st + p.oc_valid + col, (double)sq);
+            });
+#pragma unroll
+            for (int i = 0; i < NA; ++i) acc_s[i] = long_q[i + opaque_zero] = 0ull;
+        }
+    };
+
+    const int m_lane = q * 32 + lane, lw = m_lane & (p.bw - 1);   // (merged taps: position in the image row)
+    const float m_left = lw != 0 ? 1.f : 0.f, m_right = lw != p.bw - 1 ? 1.f : 0.f;
+    // (the next unit's coordinates are worked out while the barrier is probed, as in epilogue_loop)
+    UnitCoord c_next = decode_unit(p, walk.unit(p, walk.first < walk.count ? walk.first : 0));
+    for (int pu = walk.first; pu < walk.count; pu += walk.stride) {
+        const UnitCoord c = c_next;
+        const int n_it = unit_iters(p, c.par);
+        int buf = 0;
+        uint32_t full_now = 0;
+        if (n_it > 0) {
+            buf = jacc & (p.acc_bufs - 1);
+            full_now = mbar_try_wait(&acc_full[buf], (uint32_t)(jacc >> p.acc_shift) & 1u) ? 1u : 0u;
+        }
+        if (pu + walk.stride < walk.count) c_next = decode_unit(p, walk.unit(p, pu + walk.stride));
+        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + ((long long)c.n0 * p.os_n + (long long)c.oh0 * p.os_h + (long long)c.ow0 * p.os_w +
+                             p.off[c.par] + c.ktile * p.n_tile + my_off);
+        const int images = p.n_valid - c.n0;   // (the second tile of a pair may lie past the last image)
+        const int rows = images >= p.bn ? 128 : images > 0 ? images * p.bw * p.bh : 0;
+        if (n_it > 0) {
+            if (!__all_sync(0xffffffffu, full_now != 0u)) {
+                const long long w3 = clock64();
+                ok = true;
+                if (lane == 0) ok = mbar_wait_bounded(&acc_full[buf], (uint32_t)(jacc >> p.acc_shift) & 1u, p.spin_limit, abort_flag);
+                epi_wait += clock64() - w3;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) {
+                    if (lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
+                    break;
+                }
+            }
+            tc_fence_after();
+            ++jacc;
+        }
+        const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * p.acc_cols + col_begin);
+        auto release = [&]() {
+            if (n_it > 0) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (remote_empty) mbar_arrive_cluster(map_to_cta(smem_u32(&acc_empty[buf]), 0));
+                    else mbar_arrive(&acc_empty[buf]);
+                }
+            }
+        };
+        uint32_t r[BC / 16][16];
+        auto fetch = [&](int b) {
+#pragma unroll
+            for (int ck = 0; ck < BC / 16; ++ck) tmem_ld16(t_row + (uint32_t)(b * BC + ck * 16), r[ck]);
+        };
+        if constexpr (HM) {   // (see epilogue_loop; one block)
+#pragma unroll
+            for (int ck = 0; ck < BC / 16; ++ck) {
+                uint32_t d0[16], d1[16], d2[16];
+                tmem_ld16(t_row + (uint32_t)(ck * 16), d0);
+                tmem_ld16(t_row + (uint32_t)(p.n_tile + ck * 16), d1);
+                tmem_ld16(t_row + (uint32_t)(2 * p.n_tile + ck * 16), d2);
+                tmem_ld_wait();
+                if (ck == BC / 16 - 1) release();
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const float left = __shfl_up_sync(0xffffffffu, __uint_as_float(d0[i]), 1);
+                    const float right = __shfl_down_sync(0xffffffffu, __uint_as_float(d2[i]), 1);
+                    r[ck][i] = __float_as_uint(fmaf(left, m_left, fmaf(right, m_right, __uint_as_float(d1[i]))));
+                }
+            }
+        } else if (n_it > 0) {
+            fetch(0);
+            tmem_ld_wait();
+            if (NB == 1) release();
+        } else {
+#pragma unroll
+            for (int ck = 0; ck < BC / 16; ++ck)
+#pragma unroll
+                for (int i = 0; i < 16; ++i) r[ck][i] = 0u;
+        }
+        if constexpr (STATS) {   // the previous units' sums
+            const int next_group = p.stats_group_images > 0 ? (p.grp_shift >= 0 ? c.n0 >> p.grp_shift : c.n0 / p.stats_group_images) : 0;
+            if (cur_group >= 0 && (next_group != cur_group || held == kFoldUnits / 2)) flush_stats(next_group != cur_group);
+            ++held;
+            cur_group = next_group;
+            cur_ktile = c.ktile;
+        }
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            __syncwarp();   // the previous block has been read
+#pragma unroll
+            for (int j = 0; j < BC / 8; ++j) {
+                uint32_t w[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int col = 8 * j + 2 * i;
+                    w[i] = pack_bf16x2(__uint_as_float(r[col / 16][col % 16]), __uint_as_float(r[col / 16][col % 16 + 1]));
+                }
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(st_w + 16u * (uint32_t)(j ^ sw_w)), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+            }
+            __syncwarp();
+            if (b + 1 < NB && n_it > 0) fetch(b + 1);   // comes in while this block goes out
+            constexpr int U = LPR < 4 ? LPR : 4;
+#pragma unroll
+            for (int i0 = 0; i0 < LPR; i0 += U) {
+                uint4 v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int row = lane / LPR + RPI * (i0 + u);
+                    const uint32_t at = smem_u32(stage) + (uint32_t)row * (BC * 2) + 16u * (uint32_t)((lane % LPR) ^ swizzle(row));
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[u].x), "=r"(v[u].y), "=r"(v[u].z), "=r"(v[u].w) : "r"(at) : "memory");
+                    if (my_row + RPI * (i0 + u) < rows) {
+                        int off = b * BC;
+#pragma unroll
+                        for (int t = 0; t < 5 - LOG_RPI; ++t)
+                            if (((i0 + u) >> t) & 1) off += step_off[t];
+                        *reinterpret_cast<uint4*>(out + off) = v[u];
+                    } else {
+                        v[u] = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                }
+                if constexpr (STATS) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        f32x2 f[U];
+#pragma unroll
+                        for (int u = 0; u < U; ++u) f[u] = widen_bf16x2(k == 0 ? v[u].x : k == 1 ? v[u].y : k == 2 ? v[u].z : v[u].w);
+                        f32x2 s = add_f32x2(f[0], f[1]), sq = fma_f32x2(f[1], f[1], mul_f32x2(f[0], f[0]));
+                        if constexpr (U == 4) {
+                            s = add_f32x2(s, add_f32x2(f[2], f[3]));
+                            sq = add_f32x2(sq, fma_f32x2(f[3], f[3], mul_f32x2(f[2], f[2])));
+                        }
+                        acc_s[4 * b + k] = add_f32x2(acc_s[4 * b + k], s);
+                        acc_q[4 * b + k] = add_f32x2(acc_q[4 * b + k], sq);
+                    }
+                }
+            }
+            if (b + 1 < NB && n_it > 0) {
+                tmem_ld_wait();
+                if (b + 2 == NB) release();
+            }
+        }
+    }
+    if constexpr (STATS) asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");   // (blocks may lie where the sums go)
+    if (STATS && cur_group >= 0 && ok)
+        each_total([&](int col, float s, float sq) {
+            my_stats[col] = s;
+            my_stats[128 + col] = sq;
+        });
+    if (p.stall != nullptr && e == 0 && lane == 0) atomicAdd(p.stall + 3, (unsigned long long)epi_wait);
+    return STATS && ok ? make_int2(cur_group, cur_ktile) : make_int2(-1, 0);
+}
+
 // Issues the MMAs of one stage: NB sub-tiles (vertical taps) x KS k-steps of 16 channels, fully unrolled so that
 // the issuing thread spends a handful of independent instructions per MMA (its own dependent-issue latency, not the
 // tensor pipe, bounds small-N tiles otherwise).  Descriptor low words advance by 32 bytes per k-step inside the
@@ -715,7 +945,8 @@ __device__ __forceinline__ void mma_issuer_split(const ConvKParams& p, const Uni
 // general (one MMA per tap or vertical tap reuse, any tile width up to 128 channels), split (tiles wider than 128 channels:
 // two issuing threads share every unit), merged horizontal taps, full-halo stages.
 enum : int { KIND_GENERAL = 0, KIND_SPLIT = 1, KIND_HMERGE = 2, KIND_FULL_HALO = 3 };
-template <bool PAIR, int KIND>
+// BLOCKS: with epilogue_blocks in place of epilogue_loop (p.block_cols).
+template <bool PAIR, int KIND, bool BLOCKS>
 __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_constant__ ConvKParams p)
 {
     const int rank = PAIR ? (int)cluster_ctarank() : 0;   // 0 = leader of the pair: issues the MMAs, owns the barriers the pair shares
@@ -725,7 +956,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
     __shared__ uint32_t abort_flag;
     __shared__ int slot_stage[kMaxStages];   // per ring slot: 1 + index of the stage whose loads were issued into it last
     __shared__ int2 s_last;   // statistics group and channel tile whose sums the epilogue warps left in s_stats
-    __shared__ float s_stats[kEpiWarps][256];   // per epilogue warp (128 columns at most): [0,128) sums, [128,256) sums of squares
+    __shared__ __align__(16) float s_stats[kEpiWarps][256];   // per epilogue warp (128 columns at most): [0,128) sums, [128,256) sums of squares
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023u) & ~uintptr_t(1023));
     uint8_t* ring = smem + p.resident_bytes;
@@ -982,7 +1213,21 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
 #define B2C_EPILOGUE(NCH, EAGER, HM)                                                                                                           \
     last = p.stats != nullptr ? epilogue_loop<NCH, EAGER, HM, true>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank) \
                               : epilogue_loop<NCH, EAGER, HM, false>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], e, lane, rank)
-        if constexpr (KIND == KIND_SPLIT) {   // tiles wider than 128 channels
+#define B2C_BLOCKS(BC, NB, HM)                                                                                                                            \
+    last = p.stats != nullptr ? epilogue_blocks<BC, NB, HM, true>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], stage, e, lane, rank) \
+                              : epilogue_blocks<BC, NB, HM, false>(p, tmem_base, acc_full, acc_empty, &abort_flag, s_stats[e], stage, e, lane, rank)
+        if constexpr (BLOCKS) {
+            // (s_stats, which is written once all epilogue warps are through with their blocks, has room for two blocks of 64 columns, or for the
+            // eight of 16)
+            uint8_t* spare = reinterpret_cast<uint8_t*>(s_stats);
+            uint8_t* behind = ring + (size_t)S * stage_bytes;
+            uint8_t* stage = p.block_cols == 16 ? spare + 1024 * e : p.block_cols == 32 ? behind + 2048 * e : e < 2 ? spare + 4096 * e : behind + 4096 * (e - 2);
+            if constexpr (KIND == KIND_SPLIT) B2C_BLOCKS(64, 2, false);
+            else if constexpr (KIND == KIND_HMERGE) B2C_BLOCKS(32, 1, true);
+            else if constexpr (KIND == KIND_FULL_HALO) B2C_BLOCKS(16, 4, false);
+            else if (p.n_tile == 64) B2C_BLOCKS(32, 1, false);
+            else B2C_BLOCKS(64, 1, false);
+        } else if constexpr (KIND == KIND_SPLIT) {   // tiles wider than 128 channels
             B2C_EPILOGUE(8, false, false);
         } else if constexpr (KIND == KIND_HMERGE) {
             B2C_EPILOGUE(2, true, true);
@@ -993,6 +1238,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kmajor_kernel(const __grid_c
             else B2C_EPILOGUE(8, false, false);   // (only with issue splitting switched off)
         }
 #undef B2C_EPILOGUE
+#undef B2C_BLOCKS
         if (e == 0 && lane == 0) s_last = last;
     }
     tc_fence_before();
@@ -1288,7 +1534,10 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
         p.tiles_w = 1; p.tiles_h = gh / p.bh; p.tiles_n = pb.n;
         p.total_units = p.tiles_n * p.tiles_h * p.n_ktiles;
         const int a_bytes = (p.bh + 2) * p.bw * 128;   // multiples of 1 KB for every row length used here
-        int stages = (ring_budget - bank) / a_bytes;
+        // Five slots and the blocks of the epilogue beat six slots (a data gradient of 50 images loses 0.5 us, but the forward pass gains, and a
+        // program that runs both loads one kernel less: a kernel that comes to the SMs from DRAM costs about 5 us)
+        int stages = (ring_budget - bank - 16 * 1024) / a_bytes;
+        if (stages < 3) stages = (ring_budget - bank) / a_bytes;
         if (stages > kMaxStages) stages = kMaxStages;
         if (stages >= 3) {
             p.hm = 1; p.fh = 0; p.vreuse = 0; p.pair = 0;
@@ -1397,8 +1646,20 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
         p.issue_split = 1;
     }
     const int stage_bytes = p.gsub * (p.a_bytes + (p.resident ? 0 : p.nb * p.b_bytes));
+    // Epilogue in blocks, where shared memory has room for them beside the ring (a shorter ring costs more than they give: 256 -> 1024 1x1 at
+    // 8x8 59 -> 64 us): tiles of 64 channels 32 columns at a time; 128 and 256 channels 64 at a time, full-halo stages, which leave no room,
+    // 16 at a time in the kernel's static arrays.  Tiles of 256 channels without sums whose MMAs take more than 12000 cycles hide the
+    // epilogue anyway and are 1 % slower in blocks (256 -> 256 at 8x8 59.7 and 60.1 us); the others gain, see epilogue_blocks.
+    if (!cluster && !pb.out_f32 && pb.bias == nullptr) {
+        const int room = ring_budget - p.resident_bytes - p.stages * stage_bytes;
+        const int mma = R * R * pb.ic / 16 / n_par * (n_tile / 2);
+        if (n_tile == 64 && !p.fh && room >= 16 * 1024) p.block_cols = 32;
+        if (n_tile == 128) p.block_cols = p.fh ? 16 : room >= 24 * 1024 ? 64 : 0;
+        if (n_tile == 256 && p.issue_split && room >= 24 * 1024 && (pb.stats != nullptr || mma < 12000)) p.block_cols = 64;
+    }
+    const int block_bytes = p.block_cols == 64 ? 24 * 1024 : p.block_cols == 32 ? 16 * 1024 : 0;
     size_t smem_bytes = (size_t)p.resident_bytes + (size_t)p.stages * stage_bytes + 1024 +
-                        (cluster && !p.x_overlap ? (size_t)(p.splits - 1) * (p.n_tile / p.splits) * 512 : 0);
+                        block_bytes + (cluster && !p.x_overlap ? (size_t)(p.splits - 1) * (p.n_tile / p.splits) * 512 : 0);
     // CTAs that wait for one another (pairs, and clusters that share a tile) take more than half of an SM's shared memory, so that no two of
     // them share an SM.  Their TMEM allocations wait for columns without a limit: two clusters of different streams (or three) that met on
     // several SMs could each hold the columns that the other one's partner waits for.
@@ -1463,6 +1724,10 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
                 p.off[ph * 2 + pw] = ((long long)ph * pb.ow + pw) * pb.oc;
             }
         p.os_n = (long long)pb.oh * pb.ow * pb.oc; p.os_h = 2ll * pb.ow * pb.oc; p.os_w = 2ll * pb.oc;
+    }
+    for (int i = 0; i < 7; ++i) {
+        const int v = 1 << i;
+        p.row_bit[i] = (int)(v < p.bw ? p.os_w * v : v < p.bw * p.bh ? p.os_h * (v / p.bw) : p.os_n * (v / (p.bw * p.bh)));
     }
     p.r_filter = R;
     p.n_valid = pb.n;
@@ -1529,15 +1794,20 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
     if (p.splits > 0) return launch_conv_splitk(ctx, p, grid, smem_bytes, stream);
     // the kernel kind of the plan (merged taps run on single CTAs only)
     typedef void (*kernel_t)(const ConvKParams);
-    static const kernel_t kernels[2][4] = {
-        {conv_kmajor_kernel<false, KIND_GENERAL>, conv_kmajor_kernel<false, KIND_SPLIT>, conv_kmajor_kernel<false, KIND_HMERGE>, conv_kmajor_kernel<false, KIND_FULL_HALO>},
-        {conv_kmajor_kernel<true, KIND_GENERAL>, conv_kmajor_kernel<true, KIND_SPLIT>, nullptr, conv_kmajor_kernel<true, KIND_FULL_HALO>}};
-    const kernel_t kernel = kernels[p.pair ? 1 : 0][kernel_kind(p)];
+    static const kernel_t kernels[2][2][4] = {
+        {{conv_kmajor_kernel<false, KIND_GENERAL, false>, conv_kmajor_kernel<false, KIND_SPLIT, false>, conv_kmajor_kernel<false, KIND_HMERGE, false>,
+          conv_kmajor_kernel<false, KIND_FULL_HALO, false>},
+         {conv_kmajor_kernel<true, KIND_GENERAL, false>, conv_kmajor_kernel<true, KIND_SPLIT, false>, nullptr, conv_kmajor_kernel<true, KIND_FULL_HALO, false>}},
+        {{conv_kmajor_kernel<false, KIND_GENERAL, true>, conv_kmajor_kernel<false, KIND_SPLIT, true>, conv_kmajor_kernel<false, KIND_HMERGE, true>,
+          conv_kmajor_kernel<false, KIND_FULL_HALO, true>},
+         {conv_kmajor_kernel<true, KIND_GENERAL, true>, conv_kmajor_kernel<true, KIND_SPLIT, true>, nullptr, conv_kmajor_kernel<true, KIND_FULL_HALO, true>}}};
+    const kernel_t kernel = kernels[p.block_cols ? 1 : 0][p.pair ? 1 : 0][kernel_kind(p)];
     if (kernel == nullptr) return B2C_ERR_UNSUPPORTED_SHAPE;
     if (!(ctx->smem_optin_done & B2C_OPTIN_KMAJOR)) {   // the attribute belongs to the device: kept per context, not per process
-        for (int a = 0; a < 2; ++a)
+        for (int a = 0; a < 4; ++a)
             for (int b = 0; b < 4; ++b)
-                if (kernels[a][b] != nullptr) B2C_CUDA(cudaFuncSetAttribute(kernels[a][b], cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
+                if (kernels[a >> 1][a & 1][b] != nullptr)
+                    B2C_CUDA(cudaFuncSetAttribute(kernels[a >> 1][a & 1][b], cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
         ctx->smem_optin_done |= B2C_OPTIN_KMAJOR;
     }
     B2C_CUDA(b2c_launch(ctx, kernel, dim3((unsigned)grid), dim3(kThreads), smem_bytes, stream, p.pair ? 2u : 1u, p));

@@ -38,10 +38,12 @@ struct alignas(64) ConvKParams {
     int splits;                      // split-K plans (conv_splitk.cu): CTAs (or CTA pairs) of a cluster that share a unit's k-blocks; 0: persistent kernel
     int x_off, x_overlap;            // split-K: byte offset of the exchange area behind the ring's start; it overlaps the ring
     int pair;                        // CTA pairs (cta_group::2): M = 256 per MMA, each CTA holds half of every B tile
+    int block_cols;                  // columns that an epilogue warp turns from a row per lane into rows of 16-byte vectors at a time (0: it does not)
     int resident;                    // filter bank of this CTA's channel tile stays in shared memory
     int resident_bytes;
     int n_valid, oc_valid;           // images / output channels that exist
     long long os_n, os_h, os_w;      // output element strides along the tile grid
+    int row_bit[7];                  // output elements between rows m and m + 2^i of a tile (its sides are powers of two: bits of m add up)
     long long off[4];                // output element offset per parity
     void* out;
     int out_is_f32;
