@@ -251,6 +251,7 @@ struct LayerPlan {
     long long run_off = -1;                                                // elements into the running-statistics array
     int src_slot = -1, res_slot = -1;                                     // which gradient buffer of src / res this layer writes
     int chunk_groups = 1;          // micro-batches of a pass this layer takes per launch (divides n_conc)
+    int bwd_bn = -1;               // BatchNorm layer whose backward sums this convolution's data gradient may take (it writes the last contribution)
     int seg_index = -1;            // position of this layer's filter bank among the weight layers (conv, fc)
 };
 
@@ -273,6 +274,7 @@ struct b2c_net {
     float *w = nullptr, *v = nullptr, *g = nullptr;
     char *w_bf16 = nullptr, *w_dgrad = nullptr, *ws = nullptr;
     bool fuse_stats = true;
+    std::vector<char> bwd_sums_done;   // per layer: the BatchNorm's backward sums came with a data gradient of this pass
     // optional per-launch timing (CUDA events on the step's stream), summed per kernel family
     bool profile = false;
     struct Span { cudaEvent_t a, b; int kind, layer, pass; };   // layer -1: not a layer's launch site; pass 0 forward, 1 parameter gradient, 2 data gradient
@@ -448,6 +450,19 @@ b2c_status b2c_net_create_concurrent(b2c_ctx* ctx, const b2c_layer_desc* layers,
             if (kind != B2C_LAYER_BN && kind != B2C_LAYER_XENT && net->tensors[i + 1].n_contrib != 1) return fail(B2C_ERR_UNSUPPORTED_SHAPE);
             if ((L.src_slot = add_contrib(L.d.src)) < 0) return fail(B2C_ERR_UNSUPPORTED_SHAPE);
             if (kind == B2C_LAYER_BN && L.d.res >= 0 && (L.res_slot = add_contrib(L.d.res)) < 0) return fail(B2C_ERR_UNSUPPORTED_SHAPE);
+        }
+    }
+    // The data gradient that a BatchNorm's output gradient is complete with: of the first layer that reads the output, if that is a convolution.
+    // B2C_FUSE_BN_BWD=0: the sums of the backward pass always take a pass of their own.
+    const char* bwd_env = std::getenv("B2C_FUSE_BN_BWD");
+    net->bwd_sums_done.assign(n_layers, 0);
+    for (int i = n_layers - 1; i >= 0 && !(bwd_env && bwd_env[0] == '0') && !ctx->use_bn_grouped; --i) {
+        if (net->layers[i].d.kind != B2C_LAYER_BN || net->tensors[net->layers[i].d.src].producer < 0 ||
+            net->layers[net->tensors[net->layers[i].d.src].producer].d.kind != B2C_LAYER_CONV) continue;   // (other inputs' sums are not cleared with the pass)
+        for (int k = i + 1; k < n_layers; ++k) {
+            if (net->layers[k].d.src != i + 1 && !(net->layers[k].d.kind == B2C_LAYER_BN && net->layers[k].d.res == i + 1)) continue;
+            if (net->layers[k].d.kind == B2C_LAYER_CONV) net->layers[k].bwd_bn = i;
+            break;
         }
     }
     // small per-layer buffers; the fp64 statistics are contiguous so that one launch clears them
@@ -806,13 +821,14 @@ b2c_status b2c_train_step(b2c_net* net, const void* images, const int32_t* label
                 }
                 case B2C_LAYER_BN: {
                     const TensorPlan& in = net->tensors[d.src];
-                    ProfScope ps_(net, stream, B2C_PROF_BN_BWD, 2, i, 2);
+                    const bool sums_done = net->bwd_sums_done[i] != 0;
+                    ProfScope ps_(net, stream, B2C_PROF_BN_BWD, sums_done ? 1 : 2, i, 2);
                     B2C_TRY(launch_bn_bwd(ctx, Gc, (long long)mbs * in.h * in.w, in.c, grad(i + 1, 0, img0),
                                           o.n_contrib > 1 ? grad(i + 1, 1, img0) : nullptr, act(d.src, img0), act(i + 1, img0), net->w + L.gamma_off,
                                           reinterpret_cast<float*>(net->ws + L.mean_off) + (size_t)g0 * in.c,
                                           reinterpret_cast<float*>(net->ws + L.invstd_off) + (size_t)g0 * in.c, d.relu, grad(d.src, L.src_slot, img0),
                                           d.res >= 0 ? grad(d.res, L.res_slot, img0) : nullptr, net->g + L.gamma_off, net->g + L.beta_off, 1,
-                                          reinterpret_cast<double*>(net->ws + L.bwd_ws_off) + (size_t)g0 * 2 * in.c, /*sums_zeroed=*/in.stats_off >= 0,
+                                          reinterpret_cast<double*>(net->ws + L.bwd_ws_off) + (size_t)g0 * 2 * in.c, sums_done, /*sums_zeroed=*/in.stats_off >= 0,
                                           L.mask_off >= 0 ? net->ws + L.mask_off + (long long)img0 * in.h * in.w * in.c / 8 : nullptr,
                                           ctx->use_bn_grouped ? reinterpret_cast<unsigned*>(net->ws + L.arrive_off) + g0 : nullptr, stream));
                     break;
@@ -839,8 +855,20 @@ b2c_status b2c_train_step(b2c_net* net, const void* images, const int32_t* label
                         // channels on 16x16, 16 images, 188.4 -> 164.9 us, ResNet-18-shaped 128 images 1384 -> 1361, 4 x 50 images 3965 -> 3854,
                         // 1024 images 5774 -> 5752; with the shortcuts' convolutions 163.2, 1356, 3846.
                         pb.no_wait = true;
+                        bool sums_done = false;
+                        if (L.bwd_bn >= 0) {   // (whether it takes them depends on the plan alone: the same for every run of a pass)
+                            const LayerPlan& B = net->layers[L.bwd_bn];
+                            const TensorPlan& t = net->tensors[d.src];
+                            pb.stats = reinterpret_cast<double*>(net->ws + B.bwd_ws_off) + (size_t)g0 * 2 * t.c;
+                            pb.stats_group_images = G > 1 ? mbs : 0;
+                            pb.bwd_y = act(B.d.src, img0);
+                            pb.bwd_other = t.n_contrib > 1 ? grad(d.src, 1 - L.src_slot, img0) : nullptr;
+                            pb.bwd_mask = B.mask_off >= 0 ? net->ws + B.mask_off + (long long)img0 * t.h * t.w * t.c / 8 : nullptr;
+                            pb.bwd_done = &sums_done;
+                        }
                         ProfScope ps_(net, stream, B2C_PROF_CONV_DGRAD, 1, i, 2);
                         B2C_TRY(launch_conv_kmajor(ctx, pb, stream));
+                        if (L.bwd_bn >= 0) net->bwd_sums_done[L.bwd_bn] = sums_done ? 1 : 0;
                     }
                     break;
                 }

@@ -141,6 +141,12 @@ struct KMajorProblem {
     const float* bias;
     double* stats;         // fp64 [groups][2*oc] or nullptr
     int stats_group_images;  // images per statistics group (0: one group)
+    // Data gradient whose output is the last contribution to the gradient of a BatchNorm(+ReLU) output: `stats` takes the sums of the BatchNorm's
+    // backward pass, sum dz and sum dz*y with dz = (out + bwd_other) where bwd_mask has a bit, else 0.  A plan that cannot ignores them.
+    const void* bwd_y;       // the BatchNorm's input (nullptr: no such sums)
+    const void* bwd_other;   // the other contribution, or nullptr
+    const void* bwd_mask;    // one bit per element, or nullptr
+    bool* bwd_done;          // set to whether the launch takes the sums
     bool no_wait;          // the launch right before this one shares nothing that is written with this one, and itself waits for the one before it:
                            // the kernel starts as SMs fall free and waits for that launch only at its end
 };
@@ -162,14 +168,14 @@ b2c_status plan_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, b2c_conv_plan& 
 // save_mean / save_invstd fp32 [G][c].  G > 1 requires acc != 0 in the backward pass.  stats_ready: 1 = `stats` holds the
 // sums already (convolution epilogue), 0 = clear and compute them, 2 = compute them into `stats` the caller has cleared.  relu_mask (optional): one bit per
 // element, "stored output > 0" (a byte per 8 channels), written by the forward pass and read by the backward pass
-// in place of the output tensor.  sums_zeroed: the caller has already cleared `sums` (and `arrivals`).  arrivals (optional): G
+// in place of the output tensor.  sums_ready: `sums` holds the sums already (a data gradient's epilogue).  sums_zeroed: the caller has already cleared `sums` (and `arrivals`).  arrivals (optional): G
 // zeroed counters; with them the two passes run in one cooperative launch, group by group (bn_bwd_grouped_kernel).
 b2c_status launch_bn_fwd(b2c_ctx* ctx, int G, long long m, int c, const void* y, double* stats, int stats_ready, const float* gamma,
                          const float* beta, const void* residual, int relu, float eps, void* a, float* save_mean, float* save_invstd,
                          float* run_mean, float* run_var, float momentum, void* relu_mask, cudaStream_t stream);
 b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da1, const void* da2, const void* y, const void* a,
                          const float* gamma, const float* save_mean, const float* save_invstd, int relu, void* dy, void* dres, float* dgamma,
-                         float* dbeta, int acc, double* sums, bool sums_zeroed, const void* relu_mask, unsigned* arrivals, cudaStream_t stream);
+                         float* dbeta, int acc, double* sums, bool sums_ready, bool sums_zeroed, const void* relu_mask, unsigned* arrivals, cudaStream_t stream);
 
 // Average + SGD-momentum update of `count` elements, gradient sums cleared, and both bf16 copies, in one launch.  The segments (filter banks)
 // lie back to back from element 0 and their sizes are multiples of 8; elements behind the last one have no data-gradient layout.

@@ -77,26 +77,6 @@ __device__ __forceinline__ int unit_stages(const ConvKParams& p, int par)
     return p.gsub > 1 ? (n + p.gsub - 1) / p.gsub : n;
 }
 
-// Column sums over the 32 rows a warp holds (one row per lane, 16 columns each): a butterfly that halves the
-// number of columns each lane carries (16 -> 8 -> 4 -> 2 -> 1).  On return lane l holds in a[0], b[0] the totals of
-// column (l >> 1) of the chunk.
-__device__ __forceinline__ void butterfly16(float (&a)[16], float (&b)[16], int lane)
-{
-#pragma unroll
-    for (int width = 8, bit = 16; width >= 1; width >>= 1, bit >>= 1) {
-        const bool upper = (lane & bit) != 0;
-#pragma unroll
-        for (int i = 0; i < width; ++i) {
-            const float sa = upper ? a[i] : a[i + width], ka = upper ? a[i + width] : a[i];
-            const float sb = upper ? b[i] : b[i + width], kb_ = upper ? b[i + width] : b[i];
-            a[i] = ka + __shfl_xor_sync(0xffffffffu, sa, bit);
-            b[i] = kb_ + __shfl_xor_sync(0xffffffffu, sb, bit);
-        }
-    }
-    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
-    b[0] += __shfl_xor_sync(0xffffffffu, b[0], 1);
-}
-
 // Epilogue of one warp over all units of the CTA, for the tile widths and plans that epilogue_blocks does not take.  Epilogue warp e reads the TMEM lane quarter its warp index selects and the column half e >> 2
 // of every accumulator.  The warp owns at most NCH 16-column chunks per unit.  EAGER: it reads all
 // its columns at once and hands the accumulator back before packing and storing (narrow tiles).
@@ -1651,11 +1631,12 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     // 16 at a time in the kernel's static arrays.  Tiles of 256 channels without sums whose MMAs take more than 12000 cycles hide the
     // epilogue anyway and are 1 % slower in blocks (256 -> 256 at 8x8 59.7 and 60.1 us); the others gain, see epilogue_blocks.
     if (!cluster && !pb.out_f32 && pb.bias == nullptr) {
+        const bool sums = pb.stats != nullptr && pb.bwd_y == nullptr;
         const int room = ring_budget - p.resident_bytes - p.stages * stage_bytes;
         const int mma = R * R * pb.ic / 16 / n_par * (n_tile / 2);
         if (n_tile == 64 && !p.fh && room >= 16 * 1024) p.block_cols = 32;
         if (n_tile == 128) p.block_cols = p.fh ? 16 : room >= 24 * 1024 ? 64 : 0;
-        if (n_tile == 256 && p.issue_split && room >= 24 * 1024 && (pb.stats != nullptr || mma < 12000)) p.block_cols = 64;
+        if (n_tile == 256 && p.issue_split && room >= 24 * 1024 && (sums || mma < 12000)) p.block_cols = 64;
     }
     const int block_bytes = p.block_cols == 64 ? 24 * 1024 : p.block_cols == 32 ? 16 * 1024 : 0;
     size_t smem_bytes = (size_t)p.resident_bytes + (size_t)p.stages * stage_bytes + 1024 +
@@ -1743,6 +1724,9 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     p.nk_shift = log2_exact(p.n_ktiles);
     p.grp_shift = log2_exact(p.stats_group_images);
     p.cb_shift = log2_exact(p.c_blocks);
+    // Sums of a BatchNorm's backward pass: the one-wave kernel only, whose layers are bound by launches.  In the persistent kernel the other
+    // operands' latency comes once per unit: 64 -> 64 3x3 with 1024 images 66 -> 140 us for 45 us less in the BatchNorm.
+    if (pb.bwd_y != nullptr && (!cluster || (p.stats_group_images > 0 && p.stats_group_images % p.bn != 0))) p.stats = nullptr;
     if (p.stats && p.stats_group_images > 0 && (p.stats_group_images % p.bn) != 0) return B2C_ERR_UNSUPPORTED_SHAPE;  // a tile must not straddle groups
     return B2C_OK;
 }
@@ -1769,7 +1753,7 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
     // plans are keyed by everything the planner reads: the problem and the context's switches
     const int switches = ctx->use_pairs | ctx->use_full_halo << 4 | ctx->use_issue_split << 5 | ctx->use_hmerge << 6 | ctx->use_group_kblocks << 7 | ctx->use_split_k << 8;
     const b2c_plan_key key = {{b2c_key_pair('K', switches), b2c_key_pair(pb.n, pb.stats_group_images), b2c_key_pair(pb.ih, pb.iw), b2c_key_pair(pb.oh, pb.ow),
-                               b2c_key_pair(pb.ic, pb.oc), b2c_key_pair(pb.r, pb.stride), b2c_key_pair(pb.pad, pb.dgrad | pb.out_f32 << 1), b2c_key_ptr(pb.in),
+                               b2c_key_pair(pb.ic, pb.oc), b2c_key_pair(pb.r, pb.stride), b2c_key_pair(pb.pad, pb.dgrad | pb.out_f32 << 1 | (pb.bwd_y != nullptr) << 2), b2c_key_ptr(pb.in),
                                b2c_key_ptr(pb.wt), b2c_key_ptr(pb.out), b2c_key_ptr(pb.bias), b2c_key_ptr(pb.stats)}};
     auto it = ctx->plan_cache.find(key);
     if (it == ctx->plan_cache.end()) {
@@ -1787,6 +1771,11 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
     const int grid = plan.grid;
     const size_t smem_bytes = plan.smem_bytes;
     p.no_wait = pb.no_wait ? 1 : 0;
+    const bool bwd = pb.bwd_y != nullptr && p.stats != nullptr;
+    p.bwd_y = bwd ? pb.bwd_y : nullptr;
+    p.bwd_other = pb.bwd_other;
+    p.bwd_mask = reinterpret_cast<const uint8_t*>(pb.bwd_mask);
+    if (pb.bwd_done != nullptr) *pb.bwd_done = bwd;
     p.status = ctx->d_status;
     p.spin_limit = ctx->spin_limit;
     p.stall = ctx->stall_counters;

@@ -51,6 +51,8 @@ struct alignas(64) ConvKParams {
     const float* bias;
     double* stats;
     int stats_group_images;          // images per BatchNorm statistics group (0: one group)
+    const void *bwd_y, *bwd_other;   // sums of a BatchNorm's backward pass in place of those of the output (see KMajorProblem)
+    const uint8_t* bwd_mask;
     int no_wait;                     // starts beside the previous launch of the stream, see pdl_begin
     unsigned* status;
     unsigned spin_limit;
@@ -162,6 +164,46 @@ __device__ __forceinline__ float2 column_total(f32x2 v)
     return f;
 }
 __device__ __forceinline__ int column_of(int lane) { return (lane & 24) >> 1; }   // first of a lane's four columns; lanes with (l & 7) == 0 speak for them
+
+// Column sums over the 32 rows a warp holds (one row per lane, 16 columns each): a butterfly that halves the
+// number of columns each lane carries (16 -> 8 -> 4 -> 2 -> 1).  On return lane l holds in a[0], b[0] the totals of
+// column (l >> 1) of the chunk.
+__device__ __forceinline__ void butterfly16(float (&a)[16], float (&b)[16], int lane)
+{
+#pragma unroll
+    for (int width = 8, bit = 16; width >= 1; width >>= 1, bit >>= 1) {
+        const bool upper = (lane & bit) != 0;
+#pragma unroll
+        for (int i = 0; i < width; ++i) {
+            const float sa = upper ? a[i] : a[i + width], ka = upper ? a[i + width] : a[i];
+            const float sb = upper ? b[i] : b[i + width], kb_ = upper ? b[i + width] : b[i];
+            a[i] = ka + __shfl_xor_sync(0xffffffffu, sa, bit);
+            b[i] = kb_ + __shfl_xor_sync(0xffffffffu, sb, bit);
+        }
+    }
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+    b[0] += __shfl_xor_sync(0xffffffffu, b[0], 1);
+}
+
+// What the sums of a BatchNorm's backward pass need of 8 neighbouring elements.  The loads pass the L1 by: a launch that starts beside the one
+// before it (no_wait) may find lines there that are older than its operands.
+struct BwdVec {
+    uint4 y, other;
+    unsigned mask;
+};
+__device__ __forceinline__ void bwd_load(const ConvKParams& p, long long element, BwdVec& v)
+{
+    v.y = __ldcg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.bwd_y) + element));
+    v.other = p.bwd_other != nullptr ? __ldcg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.bwd_other) + element)) : make_uint4(0u, 0u, 0u, 0u);
+    v.mask = p.bwd_mask != nullptr ? (unsigned)__ldcg(p.bwd_mask + (element >> 3)) : 0xffu;
+}
+// dz of columns 2 k and 2 k + 1 of such a vector, from the packed pair that the convolution stores there.
+__device__ __forceinline__ f32x2 bwd_pair(uint32_t stored, uint32_t other, unsigned mask, int k)
+{
+    const float2 f = split_f32x2(add_f32x2(widen_bf16x2(stored), widen_bf16x2(other)));
+    return make_f32x2((mask >> (2 * k)) & 1u ? f.x : 0.f, (mask >> (2 * k + 1)) & 1u ? f.y : 0.f);
+}
+__device__ __forceinline__ uint32_t word_of(const uint4& v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
 
 // Clusters of `cluster` CTAs (pair: made of CTA pairs) that run at the same time on this context's device.
 int splitk_max_clusters(b2c_ctx* ctx, int cluster, bool pair);

@@ -82,7 +82,10 @@ __device__ __forceinline__ float column_sums(const uint32_t (&pk)[8], float* sta
 
 // TIMED: the instance that adds to the stall counters (read at run time, they cost the small net of tests and benchmarks 2.5 % of
 // its step: 198 -> 203 us)
-template <bool PAIR, bool TIMED>
+// BWD: the instance that takes the sums of a BatchNorm's backward pass (p.bwd_y), with shuffles: its products are fp32.  A launch of 6-8 us that
+// reads the gradient again is replaced by 2-4 us in this one (the first operands come in while the accumulator is waited for).  Steps: two
+// blocks of 64 and 128 channels on 16x16, 16 images, 162.4 -> 148.5 us, ResNet-18-shaped 128 images 1327 -> 1309, 4 x 50 images 3786 -> 3679.
+template <bool PAIR, bool TIMED, bool BWD>
 __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid_constant__ ConvKParams p)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -217,6 +220,27 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     }
 
     // ---------------------------------------------------------------- epilogue: all eight warps
+    const int q = warp & 3, half = warp >> 2;   // TMEM lane quarter of this warp, half of the columns
+    const int m = q * 32 + lane;                // accumulator row = pixel of the tile (w fastest, then h, then image)
+    const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
+    const int sw = p.n_tile / p.splits;         // columns this CTA finishes
+    const int col0 = split * sw;
+    const int lw = m % p.bw, lh = (m / p.bw) % p.bh, ln = m / (p.bw * p.bh);
+    const bool row_valid = c.n0 + ln < p.n_valid;
+    const long long row_off = (long long)(c.n0 + ln) * p.os_n + (long long)(c.oh0 + lh) * p.os_h + (long long)(c.ow0 + lw) * p.os_w + p.off[c.par];
+    // 16 columns at a time (the last step of an odd count of eights takes 8)
+    const int n16 = (sw + 15) >> 4, g_lo = half ? (n16 + 1) >> 1 : 0, g_hi = half ? n16 : (n16 + 1) >> 1;
+    // what the sums of a BatchNorm's backward pass need beside the output: read a step ahead, the first step's before the accumulator is waited for
+    BwdVec in[2];
+    auto load_bwd = [&](int g) {
+        const long long at = row_off + c.ktile * p.n_tile + col0 + g * 16;
+        in[0] = in[1] = BwdVec{make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u), 0u};
+        if (row_valid) {
+            bwd_load(p, at, in[0]);
+            if (g * 16 + 16 <= sw) bwd_load(p, at + 8, in[1]);
+        }
+    };
+    if (BWD && g_lo < g_hi) load_bwd(g_lo);
     const long long t_wait = TIMED ? clock64() : 0;
     if (n_slots > 0 && !mbar_wait_warp(&acc_bar, 0u, p.spin_limit, &abort_flag) && lane == 0) atomicOr(p.status, B2C_DEV_TIMEOUT);
     if (TIMED && rank == 0 && warp == 2 && lane == 0) atomicAdd(p.stall + 3, (unsigned long long)(clock64() - t_wait));
@@ -243,11 +267,6 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     }
     tc_fence_after();
 
-    const int q = warp & 3, half = warp >> 2;   // TMEM lane quarter of this warp, half of the columns
-    const int m = q * 32 + lane;                // accumulator row = pixel of the tile (w fastest, then h, then image)
-    const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
-    const int sw = p.n_tile / p.splits;         // columns this CTA finishes
-    const int col0 = split * sw;
     const bool exchange = p.splits > 1 && k_total > 0;
     if (exchange) {
         // partial sums of the other CTAs' columns -> their exchange areas: block (sender, four columns) = 128 rows x 16 bytes; the next columns
@@ -289,12 +308,7 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
     }
     if (clustered) cluster_sync_all();   // the partial sums have arrived; nobody reads or writes another CTA's memory after this
 
-    const int lw = m % p.bw, lh = (m / p.bw) % p.bh, ln = m / (p.bw * p.bh);
-    const bool row_valid = c.n0 + ln < p.n_valid;
-    const long long row_off = (long long)(c.n0 + ln) * p.os_n + (long long)(c.oh0 + lh) * p.os_h + (long long)(c.ow0 + lw) * p.os_w + p.off[c.par];
     const bool do_stats = p.stats != nullptr;
-    // 16 columns at a time (the last step of an odd count of eights takes 8)
-    const int n16 = (sw + 15) >> 4, g_lo = half ? (n16 + 1) >> 1 : 0, g_hi = half ? n16 : (n16 + 1) >> 1;
     auto fetch = [&](uint32_t (&r)[16], int g) {
         uint32_t lo[8], hi[8];
         tmem_ld8(t_row + (uint32_t)(col0 + g * 16), lo);
@@ -368,7 +382,26 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
 #pragma unroll
                 for (int i = 0; i < 8; ++i) pk[i] = 0u;
             }
-            s_sum[q][total_is_square(lane)][g * 16 + column_of_total(lane)] = column_sums(pk, s_stage[warp], lane);
+            if constexpr (BWD) {
+                float a[16], b[16];   // dz and dz * y of this row
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const f32x2 dz = bwd_pair(pk[4 * h + k], word_of(in[h].other, k), in[h].mask, k);
+                        const float2 s = split_f32x2(dz), sy = split_f32x2(mul_f32x2(dz, widen_bf16x2(word_of(in[h].y, k))));
+                        a[8 * h + 2 * k] = s.x; a[8 * h + 2 * k + 1] = s.y;
+                        b[8 * h + 2 * k] = sy.x; b[8 * h + 2 * k + 1] = sy.y;
+                    }
+                if (g + 1 < g_hi) load_bwd(g + 1);
+                butterfly16(a, b, lane);
+                if ((lane & 1) == 0) {
+                    s_sum[q][0][g * 16 + (lane >> 1)] = a[0];
+                    s_sum[q][1][g * 16 + (lane >> 1)] = b[0];
+                }
+            } else {
+                s_sum[q][total_is_square(lane)][g * 16 + column_of_total(lane)] = column_sums(pk, s_stage[warp], lane);
+            }
             __syncwarp();
         }
     }
@@ -402,7 +435,8 @@ __global__ void __launch_bounds__(kSkThreads, 1) conv_splitk_kernel(const __grid
 static b2c_status splitk_optin(b2c_ctx* ctx)
 {
     if (!(ctx->smem_optin_done & B2C_OPTIN_SPLITK)) {
-        for (auto* k : {conv_splitk_kernel<false, false>, conv_splitk_kernel<false, true>, conv_splitk_kernel<true, false>, conv_splitk_kernel<true, true>})
+        for (auto* k : {conv_splitk_kernel<false, false, false>, conv_splitk_kernel<false, true, false>, conv_splitk_kernel<true, false, false>, conv_splitk_kernel<true, true, false>,
+                        conv_splitk_kernel<false, false, true>, conv_splitk_kernel<true, false, true>})
             B2C_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024));
         ctx->smem_optin_done |= B2C_OPTIN_SPLITK;
     }
@@ -427,7 +461,7 @@ int splitk_max_clusters(b2c_ctx* ctx, int cluster, bool pair)
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, pair ? conv_splitk_kernel<true, false> : conv_splitk_kernel<false, false>, &cfg) == cudaSuccess) known = n;
+        if (cudaOccupancyMaxActiveClusters(&n, pair ? conv_splitk_kernel<true, false, false> : conv_splitk_kernel<false, false, false>, &cfg) == cudaSuccess) known = n;
     }
     return known;
 }
@@ -438,8 +472,9 @@ b2c_status launch_conv_splitk(b2c_ctx* ctx, const ConvKParams& p, int grid, size
     if (st != B2C_OK) return st;
     const unsigned cluster = (unsigned)(p.splits * (p.pair ? 2 : 1));
     const bool timed = p.stall != nullptr;
-    auto* kernel = p.pair ? (timed ? conv_splitk_kernel<true, true> : conv_splitk_kernel<true, false>)
-                          : (timed ? conv_splitk_kernel<false, true> : conv_splitk_kernel<false, false>);
+    auto* kernel = p.bwd_y != nullptr ? (p.pair ? conv_splitk_kernel<true, false, true> : conv_splitk_kernel<false, false, true>)
+                   : p.pair           ? (timed ? conv_splitk_kernel<true, true, false> : conv_splitk_kernel<true, false, false>)
+                                      : (timed ? conv_splitk_kernel<false, true, false> : conv_splitk_kernel<false, false, false>);
     B2C_CUDA(b2c_launch(ctx, kernel, dim3((unsigned)grid), dim3(kSkThreads), smem_bytes, stream, cluster, p));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;

@@ -1482,18 +1482,18 @@ b2c_status launch_update_pack(b2c_ctx* ctx, const b2c_weight_seg* segs, int n_se
 
 b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da1, const void* da2, const void* y, const void* a,
                          const float* gamma, const float* save_mean, const float* save_invstd, int relu, void* dy, void* dres, float* dgamma,
-                         float* dbeta, int acc, double* sums, bool sums_zeroed, const void* relu_mask, unsigned* arrivals, cudaStream_t stream)
+                         float* dbeta, int acc, double* sums, bool sums_ready, bool sums_zeroed, const void* relu_mask, unsigned* arrivals, cudaStream_t stream)
 {
     const int rows_per_iter = kEwThreads / (c / 8);
     dim3 grid((unsigned)ew_grid(ctx, G, m, rows_per_iter), (unsigned)G);
     const uint8_t* mask = relu ? reinterpret_cast<const uint8_t*>(relu_mask) : nullptr;
-    if (!sums_zeroed) {
+    if (!sums_ready && !sums_zeroed) {
         b2c_status st = launch_zero(ctx, sums, sizeof(double) * 2 * c * G, nullptr, stream);
         if (st != B2C_OK) return st;
         if (arrivals != nullptr) B2C_CUDA(cudaMemsetAsync(arrivals, 0, sizeof(unsigned) * G, stream));
     }
     // Both passes in one cooperative launch, group by group (the apply pass of a group re-reads its tensors from L2).
-    if (arrivals != nullptr) {
+    if (arrivals != nullptr && !sums_ready) {
         // Stage size (vectors per thread and tensor) and ring depth: as many stages as fit, four at most.
         const int groups = c / 8, active = rows_per_iter * groups;
         const int nt = da2 != nullptr ? 3 : 2;
@@ -1564,14 +1564,14 @@ b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da
                 B2C_CUDA(cudaFuncSetAttribute(bn_bwd_apply_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024));
                 ctx->smem_optin_done |= B2C_OPTIN_BN_BWD;
             }
-            B2C_CUDA(b2c_launch(ctx, bn_bwd_reduce_staged_kernel, reduce_grid(grid, 2.0 * nt * m * c), dim3(kStThreads), smem, stream, 1u, da1, da2, y, m, c, relu, sums, mask, ctx->spin_limit, ctx->d_status));
+            if (!sums_ready) B2C_CUDA(b2c_launch(ctx, bn_bwd_reduce_staged_kernel, reduce_grid(grid, 2.0 * nt * m * c), dim3(kStThreads), smem, stream, 1u, da1, da2, y, m, c, relu, sums, mask, ctx->spin_limit, ctx->d_status));
             B2C_CUDA(b2c_launch(ctx, bn_bwd_apply_staged_kernel, dim3(grid), dim3(kStThreads), smem, stream, 1u, da1, da2, y, m, c, gamma, save_mean, save_invstd, relu, sums, dy, dres,
                                                                             dgamma, dbeta, acc, mask, ctx->spin_limit, ctx->d_status));
             B2C_CUDA(cudaGetLastError());
             return B2C_OK;
         }
     }
-    B2C_CUDA(b2c_launch(ctx, bn_bwd_reduce_kernel, reduce_grid(grid, (da2 != nullptr ? 6.0 : 4.0) * m * c), dim3(kEwThreads), 0, stream, 1u, da1, da2, y, a, m, c, relu, sums, mask));
+    if (!sums_ready) B2C_CUDA(b2c_launch(ctx, bn_bwd_reduce_kernel, reduce_grid(grid, (da2 != nullptr ? 6.0 : 4.0) * m * c), dim3(kEwThreads), 0, stream, 1u, da1, da2, y, a, m, c, relu, sums, mask));
     B2C_CUDA(b2c_launch(ctx, bn_bwd_apply_kernel, dim3(grid), dim3(kEwThreads), 0, stream, 1u, da1, da2, y, a, m, c, gamma, save_mean, save_invstd, relu, sums, dy, dres, dgamma, dbeta,
                                                          acc, mask));
     B2C_CUDA(cudaGetLastError());
@@ -1613,7 +1613,7 @@ b2c_status b2c_bn_relu_bwd(b2c_ctx* ctx, int n, int h, int w, int c, const void*
         (dres && !b2c_aligned16(dres)) || (reinterpret_cast<uintptr_t>(ws) & 7u))
         return B2C_ERR_MISALIGNED;
     return launch_bn_bwd(ctx, 1, (long long)n * h * w, c, da1, da2, y, a, gamma, save_mean, save_invstd, relu, dy, dres, dgamma, dbeta, acc,
-                         reinterpret_cast<double*>(ws), false, relu_mask, nullptr, stream);
+                         reinterpret_cast<double*>(ws), false, false, relu_mask, nullptr, stream);
 }
 
 size_t b2c_bn_relu_bwd_groups_workspace_bytes(int c, int groups)
@@ -1643,7 +1643,7 @@ b2c_status b2c_bn_relu_bwd_groups(b2c_ctx* ctx, int groups, long long rows_per_g
         B2C_CUDA(cudaMemsetAsync(dbeta, 0, sizeof(float) * c, stream));
     }
     return launch_bn_bwd(ctx, groups, rows_per_group, c, da1, da2, y, nullptr, gamma, save_mean, save_invstd, relu, dy, dres, dgamma, dbeta,
-                         groups > 1 ? 1 : acc, sums, true, relu_mask, arrivals, stream);
+                         groups > 1 ? 1 : acc, sums, false, true, relu_mask, arrivals, stream);
 }
 
 b2c_status b2c_avgpool_fwd(b2c_ctx* ctx, int n, int hw, int c, const void* a, void* pooled, void* stream_)
@@ -1812,7 +1812,7 @@ b2c_status b2c_bn_relu_bwd_static(b2c_ctx* ctx, int n, int h, int w, int c, cons
     }
     // the array keeps the previous call's sums: the launcher clears the part this call uses
     return launch_bn_bwd(ctx, 1, (long long)n * h * w, c, da1, da2, y, a, gamma, save_mean, save_invstd, relu, dy, dres, dgamma, dbeta, acc,
-                         g_bn_bwd_static_ptr[current], false, nullptr, nullptr, stream);
+                         g_bn_bwd_static_ptr[current], false, false, nullptr, nullptr, stream);
 }
 
 }  // extern "C"
