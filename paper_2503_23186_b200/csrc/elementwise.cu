@@ -149,10 +149,22 @@ __device__ __forceinline__ void bn_moments(const double* stats, int c, int ch, d
     invstd = rsqrtf((float)v + eps);
 }
 
+__device__ __forceinline__ void load8(const float* src, float (&f)[8])   // 16-byte aligned
+{
+    const float4 a = reinterpret_cast<const float4*>(src)[0], b = reinterpret_cast<const float4*>(src)[1];
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
+    f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+}
+
+// A block works the coefficients of its channels out once, into shared memory: with each thread reading the fp64 sums of its own 8 channels the
+// loads of a warp touched 16 lines each and the rows of threads repeated each other's fp64 work, which is what the kernel took on small tensors.
+// (The reciprocal of the row count comes from the host, an fp64 division less.)  One launch behind the other: forward 50 images at 4x4
+// with 512 channels 5.2 -> 2.9 us, 128 at 16x16 with 128 channels 6.5 -> 4.6, 128 at 32x32 with 256 channels 27.7 -> 26.2; both passes of the
+// backward 10.3 -> 7.3, 15.8 -> 13.4 and 59.1 -> 55.4.
 // UNROLL independent 16-byte loads per tensor and thread are in flight: without a residual the kernel reads one tensor,
 // so it takes twice the rows per step to keep as many bytes in flight as the residual variant (HBM latency x bandwidth).
 template <int UNROLL, bool RES>
-__global__ void __launch_bounds__(kEwThreads, 2) bn_apply_kernel(const void* __restrict__ y, long long m, int c, const double* __restrict__ stats_all,
+__global__ void __launch_bounds__(kEwThreads, 2) bn_apply_kernel(const void* __restrict__ y, long long m, double inv_m, int c, const double* __restrict__ stats_all,
                                                                  const float* __restrict__ gamma, const float* __restrict__ beta,
                                                                  const void* __restrict__ residual, int relu, float eps, void* __restrict__ a,
                                                                  float* save_mean, float* save_invstd, float* run_mean, float* run_var,
@@ -160,15 +172,20 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_apply_kernel(const void* __r
 {
     pdl_wait();   // first global access comes after the previous kernel of the stream
     pdl_launch_dependents();
+    extern __shared__ __align__(16) float coef[];   // [3][c]: gamma*invstd, mean, beta
     const RowWalk rw(c);
     const int g = threadIdx.x % rw.groups, rl = threadIdx.x / rw.groups;
-    const double inv_m = 1.0 / (double)m;
-    const double* stats = stats_all + (size_t)blockIdx.y * 2 * c;
     const long long base = (long long)blockIdx.y * m * rw.groups;
-    if (blockIdx.x == 0) {
-        for (int ch = threadIdx.x; ch < c; ch += kEwThreads) {
-            float mean, invstd, var;
-            bn_moments(stats, c, ch, inv_m, eps, mean, invstd, var);
+    const double* stats = stats_all + (size_t)blockIdx.y * 2 * c;
+#pragma unroll 4
+    for (int ch = threadIdx.x; ch < c; ch += kEwThreads) {
+        float mean, invstd, var;
+        bn_moments(stats, c, ch, inv_m, eps, mean, invstd, var);
+        // z = gamma*(y-mean)*invstd + beta, evaluated as (y-mean)*(gamma*invstd) + beta
+        coef[ch] = gamma[ch] * invstd;
+        coef[c + ch] = mean;
+        coef[2 * c + ch] = beta[ch];
+        if (blockIdx.x == 0) {
             save_mean[(size_t)blockIdx.y * c + ch] = mean;
             save_invstd[(size_t)blockIdx.y * c + ch] = invstd;
             if (run_mean != nullptr) {
@@ -178,17 +195,12 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_apply_kernel(const void* __r
             }
         }
     }
+    __syncthreads();
     if (rl >= rw.rows_per_iter) return;
     float scale[8], shift[8], bt[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        float mean, invstd, var;
-        bn_moments(stats, c, g * 8 + i, inv_m, eps, mean, invstd, var);
-        // z = gamma*(y-mean)*invstd + beta, evaluated as (y-mean)*(gamma*invstd) + beta
-        scale[i] = gamma[g * 8 + i] * invstd;
-        shift[i] = mean;
-        bt[i] = beta[g * 8 + i];
-    }
+    load8(coef + 8 * g, scale);
+    load8(coef + c + 8 * g, shift);
+    load8(coef + 2 * c + 8 * g, bt);
     const long long step = (long long)gridDim.x * rw.rows_per_iter;
     for (long long r = (long long)blockIdx.x * rw.rows_per_iter + rl; r < m; r += UNROLL * step) {
         uint4 vy[UNROLL], vr[RES ? UNROLL : 1];
@@ -293,9 +305,35 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_bwd_reduce_kernel(const void
     block_reduce(slots, c, rw.groups, sb, sg, rl < rw.rows_per_iter, sums_all + (size_t)blockIdx.y * 2 * c);
 }
 
-// Pass 2: dy = gamma*invstd*(dz - dbeta/m - xhat*dgamma/m), dres = dz; block 0 of each group emits dgamma, dbeta.
+// Coefficients of pass 2 for all channels, by the first kEwThreads threads of a block into shared memory ([4][c]: mean, gamma*invstd, dbeta/m and
+// (dgamma/m)*invstd, which multiplies y - mean), as in bn_apply_kernel; block 0 of each group emits dgamma, dbeta.
+__device__ __forceinline__ void bn_bwd_coefficients(float* __restrict__ coef, const double* __restrict__ sums, const float* __restrict__ mean, const float* __restrict__ invstd,
+                                                    const float* __restrict__ gamma, int c, double inv_m, int acc, float* __restrict__ dgamma, float* __restrict__ dbeta)
+{
+#pragma unroll 4
+    for (int ch = threadIdx.x; ch < c; ch += kEwThreads) {
+        const double s1 = sums[ch], s2 = sums[c + ch];
+        const double is = (double)invstd[ch], dgam = is * (s2 - (double)mean[ch] * s1);
+        coef[ch] = mean[ch];
+        coef[c + ch] = gamma[ch] * invstd[ch];
+        coef[2 * c + ch] = (float)(s1 * inv_m);
+        coef[3 * c + ch] = (float)(dgam * inv_m * is);
+        if (blockIdx.x == 0) {
+            const float db = (float)s1, dg = (float)dgam;
+            if (gridDim.y == 1) {
+                dbeta[ch] = acc ? dbeta[ch] + db : db;
+                dgamma[ch] = acc ? dgamma[ch] + dg : dg;
+            } else {   // several groups add into the same gradient (always accumulating)
+                atomicAdd(dbeta + ch, db);
+                atomicAdd(dgamma + ch, dg);
+            }
+        }
+    }
+}
+
+// Pass 2: dy = gamma*invstd*(dz - dbeta/m - xhat*dgamma/m), dres = dz.
 __global__ void __launch_bounds__(kEwThreads, 2) bn_bwd_apply_kernel(const void* __restrict__ da1, const void* __restrict__ da2,
-                                                                     const void* __restrict__ y, const void* __restrict__ a, long long m, int c,
+                                                                     const void* __restrict__ y, const void* __restrict__ a, long long m, double inv_m, int c,
                                                                      const float* __restrict__ gamma, const float* __restrict__ mean_all,
                                                                      const float* __restrict__ invstd_all, int relu,
                                                                      const double* __restrict__ sums_all, void* __restrict__ dy,
@@ -310,32 +348,15 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_bwd_apply_kernel(const void*
     const float* mean = mean_all + (size_t)blockIdx.y * c;
     const float* invstd = invstd_all + (size_t)blockIdx.y * c;
     const long long base = (long long)blockIdx.y * m * rw.groups;
-    if (blockIdx.x == 0) {
-        for (int ch = threadIdx.x; ch < c; ch += kEwThreads) {
-            const double s1 = sums[ch], s2 = sums[c + ch];
-            const float db = (float)s1, dg = (float)((double)invstd[ch] * (s2 - (double)mean[ch] * s1));
-            if (gridDim.y == 1) {
-                dbeta[ch] = acc ? dbeta[ch] + db : db;
-                dgamma[ch] = acc ? dgamma[ch] + dg : dg;
-            } else {   // several groups add into the same gradient (always accumulating)
-                atomicAdd(dbeta + ch, db);
-                atomicAdd(dgamma + ch, dg);
-            }
-        }
-    }
+    extern __shared__ __align__(16) float coef[];
+    bn_bwd_coefficients(coef, sums, mean, invstd, gamma, c, inv_m, acc, dgamma, dbeta);
+    __syncthreads();
     if (rl >= rw.rows_per_iter) return;
-    const double inv_m = 1.0 / (double)m;
     float mu[8], k0[8], kb[8], kg[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int ch = g * 8 + i;
-        const double s1 = sums[ch], s2 = sums[c + ch];
-        const double is = (double)invstd[ch], dgam = is * (s2 - (double)mean[ch] * s1);
-        mu[i] = mean[ch];
-        k0[i] = gamma[ch] * invstd[ch];                        // gamma*invstd
-        kb[i] = (float)(s1 * inv_m);                           // dbeta/m
-        kg[i] = (float)(dgam * inv_m * is);                    // (dgamma/m)*invstd, multiplies (y-mean)
-    }
+    load8(coef + 8 * g, mu);
+    load8(coef + c + 8 * g, k0);
+    load8(coef + 2 * c + 8 * g, kb);
+    load8(coef + 3 * c + 8 * g, kg);
     const long long step = (long long)gridDim.x * rw.rows_per_iter;
     constexpr int U = 2;
     for (long long r = (long long)blockIdx.x * rw.rows_per_iter + rl; r < m; r += U * step) {
@@ -391,6 +412,7 @@ __global__ void __launch_bounds__(kEwThreads, 2) bn_bwd_apply_kernel(const void*
 //   chunk = 2 * rows_per_iter rows = 2 vectors per active thread and tensor (about 8 KB per tensor); chunk k of a group
 //   goes to block k % gridDim.x; a ragged last chunk is read with plain loads.
 static constexpr int kStStages = 4;
+__device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEwThreads) : "memory"); }
 static constexpr int kStThreads = kEwThreads + 32;   // consumer warps + the producer warp
 
 struct StagedWalk {
@@ -413,7 +435,7 @@ struct StagedWalk {
 // Producer side: one thread.  Returns the number of chunks it issued (for the drain after an aborted wait).
 __device__ __forceinline__ int staged_produce(const StagedWalk& sw, uint8_t* ring, uint64_t* full, uint64_t* empty, const void* t0, const void* t1,
                                               const void* t2, const uint8_t* mask, long long base_vec, unsigned spin_limit, uint32_t* abort_flag,
-                                              unsigned* status, bool backwards = false)
+                                              unsigned* status, bool backwards = false, uint64_t* last_two_free = nullptr)
 {
     int i = 0;
     const uint32_t tbytes = (uint32_t)sw.chunk_vecs * 16u;
@@ -421,6 +443,10 @@ __device__ __forceinline__ int staged_produce(const StagedWalk& sw, uint8_t* rin
     for (long long j = blockIdx.x; j < sw.n_full; j += gridDim.x, ++i) {
         const long long k = backwards ? sw.n_full - 1 - j : j;
         const int s = i % kStStages;
+        if (i == kStStages - 2 && last_two_free != nullptr && !mbar_wait_bounded(last_two_free, 0u, spin_limit, abort_flag)) {
+            atomicOr(status, B2C_DEV_TIMEOUT);
+            break;
+        }
         if (!mbar_wait_bounded(&empty[s], (((uint32_t)(i / kStStages)) & 1u) ^ 1u, spin_limit, abort_flag)) {
             atomicOr(status, B2C_DEV_TIMEOUT);
             break;
@@ -557,7 +583,7 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_reduce_staged_kernel(con
 }
 
 __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(const void* __restrict__ da1, const void* __restrict__ da2,
-                                                                            const void* __restrict__ y, long long m, int c,
+                                                                            const void* __restrict__ y, long long m, double inv_m, int c,
                                                                             const float* __restrict__ gamma, const float* __restrict__ mean_all,
                                                                             const float* __restrict__ invstd_all, int relu,
                                                                             const double* __restrict__ sums_all, void* __restrict__ dy,
@@ -566,10 +592,11 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(cons
                                                                             unsigned* status)
 {
     extern __shared__ uint8_t st_raw[];
-    __shared__ uint64_t full[kStStages], empty[kStStages];
+    __shared__ uint64_t full[kStStages], empty[kStStages], coef_bar;
     __shared__ uint32_t abort_flag;
     uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(st_raw) + 127u) & ~uintptr_t(127));
     const StagedWalk sw(c, m, da2 != nullptr ? 3 : 2, relu != 0);
+    if (threadIdx.x == 0) mbar_init(&coef_bar, kEwThreads / 32);
     staged_init(full, empty, &abort_flag);
     __syncthreads();
     pdl_wait();   // first global access comes after the previous kernel of the stream
@@ -582,36 +609,22 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(cons
     const uint8_t* mask = relu ? relu_mask : nullptr;
     int issued = 0;
     if (warp == kEwThreads / 32) {
-        if (lane == 0) issued = staged_produce(sw, ring, full, empty, da1, y, da2, mask, base, spin_limit, &abort_flag, status, true);
+        if (lane == 0) issued = staged_produce(sw, ring, full, empty, da1, y, da2, mask, base, spin_limit, &abort_flag, status, true, &coef_bar);
     } else {
-        if (blockIdx.x == 0) {
-            for (int ch = threadIdx.x; ch < c; ch += kEwThreads) {
-                const double s1 = sums[ch], s2 = sums[c + ch];
-                const float db = (float)s1, dg = (float)((double)invstd[ch] * (s2 - (double)mean[ch] * s1));
-                if (gridDim.y == 1) {
-                    dbeta[ch] = acc ? dbeta[ch] + db : db;
-                    dgamma[ch] = acc ? dgamma[ch] + dg : dg;
-                } else {   // several groups add into the same gradient (always accumulating)
-                    atomicAdd(dbeta + ch, db);
-                    atomicAdd(dgamma + ch, dg);
-                }
-            }
-        }
         const int g = threadIdx.x % sw.groups;
         const bool act = threadIdx.x < sw.active;
         const uint32_t tbytes = (uint32_t)sw.chunk_vecs * 16u;
-        const double inv_m = 1.0 / (double)m;
+        float* coef = reinterpret_cast<float*>(ring + (size_t)(kStStages - 2) * sw.stage_bytes);   // in the last two stages, until the threads have read theirs
+        bn_bwd_coefficients(coef, sums, mean, invstd, gamma, c, inv_m, acc, dgamma, dbeta);
+        consumer_sync();
         float mu[8], k0[8], kb[8], kg[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int ch = g * 8 + i;
-            const double s1 = sums[ch], s2 = sums[c + ch];
-            const double is = (double)invstd[ch], dgam = is * (s2 - (double)mean[ch] * s1);
-            mu[i] = mean[ch];
-            k0[i] = gamma[ch] * invstd[ch];                        // gamma*invstd
-            kb[i] = (float)(s1 * inv_m);                           // dbeta/m
-            kg[i] = (float)(dgam * inv_m * is);                    // (dgamma/m)*invstd, multiplies (y-mean)
-        }
+        load8(coef + 8 * g, mu);
+        load8(coef + c + 8 * g, k0);
+        load8(coef + 2 * c + 8 * g, kb);
+        load8(coef + 3 * c + 8 * g, kg);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(&coef_bar);
         auto emit = [&](const uint4& v1, const uint4& vy, const uint4& v2, bool two, unsigned mk, long long vi) {
             float d[8], d2[8], fy[8], o[8];
             unpack8(v1, d);
@@ -678,7 +691,6 @@ __global__ void __launch_bounds__(kStThreads, 2) bn_bwd_apply_staged_kernel(cons
 // the waiting and the coefficient arithmetic beside the streaming warps.  Small layers (whole tensor in L2
 // anyway) look further ahead; they gain the second launch.  The launch is cooperative (all blocks co-resident), every
 // wait is bounded, and a block that gives up raises the status word and winds down like the other staged kernels.
-__device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEwThreads) : "memory"); }
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p)
 {
     unsigned v;
@@ -1423,10 +1435,10 @@ b2c_status launch_bn_fwd(b2c_ctx* ctx, int G, long long m, int c, const void* y,
     }
     uint8_t* mask_out = relu ? reinterpret_cast<uint8_t*>(relu_mask) : nullptr;
     if (residual != nullptr)
-        B2C_CUDA(b2c_launch(ctx, bn_apply_kernel<4, true>, dim3(grid), dim3(kEwThreads), 0, stream, 1u, y, m, c, stats, gamma, beta, residual, relu, eps, a,
+        B2C_CUDA(b2c_launch(ctx, bn_apply_kernel<4, true>, dim3(grid), dim3(kEwThreads), 3 * sizeof(float) * c, stream, 1u, y, m, 1.0 / (double)m, c, stats, gamma, beta, residual, relu, eps, a,
                             save_mean, save_invstd, run_mean, run_var, momentum, mask_out));
     else
-        B2C_CUDA(b2c_launch(ctx, bn_apply_kernel<8, false>, dim3(grid), dim3(kEwThreads), 0, stream, 1u, y, m, c, stats, gamma, beta, residual, relu, eps, a,
+        B2C_CUDA(b2c_launch(ctx, bn_apply_kernel<8, false>, dim3(grid), dim3(kEwThreads), 3 * sizeof(float) * c, stream, 1u, y, m, 1.0 / (double)m, c, stats, gamma, beta, residual, relu, eps, a,
                             save_mean, save_invstd, run_mean, run_var, momentum, mask_out));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;
@@ -1557,7 +1569,7 @@ b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da
     if (staged) {
         const int nt = da2 != nullptr ? 3 : 2;
         const size_t stage = (size_t)nt * chunk_vecs * 16 + (relu ? ((chunk_vecs + 127) & ~127) : 0);
-        const size_t smem = kStStages * stage + 128;   // (the ring also has room for the reduction's slots: more than 128 threads' vectors, twice, per tensor)
+        const size_t smem = kStStages * stage + 128;   // (the ring also has room for the reduction's slots, more than 128 threads' vectors, twice, per tensor, and two stages for 16 bytes per channel)
         if (smem <= 110 * 1024) {
             if (!(ctx->smem_optin_done & B2C_OPTIN_BN_BWD)) {
                 B2C_CUDA(cudaFuncSetAttribute(bn_bwd_reduce_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024));
@@ -1565,14 +1577,14 @@ b2c_status launch_bn_bwd(b2c_ctx* ctx, int G, long long m, int c, const void* da
                 ctx->smem_optin_done |= B2C_OPTIN_BN_BWD;
             }
             if (!sums_ready) B2C_CUDA(b2c_launch(ctx, bn_bwd_reduce_staged_kernel, reduce_grid(grid, 2.0 * nt * m * c), dim3(kStThreads), smem, stream, 1u, da1, da2, y, m, c, relu, sums, mask, ctx->spin_limit, ctx->d_status));
-            B2C_CUDA(b2c_launch(ctx, bn_bwd_apply_staged_kernel, dim3(grid), dim3(kStThreads), smem, stream, 1u, da1, da2, y, m, c, gamma, save_mean, save_invstd, relu, sums, dy, dres,
+            B2C_CUDA(b2c_launch(ctx, bn_bwd_apply_staged_kernel, dim3(grid), dim3(kStThreads), smem, stream, 1u, da1, da2, y, m, 1.0 / (double)m, c, gamma, save_mean, save_invstd, relu, sums, dy, dres,
                                                                             dgamma, dbeta, acc, mask, ctx->spin_limit, ctx->d_status));
             B2C_CUDA(cudaGetLastError());
             return B2C_OK;
         }
     }
     if (!sums_ready) B2C_CUDA(b2c_launch(ctx, bn_bwd_reduce_kernel, reduce_grid(grid, (da2 != nullptr ? 6.0 : 4.0) * m * c), dim3(kEwThreads), 0, stream, 1u, da1, da2, y, a, m, c, relu, sums, mask));
-    B2C_CUDA(b2c_launch(ctx, bn_bwd_apply_kernel, dim3(grid), dim3(kEwThreads), 0, stream, 1u, da1, da2, y, a, m, c, gamma, save_mean, save_invstd, relu, sums, dy, dres, dgamma, dbeta,
+    B2C_CUDA(b2c_launch(ctx, bn_bwd_apply_kernel, dim3(grid), dim3(kEwThreads), 4 * sizeof(float) * c, stream, 1u, da1, da2, y, a, m, 1.0 / (double)m, c, gamma, save_mean, save_invstd, relu, sums, dy, dres, dgamma, dbeta,
                                                          acc, mask));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;
