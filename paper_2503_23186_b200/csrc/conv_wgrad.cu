@@ -13,6 +13,9 @@
 // Layers with 64 output channels would leave half of M = 128 empty.  There two copies of dy, the
 // second gathered one row higher, are stacked on M: with x gathered at (r0 - pad, s - pad) the rows of
 // copy a accumulate tap (r0 + a, s), since sum_p dy[p - (a,0)] x[p + t] = sum_p dy[p] x[p + t + (a,0)].
+// Other channel counts whose last tile of 128 would be partly empty in every filter row put all three rows on M (row_blocks): with x gathered at
+// the middle row, sum_p dy[p] x[p + (r - 1, s - 1)] = sum_p dy[p - (r - 1, 0)] x[p + (0, s - 1)], so M holds (filter row, block of channels)
+// pairs back to back, each block of dy gathered at its row's height: 160 channels fill 3.75 tiles instead of 3 x 1.25 in 3 x 2.
 // Partial sums of the pixel ranges are added to dw with vector fp32 reductions.
 //
 // Framed x stages (3x3, stride 1, image rows of at least 8 pixels, 64-channel x boxes): instead of one x box per
@@ -39,6 +42,7 @@ struct alignas(64) WgradParams {
     WgGroup groups[3];
     int n_groups;
     int stack;                         // two dy copies stacked on M (64 output channels)
+    int row_blocks;                    // 3x3, stride 1: blocks of cw_a output channels per filter row; M holds (filter row, block) pairs back to back (0: it does not)
     int bw, bh, bn, tiles_w, tiles_h;  // pixel chunk box and chunk grid (tiles_h covers one extra row when stacked)
     int pb;                            // pixels per chunk
     int cw_a, swz_a, cw_b, swz_b;      // channels per box (= one swizzle row) and descriptor swizzle code: dy, x
@@ -210,6 +214,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                 const uint32_t tx = p.fx ? (uint32_t)(p.a_bytes + p.b_boxes * p.fx_tx) : (uint32_t)(p.a_bytes + grp.nb * p.b_boxes * p.box_b);
                 const bool timed = p.stall != nullptr && w == 0 && lane == 0;
                 long long waited = 0;
+                // filter row and channel block of the tile's first dy box
+                const int row0 = p.row_blocks ? ktile * p.a_boxes / p.row_blocks : 0, block0 = ktile * p.a_boxes - row0 * p.row_blocks;
                 const int G = p.gsub;   // a slot holds G consecutive chunks (the tile's last one possibly fewer)
                 while (slot < first_slot + n_slots) {
                     const int it = slot - first_slot;
@@ -234,6 +240,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                                 // one box with a halo row on top: copy 1 of dy (gathered one row higher) is its first pb pixels,
                                 // copy 0 starts one image row further down
                                 tma_load_4d(dst, &p.tmDy, &full_bar[s], 0, ow0, oh0 - 1, n0);
+                            } else if (p.row_blocks) {
+                                // x is gathered at the middle filter row; row r wants dy one image row further up or down (boxes past the last
+                                // pair lie behind the last channel and are zero-filled)
+                                int r = row0, kb = block0;
+                                for (int j = 0; j < p.a_boxes; ++j) {
+                                    tma_load_4d(dst + (size_t)j * p.box_a, &p.tmDy, &full_bar[s], r < 3 ? kb * p.cw_a : p.k_total, ow0, r < 3 ? oh0 + 1 - r : oh0, n0);
+                                    if (++kb == p.row_blocks) { kb = 0; ++r; }
+                                }
                             } else {
                                 for (int j = 0; j < p.a_boxes; ++j)  // boxes past the last channel are zero-filled
                                     tma_load_4d(dst + (size_t)j * p.box_a, &p.tmDy, &full_bar[s], ktile * 128 + j * p.cw_a, ow0, oh0, n0);
@@ -366,7 +380,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
             const int q = warp & 3, part = warp >> 2;
             const int m = q * 32 + lane;
             const int copy = p.stack ? 1 - (m >> 6) : 0;                   // which dy copy this accumulator row belongs to (copy 1 comes first)
-            const int k = p.stack ? (m & 63) : ktile * 128 + m;
+            int k = p.stack ? (m & 63) : ktile * 128 + m, row = 0;   // output channel, and filter row where M holds several
+            if (p.row_blocks) {
+                const int pair = ktile * p.a_boxes + m / p.cw_a;
+                row = pair / p.row_blocks;
+                k = row < 3 ? (pair - row * p.row_blocks) * p.cw_a + m % p.cw_a : p.k_total;
+            }
             __syncwarp();
             bool ok = n_chunks > 0;
             if (ok) {
@@ -379,13 +398,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
             // their vectors as they are, unless many CTAs add to the same rows; warps whose rows all lie past the last filter row have nothing to
             // send.  640 -> 16 channels at 2x2 with 7 images 9.2 us with the exchange, 6.6 without; 49 CTAs per row (160 -> 16 at 32x32 with 13
             // images) 15.7 and 12.6, but 148 (64 -> 32 1x1 at 32x32 with 256 images) 12.3 and 13.5.
-            const bool few_rows = !p.stack && p.k_total - ktile * 128 <= 32 && p.n_splits <= 64;
-            if (ok && (p.stack || ktile * 128 + q * 32 < p.k_total)) {
+            const bool few_rows = !p.stack && !p.row_blocks && p.k_total - ktile * 128 <= 32 && p.n_splits <= 64;
+            if (ok && (p.stack || (p.row_blocks ? ktile * 128 + q * 32 < 3 * p.k_total : ktile * 128 + q * 32 < p.k_total))) {
                 const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
                 const int n_ck = p.ct >> 4;
                 const int ck_begin = part == 0 ? 0 : (n_ck + 1) >> 1, ck_end = part == 0 ? (n_ck + 1) >> 1 : n_ck;   // this warp's chunks
                 for (int b = 0; b < grp.nb && ck_begin < ck_end; ++b) {
-                    const int rs = grp.rs[copy][b];
+                    const int rs = p.row_blocks ? 3 * row + b : grp.rs[copy][b];
                     const bool live = rs >= 0 && k < p.k_total;
                     float* dst = p.dw + ctile * p.ct;
                     // offset of the row in dw in units of 16 elements: a filter bank may exceed 2^31 elements, but not 2^36 (256 GB)
@@ -538,7 +557,16 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
             if (pb.c % (nb * p.cw_b) == 0) { p.ct = nb * p.cw_b; break; }
     }
     p.n_ctiles = pb.c / p.ct;
-    p.n_ktiles = p.stack ? 1 : (pb.k + 127) / 128;
+    // Filter rows on M: 3x3, stride 1, where the three rows' channels fill fewer tiles of 128 back to back than each row for itself, and the fewer
+    // tiles still make 64 CTAs of four chunks (below that the chip is idle either way and a tile has more to send: 64 -> 32 at 16x16 with 16
+    // images 6.6 us in 48 CTAs, 7.9 in 16).  160 -> 160 at 32x32 with 256 images 151 -> 112 us, 16 -> 160 61 -> 44, 320 -> 320 at 16x16 118 -> 113,
+    // 16 -> 16 at 32x32 with 512 images 72 -> 29, 32 -> 32 at 16x16 with 1024 25 -> 13, 48 -> 48 at 32x32 with 128 33 -> 24.
+    {
+        const int tiles = (3 * pb.k + 127) / 128;
+        const long long chunks = ((long long)pb.n * pb.p * pb.q + 63) / 64;
+        if (R == 3 && pb.stride == 1 && !p.stack && tiles < 3 * ((pb.k + 127) / 128) && tiles * p.n_ctiles * (chunks / 4) >= 64) p.row_blocks = pb.k / p.cw_a;
+    }
+    p.n_ktiles = p.stack ? 1 : p.row_blocks ? (3 * pb.k + 127) / 128 : (pb.k + 127) / 128;
     p.a_boxes = p.stack ? 2 : 128 / p.cw_a;
     p.b_boxes = p.ct / p.cw_b;
     const int shifts = R == 3 ? 3 : 1;
@@ -565,6 +593,11 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
         WgGroup& g = p.groups[0];
         g.nb = 1; g.map[0] = fw.map[0]; g.dh[0] = fw.dh[0]; g.dw[0] = fw.dw[0];
         g.rs[0][0] = 0; g.rs[1][0] = -1;
+    } else if (p.row_blocks) {
+        p.n_groups = 1;   // x at the middle filter row
+        WgGroup& g = p.groups[0];
+        g.nb = 3;
+        for (int s = 0; s < 3; ++s) { g.map[s] = fw.map[3 + s]; g.dh[s] = fw.dh[3 + s]; g.dw[s] = fw.dw[3 + s]; g.rs[0][s] = g.rs[1][s] = -1; }
     } else if (!p.stack) {
         p.n_groups = 3;   // one group per filter row
         for (int r = 0; r < 3; ++r) {
