@@ -134,7 +134,8 @@ __device__ __forceinline__ void wg_issue(uint32_t d_tmem, uint32_t a_lo, uint32_
 
 // STREAM: the launch deals out equal runs of (tile, chunk) pairs (p.stream); otherwise a CTA has one tile, and the code for more is left out
 // (it cost short launches 0.2-1.7 us).
-template <bool STREAM>
+// ROWS: M holds (filter row, channel block) pairs (p.row_blocks); with both in one kernel the others ran 1-3 % slower.
+template <bool STREAM, bool ROWS>
 __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_constant__ WgradParams p)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                 const bool timed = p.stall != nullptr && w == 0 && lane == 0;
                 long long waited = 0;
                 // filter row and channel block of the tile's first dy box
-                const int row0 = p.row_blocks ? ktile * p.a_boxes / p.row_blocks : 0, block0 = ktile * p.a_boxes - row0 * p.row_blocks;
+                const int row0 = ROWS ? ktile * p.a_boxes / p.row_blocks : 0, block0 = ROWS ? ktile * p.a_boxes - row0 * p.row_blocks : 0;
                 const int G = p.gsub;   // a slot holds G consecutive chunks (the tile's last one possibly fewer)
                 while (slot < first_slot + n_slots) {
                     const int it = slot - first_slot;
@@ -240,7 +241,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
                                 // one box with a halo row on top: copy 1 of dy (gathered one row higher) is its first pb pixels,
                                 // copy 0 starts one image row further down
                                 tma_load_4d(dst, &p.tmDy, &full_bar[s], 0, ow0, oh0 - 1, n0);
-                            } else if (p.row_blocks) {
+                            } else if (ROWS) {
                                 // x is gathered at the middle filter row; row r wants dy one image row further up or down (boxes past the last
                                 // pair lie behind the last channel and are zero-filled)
                                 int r = row0, kb = block0;
@@ -381,7 +382,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
             const int m = q * 32 + lane;
             const int copy = p.stack ? 1 - (m >> 6) : 0;                   // which dy copy this accumulator row belongs to (copy 1 comes first)
             int k = p.stack ? (m & 63) : ktile * 128 + m, row = 0;   // output channel, and filter row where M holds several
-            if (p.row_blocks) {
+            if constexpr (ROWS) {
                 const int pair = ktile * p.a_boxes + m / p.cw_a;
                 row = pair / p.row_blocks;
                 k = row < 3 ? (pair - row * p.row_blocks) * p.cw_a + m % p.cw_a : p.k_total;
@@ -398,13 +399,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv_wgrad_kernel(const __grid_
             // their vectors as they are, unless many CTAs add to the same rows; warps whose rows all lie past the last filter row have nothing to
             // send.  640 -> 16 channels at 2x2 with 7 images 9.2 us with the exchange, 6.6 without; 49 CTAs per row (160 -> 16 at 32x32 with 13
             // images) 15.7 and 12.6, but 148 (64 -> 32 1x1 at 32x32 with 256 images) 12.3 and 13.5.
-            const bool few_rows = !p.stack && !p.row_blocks && p.k_total - ktile * 128 <= 32 && p.n_splits <= 64;
-            if (ok && (p.stack || (p.row_blocks ? ktile * 128 + q * 32 < 3 * p.k_total : ktile * 128 + q * 32 < p.k_total))) {
+            const bool few_rows = !p.stack && !ROWS && p.k_total - ktile * 128 <= 32 && p.n_splits <= 64;
+            if (ok && (p.stack || (ROWS ? ktile * 128 + q * 32 < 3 * p.k_total : ktile * 128 + q * 32 < p.k_total))) {
                 const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
                 const int n_ck = p.ct >> 4;
                 const int ck_begin = part == 0 ? 0 : (n_ck + 1) >> 1, ck_end = part == 0 ? (n_ck + 1) >> 1 : n_ck;   // this warp's chunks
                 for (int b = 0; b < grp.nb && ck_begin < ck_end; ++b) {
-                    const int rs = p.row_blocks ? 3 * row + b : grp.rs[copy][b];
+                    const int rs = ROWS ? 3 * row + b : grp.rs[copy][b];
                     const bool live = rs >= 0 && k < p.k_total;
                     float* dst = p.dw + ctile * p.ct;
                     // offset of the row in dw in units of 16 elements: a filter bank may exceed 2^31 elements, but not 2^36 (256 GB)
@@ -556,16 +557,43 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
         for (int nb = max_boxes; nb >= 1; --nb)
             if (pb.c % (nb * p.cw_b) == 0) { p.ct = nb * p.cw_b; break; }
     }
-    p.n_ctiles = pb.c / p.ct;
-    // Filter rows on M: 3x3, stride 1, where the three rows' channels fill fewer tiles of 128 back to back than each row for itself, and the fewer
-    // tiles still make 64 CTAs of four chunks (below that the chip is idle either way and a tile has more to send: 64 -> 32 at 16x16 with 16
-    // images 6.6 us in 48 CTAs, 7.9 in 16).  160 -> 160 at 32x32 with 256 images 151 -> 112 us, 16 -> 160 61 -> 44, 320 -> 320 at 16x16 118 -> 113,
-    // 16 -> 16 at 32x32 with 512 images 72 -> 29, 32 -> 32 at 16x16 with 1024 25 -> 13, 48 -> 48 at 32x32 with 128 33 -> 24.
-    {
-        const int tiles = (3 * pb.k + 127) / 128;
+    // 3x3 layers: a narrower tile, and filter rows that share tiles of M (stride 1), where the estimate is better.  A CTA ends with the sending of
+    // its partial sums, 23 cycles per column, and all CTAs together send n_splits filter banks: with few chunks per CTA that is most of the
+    // launch.  Measured with the widest tile / half of it: 128 -> 128 at 16x16 with 50 / 128 / 300 / 600 images 12.8 / 16.0 / 22.6 / 35.8 us and
+    // 9.8 / 13.8 / 21.1 / 38.0, 256 -> 512 at 8x8 stride 2 with 50 / 128 11.9 / 13.9 and 8.3 / 10.7, 512 -> 512 at 4x4 with 50 / 128 13.0 /
+    // 17.0 and 11.2 / 18.2, 128 -> 256 at 16x16 stride 2 with 1024 40.9 and 46.1.  Filter rows on M: 160 -> 160 at 32x32 with 256 images
+    // 151 -> 112 us, 16 -> 160 61 -> 44, 16 -> 16 at 32x32 with 512 images 72 -> 29, 32 -> 32 at 16x16 with 1024 25 -> 13, 48 -> 48 at 32x32 with
+    // 128 33 -> 24; not where they save nothing: 64 -> 32 at 16x16 with 16 6.6 -> 7.9.
+    if (R == 3) {
         const long long chunks = ((long long)pb.n * pb.p * pb.q + 63) / 64;
-        if (R == 3 && pb.stride == 1 && !p.stack && tiles < 3 * ((pb.k + 127) / 128) && tiles * p.n_ctiles * (chunks / 4) >= 64) p.row_blocks = pb.k / p.cw_a;
+        const int m_rows = p.stack ? 2 : 3 * ((pb.k + 127) / 128), m_shared = (3 * pb.k + 127) / 128;   // tiles of M
+        auto cycles = [&](int ct, int m_tiles) {
+            const int tiles = m_tiles * (pb.c / ct);
+            long long splits = ctx->sm_count / tiles < chunks / 4 ? ctx->sm_count / tiles : chunks / 4;
+            if (splits < 1) splits = 1;
+            // MMAs of a chunk of 64 pixels (128 x n x 16: n / 2 cycles, or its operands at 128 B/clk) and its loads at about 60 B/clk
+            auto mma = [](int n) { return 4 * (n / 2 > 32 + n / 4 ? n / 2 : 32 + n / 4); };
+            const int work = p.fx ? ct / p.cw_b * mma(3 * p.cw_b) : 3 * ct <= 256 ? mma(3 * ct) : 2 * ct <= 256 ? mma(2 * ct) + mma(ct) : 3 * mma(ct);
+            const int load = (128 + (p.fx ? ct * 5 / 4 : 3 * ct)) * 128 / 60, chunk = work > load ? work : load, tail = 1500 + 69 * ct;
+            const long long plain = (tiles * splits + ctx->sm_count - 1) / ctx->sm_count * ((chunks + splits - 1) / splits * chunk + tail);
+            const long long equal = (tiles * chunks / ctx->sm_count + 1) * chunk + (tiles + ctx->sm_count) * (long long)tail / ctx->sm_count;   // (equal runs, see below)
+            return tiles * chunks >= 8ll * ctx->sm_count && equal * 100 < plain * 85 ? equal : plain;
+        };
+        const bool may_share = pb.stride == 1 && !p.stack && m_shared < m_rows;
+        const int widest_ct = p.ct;
+        bool share = may_share && cycles(widest_ct, m_shared) * 100 < cycles(widest_ct, m_rows) * 97;
+        long long best = cycles(widest_ct, share ? m_shared : m_rows);
+        best = best * (p.cw_a == 64 && p.cw_b == 64 ? 97 : 75) / 100;   // (narrow boxes: many loads per chunk, which the estimate leaves out)
+        for (int cand = widest_ct - p.cw_b; cand >= p.cw_b; cand -= p.cw_b) {
+            if (pb.c % cand) continue;
+            for (int sh = 0; sh <= (may_share ? 1 : 0); ++sh) {
+                const long long est = cycles(cand, sh ? m_shared : m_rows);
+                if (est < best) { best = est; p.ct = cand; share = sh != 0; }
+            }
+        }
+        if (share) p.row_blocks = pb.k / p.cw_a;
     }
+    p.n_ctiles = pb.c / p.ct;
     p.n_ktiles = p.stack ? 1 : p.row_blocks ? (3 * pb.k + 127) / 128 : (pb.k + 127) / 128;
     p.a_boxes = p.stack ? 2 : 128 / p.cw_a;
     p.b_boxes = p.ct / p.cw_b;
@@ -750,13 +778,15 @@ b2c_status launch_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, cudaStream_t 
     p.stall = ctx->stall_counters;
 
     if (!(ctx->smem_optin_done & B2C_OPTIN_WGRAD)) {
-        B2C_CUDA(cudaFuncSetAttribute(conv_wgrad_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
-        B2C_CUDA(cudaFuncSetAttribute(conv_wgrad_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
+        for (auto* k : {conv_wgrad_kernel<false, false>, conv_wgrad_kernel<false, true>, conv_wgrad_kernel<true, false>, conv_wgrad_kernel<true, true>})
+            B2C_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024));
         ctx->smem_optin_done |= B2C_OPTIN_WGRAD;
     }
     const size_t smem_bytes = plan.smem_bytes;
     dim3 grid((unsigned)plan.grid);
-    B2C_CUDA(b2c_launch(ctx, p.stream ? conv_wgrad_kernel<true> : conv_wgrad_kernel<false>, grid, dim3(kWgThreads), smem_bytes, stream, 1u, p));
+    auto* kernel = p.row_blocks ? (p.stream ? conv_wgrad_kernel<true, true> : conv_wgrad_kernel<false, true>)
+                                : (p.stream ? conv_wgrad_kernel<true, false> : conv_wgrad_kernel<false, false>);
+    B2C_CUDA(b2c_launch(ctx, kernel, grid, dim3(kWgThreads), smem_bytes, stream, 1u, p));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;
 }
