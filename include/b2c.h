@@ -239,6 +239,14 @@ typedef struct {
     int slot_k_blocks;     /* k-blocks per ring slot */
 } b2c_conv_plan;
 b2c_status b2c_conv2d_plan(b2c_ctx* ctx, const b2c_conv_desc* d, int pass, b2c_conv_plan* out);
+/* The same with more of the plan.  A forward call with ch_stats may have another epilogue, and with it other shared memory, than one
+ * without: ch_stats != 0 asks for the former (pass 0 only; b2c_conv2d_plan answers for the latter). */
+typedef struct {
+    b2c_conv_plan plan;
+    int block_cols;        /* forward / data gradient: columns per block of the persistent kernel's epilogue (0: it works by rows) */
+    int row_blocks;        /* weight gradient: channel blocks per filter row where M holds all three filter rows (0: one row at a time) */
+} b2c_conv_plan_detail;
+b2c_status b2c_conv2d_plan_detail(b2c_ctx* ctx, const b2c_conv_desc* d, int pass, int ch_stats, b2c_conv_plan_detail* out);
 
 /* db[k] (+)= sum_m dz[m, k] for bf16 dz [m, pitch]; fp32 db [k]. */
 b2c_status b2c_bias_grad(b2c_ctx* ctx, int m, int k, int pitch, const void* dz, float* db, int accumulate, void* stream);

@@ -27,7 +27,7 @@ EXPORTS = [
     "b2c_conv2d_workspace_bytes", "b2c_conv2d_fwd", "b2c_bn_relu_fwd", "b2c_avgpool_fwd", "b2c_avgpool_bwd", "b2c_pad_channels",
     "b2c_softmax_xent_fwd_bwd", "b2c_bn_relu_bwd_workspace_bytes", "b2c_bn_relu_bwd", "b2c_bn_relu_bwd_static",
     "b2c_bn_relu_bwd_groups_workspace_bytes", "b2c_bn_relu_bwd_groups", "b2c_conv2d_dgrad",
-    "b2c_conv2d_wgrad", "b2c_conv2d_plan", "b2c_bias_grad", "b2c_grad_accum_sgd_momentum", "b2c_weight_pack_dgrad",
+    "b2c_conv2d_wgrad", "b2c_conv2d_plan", "b2c_conv2d_plan_detail", "b2c_bias_grad", "b2c_grad_accum_sgd_momentum", "b2c_weight_pack_dgrad",
     "b2c_net_create", "b2c_net_create_concurrent", "b2c_net_destroy", "b2c_net_param_count", "b2c_net_param_offset",
     "b2c_net_padded_image_channels", "b2c_net_first_conv_im2col", "b2c_im2col_3x3", "b2c_net_workspace_bytes", "b2c_net_tensor_offset", "b2c_net_bind",
     "b2c_net_sync_weights", "b2c_train_step", "b2c_net_apply_update", "b2c_net_profile_enable", "b2c_net_profile_read",
@@ -44,6 +44,10 @@ class ConvDesc(Structure):
 
 class ConvPlan(Structure):
     _fields_ = [(n, c_int) for n in ("kind", "tile_channels", "pair", "splits", "overlap", "ctas", "smem_bytes", "k_block", "slot_k_blocks")]
+
+
+class ConvPlanDetail(Structure):
+    _fields_ = [("plan", ConvPlan), ("block_cols", c_int), ("row_blocks", c_int)]
 
 
 PLAN_KINDS = ["general", "shared-units", "merged-taps", "full-halo", "one-wave", "wgrad", "wgrad-runs"]
@@ -245,12 +249,13 @@ class Context:
     def conv2d_wgrad(self, d: ConvDesc, dy, x, dw, accumulate=False):
         _check(lib().b2c_conv2d_wgrad(self.handle, byref(d), _ptr(dy), _ptr(x), _ptr(dw), int(accumulate), _stream()), "b2c_conv2d_wgrad")
 
-    def conv2d_plan(self, d: ConvDesc, which: str) -> dict:
-        """The launch plan of conv2d_fwd, conv2d_dgrad or conv2d_wgrad ("fwd", "dgrad", "wgrad") for a layer; nothing is launched."""
-        plan = ConvPlan()
-        _check(lib().b2c_conv2d_plan(self.handle, byref(d), ("fwd", "dgrad", "wgrad").index(which), byref(plan)), "b2c_conv2d_plan")
+    def conv2d_plan(self, d: ConvDesc, which: str, sums: bool = False) -> dict:
+        """The launch plan of conv2d_fwd (with ch_stats if `sums`), conv2d_dgrad or conv2d_wgrad ("fwd", "dgrad", "wgrad") for a layer; nothing is launched."""
+        detail = ConvPlanDetail()
+        _check(lib().b2c_conv2d_plan_detail(self.handle, byref(d), ("fwd", "dgrad", "wgrad").index(which), int(sums), byref(detail)), "b2c_conv2d_plan_detail")
+        plan = detail.plan
         out = {name: getattr(plan, name) for name, _ in ConvPlan._fields_}
-        out["kind"] = PLAN_KINDS[plan.kind]
+        out.update(kind=PLAN_KINDS[plan.kind], block_cols=detail.block_cols, row_blocks=detail.row_blocks)
         return out
 
     def bias_grad(self, m, k, pitch, dz, db, accumulate=False):

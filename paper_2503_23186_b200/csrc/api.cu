@@ -213,14 +213,26 @@ b2c_status b2c_conv2d_wgrad(b2c_ctx* ctx, const b2c_conv_desc* d, const void* dy
     return launch_conv_wgrad(ctx, pb, (cudaStream_t)stream);
 }
 
-b2c_status b2c_conv2d_plan(b2c_ctx* ctx, const b2c_conv_desc* d, int pass, b2c_conv_plan* out)
+b2c_status b2c_conv2d_plan_detail(b2c_ctx* ctx, const b2c_conv_desc* d, int pass, int ch_stats, b2c_conv_plan_detail* out)
 {
-    if (!ctx || !out || pass < 0 || pass > 2) return B2C_ERR_INVALID_ARG;
+    if (!ctx || !out || pass < 0 || pass > 2 || (ch_stats && pass != 0)) return B2C_ERR_INVALID_ARG;
     int p, q;
     b2c_status st = check_desc(d, &p, &q);
     if (st != B2C_OK) return st;
-    *out = b2c_conv_plan{};
-    return pass == 2 ? plan_conv_wgrad(ctx, wgrad_problem(d, p, q), *out) : plan_conv_kmajor(ctx, kmajor_problem(d, p, q, pass == 1), *out);
+    *out = b2c_conv_plan_detail{};
+    if (pass == 2) return plan_conv_wgrad(ctx, wgrad_problem(d, p, q), *out);
+    KMajorProblem pb = kmajor_problem(d, p, q, pass == 1);
+    pb.ask_sums = ch_stats != 0;
+    return plan_conv_kmajor(ctx, pb, *out);
+}
+
+b2c_status b2c_conv2d_plan(b2c_ctx* ctx, const b2c_conv_desc* d, int pass, b2c_conv_plan* out)
+{
+    if (!out) return B2C_ERR_INVALID_ARG;
+    b2c_conv_plan_detail detail{};
+    const b2c_status st = b2c_conv2d_plan_detail(ctx, d, pass, 0, &detail);
+    *out = detail.plan;
+    return st;
 }
 
 }  // extern "C"

@@ -147,11 +147,12 @@ struct KMajorProblem {
     const void* bwd_other;   // the other contribution, or nullptr
     const void* bwd_mask;    // one bit per element, or nullptr
     bool* bwd_done;          // set to whether the launch takes the sums
+    bool ask_sums;         // a question about the plan of a call with `stats`
     bool no_wait;          // the launch right before this one shares nothing that is written with this one, and itself waits for the one before it:
                            // the kernel starts as SMs fall free and waits for that launch only at its end
 };
 b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_t stream);
-b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan& out);   // pointers of the problem: null
+b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan_detail& out);   // pointers of the problem: null
 
 struct WgradProblem {
     int n, h, w, c;        // x
@@ -162,7 +163,7 @@ struct WgradProblem {
     float* dw;             // [k][r*r][c] fp32, accumulated into
 };
 b2c_status launch_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, cudaStream_t stream);
-b2c_status plan_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, b2c_conv_plan& out);
+b2c_status plan_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, b2c_conv_plan_detail& out);
 
 // BatchNorm over G statistics groups (micro-batches) of m rows each; stats / sums are fp64 [G][2c],
 // save_mean / save_invstd fp32 [G][c].  G > 1 requires acc != 0 in the backward pass.  stats_ready: 1 = `stats` holds the

@@ -1631,7 +1631,7 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     // 16 at a time in the kernel's static arrays.  Tiles of 256 channels without sums whose MMAs take more than 12000 cycles hide the
     // epilogue anyway and are 1 % slower in blocks (256 -> 256 at 8x8 59.7 and 60.1 us); the others gain, see epilogue_blocks.
     if (!cluster && !pb.out_f32 && pb.bias == nullptr) {
-        const bool sums = pb.stats != nullptr && pb.bwd_y == nullptr;
+        const bool sums = (pb.stats != nullptr || pb.ask_sums) && pb.bwd_y == nullptr;
         const int room = ring_budget - p.resident_bytes - p.stages * stage_bytes;
         const int mma = R * R * pb.ic / 16 / n_par * (n_tile / 2);
         if (n_tile == 64 && !p.fh && room >= 16 * 1024) p.block_cols = 32;
@@ -1733,7 +1733,7 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
 
 static int kernel_kind(const ConvKParams& p) { return p.hm ? KIND_HMERGE : p.fh ? KIND_FULL_HALO : p.issue_split ? KIND_SPLIT : KIND_GENERAL; }
 
-b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan& out)
+b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan_detail& detail)
 {
     static_assert((int)KIND_GENERAL == B2C_PLAN_GENERAL && (int)KIND_SPLIT == B2C_PLAN_SHARED_UNITS && (int)KIND_HMERGE == B2C_PLAN_MERGED_TAPS &&
                       (int)KIND_FULL_HALO == B2C_PLAN_FULL_HALO, "the header's names of the kernel kinds");
@@ -1741,10 +1741,12 @@ b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan
     b2c_status st = build_kmajor_plan(ctx, pb, plan);
     if (st != B2C_OK) return st;
     const ConvKParams& p = plan.p;
+    b2c_conv_plan& out = detail.plan;
     out.kind = p.splits > 0 ? B2C_PLAN_ONE_WAVE : kernel_kind(p);
     out.tile_channels = p.n_tile; out.pair = p.pair; out.splits = p.splits > 0 ? p.splits : 1; out.overlap = p.x_overlap;
     out.ctas = plan.grid; out.smem_bytes = (int)plan.smem_bytes;
     out.k_block = p.kb; out.slot_k_blocks = p.gsub;
+    detail.block_cols = p.block_cols;
     return B2C_OK;
 }
 

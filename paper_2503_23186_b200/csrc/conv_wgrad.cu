@@ -742,16 +742,18 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     return B2C_OK;
 }
 
-b2c_status plan_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, b2c_conv_plan& out)
+b2c_status plan_conv_wgrad(b2c_ctx* ctx, const WgradProblem& pb, b2c_conv_plan_detail& detail)
 {
     WgradPlan plan;
     b2c_status st = build_wgrad_plan(ctx, pb, plan);
     if (st != B2C_OK) return st;
     const WgradParams& p = plan.p;
+    b2c_conv_plan& out = detail.plan;
     out.kind = p.stream ? B2C_PLAN_WGRAD_RUNS : B2C_PLAN_WGRAD;
     out.tile_channels = p.ct; out.splits = p.n_splits;
     out.ctas = plan.grid; out.smem_bytes = (int)plan.smem_bytes;
     out.k_block = p.pb; out.slot_k_blocks = p.gsub;
+    detail.row_blocks = p.row_blocks;
     return B2C_OK;
 }
 

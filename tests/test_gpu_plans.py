@@ -96,3 +96,16 @@ def test_clusters_have_their_sms_to_themselves(ctx):
                 raised += plan["smem_bytes"] == 115 * 1024
                 assert plan["smem_bytes"] > 114 * 1024, (shape, plan)
     assert clusters >= 200 and raised >= 5, (clusters, raised)
+
+
+def test_plan_of_a_call_with_sums(ctx):
+    """256-channel tiles whose MMAs hide the epilogue work in blocks only where they take sums: the query tells both apart, and the
+    shared memory that it reports holds the blocks."""
+    from paper_2503_23186_b200 import binding
+    d = binding.conv_desc(1024, 8, 8, 256, 256, 3, 1)
+    plain, sums = ctx.conv2d_plan(d, "fwd"), ctx.conv2d_plan(d, "fwd", sums=True)
+    assert plain["block_cols"] == 0 and sums["block_cols"] == 64, (plain, sums)
+    assert sums["smem_bytes"] == plain["smem_bytes"] + 24 * 1024
+    for which in ("dgrad", "wgrad"):
+        with pytest.raises(binding.B2CError):
+            ctx.conv2d_plan(d, which, sums=True)
