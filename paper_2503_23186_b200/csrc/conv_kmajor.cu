@@ -413,6 +413,10 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
 // Layers of 1024 images inside a step, epilogue_loop -> this: with sums 64 -> 256 1x1 at 32x32 312 -> 145 us (sums in a pass of their own: 139 +
 // 95), 128 -> 512 at 16x16 166 -> 84, 64 -> 64 3x3 80 -> 71, 128 -> 128 3x3 at 16x16 77 -> 63, 64 -> 128 1x1 stride 2 60 -> 41, 512 -> 512 at 4x4
 // 65 -> 63; without sums data gradient 256 <- 64 1x1 137 -> 126, 512 <- 128 81 -> 71, 64 <- 64 3x3 66 -> 63.
+// Every four units the running squares move on to a second sum in local memory, and what that addition rounds off stays behind: squares of
+// positive outputs of 2048 images (16 -> 64 1x1) are 2.1e-9 off, 4.3e-8 without the remainder, of 1024 images (128 -> 512 1x1) 7.9e-9 and 1.0e-8.
+// Tiles of 64 channels have registers for a second plain sum too (16 -> 64 1x1 with 1024 images 49.7 -> 50.6 us for both); wider ones keep
+// one for the whole statistics group, as in epilogue_loop: sums of 1024 images with a mean are 0.2-1.4e-9 of their magnitudes off, there and here.
 template <int BC, int NB, bool HM, bool STATS>
 __device__ __forceinline__ int2 epilogue_blocks(const ConvKParams& p, uint32_t tmem_base, uint64_t* acc_full, uint64_t* acc_empty, uint32_t* abort_flag,
                                                 float* my_stats, uint8_t* stage, int e, int lane, int rank)
@@ -438,12 +442,15 @@ __device__ __forceinline__ int2 epilogue_blocks(const ConvKParams& p, uint32_t t
     const int sw_w = swizzle(lane);
 
     constexpr int NA = STATS ? 4 * NB : 1;   // column pairs this lane sums
-    f32x2 acc_s[NA], acc_q[NA], long_q[NA];
+    constexpr bool LONG_S = STATS && BC == 32;   // tiles of 64 channels have registers for a second running sum
+    f32x2 acc_s[NA], acc_q[NA], long_s[LONG_S ? NA : 1], long_q[NA];
     int opaque_zero = 0, held = 0;   // (an index that the compiler cannot see through keeps long_q out of the registers)
     if constexpr (STATS) {
         asm volatile("mov.u32 %0, 0;" : "=r"(opaque_zero));
 #pragma unroll
         for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = long_q[i + opaque_zero] = 0ull;
+#pragma unroll
+        for (int i = 0; i < (LONG_S ? NA : 1); ++i) long_s[i] = 0ull;
     }
     int jacc = 0, cur_group = -1, cur_ktile = 0;
     bool ok = true;
@@ -452,7 +459,7 @@ __device__ __forceinline__ int2 epilogue_blocks(const ConvKParams& p, uint32_t t
     auto each_total = [&](auto emit) {   // emit(column of the warp, sum, sum of squares) in one lane per column
 #pragma unroll
         for (int i = 0; i < NA; ++i) {
-            float2 s = split_f32x2(acc_s[i]), sq = split_f32x2(add_f32x2(acc_q[i], long_q[i + opaque_zero]));
+            float2 s = split_f32x2(LONG_S ? add_f32x2(acc_s[i], long_s[LONG_S ? i : 0]) : acc_s[i]), sq = split_f32x2(add_f32x2(acc_q[i], long_q[i + opaque_zero]));
 #pragma unroll
             for (int bit = LPR; bit < 32; bit <<= 1) {
                 s.x += __shfl_xor_sync(0xffffffffu, s.x, bit);
@@ -470,10 +477,17 @@ __device__ __forceinline__ int2 epilogue_blocks(const ConvKParams& p, uint32_t t
     };
     auto flush_stats = [&](bool group_done) {
         held = 0;
+        const f32x2 minus_one = make_f32x2(-1.f, -1.f);
 #pragma unroll
         for (int i = 0; i < NA; ++i) {
-            long_q[i + opaque_zero] = add_f32x2(long_q[i + opaque_zero], acc_q[i]);
-            acc_q[i] = 0ull;
+            // (what the addition rounds off stays behind)
+            const f32x2 old_q = long_q[i + opaque_zero], new_q = add_f32x2(old_q, acc_q[i]);
+            long_q[i + opaque_zero] = new_q;
+            acc_q[i] = add_f32x2(acc_q[i], fma_f32x2(new_q, minus_one, old_q));
+            if constexpr (LONG_S) {
+                long_s[i] = add_f32x2(long_s[i], acc_s[i]);
+                acc_s[i] = 0ull;
+            }
         }
         if (group_done) {
             double* st = p.stats + (size_t)cur_group * 2 * p.oc_valid + cur_ktile * p.n_tile + col_begin;
@@ -482,7 +496,9 @@ __device__ __forceinline__ int2 epilogue_blocks(const ConvKParams& p, uint32_t t
                 atomicAdd(st + p.oc_valid + col, (double)sq);
             });
 #pragma unroll
-            for (int i = 0; i < NA; ++i) acc_s[i] = long_q[i + opaque_zero] = 0ull;
+            for (int i = 0; i < NA; ++i) acc_s[i] = acc_q[i] = long_q[i + opaque_zero] = 0ull;
+#pragma unroll
+            for (int i = 0; i < (LONG_S ? NA : 1); ++i) long_s[i] = 0ull;
         }
     };
 

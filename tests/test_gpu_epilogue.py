@@ -59,3 +59,36 @@ def test_blocks_of_the_epilogue(shape, monkeypatch):
         assert bool(((stats[K:] - (f * f).sum(0)).abs() <= 32 * 2.0 ** -24 * (f * f).sum(0)).all())
     finally:
         ctx.close()
+
+
+# 221 and 110 units per CTA: 64-channel tiles, one MMA per tap and merged taps
+@pytest.mark.parametrize("shape", [(4096, 32, 32, 16, 64, 1, 1), (2048, 32, 32, 64, 64, 3, 1)], ids=lambda s: "n{}h{}w{}c{}k{}r{}s{}".format(*s))
+def test_sums_over_many_units(shape):
+    """Ones, and a small value in every row that a lane meets last: a running fp32 sum over all units of a CTA loses the small values once
+    it is large; sums of a few units, added up on their own, hold them."""
+    from paper_2503_23186_b200 import binding
+    N, H, W, C, K, R, st = shape
+    ctx = binding.Context(0)
+    try:
+        d = binding.conv_desc(*shape)
+        plan = ctx.conv2d_plan(d, "fwd", sums=True)
+        assert plan["block_cols"] == 32, plan
+        per_cta = N * H * W // 128 // plan["ctas"]
+        assert per_cta >= 50, plan
+        # a lane adds up rows l, l + 8, l + 16 and l + 24 of its warp's 32, of which the last is small: a quarter of the last bit of one running sum
+        small = 2.0 ** (np.ceil(np.log2(3 * (per_cta + 1))) - 26)
+        x = torch.zeros((N, H, W, C), dtype=torch.bfloat16, device="cuda")
+        pixel = torch.arange(W, device="cuda")   # (rows of a warp: 32 pixels of one image row)
+        x[..., 0] = torch.where(pixel >= 24, small, 1.0).to(torch.bfloat16)
+        w = torch.zeros((K, R, R, C), dtype=torch.bfloat16, device="cuda")
+        w[:, R // 2, R // 2, 0] = 1.0
+        y = torch.empty((N, H, W, K), dtype=torch.bfloat16, device="cuda")
+        stats = torch.zeros(2 * K, dtype=torch.float64, device="cuda")
+        ctx.conv2d_fwd(d, x, w, y, ch_stats=stats)
+        assert ctx.device_status() == 0
+        assert bool((y == x[..., :1]).all())
+        want = N * H * (24 + 8 * small)
+        # a lane's sums of four units, and their sum, are exact; the last units' share and three additions between lanes round, warps meet in fp64
+        assert bool(((stats[:K] - want).abs() <= 4 * 2.0 ** -24 * want).all()), ((stats[:K] - want) / want).abs().max().item()
+    finally:
+        ctx.close()
