@@ -492,9 +492,9 @@ b2c_status b2c_net_create_concurrent(b2c_ctx* ctx, const b2c_layer_desc* layers,
             const int pix = L.p * L.q;
             const int imgs_per_tile = pix >= 128 ? 1 : 128 / pix;
             o.fused_stats = net->fuse_stats && (n_concurrent == 1 || micro_batch % imgs_per_tile == 0);
-            // Tiles of up to 64 channels sum at next to no cost, and so do those of 128 and 256 channels, whose epilogue works in blocks (64 -> 256
-            // 1x1 130 us without, 145 with sums, a pass of its own 95; 256 -> 1024 51 and 57, 27).  Other wide ones are fused where that takes less
-            // than one more pass over the output.  Cycles of a unit, measured on 1024-image layers: 530 per 32 columns for the epilogue's
+            // Tiles of up to 64 channels sum at next to no cost, and so do those of 128 and 256 channels where the epilogue works in blocks (64 -> 256
+            // 1x1 130 us without, 145 with sums, a pass of its own 95; 256 -> 1024 51 and 57, 27).  Other wide ones, and those whose ring leaves no
+            // room for blocks (3x3 64 -> 256 at 16x16: 74 without, 105 with sums, a pass of its own 29), are fused where that takes less than one more pass over the output.  Cycles of a unit, measured on 1024-image layers: 530 per 32 columns for the epilogue's
             // stores and 600 for its sums, both hidden as far as the MMAs or the unit's share of the HBM traffic (24 B/clk per SM) take longer;
             // the pass of its own 410 per 32 columns (5.5 TB/s) and about 5500 for the launch, spread over the units of a CTA.
             int n_tile = 16;
@@ -507,7 +507,14 @@ b2c_status b2c_net_create_concurrent(b2c_ctx* ctx, const b2c_layer_desc* layers,
                 const double hidden = mma > hbm ? mma : hbm;
                 const double plain = hidden > 530.0 * x ? hidden : 530.0 * x, fused = hidden > 1130.0 * x ? hidden : 1130.0 * x;
                 const char* e2 = std::getenv("B2C_FUSE_WIDE");   // 1: always; 0: never; default: by the rule above
-                const bool wide_ok = e2 ? e2[0] != '0' : n_tile == 128 || n_tile == 256 || fused - plain <= 410.0 * x + 5500.0 / (units > 1.0 ? units : 1.0);
+                bool wide_ok = fused - plain <= 410.0 * x + 5500.0 / (units > 1.0 ? units : 1.0);   // (always with up to three units per CTA)
+                if (!wide_ok) {
+                    KMajorProblem pb{};
+                    pb.n = batch; pb.ih = L.d.h; pb.iw = L.d.w; pb.ic = L.c_pad; pb.oh = L.p; pb.ow = L.q; pb.oc = L.d.k;
+                    pb.r = L.gemm_r; pb.stride = L.d.stride; pb.pad = (L.gemm_r - 1) / 2;
+                    wide_ok = kmajor_sums_in_blocks(ctx, pb);
+                }
+                if (e2) wide_ok = e2[0] != '0';
                 if (!wide_ok) o.fused_stats = false;
             }
         }

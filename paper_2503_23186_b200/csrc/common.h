@@ -152,6 +152,9 @@ struct KMajorProblem {
                            // the kernel starts as SMs fall free and waits for that launch only at its end
 };
 b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_t stream);
+// Whether a forward convolution with BatchNorm sums works in blocks in its epilogue.  Asks the planner, without launching anything; for problems
+// of more than two units per CTA it asks the device nothing.
+bool kmajor_sums_in_blocks(b2c_ctx* ctx, KMajorProblem pb);
 b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan_detail& out);   // pointers of the problem: null
 
 struct WgradProblem {

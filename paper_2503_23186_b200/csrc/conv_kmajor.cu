@@ -1749,6 +1749,15 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
 
 static int kernel_kind(const ConvKParams& p) { return p.hm ? KIND_HMERGE : p.fh ? KIND_FULL_HALO : p.issue_split ? KIND_SPLIT : KIND_GENERAL; }
 
+bool kmajor_sums_in_blocks(b2c_ctx* ctx, KMajorProblem pb)
+{
+    pb.in = pb.wt = pb.out = nullptr;
+    pb.stats = nullptr;
+    pb.ask_sums = true;
+    KMajorPlan plan;
+    return build_kmajor_plan(ctx, pb, plan) == B2C_OK && plan.p.block_cols != 0;
+}
+
 b2c_status plan_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, b2c_conv_plan_detail& detail)
 {
     static_assert((int)KIND_GENERAL == B2C_PLAN_GENERAL && (int)KIND_SPLIT == B2C_PLAN_SHARED_UNITS && (int)KIND_HMERGE == B2C_PLAN_MERGED_TAPS &&

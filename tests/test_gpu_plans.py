@@ -109,3 +109,23 @@ def test_plan_of_a_call_with_sums(ctx):
     for which in ("dgrad", "wgrad"):
         with pytest.raises(binding.B2CError):
             ctx.conv2d_plan(d, which, sums=True)
+
+
+# 256-channel outputs of 1024 images: 3x3 layers whose ring leaves no room for the epilogue's blocks take the statistics in a pass of their own
+@pytest.mark.parametrize("c,r,blocks", [(64, 3, False), (64, 1, True), (128, 1, True)])
+def test_statistics_in_the_epilogue_where_it_works_in_blocks(ctx, c, r, blocks):
+    from paper_2503_23186_b200 import binding, workloads as wl
+    n, hw, k = 1024, 16, 256
+    plan = ctx.conv2d_plan(binding.conv_desc(n, hw, hw, c, k, r, 1), "fwd", sums=True)
+    assert (plan["block_cols"] != 0) == blocks, plan
+    spec = [dict(kind="conv", src=0, C=16, K=c, R=1, stride=1, pad=0, H=hw, W=hw, name="c0"), dict(kind="bn", src=1, C=c, H=hw, W=hw, relu=True, res=-1, name="b0"),
+            dict(kind="conv", src=2, C=c, K=k, R=r, stride=1, pad=r // 2, H=hw, W=hw, name="c1"), dict(kind="bn", src=3, C=k, H=hw, W=hw, relu=True, res=-1, name="b1"),
+            dict(kind="avgpool", src=4, C=k, H=hw, W=hw, name="pool"), dict(kind="fc", src=5, C=k, K=10, name="fc"), dict(kind="xent", src=6, K=10, name="xent")]
+    net = binding.Net(ctx, spec, n)
+    net.load_params(wl.init_params(spec, 1))
+    net.profile_read()
+    net.train_step(torch.zeros((n, hw, hw, 16), dtype=torch.bfloat16, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda"), 1, 0.1, 0.9, 0.0, update=False)
+    assert ctx.device_status() == 0
+    _, launches = net.profile_read()
+    assert launches["bn_fwd"] == (2 if blocks else 3), launches   # an apply pass each, and the statistics' own
+    net.close()
