@@ -508,6 +508,59 @@ struct WgradPlan {
     size_t smem_bytes;
 };
 
+// Pixel chunk of a layer with x tiles of `ct` channels (p.stack, p.fx and the box widths are set), and the bytes of its stage.
+struct WgChunk {
+    int pb, box_a, box_b, a_bytes, fx_tx, fx_box, bytes, bw, bh, bn, tiles_w, tiles_h, total;
+};
+static WgChunk chunk_of(const WgradParams& p, const WgradProblem& pb, int ct)
+{
+    const int shifts = pb.r == 3 ? 3 : 1, b_boxes = ct / p.cw_b;
+    WgChunk k = {};
+    k.pb = 64;   // 64 pixels, or 32 when a 64-pixel stage would not leave room for three stages
+    for (;;) {
+        k.box_a = k.pb * p.cw_a * 2;
+        k.box_b = k.pb * p.cw_b * 2;
+        k.a_bytes = p.stack ? (k.pb + (pb.q < k.pb ? pb.q : k.pb)) * p.cw_a * 2 : 128 / p.cw_a * k.box_a;   // stacked: one box with a halo row
+        k.bytes = k.a_bytes + shifts * b_boxes * k.box_b;
+        if (p.fx) {
+            const int bw = pb.q < k.pb ? pb.q : k.pb, bh = k.pb / bw;
+            k.fx_tx = (bw + 2) * bh * p.cw_b * 2;
+            k.fx_box = (k.fx_tx + 1023) & ~1023;
+            k.bytes = k.a_bytes + b_boxes * k.fx_box;
+        }
+        if (k.bytes * 3 <= 200 * 1024 || k.pb == 32) break;
+        k.pb = 32;
+    }
+    k.bw = pb.q < k.pb ? pb.q : k.pb;
+    k.bh = (k.pb / k.bw) < pb.p ? (k.pb / k.bw) : pb.p;
+    k.bn = k.pb / (k.bw * k.bh);
+    k.tiles_w = pb.q / k.bw;
+    k.tiles_h = (pb.p + (p.stack ? 1 : 0) + k.bh - 1) / k.bh;   // stacked: dy copy 1 of row p-1 is met at chunk row p
+    k.total = k.tiles_w * k.tiles_h * ((pb.n + k.bn - 1) / k.bn);
+    return k;
+}
+
+// CTAs that share a tile's chunks: one wave of one CTA per SM, at least four chunks each
+static int splits_of(const b2c_ctx* ctx, int tiles, long long chunks)
+{
+    long long splits = ctx->sm_count / tiles < chunks / 4 ? ctx->sm_count / tiles : chunks / 4;
+    return splits < 1 ? 1 : (int)splits;
+}
+
+// Tiles that do not divide the SMs evenly leave many of them idle (75 tiles: one CTA each on 148 SMs: 640 -> 640 at 8x8 with 256 images 135 us, now 82).  Equal runs of (tile, chunk)
+// pairs keep all busy, at the price of one more accumulator to send for most CTAs (about 9000 cycles).
+static bool equal_runs(const b2c_ctx* ctx, const WgradParams& p, const WgradProblem& pb, int ct, int tiles)
+{
+    const WgChunk k = chunk_of(p, pb, ct);
+    const int splits = splits_of(ctx, tiles, k.total), cols = (pb.r == 3 ? 3 : 1) * ct;
+    const double mma = (k.pb / 16) * (cols / 2.0), load = k.bytes / 60.0, chunk = mma > load ? mma : load, tail = 9000.0;
+    const int waves = (tiles * splits + ctx->sm_count - 1) / ctx->sm_count;
+    const double plain = waves * (((k.total + splits - 1) / splits) * chunk + tail);
+    const double per_cta = (double)tiles * k.total / ctx->sm_count;   // chunks
+    const double equal = per_cta * chunk + ((double)tiles / ctx->sm_count + 1.0) * tail;
+    return per_cta >= 8.0 && equal < 0.85 * plain;   // (an estimated tenth was measured as a loss: 320 -> 320 at 16x16 107 -> 111 us)
+}
+
 static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPlan& plan)
 {
     WgradParams& p = plan.p;
@@ -563,21 +616,21 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     // 9.8 / 13.8 / 21.1 / 38.0, 256 -> 512 at 8x8 stride 2 with 50 / 128 11.9 / 13.9 and 8.3 / 10.7, 512 -> 512 at 4x4 with 50 / 128 13.0 /
     // 17.0 and 11.2 / 18.2, 128 -> 256 at 16x16 stride 2 with 1024 40.9 and 46.1.  Filter rows on M: 160 -> 160 at 32x32 with 256 images
     // 151 -> 112 us, 16 -> 160 61 -> 44, 16 -> 16 at 32x32 with 512 images 72 -> 29, 32 -> 32 at 16x16 with 1024 25 -> 13, 48 -> 48 at 32x32 with
-    // 128 33 -> 24; not where they save nothing: 64 -> 32 at 16x16 with 16 6.6 -> 7.9.
+    // 128 33 -> 24; not where they save nothing: 64 -> 32 at 16x16 with 16 6.6 -> 7.9.  Whether a width's tiles are walked in equal runs is decided as
+    // for the plan itself (with an estimate of its own here, half of the widest tile took 640 -> 640 at 8x8 with 8 images from 13.4 to 17.6 us,
+    // 1024 -> 640 at 8x8 with 228 from 114 to 127, 512 -> 640 at 32x32 with 24 from 95 to 103).
     if (R == 3) {
         const long long chunks = ((long long)pb.n * pb.p * pb.q + 63) / 64;
         const int m_rows = p.stack ? 2 : 3 * ((pb.k + 127) / 128), m_shared = (3 * pb.k + 127) / 128;   // tiles of M
         auto cycles = [&](int ct, int m_tiles) {
             const int tiles = m_tiles * (pb.c / ct);
-            long long splits = ctx->sm_count / tiles < chunks / 4 ? ctx->sm_count / tiles : chunks / 4;
-            if (splits < 1) splits = 1;
+            const long long splits = splits_of(ctx, tiles, chunks);
             // MMAs of a chunk of 64 pixels (128 x n x 16: n / 2 cycles, or its operands at 128 B/clk) and its loads at about 60 B/clk
             auto mma = [](int n) { return 4 * (n / 2 > 32 + n / 4 ? n / 2 : 32 + n / 4); };
             const int work = p.fx ? ct / p.cw_b * mma(3 * p.cw_b) : 3 * ct <= 256 ? mma(3 * ct) : 2 * ct <= 256 ? mma(2 * ct) + mma(ct) : 3 * mma(ct);
             const int load = (128 + (p.fx ? ct * 5 / 4 : 3 * ct)) * 128 / 60, chunk = work > load ? work : load, tail = 1500 + 69 * ct;
-            const long long plain = (tiles * splits + ctx->sm_count - 1) / ctx->sm_count * ((chunks + splits - 1) / splits * chunk + tail);
-            const long long equal = (tiles * chunks / ctx->sm_count + 1) * chunk + (tiles + ctx->sm_count) * (long long)tail / ctx->sm_count;   // (equal runs, see below)
-            return tiles * chunks >= 8ll * ctx->sm_count && equal * 100 < plain * 85 ? equal : plain;
+            if (equal_runs(ctx, p, pb, ct, tiles)) return (tiles * chunks / ctx->sm_count + 1) * chunk + (tiles + ctx->sm_count) * (long long)tail / ctx->sm_count;
+            return (tiles * splits + ctx->sm_count - 1) / ctx->sm_count * ((chunks + splits - 1) / splits * chunk + tail);
         };
         const bool may_share = pb.stride == 1 && !p.stack && m_shared < m_rows;
         const int widest_ct = p.ct;
@@ -650,27 +703,15 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
         }
     }
 
-    // pixel chunk: 64 pixels, or 32 when a 64-pixel stage would not leave room for three stages
-    p.pb = 64;
-    for (;;) {
-        p.box_a = p.pb * p.cw_a * 2;
-        p.box_b = p.pb * p.cw_b * 2;
-        p.a_bytes = p.stack ? (p.pb + (pb.q < p.pb ? pb.q : p.pb)) * p.cw_a * 2 : p.a_boxes * p.box_a;   // stacked: one box with a halo row
-        p.stage_bytes = p.a_bytes + shifts * p.b_boxes * p.box_b;
-        if (p.fx) {
-            const int bw = pb.q < p.pb ? pb.q : p.pb, bh = p.pb / bw;
-            p.fx_tx = (bw + 2) * bh * p.cw_b * 2;
-            p.fx_box = (p.fx_tx + 1023) & ~1023;
-            p.stage_bytes = p.a_bytes + p.b_boxes * p.fx_box;
-        }
-        if (p.stage_bytes * 3 <= 200 * 1024 || p.pb == 32) break;
-        p.pb = 32;
-    }
+    const WgChunk chunk = chunk_of(p, pb, p.ct);
+    p.pb = chunk.pb;
+    p.box_a = chunk.box_a; p.box_b = chunk.box_b; p.a_bytes = chunk.a_bytes;
+    p.fx_tx = chunk.fx_tx; p.fx_box = chunk.fx_box;
     if (p.fx && p.pb != 64) return B2C_ERR_UNSUPPORTED_SHAPE;   // cannot happen: a framed stage is under 40 KB
     // Chunks with few MMAs share a ring slot (an issuing thread pays 700-900 cycles per slot for the barrier wait and the
     // commits on top of its MMAs): two chunks per slot where one holds under half of that in tensor-pipe cycles and four
     // slots remain.
-    p.sub_bytes = p.stage_bytes;
+    p.sub_bytes = chunk.bytes;
     p.gsub = 1;
     {
         const int total_cols = p.fx ? p.b_boxes * 3 * p.cw_b : shifts * p.ct;
@@ -686,9 +727,9 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
     if (stages >= 4) stages &= ~1;
     p.issuers = (stages % 2 == 0 && ctx->use_wgrad_two_issuers) ? kWgIssuers : 1;
     p.stages = stages;
-    p.bw = pb.q < p.pb ? pb.q : p.pb;
-    p.bh = (p.pb / p.bw) < pb.p ? (p.pb / p.bw) : pb.p;
-    p.bn = p.pb / (p.bw * p.bh);
+    p.bw = chunk.bw;
+    p.bh = chunk.bh;
+    p.bn = chunk.bn;
     if (p.stack && p.bn != 1) return B2C_ERR_UNSUPPORTED_SHAPE;   // cannot happen: 64 pixels per image guarantee bn == 1
     if (p.fx) {
         if (p.bn != 1) return B2C_ERR_UNSUPPORTED_SHAPE;   // cannot happen: at least 64 pixels per image
@@ -698,32 +739,18 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
         }
         p.fx_sbo = (uint32_t)((p.bw == 8 ? 10 : 8) * p.cw_b * 2);   // eight pixel rows, or one framed image row of ten
     }
-    p.tiles_w = pb.q / p.bw;
+    p.tiles_w = chunk.tiles_w;
     p.tw_shift = 0;
     while ((1 << p.tw_shift) < p.tiles_w) ++p.tw_shift;
     p.a_lbo = p.stack ? p.bw * p.cw_a * 2 : p.box_a;   // stacked: copy 0 starts one image row below copy 1
-    p.tiles_h = (pb.p + (p.stack ? 1 : 0) + p.bh - 1) / p.bh;   // stacked: dy copy 1 of row p-1 is met at chunk row p
-    const int tiles_n = (pb.n + p.bn - 1) / p.bn;
-    p.chunks_total = p.tiles_w * p.tiles_h * tiles_n;
+    p.tiles_h = chunk.tiles_h;
+    p.chunks_total = chunk.total;
     const int base = p.n_ktiles * p.n_ctiles * p.n_groups;
-    int n_splits = ctx->sm_count / base;   // one wave of one CTA per SM
-    if (n_splits > p.chunks_total / 4) n_splits = p.chunks_total / 4;
-    if (n_splits < 1) n_splits = 1;
-    p.n_splits = n_splits;
-    // Tiles that do not divide the SMs evenly leave many of them idle (75 tiles: one CTA each on 148 SMs: 640 -> 640 at 8x8 with 256 images 135 us, now 82).  Equal runs of (tile, chunk)
-    // pairs keep all busy, at the price of one more accumulator to send for most CTAs (about 9000 cycles).
-    {
-        const int cols = p.fx ? p.b_boxes * 3 * p.cw_b : shifts * p.ct;
-        const double mma = (p.pb / 16) * (cols / 2.0), load = p.sub_bytes / 60.0, chunk = mma > load ? mma : load, tail = 9000.0;
-        const int waves = (base * n_splits + ctx->sm_count - 1) / ctx->sm_count;
-        const double plain = waves * (((p.chunks_total + n_splits - 1) / n_splits) * chunk + tail);
-        const double per_cta = (double)base * p.chunks_total / ctx->sm_count;   // chunks
-        const double equal = per_cta * chunk + ((double)base / ctx->sm_count + 1.0) * tail;
-        p.stream = per_cta >= 8.0 && equal < 0.85 * plain ? 1 : 0;   // (an estimated tenth was measured as a loss: 320 -> 320 at 16x16 107 -> 111 us)
-    }
+    p.n_splits = splits_of(ctx, base, p.chunks_total);
+    p.stream = equal_runs(ctx, p, pb, p.ct, base) ? 1 : 0;
 
     plan.smem_bytes = (size_t)p.stages * p.stage_bytes + 1024;
-    plan.grid = p.stream ? ctx->sm_count : base * n_splits;
+    plan.grid = p.stream ? ctx->sm_count : base * p.n_splits;
     if (pb.dy == nullptr) return B2C_OK;   // a question about the plan
 
     if (!encode_activation_map(ctx, &p.tmDy, pb.dy, pb.n, pb.p, pb.q, pb.k, 1, 0, 0, p.cw_a, p.bw, p.stack ? p.bh + 1 : p.bh, p.bn)) return B2C_ERR_CUDA;

@@ -129,3 +129,14 @@ def test_statistics_in_the_epilogue_where_it_works_in_blocks(ctx, c, r, blocks):
     _, launches = net.profile_read()
     assert launches["bn_fwd"] == (2 if blocks else 3), launches   # an apply pass each, and the statistics' own
     net.close()
+
+
+# x tiles of 3x3 weight gradients: half of the widest where the sending of partial sums is most of the launch; not where half the width makes a
+# second wave of a few CTAs, or gives up equal runs
+@pytest.mark.parametrize("shape,tile,kind", [
+    ((50, 16, 16, 128, 128, 3, 1), 64, "wgrad"), ((128, 8, 8, 256, 512, 3, 2), 64, "wgrad"), ((600, 16, 16, 128, 128, 3, 1), 128, "wgrad"),
+    ((8, 8, 8, 640, 640, 3, 1), 128, "wgrad"), ((24, 32, 32, 512, 640, 3, 1), 128, "wgrad-runs"), ((228, 8, 8, 1024, 640, 3, 1), 128, "wgrad")],
+    ids=lambda v: "n{}h{}w{}c{}k{}r{}s{}".format(*v) if isinstance(v, tuple) else str(v))
+def test_tile_width_of_weight_gradients(ctx, shape, tile, kind):
+    plan = _plan(ctx, "wgrad", shape)
+    assert plan["tile_channels"] == tile and plan["kind"] == kind, plan
