@@ -135,6 +135,7 @@ def test_statistics_in_the_epilogue_where_it_works_in_blocks(ctx, c, r, blocks):
 # second wave of a few CTAs, or gives up equal runs
 @pytest.mark.parametrize("shape,tile,kind", [
     ((50, 16, 16, 128, 128, 3, 1), 64, "wgrad"), ((128, 8, 8, 256, 512, 3, 2), 64, "wgrad"), ((600, 16, 16, 128, 128, 3, 1), 128, "wgrad"),
+    ((9, 32, 32, 256, 16, 3, 2), 128, "wgrad"), ((14, 32, 32, 160, 16, 3, 2), 160, "wgrad"), ((10, 8, 8, 640, 16, 3, 2), 64, "wgrad"),   # 16 output channels
     ((8, 8, 8, 640, 640, 3, 1), 128, "wgrad"), ((24, 32, 32, 512, 640, 3, 1), 128, "wgrad-runs"), ((228, 8, 8, 1024, 640, 3, 1), 128, "wgrad")],
     ids=lambda v: "n{}h{}w{}c{}k{}r{}s{}".format(*v) if isinstance(v, tuple) else str(v))
 def test_tile_width_of_weight_gradients(ctx, shape, tile, kind):
