@@ -436,7 +436,7 @@ static b2c_status splitk_optin(b2c_ctx* ctx)
 {
     if (!(ctx->smem_optin_done & B2C_OPTIN_SPLITK)) {
         for (auto* k : {conv_splitk_kernel<false, false, false>, conv_splitk_kernel<false, true, false>, conv_splitk_kernel<true, false, false>, conv_splitk_kernel<true, true, false>,
-                        conv_splitk_kernel<false, false, true>, conv_splitk_kernel<true, false, true>})
+                        conv_splitk_kernel<false, false, true>, conv_splitk_kernel<false, true, true>, conv_splitk_kernel<true, false, true>, conv_splitk_kernel<true, true, true>})
             B2C_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024));
         ctx->smem_optin_done |= B2C_OPTIN_SPLITK;
     }
@@ -472,9 +472,11 @@ b2c_status launch_conv_splitk(b2c_ctx* ctx, const ConvKParams& p, int grid, size
     if (st != B2C_OK) return st;
     const unsigned cluster = (unsigned)(p.splits * (p.pair ? 2 : 1));
     const bool timed = p.stall != nullptr;
-    auto* kernel = p.bwd_y != nullptr ? (p.pair ? conv_splitk_kernel<true, false, true> : conv_splitk_kernel<false, false, true>)
-                   : p.pair           ? (timed ? conv_splitk_kernel<true, true, false> : conv_splitk_kernel<true, false, false>)
-                                      : (timed ? conv_splitk_kernel<false, true, false> : conv_splitk_kernel<false, false, false>);
+    const bool bwd = p.bwd_y != nullptr;
+    auto* kernel = p.pair ? (timed ? (bwd ? conv_splitk_kernel<true, true, true> : conv_splitk_kernel<true, true, false>)
+                                   : (bwd ? conv_splitk_kernel<true, false, true> : conv_splitk_kernel<true, false, false>))
+                          : (timed ? (bwd ? conv_splitk_kernel<false, true, true> : conv_splitk_kernel<false, true, false>)
+                                   : (bwd ? conv_splitk_kernel<false, false, true> : conv_splitk_kernel<false, false, false>));
     B2C_CUDA(b2c_launch(ctx, kernel, dim3((unsigned)grid), dim3(kSkThreads), smem_bytes, stream, cluster, p));
     B2C_CUDA(cudaGetLastError());
     return B2C_OK;

@@ -55,3 +55,35 @@ def test_sums_with_the_data_gradient(name):
         net.close()
     finally:
         ctx.close()
+
+
+def test_stall_counters_of_launches_with_sums(monkeypatch):
+    """The data gradients that take sums add their cycles to the diagnostics like the others: seven of fifteen forward and data-gradient launches."""
+    from paper_2503_23186_b200 import binding
+    spec = [dict(kind="conv", src=0, C=16, K=64, R=1, stride=1, pad=0, H=8, W=8, name="c0"), dict(kind="bn", src=1, C=64, H=8, W=8, relu=True, res=-1, name="b0")]
+    for i in range(7):
+        spec.append(dict(kind="conv", src=len(spec), C=64, K=64, R=3, stride=1, pad=1, H=8, W=8, name=f"c{i + 1}"))
+        spec.append(dict(kind="bn", src=len(spec), C=64, H=8, W=8, relu=True, res=-1, name=f"b{i + 1}"))
+    spec += [dict(kind="avgpool", src=len(spec), C=64, H=8, W=8, name="pool"), dict(kind="fc", src=len(spec) + 1, C=64, K=10, name="fc"),
+             dict(kind="xent", src=len(spec) + 2, K=10, name="xent")]
+    waited = {}
+    for fuse in ("0", "1"):
+        monkeypatch.setenv("B2C_FUSE_BN_BWD", fuse)
+        ctx = binding.Context(0)
+        net = binding.Net(ctx, spec, 16)
+        net.load_params(wl.init_params(spec, 5))
+        images, labels = dev_bf16(wl.image_batch(5, 16, hw=8, c=16, classes=10)[0]), torch.zeros(16, dtype=torch.int32, device="cuda")
+        counters = torch.zeros(8, dtype=torch.int64, device="cuda")
+        for passes in (3, 10):   # the first ones load the kernels
+            net.profile_read()
+            ctx.set_stall_counters(counters.zero_())
+            for _ in range(passes):
+                net.train_step(images, labels, 1, 0.1, 0.9, 0.0, update=False)
+            assert ctx.device_status() == 0
+            _, launches = net.profile_read()
+        waited[fuse] = counters[3].item()   # (the weight gradient does not add to this one)
+        assert (launches["bn_bwd"] < 2 * 8 * 10) == (fuse == "1"), launches
+        ctx.set_stall_counters(None)
+        net.close()
+        ctx.close()
+    assert waited["1"] > 0.8 * waited["0"], waited
