@@ -1820,8 +1820,8 @@ b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_
         {{conv_kmajor_kernel<false, KIND_GENERAL, false>, conv_kmajor_kernel<false, KIND_SPLIT, false>, conv_kmajor_kernel<false, KIND_HMERGE, false>,
           conv_kmajor_kernel<false, KIND_FULL_HALO, false>},
          {conv_kmajor_kernel<true, KIND_GENERAL, false>, conv_kmajor_kernel<true, KIND_SPLIT, false>, nullptr, conv_kmajor_kernel<true, KIND_FULL_HALO, false>}},
-        {{conv_kmajor_kernel<false, KIND_GENERAL, true>, conv_kmajor_kernel<false, KIND_SPLIT, true>, conv_kmajor_kernel<false, KIND_HMERGE, true>,
-          conv_kmajor_kernel<false, KIND_FULL_HALO, true>},
+        // (128-channel tiles: the filter bank of a full-halo plan fits only halved, for a pair)
+        {{conv_kmajor_kernel<false, KIND_GENERAL, true>, conv_kmajor_kernel<false, KIND_SPLIT, true>, conv_kmajor_kernel<false, KIND_HMERGE, true>, nullptr},
          {conv_kmajor_kernel<true, KIND_GENERAL, true>, conv_kmajor_kernel<true, KIND_SPLIT, true>, nullptr, conv_kmajor_kernel<true, KIND_FULL_HALO, true>}}};
     const kernel_t kernel = kernels[p.block_cols ? 1 : 0][p.pair ? 1 : 0][kernel_kind(p)];
     if (kernel == nullptr) return B2C_ERR_UNSUPPORTED_SHAPE;
