@@ -37,8 +37,10 @@
  *       B2C_BN_GROUPED=1     b2c_train_step runs the BatchNorm backward as one cooperative launch per layer, group by group
  *                            (b2c_bn_relu_bwd_groups); off by default: measured slower inside the step
  *       B2C_FUSE_WIDE=0|1    BatchNorm statistics of tiles wider than 64 channels: never | always in the convolution epilogue
- *                            (default: where the epilogue's sums cost less than a pass of their own)
+ *                            (default: where the epilogue works in blocks, or its sums cost less than a pass of their own)
  *       B2C_FUSE_BN_STATS=0  BatchNorm statistics by a separate pass instead of the convolution epilogue (b2c_train_step)
+ *       B2C_FUSE_BN_BWD=0    sums of the BatchNorm backward always by a pass of their own instead of, where the one-wave kernel computes the
+ *                            last contribution to the gradient, in that data gradient's epilogue (b2c_train_step)
  *       B2C_CHUNK_MB=<n>     b2c_train_step takes layers whose tensors exceed n MB a few micro-batches at a time (0 = off, default)
  */
 #ifndef B2C_H_

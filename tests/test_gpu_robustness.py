@@ -178,10 +178,10 @@ def test_kernel_switches_off_and_on(name, value, monkeypatch):
 
 
 @pytest.mark.parametrize("name,value", [("B2C_FUSE_WIDE", "0"), ("B2C_FUSE_WIDE", "1"), ("B2C_FUSE_BN_STATS", "0"), ("B2C_FUSE_BN_STATS", "1"),
-                                        ("B2C_BN_GROUPED", "1"), ("B2C_BN_GROUPED", "0")], ids=lambda v: str(v))
+                                        ("B2C_BN_GROUPED", "1"), ("B2C_BN_GROUPED", "0"), ("B2C_FUSE_BN_BWD", "0"), ("B2C_FUSE_BN_BWD", "1")], ids=lambda v: str(v))
 def test_step_plan_switches_off_and_on(name, value, monkeypatch):
-    """The switches b2c_net_create / b2c_train_step read: where the BatchNorm statistics are taken, and the grouped BatchNorm
-    backward.  One pass of four micro-batches side by side, every layer against the oracle on its own device inputs."""
+    """The switches b2c_net_create / b2c_train_step read: where the BatchNorm statistics and the sums of the backward pass are taken, and the
+    grouped BatchNorm backward.  One pass of four micro-batches side by side, every layer against the oracle on its own device inputs."""
     from paper_2503_23186_b200 import binding
     from netcheck import check_step
     monkeypatch.setenv(name, value)
