@@ -640,12 +640,12 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
         for (int cand = widest_ct - p.cw_b; cand >= p.cw_b; cand -= p.cw_b) {
             if (pb.c % cand) continue;
             for (int sh = 0; sh <= (may_share ? 1 : 0); ++sh) {
-                // With 16 output channels a narrower tile means that more CTAs gather the same few 32-byte rows of dy: beyond about 48 CTAs that costs
+                // With 16 output channels a narrower tile means that more CTAs gather the same few 32-byte rows of dy: beyond about 64 CTAs that costs
                 // more than the shorter tail gives, except with one framed x box per chunk.  Widest / narrower tile, one filter row at a time: 1024 ->
                 // 16 at 4x4 with 44 images 10.5 / 14.1 us, 96 -> 16 at 8x8 with 63 9.8 / 12.4, 160 -> 16 at 32x32 stride 2 with 14 10.0 / 15.2, but
-                // 640 -> 16 at 4x4 with 12 (30 CTAs) 7.8 / 6.3 and 128 -> 16 at 32x32 with 5 (framed) 8.7 / 7.2.
+                // 640 -> 16 at 4x4 with 12 (30 CTAs) 7.8 / 6.3, 112 -> 16 at 4x4 stride 2 with 180 (63) 9.6 / 8.3 and 128 -> 16 at 32x32 with 5 (framed) 8.7 / 7.2.
                 const int tiles = (sh ? m_shared : m_rows) * (pb.c / cand);
-                if (!sh && pb.k <= 16 && tiles * splits_of(ctx, tiles, chunks) > 48 && !(p.fx && p.cw_b == 64)) continue;
+                if (!sh && pb.k <= 16 && tiles * splits_of(ctx, tiles, chunks) > 64 && !(p.fx && p.cw_b == 64)) continue;
                 const long long est = cycles(cand, sh ? m_shared : m_rows);
                 if (est < best) { best = est; p.ct = cand; share = sh != 0; }
             }
