@@ -413,8 +413,8 @@ __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tme
 // Layers of 1024 images inside a step, epilogue_loop -> this: with sums 64 -> 256 1x1 at 32x32 312 -> 145 us (sums in a pass of their own: 139 +
 // 95), 128 -> 512 at 16x16 166 -> 84, 64 -> 64 3x3 80 -> 71, 128 -> 128 3x3 at 16x16 77 -> 63, 64 -> 128 1x1 stride 2 60 -> 41, 512 -> 512 at 4x4
 // 65 -> 63; without sums data gradient 256 <- 64 1x1 137 -> 126, 512 <- 128 81 -> 71, 64 <- 64 3x3 66 -> 63.
-// Every four units the running squares move on to a second sum in local memory, and what that addition rounds off stays behind: squares of
-// positive outputs of 2048 images (16 -> 64 1x1) are 2.1e-9 off, 4.3e-8 without the remainder, of 1024 images (128 -> 512 1x1) 7.9e-9 and 1.0e-8.
+// Every four units the running squares move on to a second sum in local memory, and what that addition rounds off stays behind (not with blocks
+// of 16 columns, where the sixteen pairs' extra instructions and spills cost 128 -> 128 at 16x16 66.9 -> 74.7 us inside a step): squares of positive outputs of 2048 images (16 -> 64 1x1) are 2.1e-9 off, 4.3e-8 without the remainder, of 1024 images (128 -> 512 1x1) 7.9e-9 and 1.0e-8.
 // Tiles of 64 channels have registers for a second plain sum too (16 -> 64 1x1 with 1024 images 49.7 -> 50.6 us for both); wider ones keep
 // one for the whole statistics group, as in epilogue_loop: sums of 1024 images with a mean are 0.2-1.4e-9 of their magnitudes off, there and here.
 template <int BC, int NB, bool HM, bool STATS>
@@ -480,10 +480,10 @@ __device__ __forceinline__ int2 epilogue_blocks(const ConvKParams& p, uint32_t t
         const f32x2 minus_one = make_f32x2(-1.f, -1.f);
 #pragma unroll
         for (int i = 0; i < NA; ++i) {
-            // (what the addition rounds off stays behind)
             const f32x2 old_q = long_q[i + opaque_zero], new_q = add_f32x2(old_q, acc_q[i]);
             long_q[i + opaque_zero] = new_q;
-            acc_q[i] = add_f32x2(acc_q[i], fma_f32x2(new_q, minus_one, old_q));
+            if constexpr (BC != 16) acc_q[i] = add_f32x2(acc_q[i], fma_f32x2(new_q, minus_one, old_q));   // what the addition rounds off stays behind
+            else acc_q[i] = 0ull;
             if constexpr (LONG_S) {
                 long_s[i] = add_f32x2(long_s[i], acc_s[i]);
                 acc_s[i] = 0ull;
