@@ -76,8 +76,8 @@ struct b2c_ctx {
     } while (0)
 
 // Kernel launch.  With ctx->use_pdl the launch carries the programmatic-stream-serialization attribute: the kernel may be
-// scheduled while the previous kernel of the stream drains, and it orders itself behind that kernel with pdl_wait()
-// (every kernel of the library calls it before its first global access).  cluster > 1 launches thread-block clusters.
+// scheduled while the previous kernel of the stream drains, and it orders itself behind that kernel with pdl_wait() before its first
+// global access; convolutions launched with no_wait do so at their end (pdl_begin, pdl_end).  cluster > 1 launches thread-block clusters.
 template <typename... KArgs, typename... Args>
 static inline cudaError_t b2c_launch(const b2c_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                      unsigned cluster, Args&&... args)
@@ -148,8 +148,8 @@ struct KMajorProblem {
     const void* bwd_mask;    // one bit per element, or nullptr
     bool* bwd_done;          // set to whether the launch takes the sums
     bool ask_sums;         // a question about the plan of a call with `stats`
-    bool no_wait;          // the launch right before this one shares nothing that is written with this one, and itself waits for the one before it:
-                           // the kernel starts as SMs fall free and waits for that launch only at its end
+    bool no_wait;          // the launch right before this one shares nothing that is written with this one, and itself waits for the one before it
+                           // (it is not no_wait): the kernel starts as SMs fall free and waits for that launch only at its end
 };
 b2c_status launch_conv_kmajor(b2c_ctx* ctx, const KMajorProblem& pb, cudaStream_t stream);
 // Whether a forward convolution with BatchNorm sums works in blocks in its epilogue.  Asks the planner, without launching anything; for problems

@@ -77,22 +77,23 @@ __device__ __forceinline__ int unit_stages(const ConvKParams& p, int par)
     return p.gsub > 1 ? (n + p.gsub - 1) / p.gsub : n;
 }
 
-// Epilogue of one warp over all units of the CTA, for the tile widths and plans that epilogue_blocks does not take.  Epilogue warp e reads the TMEM lane quarter its warp index selects and the column half e >> 2
-// of every accumulator.  The warp owns at most NCH 16-column chunks per unit.  EAGER: it reads all
+// Epilogue of one warp over all units of the CTA, for the tile widths and plans that epilogue_blocks does not take (up to 48 channels, 80 to 112,
+// 144 to 240; rings that leave no room; a bias or fp32 output).  Epilogue warp e reads the TMEM lane quarter its warp index selects and the column
+// half e >> 2 of every accumulator.  The warp owns at most NCH 16-column chunks per unit.  EAGER: it reads all
 // its columns at once and hands the accumulator back before packing and storing (narrow tiles).
 // STATS: BatchNorm sums of the values as stored, kept in registers until the statistics group ends; those of the last group are left
 // in my_stats ([0, 128) sums, [128, 256) sums of squares) for the CTA to add up.  Returns that group and channel tile (-1: none).
 //   * EAGER: a lane sums its own row's columns (32 registers per chunk), a butterfly reduces over the rows once per group.
 //   * wide tiles: two exchanges between lanes first (add_chunk), a quarter of the registers and about 65 instructions per chunk.
-//     Bound: issue slots and latency of eight warps.  Measured with 1024 images, forward with sums, 128 -> 128 at 16x16 and 1x1
-//     64 -> 256 at 32x32: shuffle butterfly per chunk (150 instructions) 82 and 342 us; tensor cores (m16n8k16, which queue behind the
+//     Bound: issue slots and latency of eight warps.  Measured with 1024 images, forward with sums, on layers that have since gone to the blocks,
+//     128 -> 128 at 16x16 and 1x1 64 -> 256 at 32x32: shuffle butterfly per chunk (150 instructions) 82 and 342 us; tensor cores (m16n8k16, which queue behind the
 //     convolution's own MMAs) 90 and 224; transposed through shared memory (two warp barriers and a chain of eight adds) 72 and 253;
 //     read from TMEM once more in the fragment layout 72 and 244; this 72 and 273 us (a rolled loop: 79 and 219).
 // The squares of bf16 values end in the same few bits: added one by one to a running fp32 sum they are rounded down more often than up,
 // and a chain of 200 comes out 5e-7 low.  So four squares of a wide tile meet before they reach the running sum, which moves on to a second
 // one in local memory after every few units; narrow tiles, which have no registers to spare, add their rows up in my_stats instead.
-// Sums of squares of 1024 images are 1.2e-8 off (without: 3.3e-7 on 64 -> 256 1x1, 4.6e-8 on 32 -> 64 1x1), for 275 -> 280 us on
-// 64 -> 256 1x1, 64.9 -> 66.1 on 128 -> 128 at 16x16, 76.6 -> 80.8 on 64 -> 64 at 32x32.
+// Sums of squares of 1024 images are 1.2e-8 off (measured on the same layers, without it: 3.3e-7 on 64 -> 256 1x1, 4.6e-8 on 32 -> 64 1x1; with it 1.2e-8 too on 16 -> 32 1x1, 1.3e-8 on 160 -> 160 and 64 -> 256 3x3),
+// for 275 -> 280 us on 64 -> 256 1x1, 64.9 -> 66.1 on 128 -> 128 at 16x16, 76.6 -> 80.8 on 64 -> 64 at 32x32.
 // Without STATS the code carries no accumulators: 1x1 64 -> 256 154 -> 126 us, 32 -> 64 57 -> 48 us, data gradient 256 -> 64 159 -> 132 us.
 template <int NCH, bool EAGER, bool HM, bool STATS>
 __device__ __forceinline__ int2 epilogue_loop(const ConvKParams& p, uint32_t tmem_base, uint64_t* acc_full, uint64_t* acc_empty,

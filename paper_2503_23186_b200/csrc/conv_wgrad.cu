@@ -16,6 +16,8 @@
 // Other channel counts whose last tile of 128 would be partly empty in every filter row put all three rows on M (row_blocks): with x gathered at
 // the middle row, sum_p dy[p] x[p + (r - 1, s - 1)] = sum_p dy[p - (r - 1, 0)] x[p + (0, s - 1)], so M holds (filter row, block of channels)
 // pairs back to back, each block of dy gathered at its row's height: 160 channels fill 3.75 tiles instead of 3 x 1.25 in 3 x 2.
+// (In both forms rows of dy beyond the image meet rows of x inside it as zeros: an infinity or NaN in the first or last image row of x reaches
+// all filter rows of its channel, not only those that see the row.  One filter row at a time, dy meets the zeros of x's frame instead.)
 // Partial sums of the pixel ranges are added to dw with vector fp32 reductions.
 //
 // Framed x stages (3x3, stride 1, image rows of at least 8 pixels, 64-channel x boxes): instead of one x box per
@@ -636,7 +638,8 @@ static b2c_status build_wgrad_plan(b2c_ctx* ctx, const WgradProblem& pb, WgradPl
         const int widest_ct = p.ct;
         bool share = may_share && cycles(widest_ct, m_shared) * 100 < cycles(widest_ct, m_rows) * 97;
         long long best = cycles(widest_ct, share ? m_shared : m_rows);
-        best = best * (p.cw_a == 64 && p.cw_b == 64 ? 97 : 75) / 100;   // (narrow boxes: many loads per chunk, which the estimate leaves out)
+        // (estimates within 3 % of one another, here and for the rows, decide nothing; narrow boxes: many loads per chunk, which the estimate leaves out)
+        best = best * (p.cw_a == 64 && p.cw_b == 64 ? 97 : 75) / 100;
         for (int cand = widest_ct - p.cw_b; cand >= p.cw_b; cand -= p.cw_b) {
             if (pb.c % cand) continue;
             for (int sh = 0; sh <= (may_share ? 1 : 0); ++sh) {

@@ -18,9 +18,11 @@ namespace b2c {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// The same for a kernel that needs nothing of the launch right before it (no_wait).  That launch let this one in only after its own wait,
-// so everything older has completed; reads must go through the async proxy (no stale L1 lines).  pdl_end keeps the order for the launches
-// behind this one: the grid does not complete before the one that it overtook.
+// The same for a kernel that needs nothing of the launch right before it (no_wait).  That launch let this one in only after its own wait (it
+// must not be no_wait itself), so everything older has completed; reads go through the async proxy or past the L1 (no stale lines).  pdl_end keeps
+// the order for the launches behind this one: the grid does not complete before the one that it overtook.  A kernel may thus start beside two
+// older ones, this one and the overtaken one.  TMEM allocations cannot wait in a circle: a kernel is let in only once every CTA of the one before
+// it has allocated, so a CTA waits for columns of older kernels only, and those need nothing of it.
 __device__ __forceinline__ void pdl_begin(int no_wait)
 {
     if (!no_wait) pdl_wait();
