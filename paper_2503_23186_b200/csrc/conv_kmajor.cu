@@ -1647,16 +1647,16 @@ static b2c_status build_kmajor_plan(b2c_ctx* ctx, const KMajorProblem& pb, KMajo
     // 8x8 59 -> 64 us): tiles of 64 channels 32 columns at a time; 128 and 256 channels 64 at a time, full-halo stages, which leave no room,
     // 16 at a time in the kernel's static arrays.  Tiles of 256 channels without sums whose MMAs take more than 12000 cycles hide the
     // epilogue anyway and are 1 % slower in blocks (256 -> 256 at 8x8 59.7 and 60.1 us), and so are 64-channel tiles with vertical tap reuse in
-    // k-blocks of 32 channels from 5000 cycles on, or with one k-block and no sums (rows / blocks at 32x32: 608 -> 64 with 60 images without sums
+    // k-blocks of 32 channels from 5000 cycles on, or with one k-block, no sums and more than two units per CTA (rows / blocks at 32x32: 608 -> 64 with 60 images without sums
     // 94.6 and 97.4 us, 224 -> 64 with 150 69.1 and 70.8, with sums 70.6 and 72.4, 160 -> 64 with 200 63.3 and 63.4, with sums 64.6 and 64.9; 32 ->
-    // 64 with 500 35.9 and 37.4, but with sums 38.7 and 37.5); the others gain, see epilogue_blocks.  Large 1x1 layers without sums that move as
+    // 64 with 500 35.9 and 37.4, but with sums 38.7 and 37.5, and with 4 at 64x64, one unit each, 6.6 and 6.2); the others gain, see epilogue_blocks.  Large 1x1 layers without sums that move as
     // much in as out are bound by HBM and differ by what else is in flight: 64 -> 64 at 32x32 with 1024 images on its own 47.0 by rows and 50.5
     // in blocks, as a data gradient inside a step 59 and 51.
     if (!cluster && !pb.out_f32 && pb.bias == nullptr) {
         const bool sums = (pb.stats != nullptr || pb.ask_sums) && pb.bwd_y == nullptr;
         const int room = ring_budget - p.resident_bytes - p.stages * stage_bytes;
         const int mma = R * R * pb.ic / 16 / n_par * (n_tile / 2);
-        const bool hidden = p.vreuse && p.kb == 32 && (R * R * pb.ic / 16 * 48 >= 5000 || (!sums && p.c_blocks == 1));
+        const bool hidden = p.vreuse && p.kb == 32 && (R * R * pb.ic / 16 * 48 >= 5000 || (!sums && p.c_blocks == 1 && units_per_cta > 2));
         if (n_tile == 64 && !p.fh && !hidden && room >= 16 * 1024) p.block_cols = 32;
         if (n_tile == 128) p.block_cols = p.fh ? 16 : room >= 24 * 1024 ? 64 : 0;
         if (n_tile == 256 && p.issue_split && room >= 24 * 1024 && (sums || mma < 12000)) p.block_cols = 64;

@@ -144,7 +144,7 @@ def test_tile_width_of_weight_gradients(ctx, shape, tile, kind):
 
 
 @pytest.mark.parametrize("shape,plain,sums", [((60, 32, 32, 608, 64, 3, 1), 0, 0), ((150, 32, 32, 224, 64, 3, 1), 0, 0), ((200, 32, 32, 160, 64, 3, 1), 32, 32),
-                                              ((500, 32, 32, 32, 64, 3, 1), 0, 32), ((300, 32, 32, 48, 64, 3, 1), 32, 32), ((500, 32, 32, 32, 64, 1, 1), 32, 32)],
+                                              ((500, 32, 32, 32, 64, 3, 1), 0, 32), ((300, 32, 32, 48, 64, 3, 1), 32, 32), ((500, 32, 32, 32, 64, 1, 1), 32, 32), ((4, 64, 64, 32, 64, 3, 1), 32, 32)],
                          ids=lambda v: "n{}h{}w{}c{}k{}r{}s{}".format(*v) if isinstance(v, tuple) else str(v))
 def test_blocks_where_the_mmas_hide_the_epilogue(ctx, shape, plain, sums):
     from paper_2503_23186_b200 import binding
